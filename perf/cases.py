@@ -159,7 +159,7 @@ def prepare(case, seed):
     more = {"step": c * case.get("steps", 0), "prefill": c, "generate": case.get("tokens", 0) + c,
             "request": (case.get("tokens", 0) + 1) * c + case.get("trigger", 0) + case.get("answer", 0)}[case["kind"]]
     dec = engine.Decoder(cfg, w, b, c, case["length"] + more + 8)
-    state = {"case": case, "dec": dec, "logits": dec.fc_debug_logits(True)}
+    state = {"case": case, "dec": dec, "weights": w, "logits": dec.fc_debug_logits(True)}
 
     def ids(*shape):
         return torch.randint(0, cfg.vocab, shape, generator=gen, device="cuda")
@@ -202,3 +202,105 @@ def run(state):
             out["answer"] = dec.fc_finish_with_trigger(state["trigger"], case["answer"])
     out["logits"] = state["logits"]
     return out
+
+class _Exact:
+    """The same model in 64 bits: K and V rounded to the model's type where they are stored, nothing else rounded."""
+
+    def __init__(self, cfg, w, kv):
+        self.cfg, self.w, self.kv = cfg, w, kv                       # kv [layers, 2, batch, kv heads, slots, head_dim]
+        self.rope = cfg.rope_theta ** (-torch.arange(0, cfg.head_dim, 2, dtype=torch.float64, device="cuda") / cfg.head_dim)
+
+    def _norm(self, x, gain):
+        return x * torch.rsqrt(x.square().mean(-1, keepdim=True) + self.cfg.rms_eps) * gain.double()
+
+    def _turn(self, t, pos):                                         # [rows, heads, head_dim]
+        a = (pos[:, None] * self.rope)[:, None]
+        x, y = t.chunk(2, -1)
+        return torch.cat([x * a.cos() - y * a.sin(), x * a.sin() + y * a.cos()], -1)
+
+    def forward(self, tokens, lens, head=True):
+        """tokens [n, c] behind lens[i] cached ones; the K/V of every row is stored; logits [n * c, vocab]."""
+        cfg, w = self.cfg, self.w
+        n, c = tokens.shape
+        hd, g = cfg.head_dim, cfg.n_heads // cfg.n_kv_heads
+        x = w["tok_emb"][tokens.reshape(-1)].double()
+        pos = torch.cat([torch.arange(m, m + c, device="cuda") for m in lens]).double()
+        for l in range(cfg.n_layers):
+            h = self._norm(x, w["g_attn"][l])
+            q, k, v = (h @ w[name][l].double().T for name in ("wq", "wk", "wv"))
+            q, k = self._turn(q.view(n * c, -1, hd), pos), self._turn(k.view(n * c, -1, hd), pos)
+            out = torch.empty_like(q)
+            for i, m in enumerate(lens):
+                at = slice(i * c, (i + 1) * c)
+                for half, t in enumerate((k, v.view(n * c, -1, hd))):
+                    self.kv[l, half, i, :, m:m + c] = t[at].transpose(0, 1).to(self.kv.dtype)
+                seen = torch.arange(m + c, device="cuda") <= torch.arange(m, m + c, device="cuda")[:, None]
+                for j in range(cfg.n_kv_heads):
+                    keys, values = self.kv[l, 0, i, j, :m + c].double(), self.kv[l, 1, i, j, :m + c].double()
+                    s = torch.einsum("rhd,kd->hrk", q[at, j * g:(j + 1) * g], keys) / math.sqrt(hd)
+                    p = s.masked_fill(~seen, -math.inf).softmax(-1)
+                    out[at, j * g:(j + 1) * g] = torch.einsum("hrk,kd->rhd", p, values)
+            x = x + out.reshape(n * c, -1) @ w["wo"][l].double().T
+            h = self._norm(x, w["g_ffn"][l])
+            h = torch.nn.functional.silu(h @ w["w_gate"][l].double().T) * (h @ w["w_up"][l].double().T)
+            x = x + h @ w["w_down"][l].double().T
+        if not head:
+            return None
+        logits = self._norm(x, w["g_final"]) @ w["lm_head"].double().T
+        logits[torch.arange(n * c, device="cuda"), w["bias_perm"].long()[tokens.reshape(-1)]] += cfg.bias_beta
+        return logits
+
+
+def exact(case, seed):
+    """Logits, and for a prompt the stored keys and values; the tokens are whole numbers and have no such value."""
+    if work(case)["flops"] > 1.2e14:                                 # over about 20 seconds in 64 bits
+        return None
+    state = prepare(case, seed)
+    cfg, w, kv, c, lens = state["dec"].cfg, state["weights"], state["dec"].kv_view(), case["c"], list(state["lens"])
+    n, model, logits = len(lens), _Exact(cfg, w, kv), state["logits"].double()
+    step = case["kind"] == "step"
+
+    def iterate(win, count):
+        made = [0] * n
+        for _ in range(count):
+            got = model.forward(win, lens)
+            logits[:len(got)] = got
+            best, new = got.view(n, c, -1).argmax(-1), win.clone()
+            for i in range(n):
+                k = 1
+                while k < c and int(win[i, k]) == int(best[i, k - 1]):
+                    k += 1
+                lens[i], made[i] = lens[i] + k, made[i] + k
+                new[i, :c - k + 1] = best[i, k - 1:]
+                for j in range(c - k + 1, c):
+                    new[i, j] = PAD if step else int(ids[i, (made[i] + j - 1) % size[i]])
+            win = new
+        return win, max(made)
+
+    if step:
+        iterate(torch.from_numpy(state["window"]).long().cuda(), case["steps"])
+        return {"logits": logits}
+    ids, size = state["prompts"], list(lens)
+    lens = [m - 1 for m in size]
+    for i, m in enumerate(lens):
+        sub = _Exact(cfg, w, kv[:, :, i:i + 1])
+        if m:
+            sub.forward(torch.from_numpy(ids[i:i + 1, :m]).long().cuda(), [0], head=False)
+    win = torch.tensor([[int(ids[i, m])] + [int(ids[i, (j - 1) % (m + 1)]) for j in range(1, c)] for i, m in enumerate(lens)],
+                       device="cuda")
+    if case["kind"] == "prefill":
+        iterate(win, 1)
+        return {"logits": logits, "kv": kv}
+    win, most = iterate(win, case["tokens"])
+    if case["kind"] == "generate":                                   # a sequence that is ahead ends, and its rows go
+        return {"logits": logits} if most == case["tokens"] else None
+    rest = torch.cat([win, torch.from_numpy(state["trigger"]).long().cuda().expand(n, -1)], 1)
+    if rest.shape[1] > 1:
+        model.forward(rest[:, :-1], lens, head=False)
+    lens = [m + rest.shape[1] - 1 for m in lens]
+    win = rest[:, -1:]
+    for _ in range(case["answer"]):
+        got = model.forward(win, lens)
+        logits[:n] = got
+        win, lens = got.argmax(-1)[:, None], [m + 1 for m in lens]
+    return {"logits": logits}
