@@ -53,7 +53,7 @@ struct Buffers {
 struct Dims {
   int rmax;        // rows of a decode step: max_batch * max_c
   int rows_ws;     // rows the activation buffers hold: a decode step or a prefill block, whichever is larger
-  int qd, kvd, ldq, nsplit_max, tk, pan_rows, pan_k, sync_words;
+  int qd, kvd, ldq, nsplit_max, tk, pan_rows, pan_k, sync_words, q_tiles;
   size_t esz;
 };
 
@@ -73,6 +73,7 @@ Dims dims_of(const fc_model_shape *s) {
   d.rmax = s->max_batch * s->max_c;
   d.rows_ws = d.rmax > kPrefillRows ? d.rmax : kPrefillRows;
   d.qd = s->n_heads * s->head_dim;
+  d.q_tiles = (int)attn_stream_q_tiles(d.rows_ws, s->n_heads / s->n_kv_heads, s->max_batch);
   d.kvd = s->n_kv_heads * s->head_dim;
   d.ldq = d.qd + 2 * d.kvd;
   d.tk = attn_tile_keys(s->dtype, s->head_dim);
@@ -97,7 +98,9 @@ size_t carve(const fc_model_shape *s, char *base, Buffers *b, std::vector<size_t
   c.guard();
   t.x = c.take<float>(R * s->d_model); c.guard();
   t.qkv = c.take<float>(R * d.ldq); c.guard();
-  t.qb = c.take<char>(R * d.qd * d.esz); c.guard();
+  // rotated queries: model dtype, or bf16 high + low in tiles of 16 queries per kv head
+  const size_t q_bytes = s->n_kv_heads * (size_t)d.q_tiles * 16 * s->head_dim * 4;
+  t.qb = c.take<char>(q_bytes > R * d.qd * d.esz ? q_bytes : R * d.qd * d.esz); c.guard();
   t.attn = c.take<float>(R * d.qd); c.guard();
   t.gu = c.take<float>(R * 2 * (size_t)s->d_ffn); c.guard();
   // sums of squares, then one group of synchronisation words per layer plus one for the first QKV and the LM head:
@@ -147,7 +150,9 @@ struct fc_ctx {
   bool cta_pairs;    // more than 64 rows: projections as clusters of two CTAs per 256-row weight tile
   bool chain;        // run O -> gate/up -> down -> next layer's QKV as one launch with grid barriers
   bool fused_attn;   // bf16 with head_dim 64/128: rotary embedding and K/V write happen inside the attention kernel
-  KvTensorMap kv_map; // TMA view of the whole K/V slab: (head_dim, max_seq, layers * 2 * max_batch * kv heads)
+  // TMA views of the whole K/V slab (head_dim, max_seq, layers * 2 * max_batch * kv heads), boxes of the tile size of each
+  // attention kernel
+  KvTensorMap kv_map, kv_map_stream;
   int n_sms;
   std::vector<UmmaPlan *> plan_qkv, plan_o, plan_gu, plan_down;
   std::vector<UmmaPlan *> plan_gu_half[2], plan_down_half[2];   // the FFN in two halves of d_ffn (chained launch, <= 16 rows)
@@ -367,9 +372,10 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
     if (rc == FC_OK && !(ctx->plan_head = umma_plan_create(args_head(ctx), PRO_GAIN, EPI_ARGMAX, ctx->n_sms, ctx->b.err, msg, sizeof msg))) rc = FC_ERR_CUDA;
     if (rc != FC_OK) { fprintf(stderr, "fc_init: %s\n", msg); return fail(rc); }
   }
+  const long long kv_planes = (long long)L * 2 * shape->max_batch * shape->n_kv_heads;
   if (ctx->fused_attn &&
-      make_kv_tensor_map(&ctx->kv_map, kv, shape->head_dim, shape->max_seq,
-                         (long long)L * 2 * shape->max_batch * shape->n_kv_heads) != cudaSuccess) {
+      (make_kv_tensor_map(&ctx->kv_map, kv, shape->head_dim, shape->max_seq, kv_planes, attn_fused_tile_keys()) != cudaSuccess ||
+       make_kv_tensor_map(&ctx->kv_map_stream, kv, shape->head_dim, shape->max_seq, kv_planes, attn_stream_tile_keys()) != cudaSuccess)) {
     fprintf(stderr, "fc_init: tensor map over the K/V slab could not be encoded\n");
     return fail(FC_ERR_CUDA);
   }
@@ -462,12 +468,30 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
   const long long stride_b = (long long)s.n_kv_heads * stride_h;
   const bool chained = ctx->chain;
   const bool o_panel = chained && ctx->fused_attn && R > 16 && ctx->d.pan_rows >= R;
+  const bool stream = with_head && ctx->fused_attn && attn_stream_pays(max_len_host, rows, s.n_heads, s.n_kv_heads, nb);
   for (int l = 0; l < s.n_layers; ++l) {
     if (!chained || l == 0)
       FC_CK(run_gemm(ctx, ctx->use_umma ? ctx->plan_qkv[l] : nullptr, args_qkv(ctx, l), R, PRO_GAIN, EPI_ATOMIC_ADD, FC_CLS_QKV, claim_word(ctx, l, GEMM_QKV)));
     void *kc = ctx->kv + (size_t)l * ctx->kv_layer_stride;
     void *vc = ctx->kv + (size_t)l * ctx->kv_layer_stride + ctx->kv_half_stride;
-    if (ctx->fused_attn) {
+    if (stream) {
+      QkvFinishArgs qa; memset(&qa, 0, sizeof qa);
+      qa.qkv = ctx->b.qkv; qa.ldq = d.ldq; qa.ss = ctx->b.ss_attn; qa.eps = s.rms_eps; qa.dn = s.d_model; qa.rope = ctx->b.rope;
+      qa.kv_len = ctx->b.kv_len; qa.segs.b0 = b0; qa.segs.c = rows; qa.segs.seq_map = seq_map;
+      qa.hq = s.n_heads; qa.hkv = s.n_kv_heads; qa.hd = s.head_dim; qa.q = ctx->b.qb; qa.q_tiles = d.q_tiles;
+      qa.kcache = kc; qa.vcache = vc; qa.stride_b = stride_b; qa.stride_h = stride_h; qa.pdl = ctx->pdl && !ctx->prof;
+      qa.z.p[0] = ctx->b.gu; qa.z.n[0] = Rz * 2 * s.d_ffn;
+      qa.z.p[1] = ctx->b.ss_ffn; qa.z.n[1] = Rz;
+      ++ctx->launches;
+      { ProfScope ps(ctx, FC_CLS_ROPE); FC_CK(launch_qkv_finish(qa, R, ctx->st)); }
+      StreamAttnArgs sa; memset(&sa, 0, sizeof sa);
+      sa.q = ctx->b.qb; sa.q_tiles = d.q_tiles; sa.kv_len = ctx->b.kv_len; sa.segs = qa.segs; sa.hq = s.n_heads; sa.hkv = s.n_kv_heads;
+      sa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; sa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
+      sa.err = ctx->b.err; sa.out = ctx->b.attn; sa.pdl = ctx->pdl && !ctx->prof;
+      if (o_panel) { sa.out_pan = ctx->b.pan; sa.pan_rows = d.pan_rows; }
+      ++ctx->launches;
+      { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_stream(ctx->kv_map_stream, sa, nb, rows, max_len_host, s.head_dim, ctx->n_sms, ctx->st)); }
+    } else if (ctx->fused_attn) {
       FusedAttnArgs fa; memset(&fa, 0, sizeof fa);
       fa.qkv = ctx->b.qkv; fa.ldq = d.ldq; fa.ss = ctx->b.ss_attn; fa.eps = s.rms_eps; fa.dn = s.d_model;
       fa.rope = ctx->b.rope; fa.c_magic = (unsigned int)((0x100000000ull + (unsigned)rows - 1) / (unsigned)rows);
@@ -1167,8 +1191,8 @@ extern "C" int fc_op_fused_window_attention(float *qkv_acc, float *sumsq, float 
     return FC_ERR_CUDA;
   KvTensorMap kmap, vmap;
   const long long planes = (long long)batch * n_kv_heads;
-  if (make_kv_tensor_map(&kmap, kcache, head_dim, max_seq, planes) != cudaSuccess ||
-      make_kv_tensor_map(&vmap, vcache, head_dim, max_seq, planes) != cudaSuccess) return FC_ERR_CUDA;
+  if (make_kv_tensor_map(&kmap, kcache, head_dim, max_seq, planes, attn_fused_tile_keys()) != cudaSuccess ||
+      make_kv_tensor_map(&vmap, vcache, head_dim, max_seq, planes, attn_fused_tile_keys()) != cudaSuccess) return FC_ERR_CUDA;
   FusedAttnArgs fa; memset(&fa, 0, sizeof fa);
   fa.qkv = qkv_acc; fa.ldq = (n_heads + 2 * n_kv_heads) * head_dim; fa.ss = sumsq; fa.eps = rms_eps; fa.dn = d_norm;
   fa.rope = (const float2 *)(base + off[0]);

@@ -119,6 +119,47 @@ struct FusedAttnArgs {   // bf16: rotary embedding + K/V write + window attentio
   ZeroList z;
 };
 
+// The rows of a forward as runs of consecutive positions of one sequence each.  n == 0: every sequence has c rows, row
+// block i belongs to sequence seq_map[i] (null: b0 + i).  n > 0: segment i is rows row0[i] .. row0[i + 1) of sequence
+// seq[i].  Position of a row: kv_len[sequence] + its index in the run.
+constexpr int kMaxSegs = 64;
+struct RowSegs {
+  int n, b0, c;
+  const int32_t *seq_map;
+  int seq[kMaxSegs], row0[kMaxSegs + 1];
+};
+
+struct QkvFinishArgs {    // bf16: QKV accumulators -> rotated queries (high + low) and K/V rows in the cache
+  const float *qkv;       // [R, ldq] fp32 accumulators (q | k | v) lacking 1/rms; read only
+  int ldq;
+  const float *ss;        // [R] sums of squares for 1/rms
+  float eps; int dn;
+  const float2 *rope;     // [max_seq][hd/2] (cos, sin)
+  const int32_t *kv_len;
+  RowSegs segs;
+  int hq, hkv, hd;
+  void *q;                // bf16 high + low in MMA operand order, q_tiles tiles of 16 queries per kv head
+  int q_tiles;
+  void *kcache, *vcache;  // layer base
+  long long stride_b, stride_h;
+  int pdl;
+  ZeroList z;
+};
+
+struct StreamAttnArgs {   // bf16: window attention over rows whose K/V are in the cache
+  const void *q;          // as written by qkv_finish_kernel
+  int q_tiles;
+  const int32_t *kv_len;
+  RowSegs segs;
+  int hq, hkv;
+  int k_plane0, v_plane0; // as in FusedAttnArgs
+  unsigned int *err;
+  float *out;             // [R, hq * hd] fp32, or
+  void *out_pan;          // the bf16 pair [2][pan_rows][hq * hd]
+  int pan_rows;
+  int pdl;
+};
+
 struct AcceptArgs {
   int32_t *window;                 // [batch, c] in/out
   const unsigned long long *amax;  // packed argmax per row, or null
@@ -161,7 +202,16 @@ cudaError_t launch_rope_kv(const RopeArgs &a, int dtype, cudaStream_t st);
 cudaError_t launch_attn(const AttnArgs &a, int dtype, int hd, cudaStream_t st);
 cudaError_t launch_attn_fused(const KvTensorMap &kmap, const KvTensorMap &vmap, const FusedAttnArgs &a, int hd, cudaStream_t st);
 // 3-d tensor map (head_dim, max_seq, planes) over bf16 K or V planes laid out [plane][max_seq][head_dim] from `base`.
-cudaError_t make_kv_tensor_map(KvTensorMap *out, const void *base, int hd, int max_seq, long long planes);
+// box_keys: keys per box.
+cudaError_t make_kv_tensor_map(KvTensorMap *out, const void *base, int hd, int max_seq, long long planes, int box_keys);
+cudaError_t launch_qkv_finish(const QkvFinishArgs &a, int R, cudaStream_t st);
+// map: boxes of attn_stream_tile_keys() keys; max_rows / max_len: the longest segment and (a bound on) the longest cache
+cudaError_t launch_attn_stream(const KvTensorMap &map, const StreamAttnArgs &a, int nseg, int max_rows, int max_len, int hd,
+                               int n_sms, cudaStream_t st);
+bool attn_stream_pays(int max_len, int c, int hq, int hkv, int nb);
+int attn_stream_tile_keys();
+size_t attn_stream_q_tiles(int rows, int group, int nseg);      // tiles per kv head for `rows` rows in nseg segments
+int attn_fused_tile_keys();
 // Grid of the fused attention kernel: splits per (sequence, kv head, query-tile group) and query tiles per CTA.
 void fused_attn_plan(int max_len, int c, int hq, int hkv, int nb, int hd, int n_sms, int &nsplit, int &qt);
 int attn_fused_max_rows();   // most window rows per sequence the fused kernel takes in one launch

@@ -626,7 +626,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-cudaError_t make_kv_tensor_map(KvTensorMap *out, const void *base, int hd, int max_seq, long long planes) {
+cudaError_t make_kv_tensor_map(KvTensorMap *out, const void *base, int hd, int max_seq, long long planes, int box_keys) {
   static_assert(sizeof(CUtensorMap) <= sizeof(KvTensorMap), "tensor map storage");
   static EncodeTiledFn enc = nullptr;
   if (!enc) {
@@ -639,7 +639,7 @@ cudaError_t make_kv_tensor_map(KvTensorMap *out, const void *base, int hd, int m
   if ((hd != 64 && hd != 128) || max_seq < 1 || planes < 1 || ((uintptr_t)base & 15)) return cudaErrorInvalidValue;
   cuuint64_t gdim[3] = {(cuuint64_t)hd, (cuuint64_t)max_seq, (cuuint64_t)planes};
   cuuint64_t gstr[2] = {(cuuint64_t)hd * 2, (cuuint64_t)max_seq * hd * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)kTK, 1};
+  cuuint32_t box[3] = {64, (cuuint32_t)box_keys, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(reinterpret_cast<CUtensorMap *>(out), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), gdim,
                    gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -737,5 +737,6 @@ cudaError_t launch_attn_fused(const KvTensorMap &kmap, const KvTensorMap &vmap, 
 }
 
 int attn_fused_max_rows() { return 2 * kTK; }
+int attn_fused_tile_keys() { return kTK; }
 
 }  // namespace fc
