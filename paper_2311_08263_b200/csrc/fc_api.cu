@@ -33,16 +33,20 @@ struct Carver {          // hands out aligned slices of the caller's workspace (
 };
 
 constexpr int kPrefillRows = 128;         // rows per forward while a prompt is cached (one 128-row accumulator block)
-
+constexpr int kBulkRows = 1024;           // the same where the dense GEMMs of k_bulk.cu run
+// Rows from which they run.  Measured, 4 layers of 7B, chained launch against this: 64 rows 649 us, 767; 96 rows 763, 817;
+// 128 rows 857, 860; 256 rows 1250, 1171; 512 rows 2130, 1936.
+constexpr int kBulkMin = 129;
 
 constexpr int kSyncClaim = kChainMax, kSyncPanel = 2 * kChainMax, kSyncTd = 3 * kChainMax;   // offsets in a group
 
 struct Buffers {
   float *x, *qkv, *attn, *gu, *ss_attn, *ss_ffn, *ss_final, *part_o, *part_ml;
-  void *pan;
+  void *pan, *pan_ffn;     // activation pairs; pan_ffn: the down projection's operand where the dense GEMMs run
   float2 *rope;
   void *qb;
-  unsigned int *counters, *err, *chain_bar;
+  unsigned int *counters, *err, *chain_bar, *bulk_arrived;
+  char *bulk_slots;
   unsigned long long *amax;
   int32_t *window, *kv_len, *n_gen, *done, *acc_count, *acc_tokens, *prompt, *prompt_lens, *out_tokens;
   int32_t *row_tokens;     // tokens of a forward that is not a plain decode step (answer-trigger context; the windows of
@@ -53,7 +57,9 @@ struct Buffers {
 struct Dims {
   int rmax;        // rows of a decode step: max_batch * max_c
   int rows_ws;     // rows the activation buffers hold: a decode step or a prefill block, whichever is larger
-  int qd, kvd, ldq, nsplit_max, tk, pan_rows, pan_k, sync_words, q_tiles;
+  int qd, kvd, ldq, nsplit_max, tk, pan_rows, bulk_rows, pan_k, sync_words, q_tiles;
+  bool bulk;       // the shape takes the dense GEMMs from kBulkMin rows
+  int rows_chain;  // rows the buffers of the chained launch hold
   size_t esz;
 };
 
@@ -68,10 +74,25 @@ bool shape_ok(const fc_model_shape *s) {
   return true;
 }
 
+// bf16 on the tensor cores with head_dim 64 / 128 and every weight matrix a whole number of 256-row tiles
+bool bulk_shape(const fc_model_shape *s) {
+  const int off = FC_FLAG_SIMT_GEMM | FC_FLAG_NO_CHAIN | FC_FLAG_NO_CTA_PAIRS;
+  return s->dtype == FC_BF16 && !(s->flags & off) && (s->head_dim == 64 || s->head_dim == 128) && s->d_model % 256 == 0 &&
+         s->d_ffn % 256 == 0 && s->n_heads * s->head_dim % 256 == 0 && s->n_kv_heads * s->head_dim % 256 == 0 && s->vocab % 256 == 0;
+}
+
 Dims dims_of(const fc_model_shape *s) {
   Dims d;
   d.rmax = s->max_batch * s->max_c;
   d.rows_ws = d.rmax > kPrefillRows ? d.rmax : kPrefillRows;
+  d.rows_chain = d.rows_ws;
+  d.bulk = bulk_shape(s);
+  if (d.bulk) {
+    d.rows_chain = kPrefillRows;
+    const long long all = ((long long)s->max_batch * s->max_seq + 127) / 128 * 128;       // no prompt block is larger
+    const int blk = all < kBulkRows ? (int)all : kBulkRows;
+    if (d.rows_ws < blk) d.rows_ws = blk;
+  }
   d.qd = s->n_heads * s->head_dim;
   d.q_tiles = (int)attn_stream_q_tiles(d.rows_ws, s->n_heads / s->n_kv_heads, s->max_batch);
   d.kvd = s->n_kv_heads * s->head_dim;
@@ -80,7 +101,8 @@ Dims dims_of(const fc_model_shape *s) {
   d.nsplit_max = (s->max_seq + d.tk - 1) / d.tk;
   d.esz = s->dtype == FC_F32 ? 4 : 2;
   // beyond 16 rows the tensor-core projections read their activations from a bf16 high/low panel
-  d.pan_rows = (d.rows_ws + 127) / 128 * 128;
+  d.pan_rows = (d.rows_chain + 127) / 128 * 128;
+  d.bulk_rows = (d.rows_ws + 127) / 128 * 128;
   d.pan_k = s->d_model > s->d_ffn ? s->d_model : s->d_ffn;
   if (d.qd > d.pan_k) d.pan_k = d.qd;
   // per-layer group of synchronisation words: grid barriers 0..5, work-claim counters 6..11, panel-ready barriers
@@ -94,24 +116,31 @@ size_t carve(const fc_model_shape *s, char *base, Buffers *b, std::vector<size_t
   Dims d = dims_of(s);
   Carver c{base, 0, guards};
   Buffers t;
-  const size_t R = d.rows_ws, Rs = d.rmax;
+  const size_t R = d.rows_ws, Rc = d.rows_chain, Rs = d.rmax;
   c.guard();
   t.x = c.take<float>(R * s->d_model); c.guard();
   t.qkv = c.take<float>(R * d.ldq); c.guard();
   // rotated queries: model dtype, or bf16 high + low in tiles of 16 queries per kv head
   const size_t q_bytes = s->n_kv_heads * (size_t)d.q_tiles * 16 * s->head_dim * 4;
   t.qb = c.take<char>(q_bytes > R * d.qd * d.esz ? q_bytes : R * d.qd * d.esz); c.guard();
-  t.attn = c.take<float>(R * d.qd); c.guard();
-  t.gu = c.take<float>(R * 2 * (size_t)s->d_ffn); c.guard();
+  t.attn = c.take<float>(Rc * d.qd); c.guard();
+  t.gu = c.take<float>(Rc * 2 * (size_t)s->d_ffn); c.guard();
   // sums of squares, then one group of synchronisation words per layer plus one for the first QKV and the LM head:
   // adjacent (no canary band in between) so that one pass clears them all
   t.ss_attn = c.take<float>(R);
   t.ss_ffn = c.take<float>(R);
   t.ss_final = c.take<float>(R);
   t.chain_bar = c.take<unsigned int>(((size_t)s->n_layers + 1) * d.sync_words); c.guard();
-  t.pan = c.take<char>((size_t)2 * d.pan_rows * d.pan_k * 2); c.guard();
-  t.part_o = c.take<float>(R * s->n_heads * (size_t)d.nsplit_max * s->head_dim); c.guard();
-  t.part_ml = c.take<float>(R * s->n_heads * (size_t)d.nsplit_max * 2); c.guard();
+  const size_t pan_chain = (size_t)2 * d.pan_rows * d.pan_k * 2;
+  const size_t pan_bulk = d.bulk ? (size_t)2 * d.bulk_rows * (s->d_model > d.qd ? s->d_model : d.qd) * 2 : 0;
+  t.pan = c.take<char>(pan_chain > pan_bulk ? pan_chain : pan_bulk); c.guard();
+  t.pan_ffn = c.take<char>(d.bulk ? (size_t)2 * d.bulk_rows * s->d_ffn * 2 : 0); c.guard();
+  t.bulk_slots = c.take<char>(d.bulk ? bulk_slot_bytes() : 0); c.guard();
+  t.bulk_arrived = c.take<unsigned int>(d.bulk ? kBulkArrived : 0); c.guard();
+  // split-KV partials of the FMA attention kernel
+  const size_t Rp = d.bulk ? 0 : R;
+  t.part_o = c.take<float>(Rp * s->n_heads * (size_t)d.nsplit_max * s->head_dim); c.guard();
+  t.part_ml = c.take<float>(Rp * s->n_heads * (size_t)d.nsplit_max * 2); c.guard();
   t.rope = c.take<float2>((size_t)s->max_seq * (s->head_dim / 2)); c.guard();
   t.counters = c.take<unsigned int>((size_t)s->max_batch * s->n_kv_heads + 1);   // + one grid-wide word
   t.err = c.take<unsigned int>(1);
@@ -130,8 +159,6 @@ size_t carve(const fc_model_shape *s, char *base, Buffers *b, std::vector<size_t
   if (b) *b = t;
   return c.off;
 }
-
-__global__ void bump_kernel(int32_t *v, int n) { if (threadIdx.x == 0 && blockIdx.x == 0) *v += n; }
 
 }  // namespace
 
@@ -444,6 +471,85 @@ static cudaError_t run_gemm(fc_ctx *ctx, const UmmaPlan *plan, GemmArgs a, int R
   return launch_gemm_simt(a, ctx->s.dtype, pro, epi, ctx->st);
 }
 
+static int run_accept(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *seq_map, int commit) {
+  const fc_model_shape &s = ctx->s;
+  AcceptArgs ac; memset(&ac, 0, sizeof ac);
+  ac.window = ctx->b.window; ac.amax = ctx->b.amax; ac.amax_clear = ctx->b.amax;
+  ac.kv_len = ctx->b.kv_len; ac.n_gen = ctx->b.n_gen; ac.done = ctx->b.done;
+  ac.accepted_count = ctx->b.acc_count; ac.accepted_tokens = ctx->b.acc_tokens;
+  ac.prompt = ctx->b.prompt; ac.prompt_lens = ctx->b.prompt_lens;
+  ac.out_tokens = ctx->b.out_tokens; ac.out_stride = s.max_seq;
+  ac.b0 = b0; ac.nb = nb; ac.c = rows; ac.p_stride = s.max_seq; ac.refill = ctx->refill; ac.pad_id = ctx->pad_id;
+  ac.seq_map = seq_map;
+  ac.max_tokens = ctx->gen_max_tokens; ac.eos_id = ctx->gen_eos; ac.commit = commit;
+  if (ctx->inject_timeout) { ac.err_inject = ctx->b.err; ctx->inject_timeout = false; }
+  ++ctx->launches;
+  ProfScope ps(ctx, FC_CLS_ACCEPT);
+  FC_CK(launch_accept(ac, ctx->st));
+  return FC_OK;
+}
+
+// A forward of many rows: one dense GEMM per projection, the attention over the cache that already holds the rows' K/V.
+// segs / nseg: which rows belong to which sequence; max_rows, max_len: the longest segment, a bound on the longest cache.
+// tokens: [R], or [sequence][max_seq] with segs.n > 0.  Every buffer is written before it is read: nothing to clear.
+static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int max_rows, int max_len, const int32_t *tokens, bool with_head) {
+  const fc_model_shape &s = ctx->s;
+  const Dims &d = ctx->d;
+  const int pdl = ctx->pdl && !ctx->prof;
+  EmbedArgs ea; memset(&ea, 0, sizeof ea);
+  ea.tokens = tokens; ea.emb = ctx->tok_emb; ea.x = ctx->b.x; ea.R = R; ea.d = s.d_model;
+  if (segs.n > 0) { ea.segs = segs; ea.kv_len = ctx->b.kv_len; ea.t_stride = s.max_seq; }
+  ++ctx->launches;
+  { ProfScope ps(ctx, FC_CLS_EMBED); FC_CK(launch_embed(ea, s.dtype, ctx->st)); }
+  BulkArgs ba; memset(&ba, 0, sizeof ba);
+  ba.slots = ctx->b.bulk_slots; ba.arrived = ctx->b.bulk_arrived;
+  ba.pan_rows = d.bulk_rows; ba.R = R; ba.eps = s.rms_eps; ba.dn = s.d_model;
+  const long long stride_h = (long long)s.max_seq * s.head_dim, stride_b = (long long)s.n_kv_heads * stride_h;
+  auto norm = [&](const void *gain, float *ss, int cls) {
+    ProfScope ps(ctx, cls);
+    ++ctx->launches;
+    return launch_norm_pair(ctx->b.x, gain, ss, ctx->b.pan, d.bulk_rows, R, s.d_model, pdl, ctx->st);
+  };
+  auto gemm = [&](const UmmaPlan *plan, int epi, int cls) {
+    ProfScope ps(ctx, cls);
+    ++ctx->launches;
+    return launch_bulk_gemm(plan, ba, epi, ctx->n_sms, pdl, ctx->st);
+  };
+  for (int l = 0; l < s.n_layers; ++l) {
+    FC_CK(norm(ctx->g_attn[l], ctx->b.ss_attn, FC_CLS_EMBED));
+    ba.pan = ctx->b.pan; ba.y = ctx->b.qkv; ba.ldy = d.ldq;
+    FC_CK(gemm(ctx->plan_qkv[l], BULK_STORE, FC_CLS_QKV));
+    QkvFinishArgs qa; memset(&qa, 0, sizeof qa);
+    qa.qkv = ctx->b.qkv; qa.ldq = d.ldq; qa.ss = ctx->b.ss_attn; qa.eps = s.rms_eps; qa.dn = s.d_model; qa.rope = ctx->b.rope;
+    qa.kv_len = ctx->b.kv_len; qa.segs = segs; qa.hq = s.n_heads; qa.hkv = s.n_kv_heads; qa.hd = s.head_dim;
+    qa.q = ctx->b.qb; qa.q_tiles = d.q_tiles;
+    qa.kcache = ctx->kv + (size_t)l * ctx->kv_layer_stride; qa.vcache = (char *)qa.kcache + ctx->kv_half_stride;
+    qa.stride_b = stride_b; qa.stride_h = stride_h; qa.pdl = pdl;
+    ++ctx->launches;
+    { ProfScope ps(ctx, FC_CLS_ROPE); FC_CK(launch_qkv_finish(qa, R, ctx->st)); }
+    StreamAttnArgs sa; memset(&sa, 0, sizeof sa);
+    sa.q = ctx->b.qb; sa.q_tiles = d.q_tiles; sa.kv_len = ctx->b.kv_len; sa.segs = segs; sa.hq = s.n_heads; sa.hkv = s.n_kv_heads;
+    sa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; sa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
+    sa.err = ctx->b.err; sa.out_pan = ctx->b.pan; sa.pan_rows = d.bulk_rows; sa.pdl = pdl;
+    ++ctx->launches;
+    { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_stream(ctx->kv_map_stream, sa, nseg, max_rows, max_len, s.head_dim, ctx->n_sms, ctx->st)); }
+    ba.y = ctx->b.x; ba.ldy = s.d_model;
+    FC_CK(gemm(ctx->plan_o[l], BULK_ADD, FC_CLS_OPROJ));
+    FC_CK(norm(ctx->g_ffn[l], ctx->b.ss_ffn, FC_CLS_EMBED));
+    ba.ss = ctx->b.ss_ffn; ba.out_pan = ctx->b.pan_ffn;
+    FC_CK(gemm(ctx->plan_gu[l], BULK_SWIGLU, FC_CLS_GATEUP));
+    ba.pan = ctx->b.pan_ffn;
+    FC_CK(gemm(ctx->plan_down[l], BULK_ADD, FC_CLS_DOWN));
+  }
+  if (with_head) {
+    FC_CK(norm(ctx->g_final, ctx->b.ss_final, FC_CLS_HEAD));
+    ba.pan = ctx->b.pan; ba.ss = ctx->b.ss_final; ba.tokens = tokens; ba.amax = ctx->b.amax; ba.logits = ctx->dbg_logits;
+    ba.perm = s.bias_beta != 0.f ? ctx->bias_perm : nullptr; ba.beta = s.bias_beta;
+    FC_CK(gemm(ctx->plan_head, BULK_HEAD, FC_CLS_HEAD));
+  }
+  return FC_OK;
+}
+
 // One decoder forward over nb sequences (b0 .. b0+nb-1) with `rows` rows each.  tokens: device [nb*rows].
 // with_head: LM head + argmax + accept (a decode step); otherwise the rows are committed (prefill chunk).
 // seq_map (device, optional): row block i belongs to sequence seq_map[i] instead of b0 + i (finished sequences skipped).
@@ -452,6 +558,16 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
   const fc_model_shape &s = ctx->s;
   const Dims &d = ctx->d;
   const int R = nb * rows;
+  RowSegs segs; memset(&segs, 0, sizeof segs);
+  segs.b0 = b0; segs.c = rows; segs.seq_map = seq_map;
+  if (ctx->d.bulk && R >= kBulkMin) {
+    int rc = forward_bulk(ctx, segs, nb, R, rows, max_len_host, tokens, with_head);
+    if (rc != FC_OK) return rc;
+    if (with_head) return run_accept(ctx, b0, nb, rows, seq_map, commit);
+    ++ctx->launches;
+    FC_CK(launch_advance(ctx->b.kv_len, segs, nb, ctx->st));
+    return FC_OK;
+  }
   const size_t Rz = R;
   EmbedArgs ea; memset(&ea, 0, sizeof ea);
   ea.tokens = tokens; ea.emb = ctx->tok_emb; ea.x = ctx->b.x; ea.R = R; ea.d = s.d_model;
@@ -477,7 +593,7 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
     if (stream) {
       QkvFinishArgs qa; memset(&qa, 0, sizeof qa);
       qa.qkv = ctx->b.qkv; qa.ldq = d.ldq; qa.ss = ctx->b.ss_attn; qa.eps = s.rms_eps; qa.dn = s.d_model; qa.rope = ctx->b.rope;
-      qa.kv_len = ctx->b.kv_len; qa.segs.b0 = b0; qa.segs.c = rows; qa.segs.seq_map = seq_map;
+      qa.kv_len = ctx->b.kv_len; qa.segs = segs;
       qa.hq = s.n_heads; qa.hkv = s.n_kv_heads; qa.hd = s.head_dim; qa.q = ctx->b.qb; qa.q_tiles = d.q_tiles;
       qa.kcache = kc; qa.vcache = vc; qa.stride_b = stride_b; qa.stride_h = stride_h; qa.pdl = ctx->pdl && !ctx->prof;
       qa.z.p[0] = ctx->b.gu; qa.z.n[0] = Rz * 2 * s.d_ffn;
@@ -576,34 +692,26 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
     GemmArgs ha = args_head(ctx);
     ha.tokens = tokens;
     FC_CK(run_gemm(ctx, ctx->plan_head, ha, R, PRO_GAIN, EPI_ARGMAX, FC_CLS_HEAD, claim_word(ctx, 0, GEMM_HEAD)));
-    AcceptArgs ac; memset(&ac, 0, sizeof ac);
-    ac.window = ctx->b.window; ac.amax = ctx->b.amax; ac.amax_clear = ctx->b.amax;
-    ac.kv_len = ctx->b.kv_len; ac.n_gen = ctx->b.n_gen; ac.done = ctx->b.done;
-    ac.accepted_count = ctx->b.acc_count; ac.accepted_tokens = ctx->b.acc_tokens;
-    ac.prompt = ctx->b.prompt; ac.prompt_lens = ctx->b.prompt_lens;
-    ac.out_tokens = ctx->b.out_tokens; ac.out_stride = s.max_seq;
-    ac.b0 = b0; ac.nb = nb; ac.c = rows; ac.p_stride = s.max_seq; ac.refill = ctx->refill; ac.pad_id = ctx->pad_id;
-    ac.seq_map = seq_map;
-    ac.max_tokens = ctx->gen_max_tokens; ac.eos_id = ctx->gen_eos; ac.commit = commit;
-    if (ctx->inject_timeout) { ac.err_inject = ctx->b.err; ctx->inject_timeout = false; }
-    ++ctx->launches;
-    { ProfScope ps(ctx, FC_CLS_ACCEPT); FC_CK(launch_accept(ac, ctx->st)); }
-  } else {
-    for (int b = b0; b < b0 + nb; ++b) {
-      ++ctx->launches;
-      bump_kernel<<<1, 32, 0, ctx->st>>>(ctx->b.kv_len + b, rows);
-      FC_CK(cudaGetLastError());
-    }
+    return run_accept(ctx, b0, nb, rows, seq_map, commit);
   }
+  ++ctx->launches;
+  FC_CK(launch_advance(ctx->b.kv_len, segs, nb, ctx->st));
   return FC_OK;
 }
 
 // Rows of one forward while tokens are only cached (prompt, answer-trigger context): what the activation buffers
 // hold, and no more than the fused attention kernel takes as one window.
 static int block_rows(const fc_ctx *ctx) {
-  int r = ctx->d.rows_ws;
+  int r = ctx->d.rows_chain;
   if (ctx->fused_attn && r > attn_fused_max_rows()) r = attn_fused_max_rows();
   return r;
+}
+
+// After a bounded wait gave up: the sequences are lost, the words that launches leave at zero may not be.
+static void clear_device_error(fc_ctx *ctx) {
+  cudaMemsetAsync(ctx->b.err, 0, sizeof(unsigned int), ctx->st);
+  if (ctx->d.bulk) cudaMemsetAsync(ctx->b.bulk_arrived, 0, kBulkArrived * sizeof(unsigned int), ctx->st);
+  ctx->ready = false;
 }
 
 static int check_device_error(fc_ctx *ctx) {
@@ -612,10 +720,42 @@ static int check_device_error(fc_ctx *ctx) {
   FC_CK(cudaStreamSynchronize(ctx->st));
   e = (unsigned int)ctx->pin[0];
   if (e) {
-    cudaMemsetAsync(ctx->b.err, 0, sizeof(e), ctx->st);
-    ctx->ready = false;
+    clear_device_error(ctx);
     return FC_ERR_DEVICE_TIMEOUT;
   }
+  return FC_OK;
+}
+
+// The prompts of a batch one behind the other (n_all rows), cut into as few blocks as the buffers allow, of nearly equal
+// size and, but for the last, whole 128-row tiles.
+static int prefill_packed(fc_ctx *ctx, int batch, const int32_t *prompt_lens, long long n_all) {
+  const long long n_blk = (n_all + ctx->d.bulk_rows - 1) / ctx->d.bulk_rows;
+  int b = 0, at = 0, blk_no = 0;                                      // next row: id `at` of prompt b
+  while (b < batch) {
+    RowSegs segs; memset(&segs, 0, sizeof segs);
+    int R = 0, max_rows = 0, max_len = 0;
+    const long long tiles = (n_all + 127) / 128;           // block i: tiles [i * tiles / n_blk, (i + 1) * tiles / n_blk)
+    const int blk = blk_no < n_blk ? (int)((blk_no + 1) * tiles / n_blk - blk_no * tiles / n_blk) * 128 : ctx->d.bulk_rows;
+    ++blk_no;
+    while (b < batch && R < blk && segs.n < kMaxSegs) {
+      const int n = prompt_lens[b] - 1 - at;
+      const int take = n < blk - R ? n : blk - R;
+      if (take > 0) {
+        segs.seq[segs.n] = b; segs.row0[segs.n] = R;
+        if (take > max_rows) max_rows = take;
+        if (at > max_len) max_len = at;
+        R += take; at += take;
+        segs.row0[++segs.n] = R;
+      }
+      if (at >= prompt_lens[b] - 1) { ++b; at = 0; }
+    }
+    if (R == 0) break;
+    int rc = forward_bulk(ctx, segs, segs.n, R, max_rows, max_len, ctx->b.prompt, false);
+    if (rc != FC_OK) return rc;
+    ++ctx->launches;
+    FC_CK(launch_advance(ctx->b.kv_len, segs, segs.n, ctx->st));
+  }
+  for (int i = 0; i < batch; ++i) ctx->kv_len_h[i] = prompt_lens[i] - 1;
   return FC_OK;
 }
 
@@ -660,7 +800,14 @@ extern "C" int fc_prefill(fc_ctx *ctx, int32_t batch, const int32_t *prompt_ids,
   // K/V of prompt[0 .. P-2]: one sequence at a time, in blocks of as many rows as the activation buffers hold
   // (at least one 128-row accumulator block, so that a prompt of P ids streams the weights ~P / 128 times)
   FC_CK(cudaEventRecord(ctx->ev0, ctx->st));
-  for (int b = 0; b < batch; ++b) {
+  long long n_all = 0;
+  for (int b = 0; b < batch; ++b) n_all += prompt_lens[b] - 1;
+  if (ctx->d.bulk && n_all >= kBulkMin) {
+    int rc = prefill_packed(ctx, batch, prompt_lens, n_all);
+    if (rc != FC_OK) return rc;
+    n_all = 0;
+  }
+  for (int b = 0; b < batch && n_all > 0; ++b) {
     const int n = prompt_lens[b] - 1;
     const int blk = block_rows(ctx);
     for (int start = 0; start < n; start += blk) {
@@ -688,8 +835,7 @@ static int collect_step(fc_ctx *ctx, int32_t *accepted_count, int32_t *accepted_
   FC_CK(cudaMemcpyAsync(p_err, ctx->b.err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->st));
   FC_CK(cudaStreamSynchronize(ctx->st));
   if (*p_err) {
-    cudaMemsetAsync(ctx->b.err, 0, sizeof(int32_t), ctx->st);
-    ctx->ready = false;
+    clear_device_error(ctx);
     return FC_ERR_DEVICE_TIMEOUT;
   }
   for (int b = 0; b < B; ++b) {

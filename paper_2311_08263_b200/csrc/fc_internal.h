@@ -1,5 +1,6 @@
 // Internal declarations shared by the CUDA sources of the Jacobi-window decode library.
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -179,7 +180,10 @@ struct AcceptArgs {
 };
 
 struct EmbedArgs {
-  const int32_t *tokens;   // [R]
+  const int32_t *tokens;   // [R], or with segs.n > 0 [sequence][t_stride]: row j of a segment is token kv_len[sequence] + j
+  RowSegs segs;
+  const int32_t *kv_len;
+  int t_stride;
   const void *emb;         // [vocab, d]
   float *x;                // [R, d]
   int R, d;
@@ -239,6 +243,37 @@ void umma_plan_destroy(UmmaPlan *p);
 // CTAs that share a tile (tcgen05 cta_group::2).
 cudaError_t launch_gemm_umma(const UmmaPlan *p, const GemmArgs &a, unsigned int *claim, unsigned int *bar_b,
                              const ZeroList *zero, int pdl, cudaStream_t st, int cta_pairs = 0);
+// What other launchers need of a plan: tensor maps (boxes of 64 k x 128 rows), rows and output offsets of the matrices.
+void umma_plan_view(const UmmaPlan *p, CUtensorMap *maps, int *n_rows, int *y_off, int &n_mats, int &K, unsigned int *&err);
+// Tensor map over an activation pair [2][pan_rows][K] (bf16), boxes of 64 k x box_rows.
+cudaError_t make_pair_tensor_map(CUtensorMap *out, const void *pan, int pan_rows, int K, int box_rows);
+
+// ---- many rows: one dense GEMM per projection (k_bulk.cu); every weight matrix a whole number of 256-row tiles
+enum BulkEpi : int {
+  BULK_STORE = 0,     // y = acc
+  BULK_ADD = 1,       // y += acc (the residual)
+  BULK_SWIGLU = 2,    // plan of gate and up: silu(s g) * (s u) as the pair out_pan, s = 1/rms from ss
+  BULK_HEAD = 3       // logits = s * acc + bias; per-row (max, lowest index)
+};
+struct BulkArgs {
+  const void *pan;        // activation pair [2][pan_rows][K]
+  int pan_rows, R;
+  float *y; int ldy;
+  const float *ss; float eps; int dn;
+  void *out_pan;          // [2][pan_rows][d_ffn]
+  void *slots;            // bulk_slot_bytes(): pieces of tiles that several pairs work on
+  unsigned int *arrived;  // kBulkArrived words, zero before the first launch; every launch leaves them zero
+  const int32_t *tokens, *perm; float beta; unsigned long long *amax; float *logits;
+};
+constexpr int kBulkPairs = 80;                       // CTA pairs the slots are laid out for
+constexpr int kBulkArrived = kBulkPairs * 16;        // fewer units than pairs are ever shared; two ranks, eight warps
+size_t bulk_slot_bytes();
+cudaError_t launch_bulk_gemm(const UmmaPlan *plan, const BulkArgs &a, int epi, int n_sms, int pdl, cudaStream_t st);
+// pan = x * gain as a pair, ss[r] = sum x^2; one row per block
+cudaError_t launch_norm_pair(const float *x, const void *gain, float *ss, void *pan, int pan_rows, int R, int d, int pdl, cudaStream_t st);
+// kv_len[sequence] += rows for every segment
+cudaError_t launch_advance(int32_t *kv_len, const RowSegs &segs, int nseg, cudaStream_t st);
+
 // Up to four projections in one launch, each consuming the previous one's reduced output; bar: n-1 zeroed words.
 // bar_b: n zeroed words (panel-ready barriers), needed when the rows exceed 16 and the plans have panels.
 // sync (optional, used up to 16 rows): how each projection is tied to the others, instead of a grid barrier

@@ -43,14 +43,33 @@ __device__ __forceinline__ unsigned long long pack_max(float v, int idx) {
 }
 
 // ------------------------------------------------------------------------------------ embed
+// A block takes whole rows, a thread eight elements at a time (d is a multiple of 8).
 template <typename T>
-__global__ void embed_kernel(EmbedArgs a) {
-  const T *emb = (const T *)a.emb;
-  const long long total = (long long)a.R * a.d;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    int r = (int)(i / a.d), k = (int)(i % a.d);
-    a.x[i] = to_f32(emb[(long long)a.tokens[r] * a.d + k]);
+__global__ void embed_kernel(const __grid_constant__ EmbedArgs a) {
+  for (int r = blockIdx.x; r < a.R; r += gridDim.x) {
+    int tok;
+    if (a.segs.n > 0) {
+      int i = 0;
+      while (i + 1 < a.segs.n && r >= a.segs.row0[i + 1]) ++i;
+      tok = a.tokens[(long long)a.segs.seq[i] * a.t_stride + a.kv_len[a.segs.seq[i]] + (r - a.segs.row0[i])];
+    } else {
+      tok = a.tokens[r];
+    }
+    const T *src = (const T *)a.emb + (long long)tok * a.d;
+    float *dst = a.x + (long long)r * a.d;
+    for (int k = threadIdx.x * 8; k < a.d; k += blockDim.x * 8) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float4 v;
+        if constexpr (sizeof(T) == 4) {
+          v = *reinterpret_cast<const float4 *>(src + k + 4 * h);
+        } else {
+          const uint2 w = *reinterpret_cast<const uint2 *>(src + k + 4 * h);
+          v = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
+        }
+        *reinterpret_cast<float4 *>(dst + k + 4 * h) = v;
+      }
+    }
   }
   zero_side(a.z);
 }
@@ -59,6 +78,19 @@ cudaError_t launch_embed(const EmbedArgs &a, int dtype, cudaStream_t st) {
   int blocks = 148 * 2;
   if (dtype == FC_F32) embed_kernel<float><<<blocks, 256, 0, st>>>(a);
   else embed_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+__global__ void advance_kernel(int32_t *kv_len, const __grid_constant__ RowSegs g, int nseg) {
+  for (int i = threadIdx.x; i < nseg; i += blockDim.x) {
+    if (g.n > 0) kv_len[g.seq[i]] += g.row0[i + 1] - g.row0[i];
+    else kv_len[g.seq_map ? g.seq_map[i] : g.b0 + i] += g.c;
+  }
+}
+
+cudaError_t launch_advance(int32_t *kv_len, const RowSegs &segs, int nseg, cudaStream_t st) {
+  if (nseg < 1) return cudaErrorInvalidValue;
+  advance_kernel<<<1, 64, 0, st>>>(kv_len, segs, nseg);
   return cudaGetLastError();
 }
 

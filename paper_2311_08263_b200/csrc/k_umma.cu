@@ -894,6 +894,28 @@ UmmaPlan *umma_plan_create(const GemmArgs &a, int pro, int epi, int n_sms, unsig
 
 void umma_plan_destroy(UmmaPlan *p) { delete p; }
 
+void umma_plan_view(const UmmaPlan *pl, CUtensorMap *maps, int *n_rows, int *y_off, int &n_mats, int &K, unsigned int *&err) {
+  for (int m = 0; m < kMaxMats; ++m) {
+    maps[m] = pl->maps[m];
+    n_rows[m] = m < pl->d.g.n_mats ? pl->d.g.n_rows[m] : 0;
+    y_off[m] = m < pl->d.g.n_mats ? pl->d.g.y_off[m] : 0;
+  }
+  n_mats = pl->d.g.n_mats; K = pl->d.g.K; err = pl->err;
+}
+
+cudaError_t make_pair_tensor_map(CUtensorMap *out, const void *pan, int pan_rows, int K, int box_rows) {
+  EncodeTiledFn enc = get_encode_fn();
+  if (!enc) return cudaErrorNotSupported;
+  if (pan_rows < 1 || K < kTileK || K % 8 || box_rows < 8 || box_rows > 256 || ((uintptr_t)pan & 15)) return cudaErrorInvalidValue;
+  cuuint64_t gdim[2] = {(cuuint64_t)K, (cuuint64_t)2 * pan_rows};
+  cuuint64_t gstr[1] = {(cuuint64_t)K * 2};
+  cuuint32_t box[2] = {(cuuint32_t)kTileK, (cuuint32_t)box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  return enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(pan), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 template <int EPI, int BN, bool PANEL>
 static cudaError_t launch_one(const MapPack &maps, const UmmaParams &p, int grid, cudaStream_t st) {
   const size_t smem = (size_t)p.stages * (kWBytes + x_parts(BN) * BN * 128) + 1024;

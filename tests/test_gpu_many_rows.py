@@ -1,0 +1,67 @@
+"""Forwards of many rows (one dense GEMM per projection), against the oracle: prompts packed into blocks that cut through
+sequences, steps whose rows end inside a row tile, grouped queries, both head sizes.  Bars and margin rule as in
+test_gpu_full_configs."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2311_08263_b200 import engine, workload as wl
+from test_gpu_full_configs import _check_step, _random_kv_case
+
+pytestmark = pytest.mark.gpu
+
+
+def _cfg(hq, hkv, hd, d_ffn=768, **kw):
+    return wl.small_config(n_layers=2, n_heads=hq, n_kv_heads=hkv, head_dim=hd, d_model=512, d_ffn=d_ffn, vocab=1024, **kw)
+
+
+STEPS = [
+    # hq, hkv, hd, d_ffn, c, lens: rows = c x sequences
+    (8, 4, 64, 768, 43, [0, 33, 70]),                      # 129 rows: one more than the chained launch takes
+    (4, 4, 128, 512, 20, [100, 0, 1, 31, 32, 33, 64, 95]),  # 160
+    (8, 8, 64, 1280, 61, [40, 0, 7, 64, 129]),              # 305: a ragged third row tile
+    (4, 2, 128, 256, 64, [5, 200, 64, 0, 17, 90, 128, 33]),  # 512: one tile of weights in the feed-forward block
+]
+
+
+@pytest.mark.parametrize("hq,hkv,hd,d_ffn,c,lens", STEPS)
+def test_many_row_step(hq, hkv, hd, d_ffn, c, lens):
+    cfg = _cfg(hq, hkv, hd, d_ffn, seed=300 + c)
+    dec, _ = _random_kv_case(cfg, lens, c, range(len(lens)))
+    assert dec.fc_last_launch_count() == 8 * cfg.n_layers + 4
+
+
+PROMPTS = [
+    (8, 4, 64, [130]),                                      # 129 rows of one sequence
+    (8, 2, 128, [1, 2, 130, 300, 65, 64, 33, 1]),           # empty and one-row segments between longer ones
+    (4, 4, 64, [700, 517, 300, 41]),                        # 1554 rows: two blocks, the cut inside the second prompt
+]
+
+
+@pytest.mark.parametrize("hq,hkv,hd,lens", PROMPTS)
+def test_packed_prompts(hq, hkv, hd, lens):
+    cfg = _cfg(hq, hkv, hd, seed=500 + len(lens), prompt_len=max(lens))
+    c, B = 4, len(lens)
+    w = wl.make_weights(cfg)
+    ids, _ = wl.make_prompts(cfg, batch=B, lens=lens)
+    dec = engine.Decoder(cfg, w, B, c, max(lens) + 2 * c)
+    dec.fc_prefill(ids.numpy(), lens, c)
+    kv = dec.kv_view().float().cpu().numpy()
+    logits = dec.fc_debug_logits(True)
+    cnt, tok, win = dec.fc_jacobi_step()
+    lg = logits.cpu().numpy().reshape(B, c, cfg.vocab)
+    for b, P in enumerate(lens):
+        o = oracle.Oracle(cfg, w, max(lens) + 2 * c)
+        o.prefill(ids[b, :P].numpy(), c)
+        window = np.array([ids[b, P - 1]] + [ids[b, (j - 1) % P] for j in range(1, c)], np.int32)
+        k_ref, acc_ref, win_ref, lg_ref = o.jacobi_step(want_logits=True)
+        _check_step(lg[b], lg_ref, window, cnt[b], tok[b], win[b], k_ref, acc_ref, win_ref)
+        if P > 1:
+            # layer 0 has no attention in front of it: fp32 sums in another order, so a stored value is at most one bf16
+            # step (2^-8 of its size, 2^-7 above a power of two) away, and nearly all are the same
+            for half, ref in enumerate(o.get_kv(0, P - 1)):
+                got = kv[0, half, b, :, :P - 1].transpose(1, 0, 2).reshape(P - 1, -1)
+                assert np.all(np.abs(got - ref) <= 2.0 ** -7 * np.abs(ref) + 1e-6)
+                assert np.mean(got != ref) < 0.01
+        o.close()
+    assert dec.fc_debug_check_guards() == 0
