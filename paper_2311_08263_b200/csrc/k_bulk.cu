@@ -9,10 +9,11 @@
 // tiles, 128 activation rows, two accumulators in the same lanes, so the epilogue has both factors of SwiGLU in one thread
 // and writes the down projection's operand itself.
 //
-// An accumulator in tensor memory runs over eight k-blocks only; then the epilogue warps add it to fp32 sums in their
-// registers, while the next eight run in the other accumulator.  (The tensor core's own additions are not rounded to
-// nearest: over a whole k range of 5120 the error of a 13B step grew by half, over eight k-blocks, 64 additions of either
-// half, it is the chained launch's.)
+// An accumulator in tensor memory runs over six k-blocks only; then the epilogue warps add it to fp32 sums in their
+// registers, while the next six run in the other accumulator.  The tensor core's own additions are not rounded to
+// nearest, so their number sets the error.  Logits of a 13B step of 256 rows against 64 bits (three seeds), and the time
+// of 4 layers: chained launch 1.07 / 1.25 / 1.29e-3; whole k range in one accumulator above 1.5e-3; 8 k-blocks 1.09 / 1.32 /
+// 1.28e-3, 1.77 ms; 6: 1.07 / 1.23 / 1.22e-3, 1.82 ms; 4: 1.03 / 1.20 / 1.06e-3, 1.88 ms.
 //
 // The tiles of a projection seldom are a whole number of rounds over the pairs: whole rounds run tile by tile, the tiles
 // that are left over are dealt as one run of k-blocks, cut into equal shares for all pairs (a share ends in one tile and may
@@ -34,7 +35,7 @@ constexpr int kBulkThreads = 320;
 constexpr int kEpiWarps = 8;
 constexpr int kMaxStages = 8;
 constexpr int kWTile = kTileM * kTileK * 2;        // 16 KB: this CTA's 128 weight rows of a k-block
-constexpr int kAccKb = 8;                          // k-blocks an accumulator runs over before it is added up in registers
+constexpr int kAccKb = 6;                          // k-blocks an accumulator runs over before it is added up in registers
 constexpr int kSlotF4 = 1024;                      // one warp's part of a piece: 16 KB
 constexpr size_t kBulkSmem = 225 * 1024;           // ring + alignment; static shared memory takes the rest of 227 KB
 
