@@ -198,6 +198,9 @@ struct fc_ctx {
   std::vector<size_t> guards;    // offsets of the canary bands inside the workspace
   // pinned staging: [count | tokens | window | err]
   int32_t *pin = nullptr;
+  // what the accept kernel reports, in pinned memory: [max_batch] counts, [max_batch * max_c] tokens, windows, error word
+  int32_t *res_count = nullptr, *res_tokens = nullptr, *res_window = nullptr, *res_err = nullptr;
+  bool small = false;            // fp32 model whose forward is one kernel
   int32_t *pin_map = nullptr;    // pinned [max_batch]: the live sequences of a compacted step
   int64_t launches = 0;
   char cuda_err[256] = {0};
@@ -261,6 +264,7 @@ extern "C" void fc_destroy(fc_ctx *ctx) {
   destroy_plans(ctx);
   if (ctx->pin) cudaFreeHost(ctx->pin);
   if (ctx->pin_map) cudaFreeHost(ctx->pin_map);
+  if (ctx->res_count) cudaFreeHost(ctx->res_count);
   if (ctx->ev0) cudaEventDestroy(ctx->ev0);
   if (ctx->ev1) cudaEventDestroy(ctx->ev1);
   delete ctx;
@@ -409,6 +413,14 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
   const size_t pin_ints = (size_t)shape->max_batch * (1 + 2 * shape->max_c) + 4;
   if (cudaMallocHost((void **)&ctx->pin, pin_ints * sizeof(int32_t)) != cudaSuccess) return fail(FC_ERR_CUDA);
   if (cudaMallocHost((void **)&ctx->pin_map, (size_t)shape->max_batch * sizeof(int32_t)) != cudaSuccess) return fail(FC_ERR_CUDA);
+  const size_t res_ints = (size_t)shape->max_batch * (1 + 2 * shape->max_c) + 1;
+  if (cudaMallocHost((void **)&ctx->res_count, res_ints * sizeof(int32_t)) != cudaSuccess) return fail(FC_ERR_CUDA);
+  memset(ctx->res_count, 0, res_ints * sizeof(int32_t));
+  ctx->res_tokens = ctx->res_count + shape->max_batch;
+  ctx->res_window = ctx->res_tokens + (size_t)shape->max_batch * shape->max_c;
+  ctx->res_err = ctx->res_window + (size_t)shape->max_batch * shape->max_c;
+  ctx->small = shape->dtype == FC_F32 && !(shape->flags & (FC_FLAG_SIMT_GEMM | FC_FLAG_NO_CHAIN)) &&
+               small_model_fits(shape->d_model, ctx->d.qd, ctx->d.kvd, shape->d_ffn, shape->head_dim, shape->vocab, L);
   if (cudaEventCreate(&ctx->ev0) != cudaSuccess || cudaEventCreate(&ctx->ev1) != cudaSuccess) return fail(FC_ERR_CUDA);
   if (cudaMemsetAsync(ws, 0, fc_workspace_bytes(shape), ctx->st) != cudaSuccess) return fail(FC_ERR_CUDA);
   for (size_t off : ctx->guards)      // canary bands between the slices (checked by fc_debug_check_guards)
@@ -471,7 +483,7 @@ static cudaError_t run_gemm(fc_ctx *ctx, const UmmaPlan *plan, GemmArgs a, int R
   return launch_gemm_simt(a, ctx->s.dtype, pro, epi, ctx->st);
 }
 
-static int run_accept(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *seq_map, int commit) {
+static AcceptArgs accept_args(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *seq_map, int commit) {
   const fc_model_shape &s = ctx->s;
   AcceptArgs ac; memset(&ac, 0, sizeof ac);
   ac.window = ctx->b.window; ac.amax = ctx->b.amax; ac.amax_clear = ctx->b.amax;
@@ -482,10 +494,38 @@ static int run_accept(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *seq_
   ac.b0 = b0; ac.nb = nb; ac.c = rows; ac.p_stride = s.max_seq; ac.refill = ctx->refill; ac.pad_id = ctx->pad_id;
   ac.seq_map = seq_map;
   ac.max_tokens = ctx->gen_max_tokens; ac.eos_id = ctx->gen_eos; ac.commit = commit;
+  ac.host_count = ctx->res_count; ac.host_tokens = ctx->res_tokens; ac.host_window = ctx->res_window; ac.host_err = ctx->res_err;
+  ac.err = ctx->b.err;
   if (ctx->inject_timeout) { ac.err_inject = ctx->b.err; ctx->inject_timeout = false; }
+  return ac;
+}
+static int run_accept(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *seq_map, int commit) {
   ++ctx->launches;
   ProfScope ps(ctx, FC_CLS_ACCEPT);
-  FC_CK(launch_accept(ac, ctx->st));
+  FC_CK(launch_accept(accept_args(ctx, b0, nb, rows, seq_map, commit), ctx->st));
+  return FC_OK;
+}
+
+// A small fp32 model: the whole forward, and with the head the accept step, in one kernel.
+static int forward_small(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, const int32_t *tokens, bool with_head, int commit) {
+  const fc_model_shape &s = ctx->s;
+  SmallArgs a; memset(&a, 0, sizeof a);
+  for (int l = 0; l < s.n_layers; ++l)
+    a.layers[l] = SmallLayer{(const float *)ctx->wq[l], (const float *)ctx->wk[l], (const float *)ctx->wv[l], (const float *)ctx->wo[l],
+                             (const float *)ctx->w_gate[l], (const float *)ctx->w_up[l], (const float *)ctx->w_down[l],
+                             (const float *)ctx->g_attn[l], (const float *)ctx->g_ffn[l]};
+  a.n_layers = s.n_layers; a.d = s.d_model; a.hq = s.n_heads; a.hkv = s.n_kv_heads; a.hd = s.head_dim; a.f = s.d_ffn; a.vocab = s.vocab;
+  a.emb = (const float *)ctx->tok_emb; a.g_final = (const float *)ctx->g_final; a.lm_head = (const float *)ctx->lm_head;
+  a.eps = s.rms_eps; a.rope = ctx->b.rope; a.tokens = tokens; a.kv_len = ctx->b.kv_len; a.seq_map = segs.seq_map;
+  a.b0 = segs.b0; a.c = rows; a.R = nb * rows;
+  a.kv = (float *)ctx->kv; a.half_stride = (long long)(ctx->kv_half_stride / sizeof(float));
+  a.stride_h = (long long)s.max_seq * s.head_dim; a.stride_b = s.n_kv_heads * a.stride_h;
+  a.x = ctx->b.x; a.q = (float *)ctx->b.qb; a.attn = ctx->b.attn; a.h = ctx->b.gu;
+  a.with_head = with_head; a.perm = s.bias_beta != 0.f ? ctx->bias_perm : nullptr; a.beta = s.bias_beta; a.logits = ctx->dbg_logits;
+  if (with_head) a.accept = accept_args(ctx, segs.b0, nb, rows, segs.seq_map, commit);
+  ++ctx->launches;
+  ProfScope ps(ctx, FC_CLS_CHAIN);
+  FC_CK(launch_small_forward(a, ctx->st));
   return FC_OK;
 }
 
@@ -560,6 +600,13 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
   const int R = nb * rows;
   RowSegs segs; memset(&segs, 0, sizeof segs);
   segs.b0 = b0; segs.c = rows; segs.seq_map = seq_map;
+  if (ctx->small) {
+    int rc = forward_small(ctx, segs, nb, rows, tokens, with_head, commit);
+    if (rc != FC_OK || with_head) return rc;
+    ++ctx->launches;
+    FC_CK(launch_advance(ctx->b.kv_len, segs, nb, ctx->st));
+    return FC_OK;
+  }
   if (ctx->d.bulk && R >= kBulkMin) {
     int rc = forward_bulk(ctx, segs, nb, R, rows, max_len_host, tokens, with_head);
     if (rc != FC_OK) return rc;
@@ -825,16 +872,17 @@ extern "C" int fc_prefill(fc_ctx *ctx, int32_t batch, const int32_t *prompt_ids,
   return FC_OK;
 }
 
-// Copy (count | tokens | window | err) of the finished step to the host and refresh the host mirrors.
+// Wait for the step and refresh the host mirrors from what its accept kernel reported.
 static int collect_step(fc_ctx *ctx, int32_t *accepted_count, int32_t *accepted_tokens, int32_t *window_out) {
   const int B = ctx->batch, c = ctx->c;
-  int32_t *p_cnt = ctx->pin, *p_tok = p_cnt + B, *p_win = p_tok + (size_t)B * c, *p_err = p_win + (size_t)B * c;
-  FC_CK(cudaMemcpyAsync(p_cnt, ctx->b.acc_count, sizeof(int32_t) * B, cudaMemcpyDeviceToHost, ctx->st));
-  FC_CK(cudaMemcpyAsync(p_tok, ctx->b.acc_tokens, sizeof(int32_t) * B * c, cudaMemcpyDeviceToHost, ctx->st));
-  FC_CK(cudaMemcpyAsync(p_win, ctx->b.window, sizeof(int32_t) * B * c, cudaMemcpyDeviceToHost, ctx->st));
-  FC_CK(cudaMemcpyAsync(p_err, ctx->b.err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->st));
+  int32_t *p_cnt = ctx->res_count, *p_tok = ctx->res_tokens, *p_win = ctx->res_window;
+  bool all_live = true;
+  for (int b = 0; b < B; ++b) all_live = all_live && !ctx->done_h[b];
+  // finished sequences are not part of the step: their windows are only on the device
+  if (!all_live) FC_CK(cudaMemcpyAsync(p_win, ctx->b.window, sizeof(int32_t) * B * c, cudaMemcpyDeviceToHost, ctx->st));
   FC_CK(cudaStreamSynchronize(ctx->st));
-  if (*p_err) {
+  if (*ctx->res_err) {
+    *ctx->res_err = 0;
     clear_device_error(ctx);
     return FC_ERR_DEVICE_TIMEOUT;
   }

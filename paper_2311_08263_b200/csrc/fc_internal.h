@@ -177,7 +177,32 @@ struct AcceptArgs {
   int max_tokens, eos_id;          // max_tokens <= 0: unlimited
   int commit;                      // 0: leave kv_len / n_gen / window untouched (latency measurement)
   unsigned int *err_inject;        // test aid: when non-null the kernel raises this error word (no wait involved)
+  // what the host wants to know, written to its (pinned) memory as well; all null: nothing
+  int32_t *host_count, *host_tokens, *host_window, *host_err;
+  const unsigned int *err;         // the device error word behind host_err
 };
+
+// A small fp32 model's forward as one kernel (k_small.cu).
+constexpr int kSmallLayers = 16;
+struct SmallLayer { const float *wq, *wk, *wv, *wo, *w_gate, *w_up, *w_down, *g_attn, *g_ffn; };
+struct SmallArgs {
+  SmallLayer layers[kSmallLayers];
+  int n_layers, d, hq, hkv, hd, f, vocab;
+  const float *emb, *g_final, *lm_head;
+  float eps;
+  const float2 *rope;
+  const int32_t *tokens;           // [R]
+  const int32_t *kv_len, *seq_map; // row block i belongs to sequence seq_map[i] (null: b0 + i)
+  int b0, c, R;
+  float *kv;                       // K and V planes of a layer half_stride elements apart
+  long long half_stride, stride_b, stride_h;
+  float *x, *q, *attn, *h;         // [R, d], [R, qd], [R, qd], [R, f]
+  int with_head;
+  const int32_t *perm; float beta; float *logits;
+  AcceptArgs accept;               // with_head: runs behind the LM head; accept.amax_clear is the argmax buffer, zero on entry
+};
+bool small_model_fits(int d, int qd, int kvd, int f, int hd, int vocab, int n_layers);
+cudaError_t launch_small_forward(const SmallArgs &a, cudaStream_t st);
 
 struct EmbedArgs {
   const int32_t *tokens;   // [R], or with segs.n > 0 [sequence][t_stride]: row j of a segment is token kv_len[sequence] + j

@@ -1,7 +1,7 @@
 // FMA (non-tensor-core) kernels of the Jacobi-window decode step: embedding gather, the plain
 // projection kernel used by the fp32 configuration, rotary embedding + K/V write, split-KV window
 // attention, and the accept / commit / shift / refill kernel.
-#include "fc_internal.h"
+#include "fc_accept.cuh"
 
 namespace fc {
 
@@ -393,59 +393,8 @@ cudaError_t launch_attn(const AttnArgs &a, int dtype, int hd, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------------------------------ accept / commit / shift / refill
-// One thread per sequence (all integer work; c <= 64).  a[j] = greedy token after window slot j.
-// a[0] is always exact; a[j] is exact while every guess w[1..j] matched the exact token before it
-// (checked one by one, Eq. 5).  K/V of the accepted rows already sit at their final slots, so the
-// commit is kv_len += k.  New window: pending token a[k-1], the unverified outputs a[k..c-1] as next
-// guesses, then refill ids for the k-1 positions no forward has predicted yet.
-__global__ void accept_kernel(AcceptArgs a) {
-  const int bl = blockIdx.x * blockDim.x + threadIdx.x;
-  if (bl >= a.nb) return;
-  const int b = a.seq_map ? a.seq_map[bl] : a.b0 + bl, c = a.c;
-  int32_t *w = a.window + (long long)b * c;
-  int32_t arg[64];
-  for (int j = 0; j < c; ++j) {
-    const int r = bl * c + j;
-    if (a.amax) {
-      arg[j] = (int32_t)(0xFFFFFFFFu - (unsigned int)(a.amax[r] & 0xFFFFFFFFull));
-      if (a.amax_clear) a.amax_clear[r] = 0ull;
-    } else {
-      arg[j] = a.argmax[r];
-    }
-  }
-  if (a.err_inject && bl == 0) atomicExch(a.err_inject, 1u);
-  if (a.done && a.done[b]) { a.accepted_count[b] = 0; return; }
-  int k = 1;
-  while (k < c && w[k] == arg[k - 1]) ++k;
-  // stop rules: cut at max_tokens and just after the first EOS
-  const int n0 = a.n_gen[b];
-  int kept = 0, finished = 0;
-  for (int j = 0; j < k && !finished; ++j) {
-    if (a.max_tokens > 0 && n0 + kept >= a.max_tokens) { finished = 1; break; }
-    a.accepted_tokens[(long long)b * c + j] = arg[j];
-    if (a.out_tokens && n0 + kept < a.out_stride) a.out_tokens[(long long)b * a.out_stride + n0 + kept] = arg[j];
-    ++kept;
-    if (a.eos_id >= 0 && arg[j] == a.eos_id) finished = 1;
-  }
-  if (a.max_tokens > 0 && n0 + kept >= a.max_tokens) finished = 1;
-  a.accepted_count[b] = kept;
-  if (!a.commit) return;
-  if (finished && a.done) a.done[b] = 1;
-  k = kept;                      // after a cut the remaining state is only reported, never used
-  if (k == 0) return;
-  a.kv_len[b] += k;
-  const int n1 = n0 + k;
-  a.n_gen[b] = n1;
-  const int P = a.prompt_lens ? a.prompt_lens[b] : 1;
-  int32_t nw[64];
-  nw[0] = arg[k - 1];
-  for (int j = 1; j < c; ++j) {
-    if (j <= c - k) nw[j] = arg[k - 1 + j];
-    else nw[j] = (a.refill == FC_REFILL_PAD || !a.prompt) ? a.pad_id
-                                                          : a.prompt[(long long)b * a.p_stride + (n1 + j - 1) % P];
-  }
-  for (int j = 0; j < c; ++j) w[j] = nw[j];
-}
+// One warp per sequence.
+__global__ void accept_kernel(const __grid_constant__ AcceptArgs a) { accept_warp(a, blockIdx.x, threadIdx.x); }
 
 __global__ void gather_rows_kernel(int32_t *dst, const int32_t *window, const int32_t *seq_map, int nb, int c) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -458,7 +407,7 @@ cudaError_t launch_gather_rows(int32_t *dst, const int32_t *window, const int32_
 }
 
 cudaError_t launch_accept(const AcceptArgs &a, cudaStream_t st) {
-  accept_kernel<<<(a.nb + 31) / 32, 32, 0, st>>>(a);
+  accept_kernel<<<a.nb, 32, 0, st>>>(a);
   return cudaGetLastError();
 }
 
