@@ -388,7 +388,11 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
     if (shape->d_model < 64 || shape->d_ffn < 64 || ctx->d.qd < 64) return fail(FC_ERR_SHAPE);
     char msg[200];
     // halves of d_ffn must be whole 128-row tiles (and so whole 64-wide k-blocks of the down projection)
-    ctx->ffn_split = ctx->chain && shape->d_ffn % 256 == 0 && !(shape->flags & FC_FLAG_NO_FFN_SPLIT);
+    // and long enough phases to hide a barrier: at least four chunks (128 rows x 4 k-blocks) of gate and up per CTA.
+    // Below that every phase is one round of chunks, and two phases more are only latency (16 layers, split against not: 1.1B,
+    // 2.4 chunks per CTA, 16 rows 866 against 831 us, 1 row 749 against 709; 7B, 9.3 chunks, 1658 against 1664).
+    const long long gu_chunks = 2ll * (shape->d_ffn / 128) * ((shape->d_model + 255) / 256);
+    ctx->ffn_split = ctx->chain && shape->d_ffn % 256 == 0 && gu_chunks >= 8ll * ctx->n_sms && !(shape->flags & FC_FLAG_NO_FFN_SPLIT);
     for (int l = 0; l < L && rc == FC_OK; ++l) {
       UmmaPlan *p;
       if (!(p = umma_plan_create(args_qkv(ctx, l), PRO_GAIN, EPI_ATOMIC_ADD, ctx->n_sms, ctx->b.err, msg, sizeof msg))) rc = FC_ERR_CUDA; else ctx->plan_qkv.push_back(p);
