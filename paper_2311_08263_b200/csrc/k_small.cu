@@ -98,6 +98,21 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
     s1 = w1 ? sum8(q, lane) : 0.f;
   };
 
+  // This warp's first weight row of a coming step on its way into the first-level cache while the barrier in front of
+  // that step is waited for: nobody waits for these loads.
+  auto touch = [&](const float *row, int K) {
+    for (int k = lane * 4; k < K; k += 128) {
+      float t;
+      asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(t) : "l"(row + k));
+    }
+  };
+  // the first row of the rotary pair that is unit u of the QKV step
+  auto pair_row = [&](const SmallLayer &w, int u) -> const float * {
+    const int h = u / half, i = u - h * half;
+    return (h < a.hq ? w.wq + (long long)h * hd * d : h < a.hq + a.hkv ? w.wk + (long long)(h - a.hq) * hd * d : w.wv + (long long)(h - a.hq - a.hkv) * hd * d) + (long long)i * d;
+  };
+  const int n_pairs = (a.hq + 2 * a.hkv) * half;
+
   for (int l = 0; l < a.n_layers; ++l) {
     const SmallLayer &w = a.layers[l];
     const float *x_in = l == 0 ? nullptr : a.x;                   // layer 0 reads the embedding rows themselves
@@ -106,21 +121,20 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
     for (int r0 = 0; r0 < R; r0 += kSmRows) {
       const int n = min(kSmRows, R - r0);
       stage(x_in, d, d, w.g_attn, r0, n);
-      for (int u = gw; u < (a.hq + 2 * a.hkv) * half; u += kUnits) {
+      for (int u = gw; u < n_pairs; u += kUnits) {
         const int h = u / half, i = u - h * half;
-        const float *m = h < a.hq ? w.wq + (long long)h * hd * d : h < a.hq + a.hkv ? w.wk + (long long)(h - a.hq) * hd * d : w.wv + (long long)(h - a.hq - a.hkv) * hd * d;
+        const float *m = pair_row(w, u);
         for (int c0 = 0; c0 < n; c0 += 8) {
-          float v0, v1;
-          dots(m + (long long)i * d, m + (long long)(i + half) * d, d, xs + c0 * d, v0, v1);
-          const int rr = c0 + (lane >> 2);
-          if ((lane & 3) || rr >= n) continue;
-          const int r = r0 + rr;
+          const int rr = c0 + (lane >> 2), r = r0 + min(rr, n - 1);
           int b, j;
           seq_of(r, b, j);
-          const int pos = a.kv_len[b] + j;
+          const int pos = a.kv_len[b] + j;                          // on its way, with the rotation, beside the weights
+          const float2 rot = __ldg(a.rope + (long long)pos * half + i);
+          float v0, v1;
+          dots(m, m + (long long)half * d, d, xs + c0 * d, v0, v1);
+          if ((lane & 3) || rr >= n) continue;
           v0 *= s_rms[rr]; v1 *= s_rms[rr];
           if (h < a.hq + a.hkv) {
-            const float2 rot = __ldg(a.rope + (long long)pos * half + i);
             const float o0 = v0 * rot.x - v1 * rot.y, o1 = v0 * rot.y + v1 * rot.x;
             v0 = o0; v1 = o1;
           }
@@ -130,6 +144,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
         }
       }
     }
+    if (gw < d) touch(w.wo + (long long)gw * qd, qd);
     cluster_sync_all();
     // ---- attention: a (row, head) per group of warps, keys dealt in blocks of eight
     {
@@ -216,23 +231,27 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
     }
     cluster_sync_all();
     // ---- x += attn . Wo
-    auto add_to_x = [&](const float *src, int K, const float *m, bool from_emb) {
+    auto add_to_x = [&](const float *src, int K, const float *m, bool from_emb, auto &&next) {
       for (int r0 = 0; r0 < R; r0 += kSmRows) {
         const int n = min(kSmRows, R - r0);
         stage(src, K, K, nullptr, r0, n);
         for (int u = gw; u < d; u += kUnits)
           for (int c0 = 0; c0 < n; c0 += 8) {
+            const int rr = c0 + (lane >> 2), r = r0 + min(rr, n - 1);
+            float *x = a.x + (long long)r * d + u;
+            const float before = from_emb ? a.emb[(long long)a.tokens[r] * d + u] : __ldcg(x);
             float v, none;
             dots(m + (long long)u * K, nullptr, K, xs + c0 * K, v, none);
-            const int rr = c0 + (lane >> 2);
             if ((lane & 3) || rr >= n) continue;
-            float *x = a.x + (long long)(r0 + rr) * d + u;
-            *x = (from_emb ? a.emb[(long long)a.tokens[r0 + rr] * d + u] : __ldcg(x)) + v;
+            *x = before + v;
           }
       }
+      next();
       cluster_sync_all();
     };
-    add_to_x(a.attn, qd, w.wo, l == 0);
+    add_to_x(a.attn, qd, w.wo, l == 0, [&] {
+      if (gw < F) { touch(w.w_gate + (long long)gw * d, d); touch(w.w_up + (long long)gw * d, d); }
+    });
     // ---- silu(gate) * up
     for (int r0 = 0; r0 < R; r0 += kSmRows) {
       const int n = min(kSmRows, R - r0);
@@ -247,8 +266,15 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
           a.h[(long long)(r0 + rr) * F + u] = (g / (1.0f + expf(-g))) * up;
         }
     }
+    if (gw < d) touch(w.w_down + (long long)gw * F, F);
     cluster_sync_all();
-    add_to_x(a.h, F, w.w_down, false);
+    add_to_x(a.h, F, w.w_down, false, [&] {
+      if (l + 1 < a.n_layers) {
+        if (gw < n_pairs) { const float *m = pair_row(a.layers[l + 1], gw); touch(m, d); touch(m + (long long)half * d, d); }
+      } else if (a.with_head && gw < a.vocab) {
+        touch(a.lm_head + (long long)gw * d, d);
+      }
+    });
   }
   if (!a.with_head) return;
   // ---- LM head, greedy token per row
@@ -259,13 +285,13 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
     __syncthreads();
     for (int u = gw; u < a.vocab; u += kUnits)
       for (int c0 = 0; c0 < n; c0 += 8) {
+        const int rr = c0 + (lane >> 2), r = r0 + min(rr, n - 1);
+        const int favoured = a.perm ? a.perm[a.tokens[r]] : -1;
         float v, none;
         dots(a.lm_head + (long long)u * d, nullptr, d, xs + c0 * d, v, none);
-        const int rr = c0 + (lane >> 2);
         if ((lane & 3) || rr >= n) continue;
-        const int r = r0 + rr;
         float logit = v * s_rms[rr];
-        if (a.perm && a.perm[a.tokens[r]] == u) logit += a.beta;
+        if (favoured == u) logit += a.beta;
         if (a.logits) a.logits[(long long)r * a.vocab + u] = logit;
         atomicMax(&best[rr], ((unsigned long long)ordered_key_u(logit) << 32) | (unsigned long long)(0xFFFFFFFFu - (unsigned int)u));
       }
@@ -278,7 +304,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
 }
 
 // Models whose steps this kernel is made for: sixteen SMs hold and stream their layers.  Measured, this kernel against the
-// separate ones, per step: 2 layers, d 128, ffn 512 (1 MB of weights a layer), 8 rows over 64 keys 43 against 211 us, 4 x 16
+// separate ones, per step: 2 layers, d 128, ffn 512 (1 MB of weights a layer), 8 rows over 64 keys 41 against 211 us, 4 x 16
 // rows over 200 keys 150 against 1200; 8 layers, d 256, ffn 768 (3.3 MB), 8 rows over 512 keys 271 against 1144, 4 x 16 rows
 // 1530 against 7142; a prompt of 512 8.1 against 56.7 ms; 4 layers, d 512, ffn 1024 (10 MB), 1 row 189 against 337, 8 rows 218
 // against 803.  At 34 MB a layer and 131 MB of LM head one row costs more here (851 against 810).
