@@ -571,6 +571,7 @@ static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int m
     qa.stride_b = stride_b; qa.stride_h = stride_h; qa.pdl = pdl;
     ++ctx->launches;
     { ProfScope ps(ctx, FC_CLS_ROPE); FC_CK(launch_qkv_finish(qa, R, ctx->st)); }
+    if (!with_head && l + 1 == s.n_layers) break;      // rows that are only cached: nothing reads what follows the last K/V rows
     StreamAttnArgs sa; memset(&sa, 0, sizeof sa);
     sa.q = ctx->b.qb; sa.q_tiles = d.q_tiles; sa.kv_len = ctx->b.kv_len; sa.segs = segs; sa.hq = s.n_heads; sa.hkv = s.n_kv_heads;
     sa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; sa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
@@ -703,6 +704,7 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
     zl.p[0] = ctx->b.qkv; zl.n[0] = Rz * d.ldq;
     zl.p[1] = ctx->b.ss_attn; zl.n[1] = Rz;
     const ZeroList *zero = ctx->fused_attn ? &zl : nullptr;
+    if (!with_head && l + 1 == s.n_layers) break;      // rows that are only cached: nothing reads what follows the last K/V rows
     if (chained) {
       // O projection, gate/up, down and the next layer's QKV: one persistent launch.
       // Up to 16 rows the phases are tied together without a stall where the data allow it (see ChainSync): gate/up

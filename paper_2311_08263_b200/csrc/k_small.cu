@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
         }
       }
     }
+    if (!a.with_head && l + 1 == a.n_layers) break;                 // rows that are only cached: nothing reads what follows
     if (gw < d) touch(w.wo + (long long)gw * qd, qd);
     cluster_sync_all();
     // ---- attention: a (row, head) per group of warps, keys dealt in blocks of eight
