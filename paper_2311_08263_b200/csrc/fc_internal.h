@@ -269,8 +269,8 @@ void umma_plan_destroy(UmmaPlan *p);
 cudaError_t launch_gemm_umma(const UmmaPlan *p, const GemmArgs &a, unsigned int *claim, unsigned int *bar_b,
                              const ZeroList *zero, int pdl, cudaStream_t st, int cta_pairs = 0);
 // What other launchers need of a plan: tensor maps (boxes of 64 k x 128 rows), rows and output offsets of the matrices.
-void umma_plan_view(const UmmaPlan *p, CUtensorMap *maps, int *n_rows, int *y_off, int &n_mats, int &K, unsigned int *&err);
-// Tensor map over an activation pair [2][pan_rows][K] (bf16), boxes of 64 k x box_rows.
+void umma_plan_view(const UmmaPlan *p, CUtensorMap *maps, const void **w, int *n_rows, int *y_off, int &n_mats, int &K, unsigned int *&err);
+// Tensor map over 2 * pan_rows rows of K elements (bf16; an activation pair, or a weight matrix), boxes of 64 k x box_rows.
 cudaError_t make_pair_tensor_map(CUtensorMap *out, const void *pan, int pan_rows, int K, int box_rows);
 
 // ---- many rows: one dense GEMM per projection (k_bulk.cu); every weight matrix a whole number of 256-row tiles

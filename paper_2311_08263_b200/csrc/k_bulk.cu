@@ -5,9 +5,11 @@
 // operand bytes out of L2.  So the tile is as large as tensor memory allows with two accumulators: a cluster of two CTAs
 // (tcgen05 cta_group::2, M = 256) multiplies 256 weight rows by up to 256 activation rows, and the high and the low products
 // go to the SAME accumulator - per k-block of 64 a CTA loads 16 KB of weights once for both halves (48 KB per 2 x 256 x 256 x
-// 64 products of the pair; the chained kernel's pairs load 32 KB for half as many).  Gate and up run together: two weight
-// tiles, 128 activation rows, two accumulators in the same lanes, so the epilogue has both factors of SwiGLU in one thread
-// and writes the down projection's operand itself.
+// 64 products of the pair; the chained kernel's pairs load 32 KB for half as many).  Gate and up run together: a CTA's 128
+// weight rows are 64 of the gate and the same 64 of up, so the two factors of SwiGLU lie 64 lanes apart in one accumulator; the
+// two epilogue warps that hold them swap halves of each 16-row block through shared memory and write the down projection's
+// operand themselves.  (Two accumulators of 128 rows in the same lanes need no exchange but MMAs of half the width: gate/up of
+// 13B at about 1000 rows 444 us that way, 390 this way; a prompt batch of 13B, 8 layers, 63.1 -> 60.1 ms.)
 //
 // An accumulator in tensor memory runs over six k-blocks only; then the epilogue warps add it to fp32 sums in their
 // registers, while the next six run in the other accumulator.  The tensor core's own additions are not rounded to
@@ -33,6 +35,7 @@ namespace fc {
 namespace {
 constexpr int kBulkThreads = 320;
 constexpr int kEpiWarps = 8;
+constexpr int kSwapBytes = 16 * 1024;              // BULK_SWIGLU: four pairs of epilogue warps x two buffers x two directions x 1 KB
 constexpr int kMaxStages = 8;
 constexpr int kWTile = kTileM * kTileK * 2;        // 16 KB: this CTA's 128 weight rows of a k-block
 constexpr int kAccKb = 6;                          // k-blocks an accumulator runs over before it is added up in registers
@@ -64,6 +67,21 @@ struct BulkParams {
   unsigned int *err;
 };
 
+// Two warps (64 threads) meet at named barrier `id`; the verdict is true where it is for every lane of both.
+__device__ __forceinline__ bool meet_and(int id, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "bar.red.and.pred p, %2, 64, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r) : "r"((uint32_t)ok), "r"(id) : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void meet(int id) {
+  __syncwarp();
+  asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
+}
 __device__ __forceinline__ uint32_t pack_pair(float a, float b) {
   __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t *>(&v);
@@ -113,12 +131,12 @@ __global__ void __launch_bounds__(256) norm_pair_kernel(const float *x, const __
 // ------------------------------------------------------------------------------------ GEMM
 template <int EPI>
 __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid_constant__ BulkMaps maps, const __grid_constant__ BulkParams p) {
-  constexpr bool kDual = EPI == BULK_SWIGLU;                      // two weight tiles share the activation rows
-  constexpr int kNW = kDual ? 2 : 1;
+  constexpr bool kMixed = EPI == BULK_SWIGLU;                     // a CTA's weight rows: 64 of gate, 64 of up
   extern __shared__ unsigned char smem_dyn[];
   __shared__ __align__(8) unsigned long long full_b[kMaxStages], empty_b[kMaxStages], accum_full[2], tmem_empty[2], drain_bar;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
+  __shared__ unsigned int last_s[4];                              // per pair of epilogue warps: pieces of the tile that were there
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int S = p.stages;
@@ -160,7 +178,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
     t.rt = t.u % p.n_rt;
     t.lt = t.u / p.n_rt;
     t.m = 0;
-    if (!kDual)
+    if (!kMixed)
       while (t.m + 1 < p.n_mats && t.lt >= p.n_tiles[t.m]) { t.lt -= p.n_tiles[t.m]; ++t.m; }
     return true;
   };
@@ -171,16 +189,20 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
     if (lane == 0) {
       bool ok = true;
       int it = 0;
-      const uint32_t tx = 2u * (uint32_t)(kNW * kWTile + 2 * x_bytes);        // both CTAs' bytes count on the leader's barrier
+      const uint32_t tx = 2u * (uint32_t)(kWTile + 2 * x_bytes);        // both CTAs' bytes count on the leader's barrier
       auto load_w = [&](int stage, int m, int lt, int kb) {
         const uint32_t bar = map_to_cta(smem_u32(&full_b[stage]), 0), dst = base + (uint32_t)(stage * p.stage_bytes);
-        const int row = lt * 2 * kTileM + (int)rank * kTileM;
         if (rank == 0) mbar_expect_tx(smem_u32(&full_b[stage]), tx);
-        tma_load_2d_pair(dst, &maps.w[kDual ? 0 : m], kb * kTileK, row, bar);
-        if (kDual) tma_load_2d_pair(dst + kWTile, &maps.w[1], kb * kTileK, row, bar);
+        if (kMixed) {
+          const int row = lt * kTileM + (int)rank * (kTileM / 2);
+          tma_load_2d_pair(dst, &maps.w[0], kb * kTileK, row, bar);
+          tma_load_2d_pair(dst + kWTile / 2, &maps.w[1], kb * kTileK, row, bar);
+        } else {
+          tma_load_2d_pair(dst, &maps.w[m], kb * kTileK, lt * 2 * kTileM + (int)rank * kTileM, bar);
+        }
       };
       auto load_x = [&](int stage, int rt, int kb) {
-        const uint32_t bar = map_to_cta(smem_u32(&full_b[stage]), 0), dst = base + (uint32_t)(stage * p.stage_bytes + kNW * kWTile);
+        const uint32_t bar = map_to_cta(smem_u32(&full_b[stage]), 0), dst = base + (uint32_t)(stage * p.stage_bytes + kWTile);
         const int row = rt * p.bn + (int)rank * (p.bn >> 1);
         tma_load_2d_pair(dst, &maps.x, kb * kTileK, row, bar);
         tma_load_2d_pair(dst + x_bytes, &maps.x, kb * kTileK, p.pan_rows + row, bar);
@@ -223,25 +245,21 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
           const int acc = seg & 1;
           if (seg >= 2 && !mbar_wait(smem_u32(&tmem_empty[acc]), ((uint32_t)(seg >> 1) - 1u) & 1u, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t d0 = tmem_base + (uint32_t)(acc * 256), d1 = d0 + 128u;
+          const uint32_t d0 = tmem_base + (uint32_t)(acc * 256);
           const int kc1 = min(kc + kAccKb, t.kb1);
           for (int kb = kc; kb < kc1; ++kb, ++it) {
             const int stage = it % S;
             if (!mbar_wait(smem_u32(&full_b[stage]), (uint32_t)(it / S) & 1u, abort_flag)) { ok = false; break; }
             tc_fence_after();
             const uint32_t sb = base + (uint32_t)(stage * p.stage_bytes);
-            const uint64_t a0 = smem_desc_sw128(sb), a1 = smem_desc_sw128(sb + kWTile);
-            const uint64_t bh = smem_desc_sw128(sb + kNW * kWTile), bl = smem_desc_sw128(sb + kNW * kWTile + x_bytes);
+            const uint64_t a0 = smem_desc_sw128(sb);
+            const uint64_t bh = smem_desc_sw128(sb + kWTile), bl = smem_desc_sw128(sb + kWTile + x_bytes);
 #pragma unroll
             for (int kk = 0; kk < kTileK / 16; ++kk) {
               const uint64_t o = (uint64_t)(kk * 2);
               const uint32_t more = (kb > kc || kk > 0) ? 1u : 0u;
               umma_bf16_pair(d0, a0 + o, bh + o, idesc, more);
               umma_bf16_pair(d0, a0 + o, bl + o, idesc, 1u);
-              if (kDual) {
-                umma_bf16_pair(d1, a1 + o, bh + o, idesc, more);
-                umma_bf16_pair(d1, a1 + o, bl + o, idesc, 1u);
-              }
             }
             umma_commit_pair(smem_u32(&empty_b[stage]));
           }
@@ -255,8 +273,11 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
     asm volatile("griddepcontrol.wait;" ::: "memory");            // outputs may still be read by the kernel in front
     const int q = warp & 3, half = (warp - 2) >> 2;               // tensor-memory lanes 32 q .. 32 q + 31; every second block of 16 rows
     const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
-    constexpr int kBlocks = kDual ? 4 : 8;                        // blocks of 16 rows of a tile that this warp holds
-    float sum[kBlocks][kNW][16];
+    constexpr int kBlocks = 8;                                    // blocks of 16 rows of a tile that this warp holds
+    float sum[kBlocks][16];
+    const int duo = half * 2 + (q & 1);                            // BULK_SWIGLU: the two warps of the same columns
+    const bool is_up = q >= 2;
+    float *swap = reinterpret_cast<float *>(smem_dyn + (base - smem_u32(smem_dyn)) + (size_t)S * p.stage_bytes) + duo * 1024;
     Item t;
     int seg = 0;
     bool ok = true;
@@ -267,19 +288,17 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
       for (int kc = t.kb0; kc < t.kb1; kc += kAccKb, ++seg) {
         const int acc = seg & 1;
         ok = mbar_wait_warp(smem_u32(&accum_full[acc]), ((uint32_t)seg >> 1) & 1u, abort_flag);
+        if (kMixed) ok = meet_and(1 + duo, ok);                    // both go on or both leave
         if (!ok) break;
         tc_fence_after();
         const uint32_t t_acc = t_lane + (uint32_t)(acc * 256 + half * 16);
 #pragma unroll
         for (int i = 0; i < kBlocks; ++i) {
           if (i < blocks) {
+            float v[16];
+            tmem_ld16(t_acc + (uint32_t)(i * 32), v);
 #pragma unroll
-            for (int d = 0; d < kNW; ++d) {
-              float v[16];
-              tmem_ld16(t_acc + (uint32_t)(d * 128 + i * 32), v);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) sum[i][d][j] = kc > t.kb0 ? sum[i][d][j] + v[j] : v[j];
-            }
+            for (int j = 0; j < 16; ++j) sum[i][j] = kc > t.kb0 ? sum[i][j] + v[j] : v[j];
           }
         }
         tc_fence_before();
@@ -299,19 +318,25 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
         for (int i = 0; i < kBlocks; ++i)
           if (i < blocks)
 #pragma unroll
-            for (int d = 0; d < kNW; ++d)
-#pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4)
-                __stcg(dst + ((i * kNW + d) * 4 + k4) * 32, make_float4(sum[i][d][4 * k4], sum[i][d][4 * k4 + 1], sum[i][d][4 * k4 + 2], sum[i][d][4 * k4 + 3]));
+            for (int k4 = 0; k4 < 4; ++k4)
+              __stcg(dst + (i * 4 + k4) * 32, make_float4(sum[i][4 * k4], sum[i][4 * k4 + 1], sum[i][4 * k4 + 2], sum[i][4 * k4 + 3]));
         __threadfence();                                           // this lane's piece is visible before the count
         __syncwarp();
+        if (kMixed) meet(1 + duo);                                 // the two warps of a column count as one
         unsigned int before = 0;
-        if (lane == 0) {
-          unsigned int *word = p.arrived + ((size_t)tile * 2 + rank) * kEpiWarps + (warp - 2);
+        if (lane == 0 && !(kMixed && is_up)) {
+          unsigned int *word = p.arrived + ((size_t)tile * 2 + rank) * kEpiWarps + (kMixed ? duo : warp - 2);
+          __threadfence();
           before = atomicAdd(word, 1u);
           if (before == (unsigned int)(to - from)) *word = 0u;     // the last one: nobody else touches it in this launch
+          if (kMixed) last_s[duo] = before;
         }
-        before = __shfl_sync(0xffffffffu, before, 0);
+        if (kMixed) {
+          meet(1 + duo);
+          before = last_s[duo];
+        } else {
+          before = __shfl_sync(0xffffffffu, before, 0);
+        }
         if (before != (unsigned int)(to - from)) continue;
         __threadfence();
         for (int pr = from; pr <= to; ++pr) {
@@ -320,26 +345,22 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
           for (int i = 0; i < kBlocks; ++i)
             if (i < blocks)
 #pragma unroll
-              for (int d = 0; d < kNW; ++d)
-#pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4) {
-                  const float4 x = __ldcg(src + ((i * kNW + d) * 4 + k4) * 32);
-                  float *sd = &sum[i][d][4 * k4];
-                  if (pr == from) { sd[0] = x.x; sd[1] = x.y; sd[2] = x.z; sd[3] = x.w; }
-                  else { sd[0] += x.x; sd[1] += x.y; sd[2] += x.z; sd[3] += x.w; }
-                }
+              for (int k4 = 0; k4 < 4; ++k4) {
+                const float4 x = __ldcg(src + (i * 4 + k4) * 32);
+                float *sd = &sum[i][4 * k4];
+                if (pr == from) { sd[0] = x.x; sd[1] = x.y; sd[2] = x.z; sd[3] = x.w; }
+                else { sd[0] += x.x; sd[1] += x.y; sd[2] += x.z; sd[3] += x.w; }
+              }
         }
       }
       // a lane holds output column n0 + lane for 16 rows of a block; quads are transposed, so that a lane then holds four
       // adjacent columns of rows (lane & 3) + 4 i
-      const int n0 = t.lt * 2 * kTileM + (int)rank * kTileM + q * 32;
+      const int n0 = kMixed ? t.lt * kTileM + (int)rank * (kTileM / 2) + (q & 1) * 32 : t.lt * 2 * kTileM + (int)rank * kTileM + q * 32;
 #pragma unroll
       for (int i = 0; i < kBlocks; ++i) {
         if (i >= blocks) break;
         const int r0 = r_base + i * 32;
-        float (&v)[16] = sum[i][0];
-        float (&w)[16] = sum[i][kNW - 1];
-        (void)w;
+        float (&v)[16] = sum[i];
         if constexpr (EPI == BULK_STORE || EPI == BULK_ADD) {
           float *yb = p.y + p.y_off[m] + n0 + (lane & ~3);
 #pragma unroll
@@ -353,24 +374,31 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
             }
           }
         } else if constexpr (EPI == BULK_SWIGLU) {
-          const int rs = r0 + (lane & 15);
-          const float s_mine = rs < p.R ? rsqrtf(__ldcg(p.ss + rs) / (float)p.dn + p.eps) : 0.f;
+          // the gate warp keeps rows 0-7 of the block and gets their up factors, the up warp rows 8-15 and their gates
+          float *out = swap + (i & 1) * 512 + (is_up ? 256 : 0) + lane, *in = swap + (i & 1) * 512 + (is_up ? 0 : 256) + lane;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
+          for (int j = 0; j < 8; ++j) out[j * 32] = is_up ? v[j] : v[8 + j];
+          const int ra = r0 + (is_up ? 8 : 0), rs = ra + (lane & 7);
+          const float s_mine = rs < p.R ? rsqrtf(__ldcg(p.ss + rs) / (float)p.dn + p.eps) : 0.f;
+          meet(1 + duo);                                           // (two buffers in turn: a block's reader is past it one barrier later)
+          float y[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float other = in[j * 32], own = is_up ? v[8 + j] : v[j];
             const float s = __shfl_sync(0xffffffffu, s_mine, j);
-            const float gt = s * v[j];
-            v[j] = __fdividef(gt, 1.0f + __expf(-gt)) * (s * w[j]);
+            const float gt = s * (is_up ? other : own);
+            y[j] = __fdividef(gt, 1.0f + __expf(-gt)) * (s * (is_up ? own : other));
           }
 #pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4) {
-            quad_transpose(v[4 * k4], v[4 * k4 + 1], v[4 * k4 + 2], v[4 * k4 + 3], lane);
-            const int r = r0 + 4 * k4 + (lane & 3);
+          for (int k4 = 0; k4 < 2; ++k4) {
+            quad_transpose(y[4 * k4], y[4 * k4 + 1], y[4 * k4 + 2], y[4 * k4 + 3], lane);
+            const int r = ra + 4 * k4 + (lane & 3);
             if (r < p.R) {
-              const uint32_t h0 = pack_pair(v[4 * k4], v[4 * k4 + 1]), h1 = pack_pair(v[4 * k4 + 2], v[4 * k4 + 3]);
+              const uint32_t h0 = pack_pair(y[4 * k4], y[4 * k4 + 1]), h1 = pack_pair(y[4 * k4 + 2], y[4 * k4 + 3]);
               __nv_bfloat16 *dst = p.out_pan + (long long)r * p.out_ld + n0 + (lane & ~3);
               *reinterpret_cast<uint2 *>(dst) = make_uint2(h0, h1);
               *reinterpret_cast<uint2 *>(dst + (long long)p.out_rows * p.out_ld) =
-                  make_uint2(pack_pair(v[4 * k4] - lo_of(h0), v[4 * k4 + 1] - hi_of(h0)), pack_pair(v[4 * k4 + 2] - lo_of(h1), v[4 * k4 + 3] - hi_of(h1)));
+                  make_uint2(pack_pair(y[4 * k4] - lo_of(h0), y[4 * k4 + 1] - hi_of(h0)), pack_pair(y[4 * k4 + 2] - lo_of(h1), y[4 * k4 + 3] - hi_of(h1)));
             }
           }
         } else {                                                  // BULK_HEAD: logits, bias, running maximum per row
@@ -439,15 +467,14 @@ cudaError_t launch_norm_pair(const float *x, const void *gain, float *ss, void *
 }
 
 // Rows per tile (a multiple of 32: the N step of a two-CTA MMA) and how the units are dealt.  Cost in tensor cycles: a
-// k-block takes the slower of its MMAs (4 cycles per row and weight tile) and its operand loads (about 56 bytes per cycle and
+// k-block takes the slower of its MMAs (4 cycles per row) and its operand loads (about 56 bytes per cycle and
 // SM out of L2); whole rounds take nkb of them, the shares of what is left over `share`, and pieces that have to be stored
 // and added up about 9000 besides.
-static void bulk_plan(int n_wt, int nkb, int R, int n_pairs, bool dual, bool add, bool may_share, int &bn, int &rounds, int &share) {
-  const int max_bn = dual ? 128 : 256;
+static void bulk_plan(int n_wt, int nkb, int R, int n_pairs, bool add, bool may_share, int &bn, int &rounds, int &share) {
   double best = 0;
-  for (int b = 64; b <= max_bn; b += 32) {
+  for (int b = 64; b <= 256; b += 32) {
     const long long units = (long long)n_wt * ((R + b - 1) / b);
-    const double mma = (dual ? 8.0 : 4.0) * b, load = ((dual ? 2 : 1) * 16384 + b * 128) / 56.0, kb = mma > load ? mma : load;
+    const double mma = 4.0 * b, load = (16384 + b * 128) / 56.0, kb = mma > load ? mma : load;
     const long long whole = units / n_pairs, left = units - whole * n_pairs;
     double cost = (double)(whole + (left > 0)) * nkb * kb;
     int r = (int)(whole + (left > 0)), s = 0;
@@ -488,36 +515,36 @@ cudaError_t launch_bulk_gemm(const UmmaPlan *plan, const BulkArgs &a, int epi, i
   BulkParams p;
   memset(&p, 0, sizeof p);
   int n_rows[kMaxMats], K;
-  umma_plan_view(plan, maps.w, n_rows, p.y_off, p.n_mats, K, p.err);
+  const void *weights[kMaxMats];
+  umma_plan_view(plan, maps.w, weights, n_rows, p.y_off, p.n_mats, K, p.err);
   int n_wt = 0;
   for (int m = 0; m < p.n_mats; ++m) {
     if (n_rows[m] % (2 * kTileM)) return cudaErrorInvalidValue;
     p.n_tiles[m] = n_rows[m] / (2 * kTileM);
     n_wt += p.n_tiles[m];
   }
-  const bool dual = epi == BULK_SWIGLU;
-  if (dual) {
-    if (p.n_mats != 2 || n_rows[0] != n_rows[1]) return cudaErrorInvalidValue;
-    n_wt = p.n_tiles[0];
-  }
+  const bool mixed = epi == BULK_SWIGLU;
+  if (mixed && (p.n_mats != 2 || n_rows[0] != n_rows[1])) return cudaErrorInvalidValue;      // n_wt: tiles of 128 + 128 rows
   if (epi == BULK_HEAD && p.n_mats != 1) return cudaErrorInvalidValue;
   if (a.R < 1 || a.R > a.pan_rows) return cudaErrorInvalidValue;
   const int n_pairs = n_sms / 2;
   p.nkb = (K + kTileK - 1) / kTileK;
   const bool add = epi == BULK_ADD;
-  bulk_plan(n_wt, p.nkb, a.R, n_pairs, dual, add, add || (a.slots && n_pairs <= kBulkPairs), p.bn, p.rounds, p.share);
+  bulk_plan(n_wt, p.nkb, a.R, n_pairs, add, add || (a.slots && n_pairs <= kBulkPairs), p.bn, p.rounds, p.share);
   p.slots = (float4 *)a.slots; p.arrived = a.arrived;
   p.n_rt = (a.R + p.bn - 1) / p.bn;
   const long long units = (long long)n_wt * p.n_rt;
   if (units > 0x3fffffff) return cudaErrorInvalidValue;
   p.n_units = (int)units;
-  p.stage_bytes = (dual ? 2 : 1) * kWTile + p.bn * 128;
-  p.stages = (int)((kBulkSmem - 1024) / p.stage_bytes);
+  p.stage_bytes = kWTile + p.bn * 128;
+  p.stages = (int)((kBulkSmem - 1024 - (mixed ? kSwapBytes : 0)) / p.stage_bytes);
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   cudaError_t e = make_pair_tensor_map(&maps.x, a.pan, a.pan_rows, K, p.bn / 2);
+  // gate and up: boxes of 64 weight rows
+  for (int m = 0; m < 2 && mixed && e == cudaSuccess; ++m) e = make_pair_tensor_map(&maps.w[m], weights[m], n_rows[m] / 2, K, kTileM / 2);
   if (e != cudaSuccess) return e;
   p.R = a.R; p.pan_rows = a.pan_rows; p.y = a.y; p.ldy = a.ldy; p.ss = a.ss; p.eps = a.eps; p.dn = a.dn;
-  p.out_pan = (__nv_bfloat16 *)a.out_pan; p.out_rows = a.pan_rows; p.out_ld = dual ? n_rows[0] : 0;
+  p.out_pan = (__nv_bfloat16 *)a.out_pan; p.out_rows = a.pan_rows; p.out_ld = mixed ? n_rows[0] : 0;
   p.tokens = a.tokens; p.perm = a.perm; p.beta = a.beta; p.amax = a.amax; p.logits = a.logits; p.vocab = n_rows[0];
   // the shares are cut for all pairs; whole units need no more pairs than there are units
   const int grid = 2 * (p.share > 0 || p.n_units > n_pairs ? n_pairs : p.n_units);

@@ -894,9 +894,10 @@ UmmaPlan *umma_plan_create(const GemmArgs &a, int pro, int epi, int n_sms, unsig
 
 void umma_plan_destroy(UmmaPlan *p) { delete p; }
 
-void umma_plan_view(const UmmaPlan *pl, CUtensorMap *maps, int *n_rows, int *y_off, int &n_mats, int &K, unsigned int *&err) {
+void umma_plan_view(const UmmaPlan *pl, CUtensorMap *maps, const void **w, int *n_rows, int *y_off, int &n_mats, int &K, unsigned int *&err) {
   for (int m = 0; m < kMaxMats; ++m) {
     maps[m] = pl->maps[m];
+    w[m] = pl->d.g.w[m];
     n_rows[m] = m < pl->d.g.n_mats ? pl->d.g.n_rows[m] : 0;
     y_off[m] = m < pl->d.g.n_mats ? pl->d.g.y_off[m] : 0;
   }
