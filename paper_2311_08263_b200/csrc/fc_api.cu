@@ -263,8 +263,6 @@ extern "C" void fc_destroy(fc_ctx *ctx) {
   if (!ctx) return;
   destroy_plans(ctx);
   if (ctx->pin) cudaFreeHost(ctx->pin);
-  if (ctx->pin_map) cudaFreeHost(ctx->pin_map);
-  if (ctx->res_count) cudaFreeHost(ctx->res_count);
   if (ctx->ev0) cudaEventDestroy(ctx->ev0);
   if (ctx->ev1) cudaEventDestroy(ctx->ev1);
   delete ctx;
@@ -414,15 +412,16 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
     fprintf(stderr, "fc_init: tensor map over the K/V slab could not be encoded\n");
     return fail(FC_ERR_CUDA);
   }
-  const size_t pin_ints = (size_t)shape->max_batch * (1 + 2 * shape->max_c) + 4;
-  if (cudaMallocHost((void **)&ctx->pin, pin_ints * sizeof(int32_t)) != cudaSuccess) return fail(FC_ERR_CUDA);
-  if (cudaMallocHost((void **)&ctx->pin_map, (size_t)shape->max_batch * sizeof(int32_t)) != cudaSuccess) return fail(FC_ERR_CUDA);
-  const size_t res_ints = (size_t)shape->max_batch * (1 + 2 * shape->max_c) + 1;
-  if (cudaMallocHost((void **)&ctx->res_count, res_ints * sizeof(int32_t)) != cudaSuccess) return fail(FC_ERR_CUDA);
-  memset(ctx->res_count, 0, res_ints * sizeof(int32_t));
-  ctx->res_tokens = ctx->res_count + shape->max_batch;
-  ctx->res_window = ctx->res_tokens + (size_t)shape->max_batch * shape->max_c;
-  ctx->res_err = ctx->res_window + (size_t)shape->max_batch * shape->max_c;
+  // one pinned block: staging, the live sequences of a compacted step, what the accept kernel reports
+  const size_t n_seq = shape->max_batch, n_rows = n_seq * shape->max_c, pin_ints = n_seq + 2 * n_rows + 4;
+  const size_t all_ints = pin_ints + n_seq + (n_seq + 2 * n_rows + 1);
+  if (cudaMallocHost((void **)&ctx->pin, all_ints * sizeof(int32_t)) != cudaSuccess) return fail(FC_ERR_CUDA);
+  memset(ctx->pin, 0, all_ints * sizeof(int32_t));
+  ctx->pin_map = ctx->pin + pin_ints;
+  ctx->res_count = ctx->pin_map + n_seq;
+  ctx->res_tokens = ctx->res_count + n_seq;
+  ctx->res_window = ctx->res_tokens + n_rows;
+  ctx->res_err = ctx->res_window + n_rows;
   ctx->small = shape->dtype == FC_F32 && !(shape->flags & (FC_FLAG_SIMT_GEMM | FC_FLAG_NO_CHAIN)) &&
                small_model_fits(shape->d_model, ctx->d.qd, ctx->d.kvd, shape->d_ffn, shape->head_dim, shape->vocab, L);
   if (cudaEventCreate(&ctx->ev0) != cudaSuccess || cudaEventCreate(&ctx->ev1) != cudaSuccess) return fail(FC_ERR_CUDA);
