@@ -34,8 +34,9 @@ struct Carver {          // hands out aligned slices of the caller's workspace (
 
 constexpr int kPrefillRows = 128;         // rows per forward while a prompt is cached (one 128-row accumulator block)
 constexpr int kBulkRows = 1024;           // the same where the dense GEMMs of k_bulk.cu run
-// Rows from which they run.  Measured, 4 layers of 7B, chained launch against this: 64 rows 649 us, 767; 96 rows 763, 817;
-// 128 rows 857, 860; 256 rows 1250, 1171; 512 rows 2130, 1936.
+// Rows from which they run.  Measured, 4 layers and LM head, K/V 512, chained launch against this: 7B, 64 rows 651 us, 809; 96 rows
+// 759, 880; 128 rows 857, 966; 256 rows (two row blocks of the chain) 1461, 1303; 512 rows 2583, 2175; 13B, 128 rows 1117, 1154;
+// 256 rows over 1024 keys 2141, 1800.
 constexpr int kBulkMin = 129;
 
 constexpr int kSyncClaim = kChainMax, kSyncPanel = 2 * kChainMax, kSyncTd = 3 * kChainMax;   // offsets in a group
