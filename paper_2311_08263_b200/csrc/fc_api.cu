@@ -39,6 +39,12 @@ constexpr int kBulkRows = 1024;           // the same where the dense GEMMs of k
 // 256 rows over 1024 keys 2141, 1800.
 constexpr int kBulkMin = 129;
 
+// Steps of more rows than this add up as the chained launch does (BulkArgs::split): the more rows, the larger the worst of
+// them.  Largest logit difference from the chained launch in units of the logits' rms: 7B, 512 rows, six-block sums 0.0259, split
+// 0.0169, that launch against itself 0.0152 (24 seeds); 13B, 256 rows, six-block sums 0.0150, that launch against itself 0.0212 (5
+// seeds): nothing to gain there.  It costs 3.5 % of the 512-row step (5 % at 256 rows).
+constexpr int kBulkSplit = 256;
+
 constexpr int kSyncClaim = kChainMax, kSyncPanel = 2 * kChainMax, kSyncTd = 3 * kChainMax;   // offsets in a group
 
 struct Buffers {
@@ -548,6 +554,7 @@ static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int m
   BulkArgs ba; memset(&ba, 0, sizeof ba);
   ba.slots = ctx->b.bulk_slots; ba.arrived = ctx->b.bulk_arrived;
   ba.pan_rows = d.bulk_rows; ba.R = R; ba.eps = s.rms_eps; ba.dn = s.d_model;
+  ba.split = with_head && R > kBulkSplit;
   const long long stride_h = (long long)s.max_seq * s.head_dim, stride_b = (long long)s.n_kv_heads * stride_h;
   auto norm = [&](const void *gain, float *ss, int cls) {
     ProfScope ps(ctx, cls);

@@ -289,6 +289,7 @@ struct BulkArgs {
   void *slots;            // bulk_slot_bytes(): pieces of tiles that several pairs work on
   unsigned int *arrived;  // kBulkArrived words, zero before the first launch; every launch leaves them zero
   const int32_t *tokens, *perm; float beta; unsigned long long *amax; float *logits;
+  int split;              // add up as the chained launch does (k_bulk.cu)
 };
 constexpr int kBulkPairs = 80;                       // CTA pairs the slots are laid out for
 constexpr int kBulkArrived = kBulkPairs * 16;        // fewer units than pairs are ever shared; two ranks, eight warps

@@ -17,6 +17,15 @@
 // of 4 layers: chained launch 1.07 / 1.25 / 1.29e-3; whole k range in one accumulator above 1.5e-3; 8 k-blocks 1.09 / 1.32 /
 // 1.28e-3, 1.77 ms; 6: 1.07 / 1.23 / 1.22e-3, 1.82 ms; 4: 1.03 / 1.20 / 1.06e-3, 1.88 ms.
 //
+// Steps of many rows (BulkArgs::split) add up as the chained launch does: a high and a low accumulator over the chained launch's
+// chunks of 16 k-blocks, shares cut between chunks.  Their results differ from that launch's by the order of fp32 additions
+// only.  With other sums the tensor core's rounding differs, which moves more stored K/V values over a bf16 rounding boundary
+// (7.0e-4 of layer 0's instead of 3.4e-5), and one such value moves its row of logits by up to a few per cent.  Largest difference
+// of two steps of 7B from the chained launch, 512 rows, 24 seeds, in units of the logits' rms: six-block sums 0.0259 (median 0.0085),
+// split 0.0169 (0.0041), two runs of the chained launch 0.0152 (0.0022); the distance from 64 bits is the same for all three.  The
+// accumulators cannot alternate then: the high one is added up while the last low products run, and the next chunk waits for
+// the rest (these two steps: six-block sums 30.7 ms, split 31.8, chained launch 35.1).
+//
 // The tiles of a projection seldom are a whole number of rounds over the pairs: whole rounds run tile by tile, the tiles
 // that are left over are dealt as one run of k-blocks, cut into equal shares for all pairs (a share ends in one tile and may
 // begin the next).  The pieces of a tile meet in L2: on the residual as fp32 reductions; elsewhere each piece is
@@ -39,6 +48,7 @@ constexpr int kSwapBytes = 16 * 1024;              // BULK_SWIGLU: four pairs of
 constexpr int kMaxStages = 8;
 constexpr int kWTile = kTileM * kTileK * 2;        // 16 KB: this CTA's 128 weight rows of a k-block
 constexpr int kAccKb = 6;                          // k-blocks an accumulator runs over before it is added up in registers
+constexpr int kSplitKb = 16;                       // the same with a high and a low accumulator: the chunks of the chained launch
 constexpr int kSlotF4 = 1024;                      // one warp's part of a piece: 16 KB
 constexpr size_t kBulkSmem = 225 * 1024;           // ring + alignment; static shared memory takes the rest of 227 KB
 
@@ -51,6 +61,7 @@ struct BulkParams {
   int n_tiles[kMaxMats], n_mats;  // 256-row weight tiles per matrix
   int y_off[kMaxMats];
   int nkb;                        // 64-wide k-blocks
+  int cut_kb;                     // length of a tile in the run that is cut into shares (split: rounded up to whole chunks)
   int n_rt, bn;                   // row tiles, rows per tile
   int n_units;                    // weight tiles x row tiles
   int rounds;                     // rounds of whole units (the last may be partial)
@@ -129,7 +140,7 @@ __global__ void __launch_bounds__(256) norm_pair_kernel(const float *x, const __
 }
 
 // ------------------------------------------------------------------------------------ GEMM
-template <int EPI>
+template <int EPI, bool SPLIT>
 __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid_constant__ BulkMaps maps, const __grid_constant__ BulkParams p) {
   constexpr bool kMixed = EPI == BULK_SWIGLU;                     // a CTA's weight rows: 64 of gate, 64 of up
   extern __shared__ unsigned char smem_dyn[];
@@ -168,10 +179,10 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
       if (t.u >= p.n_units) return false;
       t.kb0 = 0; t.kb1 = p.nkb;
     } else {
-      const int g0 = pair * p.share, g1 = min(g0 + p.share, (p.n_units - p.rounds * n_pairs) * p.nkb);
-      const int tile = g0 / p.nkb + (n - p.rounds);
-      t.kb0 = max(0, g0 - tile * p.nkb);
-      t.kb1 = min(p.nkb, g1 - tile * p.nkb);
+      const int g0 = pair * p.share, g1 = min(g0 + p.share, (p.n_units - p.rounds * n_pairs) * p.cut_kb);
+      const int tile = g0 / p.cut_kb + (n - p.rounds);
+      t.kb0 = max(0, g0 - tile * p.cut_kb);
+      t.kb1 = min(p.nkb, g1 - tile * p.cut_kb);
       if (p.share == 0 || t.kb0 >= t.kb1) return false;
       t.u = p.rounds * n_pairs + tile;
     }
@@ -182,6 +193,8 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
       while (t.m + 1 < p.n_mats && t.lt >= p.n_tiles[t.m]) { t.lt -= p.n_tiles[t.m]; ++t.m; }
     return true;
   };
+  // Accumulations [kc, acc_end) of an item.  Use u of an accumulator is in buffer u & 1; split: 2 n and 2 n + 1 run side by side.
+  auto acc_end = [&](int kc, int kb1) { return min(SPLIT ? (kc / kSplitKb + 1) * kSplitKb : kc + kAccKb, kb1); };
   const uint32_t x_bytes = (uint32_t)p.bn * 64u;                  // one half (high or low) of this CTA's bn / 2 activation rows
   int issued = 0;
 
@@ -237,16 +250,19 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
       bool ok = true;
-      int it = 0, seg = 0;
+      int it = 0, uses = 0;
+      auto drained = [&](int u) {                                  // buffer u & 1 has been added up since its last use
+        if (u >= 2 && !mbar_wait(smem_u32(&tmem_empty[u & 1]), ((uint32_t)(u >> 1) - 1u) & 1u, abort_flag)) return false;
+        tc_fence_after();
+        return true;
+      };
       const uint32_t idesc = make_idesc(p.bn, 2 * kTileM);
       Item t;
       for (int n = 0; ok && item(n, t); ++n)
-        for (int kc = t.kb0; kc < t.kb1 && ok; kc += kAccKb, ++seg) {
-          const int acc = seg & 1;
-          if (seg >= 2 && !mbar_wait(smem_u32(&tmem_empty[acc]), ((uint32_t)(seg >> 1) - 1u) & 1u, abort_flag)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t d0 = tmem_base + (uint32_t)(acc * 256);
-          const int kc1 = min(kc + kAccKb, t.kb1);
+        for (int kc = t.kb0, kc1; kc < t.kb1 && ok; kc = kc1, uses += SPLIT ? 2 : 1) {
+          kc1 = acc_end(kc, t.kb1);
+          if (!drained(uses)) { ok = false; break; }
+          const uint32_t d0 = tmem_base + (uint32_t)((uses & 1) * 256);
           for (int kb = kc; kb < kc1; ++kb, ++it) {
             const int stage = it % S;
             if (!mbar_wait(smem_u32(&full_b[stage]), (uint32_t)(it / S) & 1u, abort_flag)) { ok = false; break; }
@@ -254,20 +270,31 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
             const uint32_t sb = base + (uint32_t)(stage * p.stage_bytes);
             const uint64_t a0 = smem_desc_sw128(sb);
             const uint64_t bh = smem_desc_sw128(sb + kWTile), bl = smem_desc_sw128(sb + kWTile + x_bytes);
+            if constexpr (SPLIT) {
 #pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk) {
-              const uint64_t o = (uint64_t)(kk * 2);
-              const uint32_t more = (kb > kc || kk > 0) ? 1u : 0u;
-              umma_bf16_pair(d0, a0 + o, bh + o, idesc, more);
-              umma_bf16_pair(d0, a0 + o, bl + o, idesc, 1u);
+              for (int kk = 0; kk < kTileK / 16; ++kk)
+                umma_bf16_pair(d0, a0 + (uint64_t)(kk * 2), bh + (uint64_t)(kk * 2), idesc, (kb > kc || kk > 0) ? 1u : 0u);
+              if (kb + 1 == kc1) umma_commit_pair(smem_u32(&accum_full[0]));
+              if (kb == kc && !drained(uses + 1)) { ok = false; break; }
+#pragma unroll
+              for (int kk = 0; kk < kTileK / 16; ++kk)
+                umma_bf16_pair(d0 + 256, a0 + (uint64_t)(kk * 2), bl + (uint64_t)(kk * 2), idesc, (kb > kc || kk > 0) ? 1u : 0u);
+            } else {
+#pragma unroll
+              for (int kk = 0; kk < kTileK / 16; ++kk) {
+                const uint64_t o = (uint64_t)(kk * 2);
+                const uint32_t more = (kb > kc || kk > 0) ? 1u : 0u;
+                umma_bf16_pair(d0, a0 + o, bh + o, idesc, more);
+                umma_bf16_pair(d0, a0 + o, bl + o, idesc, 1u);
+              }
             }
             umma_commit_pair(smem_u32(&empty_b[stage]));
           }
-          if (ok) umma_commit_pair(smem_u32(&accum_full[acc]));
+          if (ok) umma_commit_pair(smem_u32(&accum_full[(uses + SPLIT) & 1]));
         }
-      // the peer's epilogue warps arrive on this CTA's accumulator barriers: wait for the last two rounds
-      for (int sg = (seg > 2 ? seg - 2 : 0); sg < seg && ok; ++sg)
-        ok = mbar_wait(smem_u32(&tmem_empty[sg & 1]), ((uint32_t)sg >> 1) & 1u, abort_flag);
+      // the peer's epilogue warps arrive on this CTA's accumulator barriers: wait for the last two uses
+      for (int u = (uses > 2 ? uses - 2 : 0); u < uses && ok; ++u)
+        ok = mbar_wait(smem_u32(&tmem_empty[u & 1]), ((uint32_t)u >> 1) & 1u, abort_flag);
     }
   } else {
     asm volatile("griddepcontrol.wait;" ::: "memory");            // outputs may still be read by the kernel in front
@@ -279,38 +306,41 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_gemm_kernel(const __grid
     const bool is_up = q >= 2;
     float *swap = reinterpret_cast<float *>(smem_dyn + (base - smem_u32(smem_dyn)) + (size_t)S * p.stage_bytes) + duo * 1024;
     Item t;
-    int seg = 0;
+    int use = 0;
     bool ok = true;
     for (int n = 0; item(n, t); ++n) {
       const int m = t.m;
       const int r_base = t.rt * p.bn + half * 16;                  // first row of block 0
       const int blocks = min((p.bn - half * 16 + 31) >> 5, (p.R - r_base + 31) >> 5);      // blocks with rows in them
-      for (int kc = t.kb0; kc < t.kb1; kc += kAccKb, ++seg) {
-        const int acc = seg & 1;
-        ok = mbar_wait_warp(smem_u32(&accum_full[acc]), ((uint32_t)seg >> 1) & 1u, abort_flag);
+      for (int kc = t.kb0, low = 0; kc < t.kb1; ++use) {
+        const int acc = use & 1;
+        ok = mbar_wait_warp(smem_u32(&accum_full[acc]), ((uint32_t)use >> 1) & 1u, abort_flag);
         if (kMixed) ok = meet_and(1 + duo, ok);                    // both go on or both leave
         if (!ok) break;
         tc_fence_after();
         const uint32_t t_acc = t_lane + (uint32_t)(acc * 256 + half * 16);
+        const bool more = kc > t.kb0 || low;
 #pragma unroll
         for (int i = 0; i < kBlocks; ++i) {
           if (i < blocks) {
             float v[16];
             tmem_ld16(t_acc + (uint32_t)(i * 32), v);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) sum[i][j] = kc > t.kb0 ? sum[i][j] + v[j] : v[j];
+            for (int j = 0; j < 16; ++j) sum[i][j] = more ? sum[i][j] + v[j] : v[j];
           }
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&tmem_empty[acc]), 0));
+        if (SPLIT && !low) low = 1;                              // the low products of the same chunk
+        else { kc = acc_end(kc, t.kb1); low = 0; }
       }
       if (!ok) break;
       if (EPI != BULK_ADD && (t.kb0 > 0 || t.kb1 < p.nkb)) {       // a piece of a tile
         const int tile = t.u - p.rounds * n_pairs;
-        const int from = tile * p.nkb / p.share, to = ((tile + 1) * p.nkb - 1) / p.share;      // the pairs that hold its pieces
+        const int from = tile * p.cut_kb / p.share, to = ((tile + 1) * p.cut_kb - 1) / p.share;      // the pairs that hold its pieces
         auto slot_of = [&](int pr) -> float4 * {
-          const int second = pr * p.share / p.nkb != tile;
+          const int second = pr * p.share / p.cut_kb != tile;
           return p.slots + ((size_t)((pr * 2 + second) * 2 + (int)rank) * kEpiWarps + (warp - 2)) * kSlotF4 + lane;
         };
         float4 *dst = slot_of(pair);
@@ -470,7 +500,9 @@ cudaError_t launch_norm_pair(const float *x, const void *gain, float *ss, void *
 // k-block takes the slower of its MMAs (4 cycles per row) and its operand loads (about 56 bytes per cycle and
 // SM out of L2); whole rounds take nkb of them, the shares of what is left over `share`, and pieces that have to be stored
 // and added up about 9000 besides.
-static void bulk_plan(int n_wt, int nkb, int R, int n_pairs, bool add, bool may_share, int &bn, int &rounds, int &share) {
+// The shares are whole groups of four k-blocks; with split accumulators, whole chunks of them.
+static void bulk_plan(int n_wt, int nkb, int R, int n_pairs, bool add, bool may_share, bool split, int &bn, int &rounds, int &share) {
+  const int unit = split ? kSplitKb : 4;
   double best = 0;
   for (int b = 64; b <= 256; b += 32) {
     const long long units = (long long)n_wt * ((R + b - 1) / b);
@@ -479,7 +511,8 @@ static void bulk_plan(int n_wt, int nkb, int R, int n_pairs, bool add, bool may_
     double cost = (double)(whole + (left > 0)) * nkb * kb;
     int r = (int)(whole + (left > 0)), s = 0;
     if (left > 0 && may_share) {
-      const int per = (int)(((left * nkb + n_pairs - 1) / n_pairs + 3) / 4 * 4);       // whole groups of four k-blocks
+      const long long run = left * (split ? (nkb + unit - 1) / unit * unit : nkb);
+      const int per = (int)(((run + n_pairs - 1) / n_pairs + unit - 1) / unit * unit);
       const double c = (whole * (double)nkb + per) * kb + (add ? 2000.0 + 4.0 * b : 9000.0);
       if (per < nkb && c < cost) { cost = c; r = (int)whole; s = per; }
     }
@@ -489,12 +522,12 @@ static void bulk_plan(int n_wt, int nkb, int R, int n_pairs, bool add, bool may_
   }
 }
 
-template <int EPI>
+template <int EPI, bool SPLIT>
 static cudaError_t launch_bulk_t(const BulkMaps &maps, const BulkParams &p, int grid, int pdl, cudaStream_t st) {
   static bool attr_done[kMaxDevices] = {false};
   const int dev = current_device_slot();
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(bulk_gemm_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBulkSmem);
+    cudaError_t e = cudaFuncSetAttribute(bulk_gemm_kernel<EPI, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBulkSmem);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -507,7 +540,7 @@ static cudaError_t launch_bulk_t(const BulkMaps &maps, const BulkParams &p, int 
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, bulk_gemm_kernel<EPI>, maps, p);
+  return cudaLaunchKernelEx(&cfg, bulk_gemm_kernel<EPI, SPLIT>, maps, p);
 }
 
 cudaError_t launch_bulk_gemm(const UmmaPlan *plan, const BulkArgs &a, int epi, int n_sms, int pdl, cudaStream_t st) {
@@ -529,8 +562,9 @@ cudaError_t launch_bulk_gemm(const UmmaPlan *plan, const BulkArgs &a, int epi, i
   if (a.R < 1 || a.R > a.pan_rows) return cudaErrorInvalidValue;
   const int n_pairs = n_sms / 2;
   p.nkb = (K + kTileK - 1) / kTileK;
+  p.cut_kb = a.split ? (p.nkb + kSplitKb - 1) / kSplitKb * kSplitKb : p.nkb;
   const bool add = epi == BULK_ADD;
-  bulk_plan(n_wt, p.nkb, a.R, n_pairs, add, add || (a.slots && n_pairs <= kBulkPairs), p.bn, p.rounds, p.share);
+  bulk_plan(n_wt, p.nkb, a.R, n_pairs, add, add || (a.slots && n_pairs <= kBulkPairs), a.split != 0, p.bn, p.rounds, p.share);
   p.slots = (float4 *)a.slots; p.arrived = a.arrived;
   p.n_rt = (a.R + p.bn - 1) / p.bn;
   const long long units = (long long)n_wt * p.n_rt;
@@ -549,10 +583,10 @@ cudaError_t launch_bulk_gemm(const UmmaPlan *plan, const BulkArgs &a, int epi, i
   // the shares are cut for all pairs; whole units need no more pairs than there are units
   const int grid = 2 * (p.share > 0 || p.n_units > n_pairs ? n_pairs : p.n_units);
   switch (epi) {
-    case BULK_STORE: return launch_bulk_t<BULK_STORE>(maps, p, grid, pdl, st);
-    case BULK_ADD: return launch_bulk_t<BULK_ADD>(maps, p, grid, pdl, st);
-    case BULK_SWIGLU: return launch_bulk_t<BULK_SWIGLU>(maps, p, grid, pdl, st);
-    case BULK_HEAD: return launch_bulk_t<BULK_HEAD>(maps, p, grid, pdl, st);
+    case BULK_STORE: return a.split ? launch_bulk_t<BULK_STORE, true>(maps, p, grid, pdl, st) : launch_bulk_t<BULK_STORE, false>(maps, p, grid, pdl, st);
+    case BULK_ADD: return a.split ? launch_bulk_t<BULK_ADD, true>(maps, p, grid, pdl, st) : launch_bulk_t<BULK_ADD, false>(maps, p, grid, pdl, st);
+    case BULK_SWIGLU: return a.split ? launch_bulk_t<BULK_SWIGLU, true>(maps, p, grid, pdl, st) : launch_bulk_t<BULK_SWIGLU, false>(maps, p, grid, pdl, st);
+    case BULK_HEAD: return a.split ? launch_bulk_t<BULK_HEAD, true>(maps, p, grid, pdl, st) : launch_bulk_t<BULK_HEAD, false>(maps, p, grid, pdl, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -3,9 +3,10 @@ sequences, steps whose rows end inside a row tile, grouped queries, both head si
 test_gpu_full_configs."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
-from paper_2311_08263_b200 import engine, workload as wl
+from paper_2311_08263_b200 import engine, lib as _l, workload as wl
 from test_gpu_full_configs import _check_step, _random_kv_case
 
 pytestmark = pytest.mark.gpu
@@ -65,3 +66,26 @@ def test_packed_prompts(hq, hkv, hd, lens):
                 assert np.mean(got != ref) < 0.01
         o.close()
     assert dec.fc_debug_check_guards() == 0
+
+
+def test_step_of_more_than_256_rows_adds_up_as_the_chained_launch():
+    """The same step through the dense GEMMs and through the chained launch: layer 0's new K/V rows come from the same embedding
+    rows, so they differ only where an fp32 sum lies so near a bf16 rounding boundary that the order of its few additions
+    decides: some 2^-24 roundings against steps of 2^-8, 3 to 6 in 100000 (measured 3.4e-5).  Sums over other runs of k-blocks
+    add the tensor core's own rounding: 7.0e-4 with six k-blocks per accumulator."""
+    B, c = 9, 33
+    cfg = wl.small_config(n_layers=2, n_heads=16, n_kv_heads=16, head_dim=128, d_model=2048, d_ffn=4864, vocab=1024, seed=811)
+    w = wl.make_weights(cfg, device="cuda")
+    window = wl.make_random_window(cfg, B, c).numpy()
+    lens = [40 + 3 * b for b in range(B)]
+    rows = []
+    for flags in (0, _l.FC_FLAG_NO_CTA_PAIRS):
+        dec = engine.Decoder(cfg, w, B, c, max(lens) + c, flags=flags)
+        kv = dec.kv_view()
+        kv.copy_(wl.make_random_kv(cfg, kv.numel(), device="cuda").view(kv.shape))
+        dec.fc_debug_set_state(lens, window[:, 0], c)
+        dec.fc_jacobi_step(window)
+        assert dec.fc_last_launch_count() == (8 if flags == 0 else 2) * cfg.n_layers + 4
+        rows.append(torch.stack([kv[0, :, b, :, lens[b]:lens[b] + c] for b in range(B)]).float())
+        assert dec.fc_debug_check_guards() == 0
+    assert float((rows[0] != rows[1]).float().mean()) < 2e-4
