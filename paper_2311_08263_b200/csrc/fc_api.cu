@@ -63,8 +63,8 @@ struct Buffers {
 
 struct Dims {
   int rmax;        // rows of a decode step: max_batch * max_c
-  int rows_ws;     // rows the activation buffers hold: a decode step or a prefill block, whichever is larger
-  int qd, kvd, ldq, nsplit_max, tk, pan_rows, bulk_rows, pan_k, sync_words, q_tiles;
+  int rows_ws;     // rows the activation buffers hold: a decode step or a block of prompts, whichever is larger
+  int qd, kvd, ldq, nsplit_max, tk, pan_rows, pan_k, sync_words, q_tiles;
   bool bulk;       // the shape takes the dense GEMMs from kBulkMin rows
   int rows_chain;  // rows the buffers of the chained launch hold
   size_t esz;
@@ -99,6 +99,7 @@ Dims dims_of(const fc_model_shape *s) {
     const long long all = ((long long)s->max_batch * s->max_seq + 127) / 128 * 128;       // no prompt block is larger
     const int blk = all < kBulkRows ? (int)all : kBulkRows;
     if (d.rows_ws < blk) d.rows_ws = blk;
+    d.rows_ws = (d.rows_ws + 127) / 128 * 128;            // whole tiles: a block of prompts fills every buffer and no more
   }
   d.qd = s->n_heads * s->head_dim;
   d.q_tiles = (int)attn_stream_q_tiles(d.rows_ws, s->n_heads / s->n_kv_heads, s->max_batch);
@@ -109,7 +110,6 @@ Dims dims_of(const fc_model_shape *s) {
   d.esz = s->dtype == FC_F32 ? 4 : 2;
   // beyond 16 rows the tensor-core projections read their activations from a bf16 high/low panel
   d.pan_rows = (d.rows_chain + 127) / 128 * 128;
-  d.bulk_rows = (d.rows_ws + 127) / 128 * 128;
   d.pan_k = s->d_model > s->d_ffn ? s->d_model : s->d_ffn;
   if (d.qd > d.pan_k) d.pan_k = d.qd;
   // per-layer group of synchronisation words: grid barriers 0..5, work-claim counters 6..11, panel-ready barriers
@@ -139,9 +139,9 @@ size_t carve(const fc_model_shape *s, char *base, Buffers *b, std::vector<size_t
   t.ss_final = c.take<float>(R);
   t.chain_bar = c.take<unsigned int>(((size_t)s->n_layers + 1) * d.sync_words); c.guard();
   const size_t pan_chain = (size_t)2 * d.pan_rows * d.pan_k * 2;
-  const size_t pan_bulk = d.bulk ? (size_t)2 * d.bulk_rows * (s->d_model > d.qd ? s->d_model : d.qd) * 2 : 0;
+  const size_t pan_bulk = d.bulk ? (size_t)2 * R * (s->d_model > d.qd ? s->d_model : d.qd) * 2 : 0;
   t.pan = c.take<char>(pan_chain > pan_bulk ? pan_chain : pan_bulk); c.guard();
-  t.pan_ffn = c.take<char>(d.bulk ? (size_t)2 * d.bulk_rows * s->d_ffn * 2 : 0); c.guard();
+  t.pan_ffn = c.take<char>(d.bulk ? (size_t)2 * R * s->d_ffn * 2 : 0); c.guard();
   t.bulk_slots = c.take<char>(d.bulk ? bulk_slot_bytes() : 0); c.guard();
   t.bulk_arrived = c.take<unsigned int>(d.bulk ? kBulkArrived : 0); c.guard();
   // split-KV partials of the FMA attention kernel
@@ -545,6 +545,7 @@ static int forward_small(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, con
 static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int max_rows, int max_len, const int32_t *tokens, bool with_head) {
   const fc_model_shape &s = ctx->s;
   const Dims &d = ctx->d;
+  if (R < 1 || R > d.rows_ws) return FC_ERR_CAPACITY;
   const int pdl = ctx->pdl && !ctx->prof;
   EmbedArgs ea; memset(&ea, 0, sizeof ea);
   ea.tokens = tokens; ea.emb = ctx->tok_emb; ea.x = ctx->b.x; ea.R = R; ea.d = s.d_model;
@@ -553,13 +554,13 @@ static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int m
   { ProfScope ps(ctx, FC_CLS_EMBED); FC_CK(launch_embed(ea, s.dtype, ctx->st)); }
   BulkArgs ba; memset(&ba, 0, sizeof ba);
   ba.slots = ctx->b.bulk_slots; ba.arrived = ctx->b.bulk_arrived;
-  ba.pan_rows = d.bulk_rows; ba.R = R; ba.eps = s.rms_eps; ba.dn = s.d_model;
+  ba.pan_rows = d.rows_ws; ba.R = R; ba.eps = s.rms_eps; ba.dn = s.d_model;
   ba.split = with_head && R > kBulkSplit;
   const long long stride_h = (long long)s.max_seq * s.head_dim, stride_b = (long long)s.n_kv_heads * stride_h;
   auto norm = [&](const void *gain, float *ss, int cls) {
     ProfScope ps(ctx, cls);
     ++ctx->launches;
-    return launch_norm_pair(ctx->b.x, gain, ss, ctx->b.pan, d.bulk_rows, R, s.d_model, pdl, ctx->st);
+    return launch_norm_pair(ctx->b.x, gain, ss, ctx->b.pan, d.rows_ws, R, s.d_model, pdl, ctx->st);
   };
   auto gemm = [&](const UmmaPlan *plan, int epi, int cls) {
     ProfScope ps(ctx, cls);
@@ -582,7 +583,7 @@ static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int m
     StreamAttnArgs sa; memset(&sa, 0, sizeof sa);
     sa.q = ctx->b.qb; sa.q_tiles = d.q_tiles; sa.kv_len = ctx->b.kv_len; sa.segs = segs; sa.hq = s.n_heads; sa.hkv = s.n_kv_heads;
     sa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; sa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
-    sa.err = ctx->b.err; sa.out_pan = ctx->b.pan; sa.pan_rows = d.bulk_rows; sa.pdl = pdl;
+    sa.err = ctx->b.err; sa.out_pan = ctx->b.pan; sa.pan_rows = d.rows_ws; sa.pdl = pdl;
     ++ctx->launches;
     { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_stream(ctx->kv_map_stream, sa, nseg, max_rows, max_len, s.head_dim, ctx->n_sms, ctx->st)); }
     ba.y = ctx->b.x; ba.ldy = s.d_model;
@@ -789,13 +790,13 @@ static int check_device_error(fc_ctx *ctx) {
 // The prompts of a batch one behind the other (n_all rows), cut into as few blocks as the buffers allow, of nearly equal
 // size and, but for the last, whole 128-row tiles.
 static int prefill_packed(fc_ctx *ctx, int batch, const int32_t *prompt_lens, long long n_all) {
-  const long long n_blk = (n_all + ctx->d.bulk_rows - 1) / ctx->d.bulk_rows;
+  const long long n_blk = (n_all + ctx->d.rows_ws - 1) / ctx->d.rows_ws;
   int b = 0, at = 0, blk_no = 0;                                      // next row: id `at` of prompt b
   while (b < batch) {
     RowSegs segs; memset(&segs, 0, sizeof segs);
     int R = 0, max_rows = 0, max_len = 0;
     const long long tiles = (n_all + 127) / 128;           // block i: tiles [i * tiles / n_blk, (i + 1) * tiles / n_blk)
-    const int blk = blk_no < n_blk ? (int)((blk_no + 1) * tiles / n_blk - blk_no * tiles / n_blk) * 128 : ctx->d.bulk_rows;
+    const int blk = blk_no < n_blk ? (int)((blk_no + 1) * tiles / n_blk - blk_no * tiles / n_blk) * 128 : ctx->d.rows_ws;
     ++blk_no;
     while (b < batch && R < blk && segs.n < kMaxSegs) {
       const int n = prompt_lens[b] - 1 - at;

@@ -84,3 +84,20 @@ def test_init_rejects_bad_arguments_before_touching_the_device(cdll):
     cdll.fc_destroy(None)                                          # destroying nothing is allowed
     cdll.fc_last_launch_count.restype = C.c_int64
     assert cdll.fc_last_launch_count(None) == 0
+
+
+@pytest.mark.parametrize("rows", [(17, 64), (33, 32), (40, 30), (21, 50)])
+def test_workspace_of_the_dense_route_holds_whole_row_tiles(cdll, rows):
+    """Blocks of prompts are whole 128-row tiles up to the capacity, so a capacity that is no multiple of 128 needs the
+    activation buffers of the next one: what one more row costs is then no row of the residual and the QKV buffer."""
+    cdll.fc_workspace_bytes.restype = C.c_size_t
+    batch, c = rows
+    full = (batch * c + 127) // 128 * 128
+    bulk = dict(dtype=lib.FC_BF16, d_model=512, n_heads=8, n_kv_heads=8, head_dim=64, d_ffn=512, vocab=1024, max_c=1, max_seq=80)
+    got = [cdll.fc_workspace_bytes(C.byref(_shape(**bulk, max_batch=n))) for n in (batch * c, full)]
+    # per sequence and row of the step: window, accepted tokens, argmax, state words, the prompt and the output ids
+    per_seq = 4 * 12 + 2 * 4 * 80 + 4 * bulk["n_kv_heads"] + 16 * 64 * 4 * bulk["n_kv_heads"]      # and a query tile per kv head
+    slack = 256 * 16
+    assert got[0] <= got[1] <= got[0] + (full - batch * c) * per_seq + slack
+    row = 4 * (512 + 3 * 512)
+    assert (full - batch * c) * row > slack

@@ -89,3 +89,35 @@ def test_step_of_more_than_256_rows_adds_up_as_the_chained_launch():
         rows.append(torch.stack([kv[0, :, b, :, lens[b]:lens[b] + c] for b in range(B)]).float())
         assert dec.fc_debug_check_guards() == 0
     assert float((rows[0] != rows[1]).float().mean()) < 2e-4
+
+
+@pytest.mark.parametrize("batch,c,short,last", [(17, 64, 69, 65), (33, 32, 36, 33)])
+def test_packed_prompts_when_the_step_capacity_is_no_whole_tile(batch, c, short, last):
+    """17 x 64 = 1088 and 33 x 32 = 1056 rows of a step, prompts of 1152 ids in one block: its last rows are beyond what a step
+    uses.  The sequences that hold them, and the first, against the oracle."""
+    cfg = _cfg(8, 8, 64, seed=900 + c, prompt_len=short)
+    lens = [short] * (batch - 1) + [last]
+    assert sum(lens) - batch == 1152
+    w = wl.make_weights(cfg)
+    ids, _ = wl.make_prompts(cfg, batch=batch, lens=lens)
+    max_seq = short + 2 * c
+    dec = engine.Decoder(cfg, w, batch, c, max_seq)
+    dec.fc_prefill(ids.numpy(), lens, c)
+    kv = dec.kv_view().float().cpu().numpy()
+    logits = dec.fc_debug_logits(True)
+    cnt, tok, win = dec.fc_jacobi_step()
+    lg = logits.cpu().numpy().reshape(batch, c, cfg.vocab)
+    for b in (0, batch - 3, batch - 2, batch - 1):
+        P = lens[b]
+        o = oracle.Oracle(cfg, w, max_seq)
+        o.prefill(ids[b, :P].numpy(), c)
+        window = np.array([ids[b, P - 1]] + [ids[b, (j - 1) % P] for j in range(1, c)], np.int32)
+        k_ref, acc_ref, win_ref, lg_ref = o.jacobi_step(want_logits=True)
+        _check_step(lg[b], lg_ref, window, cnt[b], tok[b], win[b], k_ref, acc_ref, win_ref)
+        for layer in range(cfg.n_layers):
+            for half, ref in enumerate(o.get_kv(layer, P - 1)):
+                got = kv[layer, half, b, :, :P - 1].transpose(1, 0, 2).reshape(P - 1, -1)
+                # bf16 steps (2^-8) here and there; layer 1 has one attention over such values in front of it
+                assert np.linalg.norm(got - ref) < 2.0 ** -8 * np.linalg.norm(ref)
+        o.close()
+    assert dec.fc_debug_check_guards() == 0
