@@ -94,7 +94,9 @@ size_t fc_workspace_bytes(const fc_model_shape *shape);
  * shape, weights: host structs (copied).  kv, ws: device, >= the sizes above,
  * 256-byte aligned.  cuda_stream: a cudaStream_t (NULL = default stream).  Shape limits:
  * head_dim in {32, 64, 128}; n_heads % n_kv_heads == 0; d_model, d_ffn, n_heads*head_dim multiples of 8;
- * max_c <= 64.  The bf16 tensor-core path needs an sm_100a device; FC_F32 runs on FMA kernels. */
+ * max_c <= 64.  The bf16 tensor-core path needs an sm_100a device, and its matrices and gains on 16-byte boundaries
+ * (else FC_ERR_CUDA, FC_ERR_ARG); FC_F32 runs on FMA kernels.  All other weights need the alignment of their element type:
+ * embedding tables are read in wider pieces, and a small fp32 model's forward runs as one kernel, where all are 16-byte aligned. */
 int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weights *weights,
             void *kv, size_t kv_bytes, void *ws, size_t ws_bytes, void *cuda_stream);
 

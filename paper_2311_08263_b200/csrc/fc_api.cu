@@ -347,6 +347,14 @@ static GemmArgs args_head(const fc_ctx *c) {
   return a;
 }
 
+// Whether every weight may be read 16 bytes at a time (matrix rows and gains are whole multiples of that).
+static bool wide_weights(const fc_ctx *c) {
+  uintptr_t all = (uintptr_t)c->tok_emb | (uintptr_t)c->g_final | (uintptr_t)c->lm_head;
+  for (const auto *v : {&c->wq, &c->wk, &c->wv, &c->wo, &c->w_gate, &c->w_up, &c->w_down, &c->g_attn, &c->g_ffn})
+    for (const void *p : *v) all |= (uintptr_t)p;
+  return all % 16 == 0;
+}
+
 extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weights *w, void *kv, size_t kv_bytes,
                        void *ws, size_t ws_bytes, void *cuda_stream) {
   if (!out || !shape || !w || !kv || !ws) return FC_ERR_ARG;
@@ -391,6 +399,8 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
   if (ctx->use_umma) {
     if (prop.major != 10) return fail(FC_ERR_SHAPE);
     if (shape->d_model < 64 || shape->d_ffn < 64 || ctx->d.qd < 64) return fail(FC_ERR_SHAPE);
+    for (int l = 0; l < L; ++l)
+      if (((uintptr_t)ctx->g_attn[l] | (uintptr_t)ctx->g_ffn[l] | (uintptr_t)ctx->g_final) % 16) return fail(FC_ERR_ARG);
     char msg[200];
     // halves of d_ffn must be whole 128-row tiles (and so whole 64-wide k-blocks of the down projection)
     // and long enough phases to hide a barrier: at least four chunks (128 rows x 4 k-blocks) of gate and up per CTA.
@@ -429,7 +439,7 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
   ctx->res_tokens = ctx->res_count + n_seq;
   ctx->res_window = ctx->res_tokens + n_rows;
   ctx->res_err = ctx->res_window + n_rows;
-  ctx->small = shape->dtype == FC_F32 && !(shape->flags & (FC_FLAG_SIMT_GEMM | FC_FLAG_NO_CHAIN)) &&
+  ctx->small = shape->dtype == FC_F32 && !(shape->flags & (FC_FLAG_SIMT_GEMM | FC_FLAG_NO_CHAIN)) && wide_weights(ctx) &&
                small_model_fits(shape->d_model, ctx->d.qd, ctx->d.kvd, shape->d_ffn, shape->head_dim, shape->vocab, L);
   if (cudaEventCreate(&ctx->ev0) != cudaSuccess || cudaEventCreate(&ctx->ev1) != cudaSuccess) return fail(FC_ERR_CUDA);
   if (cudaMemsetAsync(ws, 0, fc_workspace_bytes(shape), ctx->st) != cudaSuccess) return fail(FC_ERR_CUDA);

@@ -43,9 +43,11 @@ __device__ __forceinline__ unsigned long long pack_max(float v, int idx) {
 }
 
 // ------------------------------------------------------------------------------------ embed
-// A block takes whole rows, a thread eight elements at a time (d is a multiple of 8).
+// A block takes whole rows, a thread eight elements at a time (d is a multiple of 8); element by element from a table whose
+// address does not allow loads of four.
 template <typename T>
 __global__ void embed_kernel(const __grid_constant__ EmbedArgs a) {
+  const bool wide = ((unsigned long long)a.emb & (4 * sizeof(T) - 1)) == 0;
   for (int r = blockIdx.x; r < a.R; r += gridDim.x) {
     int tok;
     if (a.segs.n > 0) {
@@ -61,7 +63,10 @@ __global__ void embed_kernel(const __grid_constant__ EmbedArgs a) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         float4 v;
-        if constexpr (sizeof(T) == 4) {
+        if (!wide) {
+          const T *e = src + k + 4 * h;
+          v = make_float4(to_f32(e[0]), to_f32(e[1]), to_f32(e[2]), to_f32(e[3]));
+        } else if constexpr (sizeof(T) == 4) {
           v = *reinterpret_cast<const float4 *>(src + k + 4 * h);
         } else {
           const uint2 w = *reinterpret_cast<const uint2 *>(src + k + 4 * h);

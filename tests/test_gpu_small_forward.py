@@ -3,6 +3,7 @@ than warps, all head sizes, grouped queries, batches, keys beyond one block per 
 kernels.  fp32 on both sides, sums in other orders: logits within 2e-4, streams and accept decisions equal."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2311_08263_b200 import engine, lib as _l, workload as wl
@@ -46,3 +47,44 @@ def test_small_forward(hq, hkv, hd, d, d_ffn, vocab, c, lens, flags):
     for o in orc:
         o.close()
     assert dec.fc_debug_check_guards() == 0
+
+
+def _shifted(t):
+    """The same values one element behind a 16-byte boundary, as in a packed buffer."""
+    flat = torch.empty(t.numel() + 1, dtype=t.dtype, device="cuda")
+    assert flat.data_ptr() % 16 == 0
+    flat[1:] = t.reshape(-1)
+    return flat[1:].view(t.shape)
+
+
+@pytest.mark.parametrize("dtype,names", [("f32", None), ("f32", ["w_down"]), ("bf16", ["tok_emb"])])
+def test_weights_off_the_16_byte_boundaries(dtype, names):
+    """Element-aligned weights are read element by element: by the separate kernels in place of the one of a small fp32 model, by
+    the embedding kernel alone for bf16.  fp32 as in test_small_forward; bf16 against the aligned table (sums in another
+    order, see test_bf16_step_run_to_run_spread_is_bounded)."""
+    cfg = wl.small_config(dtype=dtype, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256, d_ffn=512, vocab=512, prompt_len=30)
+    c = 7
+    w = wl.make_weights(cfg)
+    off = dict(w)
+    for n in names or [k for k in w if k != "bias_perm"]:
+        off[n] = [_shifted(t) for t in w[n]] if isinstance(w[n], list) else _shifted(w[n])
+    ids, lens = wl.make_prompts(cfg, batch=1)
+    got = []
+    for weights in (w, off):
+        dec = engine.Decoder(cfg, weights, 1, c, 64)
+        dec.fc_prefill(ids.numpy(), lens.numpy(), c)
+        logits = dec.fc_debug_logits(True)
+        step = dec.fc_jacobi_step()
+        got.append((logits.cpu().numpy(), step))
+        if dtype == "f32":
+            assert dec.fc_last_launch_count() == (1 if weights is w else 6 * cfg.n_layers + 3)
+    o = oracle.Oracle(cfg, w, 64)
+    o.prefill(ids[0].numpy(), c)
+    k, acc, wnew, ref = o.jacobi_step(want_logits=True)
+    lg, (cnt, tok, win) = got[1]
+    if dtype == "f32":
+        assert np.abs(lg - ref).max() < 2e-4
+        assert cnt[0] == k and tok[0, :k].tolist() == acc.tolist() and win[0].tolist() == wnew.tolist()
+    else:
+        assert np.abs(lg - got[0][0]).max() < 3e-4
+    o.close()
