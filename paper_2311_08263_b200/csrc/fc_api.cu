@@ -207,7 +207,7 @@ struct fc_ctx {
   int32_t *pin = nullptr;
   // what the accept kernel reports, in pinned memory: [max_batch] counts, [max_batch * max_c] tokens, windows, error word
   int32_t *res_count = nullptr, *res_tokens = nullptr, *res_window = nullptr, *res_err = nullptr;
-  bool small = false;            // fp32 model whose forward is one kernel
+  bool small = false;            // fp32 model whose forward is one kernel (up to a number of keys: small_forward_pays)
   int32_t *pin_map = nullptr;    // pinned [max_batch]: the live sequences of a compacted step
   int64_t launches = 0;
   char cuda_err[256] = {0};
@@ -623,7 +623,7 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
   const int R = nb * rows;
   RowSegs segs; memset(&segs, 0, sizeof segs);
   segs.b0 = b0; segs.c = rows; segs.seq_map = seq_map;
-  if (ctx->small) {
+  if (ctx->small && small_forward_pays(R, s.n_heads, max_len_host + rows)) {
     int rc = forward_small(ctx, segs, nb, rows, tokens, with_head, commit);
     if (rc != FC_OK || with_head) return rc;
     ++ctx->launches;

@@ -315,6 +315,15 @@ bool small_model_fits(int d, int qd, int kvd, int f, int hd, int vocab, int n_la
   return n_layers <= kSmallLayers && k <= 1536 && layer <= (16 << 20) && (long long)vocab * d * 4 <= (16 << 20) && hd <= 128;
 }
 
+// Whether a forward of R rows over `keys` keys takes this kernel.  Every (row, head) reads its keys for itself here, on sixteen SMs,
+// where the attention of the separate kernels shares a tile of keys among all queries of a kv head and uses every SM; what
+// those lose is 9 to 21 us per row and layer in their projections.  Measured, one kernel / separate ones: 2 layers of 4 heads x 32, 1024
+// rows, 512 keys 2.6 / 17.8 ms, 2048 keys 7.0 / 18.1, 8192 keys 27.1 / 19.0; 8 layers of 8 x 64, 256 rows, 2048 keys 20.0 / 31.3, 8192
+// keys 69.6 / 37.6; 4 layers of 4 x 128, 256 rows, 2048 keys 10.0 / 22.1, 8192 keys 27.5 / 24.7.  The lines cross at 22, 28 and
+// 27 thousand keys x heads; with up to 32 rows, where the separate kernels fill few SMs, at 50 to 107 thousand (8 x 64, 8192 keys: 1
+// row 0.64 / 0.97 ms, 32 rows 7.6 / 9.4).
+bool small_forward_pays(int R, int heads, int keys) { return (long long)heads * keys <= (R < 64 ? 66000 : 24000); }
+
 template <int ND>
 static cudaError_t launch_small_t(const SmallArgs &a, size_t smem, cudaStream_t st) {
   static size_t attr_smem[kMaxDevices] = {0};

@@ -88,3 +88,33 @@ def test_weights_off_the_16_byte_boundaries(dtype, names):
     else:
         assert np.abs(lg - got[0][0]).max() < 3e-4
     o.close()
+
+
+def test_small_model_over_a_long_cache_takes_the_separate_kernels():
+    """16 heads over 1631 keys: with 64 rows (and the later blocks of the prompts) beyond the line of small_forward_pays, with 2
+    rows of the same context below it."""
+    hq, c, lens = 16, 32, [1600, 700]
+    cfg = wl.small_config(dtype="f32", n_layers=2, n_heads=hq, n_kv_heads=4, head_dim=32, d_model=128, d_ffn=256, vocab=300,
+                          prompt_len=max(lens), bias_beta=4.0, seed=733)
+    w = wl.make_weights(cfg)
+    ids, _ = wl.make_prompts(cfg, batch=2, lens=lens)
+    dec = engine.Decoder(cfg, w, 2, c, max(lens) + 3 * c)
+    dec.fc_prefill(ids.numpy(), lens, c)
+    logits = dec.fc_debug_logits(True)
+    orc = []
+    for b, P in enumerate(lens):
+        orc.append(oracle.Oracle(cfg, w, max(lens) + 3 * c))
+        orc[b].prefill(ids[b, :P].numpy(), c)
+    for width, launches in ((c, 6 * cfg.n_layers + 3), (1, 1), (c, 6 * cfg.n_layers + 3)):
+        dec.fc_set_window(width)
+        cnt, tok, win = dec.fc_jacobi_step()
+        assert dec.fc_last_launch_count() == launches
+        lg = logits[:2 * width].cpu().numpy().reshape(2, width, cfg.vocab)
+        for b in range(2):
+            orc[b].set_window(width)
+            k, acc, wnew, ref = orc[b].jacobi_step(want_logits=True)
+            assert np.abs(lg[b] - ref).max() < 2e-4
+            assert cnt[b] == k and tok[b, :k].tolist() == acc.tolist() and win[b].tolist() == wnew.tolist()
+    for o in orc:
+        o.close()
+    assert dec.fc_debug_check_guards() == 0
