@@ -440,7 +440,8 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
   ctx->res_window = ctx->res_tokens + n_rows;
   ctx->res_err = ctx->res_window + n_rows;
   ctx->small = shape->dtype == FC_F32 && !(shape->flags & (FC_FLAG_SIMT_GEMM | FC_FLAG_NO_CHAIN)) && wide_weights(ctx) &&
-               small_model_fits(shape->d_model, ctx->d.qd, ctx->d.kvd, shape->d_ffn, shape->head_dim, shape->vocab, L);
+               small_model_fits(shape->d_model, ctx->d.qd, ctx->d.kvd, shape->d_ffn, shape->head_dim, shape->vocab, L) &&
+               small_cluster_fits(shape->d_model, ctx->d.qd, shape->d_ffn, shape->head_dim);
   if (cudaEventCreate(&ctx->ev0) != cudaSuccess || cudaEventCreate(&ctx->ev1) != cudaSuccess) return fail(FC_ERR_CUDA);
   if (cudaMemsetAsync(ws, 0, fc_workspace_bytes(shape), ctx->st) != cudaSuccess) return fail(FC_ERR_CUDA);
   for (size_t off : ctx->guards)      // canary bands between the slices (checked by fc_debug_check_guards)

@@ -202,6 +202,7 @@ struct SmallArgs {
   AcceptArgs accept;               // with_head: runs behind the LM head; accept.amax_clear is the argmax buffer, zero on entry
 };
 bool small_model_fits(int d, int qd, int kvd, int f, int hd, int vocab, int n_layers);
+bool small_cluster_fits(int d, int qd, int f, int hd);      // the device can hold the kernel's cluster
 bool small_forward_pays(int R, int heads, int keys);
 cudaError_t launch_small_forward(const SmallArgs &a, cudaStream_t st);
 

@@ -20,6 +20,7 @@ namespace fc {
 namespace {
 constexpr int kSmCtas = 16, kSmThreads = 1024, kSmWarps = kSmThreads / 32;
 constexpr int kSmRows = 32;                          // rows staged at a time
+constexpr int kSmallK = 1536;                        // widest input of a projection: the staged rows fill 192 KB
 
 // Sums of eight per-lane values over the warp: lane returns the total of value lane >> 2.
 __device__ __forceinline__ float sum8(float (&v)[8], int lane) {
@@ -310,9 +311,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_forward_kernel(const __gr
 // 1530 against 7142; a prompt of 512 8.1 against 56.7 ms; 4 layers, d 512, ffn 1024 (10 MB), 1 row 189 against 337, 8 rows 218
 // against 803.  At 34 MB a layer and 131 MB of LM head one row costs more here (851 against 810).
 bool small_model_fits(int d, int qd, int kvd, int f, int hd, int vocab, int n_layers) {
-  const int k = d > qd ? (d > f ? d : f) : (qd > f ? qd : f);
   const long long layer = (long long)d * (2 * qd + 2 * kvd + 3 * f) * 4;
-  return n_layers <= kSmallLayers && k <= 1536 && layer <= (16 << 20) && (long long)vocab * d * 4 <= (16 << 20) && hd <= 128;
+  return n_layers <= kSmallLayers && d <= kSmallK && qd <= kSmallK && f <= kSmallK && layer <= (16 << 20) &&
+         (long long)vocab * d * 4 <= (16 << 20) && hd <= 128;
 }
 
 // Whether a forward of R rows over `keys` keys takes this kernel.  Every (row, head) reads its keys for itself here, on sixteen SMs,
@@ -324,37 +325,63 @@ bool small_model_fits(int d, int qd, int kvd, int f, int hd, int vocab, int n_la
 // row 0.64 / 0.97 ms, 32 rows 7.6 / 9.4).
 bool small_forward_pays(int R, int heads, int keys) { return (long long)heads * keys <= (R < 64 ? 66000 : 24000); }
 
+static size_t small_smem(int d, int qd, int f, int hd) {
+  const int k = d > qd ? (d > f ? d : f) : (qd > f ? qd : f);
+  const size_t rows = (size_t)kSmRows * k * 4, att = (size_t)kSmWarps * (hd + 2) * 4;
+  return rows > att ? rows : att;
+}
+
+// Launch configuration; the opt-ins are the same for every model, so that contexts do not undo each other's.
 template <int ND>
-static cudaError_t launch_small_t(const SmallArgs &a, size_t smem, cudaStream_t st) {
-  static size_t attr_smem[kMaxDevices] = {0};
+static cudaError_t small_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, size_t smem, cudaStream_t st) {
+  static bool attr_done[kMaxDevices] = {false};
   const int dev = current_device_slot();
-  if (smem > attr_smem[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(small_forward_kernel<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (!attr_done[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(small_forward_kernel<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmRows * kSmallK * 4);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(small_forward_kernel<ND>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    attr_smem[dev] = smem;
+    attr_done[dev] = true;
   }
-  cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3(kSmCtas); cfg.blockDim = dim3(kSmThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kSmCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, small_forward_kernel<ND>, a);
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kSmCtas; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaSuccess;
+}
+
+template <int ND>
+static cudaError_t launch_small_t(const SmallArgs &a, size_t smem, cudaStream_t st) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  cudaError_t e = small_config<ND>(cfg, attr, smem, st);
+  return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, small_forward_kernel<ND>, a) : e;
 }
 
 cudaError_t launch_small_forward(const SmallArgs &a, cudaStream_t st) {
-  const int qd = a.hq * a.hd;
-  int k = a.d > qd ? a.d : qd;
-  if (a.f > k) k = a.f;
-  size_t smem = (size_t)kSmRows * k * 4;
-  const size_t att = (size_t)kSmWarps * (a.hd + 2) * 4;
-  if (att > smem) smem = att;
+  const size_t smem = small_smem(a.d, a.hq * a.hd, a.f, a.hd);
   if (a.hd == 32) return launch_small_t<1>(a, smem, st);
   if (a.hd == 64) return launch_small_t<2>(a, smem, st);
   if (a.hd == 128) return launch_small_t<4>(a, smem, st);
   return cudaErrorInvalidValue;
+}
+
+template <int ND>
+static int small_clusters_t(size_t smem) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  int n = 0;
+  if (small_config<ND>(cfg, attr, smem, nullptr) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, small_forward_kernel<ND>, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+// A cluster of sixteen is beyond the portable eight: not every device (or part of one) has sixteen SMs in one group.
+bool small_cluster_fits(int d, int qd, int f, int hd) {
+  const size_t smem = small_smem(d, qd, f, hd);
+  return (hd == 32 ? small_clusters_t<1>(smem) : hd == 64 ? small_clusters_t<2>(smem) : hd == 128 ? small_clusters_t<4>(smem) : 0) > 0;
 }
 
 }  // namespace fc
