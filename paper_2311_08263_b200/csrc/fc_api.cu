@@ -1106,7 +1106,7 @@ extern "C" int fc_finish_with_trigger(fc_ctx *ctx, const int32_t *trigger_ids, i
   launches += ctx->launches;
   // (2) plain greedy decoding (Eq. 1) from the last context row: steps with one row per sequence
   std::vector<int32_t> pend(B), zeros(B, 0);
-  for (int b = 0; b < B; ++b) { pend[b] = rows_h[(size_t)b * n_ctx + n_ctx - 1]; answer_lens[b] = 0; }
+  for (int b = 0; b < B; ++b) { pend[b] = rows_h[(size_t)b * n_ctx + n_ctx - 1]; answer_lens[b] = 0; ctx->done_h[b] = 0; }
   FC_CK(cudaMemcpyAsync(ctx->b.window, pend.data(), sizeof(int32_t) * B, cudaMemcpyHostToDevice, ctx->st));
   FC_CK(cudaMemcpyAsync(ctx->b.done, zeros.data(), sizeof(int32_t) * B, cudaMemcpyHostToDevice, ctx->st));
   FC_CK(cudaStreamSynchronize(ctx->st));

@@ -451,6 +451,41 @@ def test_finish_with_trigger_bf16_batch_ragged_with_eos():
     assert glens2[0] == first + 1 and got2[0, :first + 1].tolist() == got[0, :first + 1].tolist()
 
 
+@pytest.mark.parametrize("dtype,flags", [("f32", lib.FC_FLAG_NO_CHAIN), ("bf16", 0)])
+def test_finish_with_trigger_after_a_finished_generation(dtype, flags):
+    """The sequences have reached max_tokens before the hand-off, and the answers cross a 128-key tile of the FMA attention
+    (fp32 through the separate kernels, bf16 with head_dim 32): its grid follows the host's copy of the cache lengths."""
+    cfg = wl.small_config(dtype=dtype, vocab=600, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=32, d_model=128, d_ffn=256,
+                          prompt_len=100, c=6, bias_beta=1.0, seed=31)
+    B, lens, n_ans = 2, [100, 57], 80
+    w = wl.make_weights(cfg)
+    max_seq = 100 + 8 + cfg.c + 4 + n_ans + 8
+    dec = engine.Decoder(cfg, w, B, cfg.c, max_seq, flags=flags)
+    ids, _ = wl.make_prompts(cfg, batch=B, lens=lens)
+    trigger = np.array([11, 22, 33, 44], np.int32)
+    dec.fc_prefill(ids.numpy(), lens, cfg.c)
+    out, out_lens, _ = dec.fc_generate(8)
+    wins = dec.fc_jacobi_step()[2]
+    logits = dec.fc_debug_logits(True)
+    got, glens = dec.fc_finish_with_trigger(trigger, n_ans)
+    lg = logits.cpu().numpy()
+    for b in range(B):
+        assert out_lens[b] == 8 and glens[b] == n_ans
+        context = np.concatenate([ids[b, :lens[b]].numpy(), out[b], wins[b, 1:], trigger]).astype(np.int32)
+        want, margins = oracle.Oracle(cfg, w, max_seq).ar_generate(context, n_ans)
+        diff = np.nonzero(got[b] != want)[0]
+        if dtype == "f32":
+            assert len(diff) == 0
+        elif len(diff):
+            assert margins[diff[0]] < MARGIN_TOL
+        # the last answer token's logits behind this sequence's own tokens
+        o = oracle.Oracle(cfg, w, max_seq)
+        every = np.concatenate([context, got[b]]).astype(np.int32)
+        o.prefill(every[:-1], 1)
+        ref = o.jacobi_step(want_logits=True)[3]
+        assert np.abs(lg[b] - ref[0]).max() < (2e-4 if dtype == "f32" else LOGIT_TOL)
+
+
 # ------------------------------------------------------------------ long positions on the fp32 path
 def test_fp32_stream_exact_at_positions_in_the_thousands():
     """Rotary angles at positions ~3000 come from the host-built table on the FMA path too: the stream stays
