@@ -121,3 +121,103 @@ def test_packed_prompts_when_the_step_capacity_is_no_whole_tile(batch, c, short,
                 assert np.linalg.norm(got - ref) < 2.0 ** -8 * np.linalg.norm(ref)
         o.close()
     assert dec.fc_debug_check_guards() == 0
+
+
+COMPACTED = [
+    # route, hq, hkv, hd, vocab, c, lens; sequences 0, 5 and 9 have the same prompt and end at the first iteration
+    ("dense", 8, 4, 64, 1024, 16, [60, 33, 70, 1, 64, 60, 20, 95, 31, 60, 47, 80]),              # 192 rows, then 144
+    ("dense", 4, 4, 128, 1024, 40, [30, 33, 70, 2, 64, 30, 20, 95, 31, 30, 47, 80]),             # 480, then 360 (split sums)
+    ("stream", 8, 8, 64, 1000, 2, [40, 33, 960, 1, 64, 40, 20, 95, 31, 40, 47, 500]),            # 72 units x 16 tiles of 64 keys
+]
+
+
+@pytest.mark.parametrize("route,hq,hkv,hd,vocab,c,lens", COMPACTED)
+def test_finished_sequences_leave_the_rows_of_the_many_row_routes(route, hq, hkv, hd, vocab, c, lens):
+    cfg = wl.small_config(n_layers=2, n_heads=hq, n_kv_heads=hkv, head_dim=hd, d_model=512, d_ffn=768, vocab=vocab, prompt_len=max(lens),
+                          seed=1200 + c)
+    B, gone = len(lens), [0, 5, 9]
+    w = wl.make_weights(cfg)
+    ids = wl.make_prompts(cfg, batch=B, lens=lens)[0].numpy()
+    ids[5], ids[9] = ids[0], ids[0]
+    max_seq = max(lens) + 3 * c
+    orc = []
+    for b, P in enumerate(lens):
+        orc.append(oracle.Oracle(cfg, w, max_seq))
+        orc[b].prefill(ids[b, :P], c)
+    eos = int(orc[0].generate(1)[0][0])
+    orc[0].prefill(ids[0, :lens[0]], c)
+    dec = engine.Decoder(cfg, w, B, c, max_seq)
+    dec.fc_prefill(ids, lens, c)
+    out, out_lens, _ = dec.fc_generate(2 * c, eos_id=eos, max_iters=1)
+    logits = dec.fc_debug_logits(True)
+    first = [o.generate(2 * c, eos_id=eos, max_iters=1)[0].tolist() for o in orc]
+    assert [b for b in range(B) if eos in first[b]] == gone
+    for b in range(B):
+        assert out[b, :out_lens[b]].tolist() == first[b]
+    cnt, tok, win = dec.fc_jacobi_step()
+    assert dec.fc_last_launch_count() == (8 if route == "dense" else 3) * cfg.n_layers + 4 + 1      # and the gather of the windows
+    lg = logits[:(B - len(gone)) * c].cpu().numpy().reshape(B - len(gone), c, vocab)
+    live = [b for b in range(B) if b not in gone]
+    for i, b in enumerate(live):
+        k, acc, wnew, ref = orc[b].jacobi_step(want_logits=True)
+        _check_step(lg[i], ref, np.zeros(c, np.int32), cnt[b], tok[b], win[b], k, acc, wnew)
+    assert all(cnt[b] == 0 for b in gone)
+    kl, _ = dec.fc_get_state()
+    for b in live:
+        assert kl[b] == orc[b].kv_len
+    assert dec.fc_debug_check_guards() == 0
+    for o in orc:
+        o.close()
+
+
+def test_more_prompts_than_segments_of_a_block():
+    """70 prompts of 2 to 6 ids: 210 rows, but a block takes 64 segments at most."""
+    cfg = _cfg(8, 8, 64, seed=1300, prompt_len=6)
+    lens, c = [2 + (3 * b) % 5 for b in range(70)], 3
+    w = wl.make_weights(cfg)
+    ids = wl.make_prompts(cfg, batch=70, lens=lens)[0].numpy()
+    dec = engine.Decoder(cfg, w, 70, c, 16)
+    dec.fc_prefill(ids, lens, c)
+    logits = dec.fc_debug_logits(True)
+    cnt, tok, win = dec.fc_jacobi_step()
+    lg = logits.cpu().numpy().reshape(70, c, cfg.vocab)
+    for b in (0, 1, 62, 63, 64, 65, 69):
+        o = oracle.Oracle(cfg, w, 16)
+        o.prefill(ids[b, :lens[b]], c)
+        k, acc, wnew, ref = o.jacobi_step(want_logits=True)
+        _check_step(lg[b], ref, np.zeros(c, np.int32), cnt[b], tok[b], win[b], k, acc, wnew)
+        o.close()
+    assert dec.fc_debug_check_guards() == 0
+
+
+def test_dense_and_chained_steps_after_a_reported_timeout():
+    """Dense step that reports a timeout, prompts again, then a chained step (64 rows) and a dense one (132 rows) over the same
+    buffers."""
+    cfg = _cfg(8, 4, 64, seed=1400, prompt_len=60)
+    B, c, lens = 4, 33, [60, 41, 3, 50]
+    w = wl.make_weights(cfg)
+    ids = wl.make_prompts(cfg, batch=B, lens=lens)[0].numpy()
+    dec = engine.Decoder(cfg, w, B, c, 60 + 4 * c)
+    dec.fc_prefill(ids, lens, c)
+    dec.fc_debug_inject_timeout()
+    with pytest.raises(engine.FcError) as e:
+        dec.fc_jacobi_step()
+    assert e.value.code == _l.FC_ERR_DEVICE_TIMEOUT
+    dec.fc_prefill(ids, lens, c)
+    logits = dec.fc_debug_logits(True)
+    orc = []
+    for b, P in enumerate(lens):
+        orc.append(oracle.Oracle(cfg, w, 60 + 4 * c))
+        orc[b].prefill(ids[b, :P], c)
+    for width, per_layer in ((16, 2), (c, 8)):
+        dec.fc_set_window(width)
+        cnt, tok, win = dec.fc_jacobi_step()
+        assert dec.fc_last_launch_count() == per_layer * cfg.n_layers + 4
+        lg = logits[:B * width].cpu().numpy().reshape(B, width, cfg.vocab)
+        for b in range(B):
+            orc[b].set_window(width)
+            k, acc, wnew, ref = orc[b].jacobi_step(want_logits=True)
+            assert _check_step(lg[b], ref, np.zeros(width, np.int32), cnt[b], tok[b], win[b], k, acc, wnew)
+    assert dec.fc_debug_check_guards() == 0
+    for o in orc:
+        o.close()
