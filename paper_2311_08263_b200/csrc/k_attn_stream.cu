@@ -509,25 +509,8 @@ cudaError_t launch_qkv_finish(const QkvFinishArgs &a, int R, cudaStream_t st) {
   return cudaLaunchKernelEx(&cfg, qkv_finish_kernel, a);
 }
 
-// Query tiles per CTA and key splits for `nb` segments of at most `rows` rows behind at most max_len keys.
-static void stream_plan(int max_len, int rows, int group, int hkv, int nb, int n_sms, int &wq, int &ns) {
-  const int nqt = (group * rows + 15) / 16;
-  wq = nqt >= 3 ? 4 : nqt;
-  const long long units = (long long)nb * hkv * ((nqt + wq - 1) / wq);
-  const int tiles = (max_len + rows + kSKeys - 1) / kSKeys;
-  const long long slots = 2ll * n_sms;
-  // Waves of CTAs times a CTA's length in tile times; start, query loads and merge cost about as much as six tiles.
-  long long best = 0;
-  ns = 1;
-  for (int s = 1; s <= 8 && s <= tiles; ++s) {
-    const long long waves = (units * s + slots - 1) / slots;
-    const long long cost = waves * ((tiles + s - 1) / s + 6 + (s > 1 ? 2 : 0));
-    if (s == 1 || cost < best) { best = cost; ns = s; }
-  }
-}
-
 template <int HD, int WQ>
-static cudaError_t launch_stream_t(const KvTensorMap &map, const StreamAttnArgs &a, int ns, int nqg, int nseg, cudaStream_t st) {
+static cudaError_t stream_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int ns, int ny, int nz, bool pdl, cudaStream_t st) {
   const size_t smem = StreamCfg<HD>::smem();
   static bool attr_done[kMaxDevices] = {false};
   const int dev = current_device_slot();
@@ -536,12 +519,10 @@ static cudaError_t launch_stream_t(const KvTensorMap &map, const StreamAttnArgs 
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3(ns, a.hkv * nqg, nseg); cfg.blockDim = dim3(stream_threads(WQ)); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute attr[2];
+  cfg.gridDim = dim3(ns, ny, nz); cfg.blockDim = dim3(stream_threads(WQ)); cfg.dynamicSmemBytes = smem; cfg.stream = st;
   int na = 0;
-  if (a.pdl) {
+  if (pdl) {
     attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[na].val.programmaticStreamSerializationAllowed = 1;
     ++na;
@@ -552,15 +533,68 @@ static cudaError_t launch_stream_t(const KvTensorMap &map, const StreamAttnArgs 
     ++na;
   }
   cfg.attrs = attr; cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, attn_stream_kernel<HD, WQ>, *reinterpret_cast<const CUtensorMap *>(&map), a);
+  return cudaSuccess;
+}
+
+// Clusters of ns CTAs that run at the same time.  Clusters do not cross groups of SMs, so it is fewer than CTA slots / ns (B200:
+// 296 slots, 71 clusters of four, 45 of six, 37 of seven, 33 of eight); a sixteenth is left out, because the CTAs of the kernel in
+// front still hold slots when they are placed (32 clusters of eight ran in two rounds).
+template <int HD, int WQ>
+static int stream_clusters_t(int ns, int n_sms) {
+  if (ns == 1) return 2 * n_sms;
+  static int known[kMaxDevices][9] = {};
+  int &n = known[current_device_slot()][ns];
+  if (n == 0) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    int fit = 0;
+    if (stream_config<HD, WQ>(cfg, attr, ns, 1, 1, false, nullptr) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&fit, attn_stream_kernel<HD, WQ>, &cfg) != cudaSuccess || fit < 1) {
+      (void)cudaGetLastError();
+      fit = 1;
+    }
+    n = fit > 15 ? fit * 15 / 16 : fit;
+  }
+  return n;
+}
+static int stream_clusters(int hd, int wq, int ns, int n_sms) {
+  if (hd == 128) return wq == 1 ? stream_clusters_t<128, 1>(ns, n_sms) : wq == 2 ? stream_clusters_t<128, 2>(ns, n_sms) : stream_clusters_t<128, 4>(ns, n_sms);
+  return wq == 1 ? stream_clusters_t<64, 1>(ns, n_sms) : wq == 2 ? stream_clusters_t<64, 2>(ns, n_sms) : stream_clusters_t<64, 4>(ns, n_sms);
+}
+
+// Query tiles per CTA and key splits for `nb` segments of at most `rows` rows behind at most max_len keys.
+static void stream_plan(int max_len, int rows, int group, int hkv, int nb, int hd, int n_sms, int &wq, int &ns) {
+  const int nqt = (group * rows + 15) / 16;
+  wq = nqt >= 3 ? 4 : nqt;
+  const long long units = (long long)nb * hkv * ((nqt + wq - 1) / wq);
+  const int tiles = (max_len + rows + kSKeys - 1) / kSKeys;
+  // Rounds of clusters times a CTA's length in tile times; start, query loads and merge cost about as much as six tiles.  Measured
+  // by splits, 4 layers over 8000 keys: 7B, 1 x 32 rows (32 units) 4 splits 825 us, 6 742, 7 720, 8 822; 13B, 1 x 32 (40 units) 5
+  // 931, 6 894, 7 1028; 13B, 2 x 16 (80 units) 2 957, 3 914, 4 1002; 7B, 4 x 16 (128 units) 1 1084, 2 940, 3 1003.
+  long long best = 0;
+  ns = 1;
+  for (int s = 1; s <= 8 && s <= tiles; ++s) {
+    const int fit = stream_clusters(hd, wq, s, n_sms);
+    const long long rounds = (units + fit - 1) / fit;
+    const long long cost = rounds * ((tiles + s - 1) / s + 6 + (s > 1 ? 2 : 0));
+    if (s == 1 || cost < best) { best = cost; ns = s; }
+  }
+}
+
+template <int HD, int WQ>
+static cudaError_t launch_stream_t(const KvTensorMap &map, const StreamAttnArgs &a, int ns, int nqg, int nseg, cudaStream_t st) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  cudaError_t e = stream_config<HD, WQ>(cfg, attr, ns, a.hkv * nqg, nseg, a.pdl != 0, st);
+  return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, attn_stream_kernel<HD, WQ>, *reinterpret_cast<const CUtensorMap *>(&map), a) : e;
 }
 
 cudaError_t launch_attn_stream(const KvTensorMap &map, const StreamAttnArgs &a, int nseg, int max_rows, int max_len, int hd,
                                int n_sms, cudaStream_t st) {
-  if (nseg < 1 || nseg > 65535 || max_rows < 1 || !a.err || a.segs.n > kMaxSegs) return cudaErrorInvalidValue;
+  if (nseg < 1 || nseg > 65535 || max_rows < 1 || !a.err || a.segs.n > kMaxSegs || (hd != 64 && hd != 128)) return cudaErrorInvalidValue;
   const int group = a.hq / a.hkv;
   int wq, ns;
-  stream_plan(max_len, max_rows, group, a.hkv, nseg, n_sms, wq, ns);
+  stream_plan(max_len, max_rows, group, a.hkv, nseg, hd, n_sms, wq, ns);
   const int nqg = (group * max_rows + wq * 16 - 1) / (wq * 16);
   if ((long long)a.hkv * nqg > 65535) return cudaErrorInvalidValue;
   if (hd == 128) {
@@ -568,23 +602,22 @@ cudaError_t launch_attn_stream(const KvTensorMap &map, const StreamAttnArgs &a, 
     if (wq == 2) return launch_stream_t<128, 2>(map, a, ns, nqg, nseg, st);
     return launch_stream_t<128, 4>(map, a, ns, nqg, nseg, st);
   }
-  if (hd == 64) {
-    if (wq == 1) return launch_stream_t<64, 1>(map, a, ns, nqg, nseg, st);
-    if (wq == 2) return launch_stream_t<64, 2>(map, a, ns, nqg, nseg, st);
-    return launch_stream_t<64, 4>(map, a, ns, nqg, nseg, st);
-  }
-  return cudaErrorInvalidValue;
+  if (wq == 1) return launch_stream_t<64, 1>(map, a, ns, nqg, nseg, st);
+  if (wq == 2) return launch_stream_t<64, 2>(map, a, ns, nqg, nseg, st);
+  return launch_stream_t<64, 4>(map, a, ns, nqg, nseg, st);
 }
 
 // Where this pair of kernels is faster than the fused one (attn_tma_kernel): with at least 64 units (kv head of a sequence x
-// 16 queries) that read together at least a thousand tiles of 64 keys.  Measured, time of an 8-layer step, fused -> this:
-// 7B, 16 x 1 row, 512 keys 1107 -> 1048 us, 16 x 4 rows, 1024 keys 1608 -> 1470; 4 x 16 rows, 512 keys 1220 -> 1176;
-// 1.1B, 16 x 1, 1024 keys 508 -> 473, 16 x 16, 512 keys 1331 -> 1210; 13B, 8 x 32, 2048 keys 4600 -> 4230.  Below the
-// line the second launch per layer costs more than it brings: 7B, 2 x 8, 512 keys 882 -> 894; 1 x 16, 2048 keys 928 -> 944;
-// 1.1B, 4 x 4, 1024 keys 469 -> 476, 1 x 16, 8192 keys 667 -> 685.
+// 16 queries) that read together at least a thousand tiles of 64 keys, three or more each.  Measured, time of an 8-layer step,
+// fused -> this: 7B, 16 x 1 row, 512 keys 1107 -> 1048 us, 16 x 4 rows, 1024 keys 1608 -> 1470; 4 x 16 rows, 512 keys 1220 -> 1176;
+// 1.1B, 16 x 1, 1024 keys 508 -> 473, 16 x 16, 512 keys 1331 -> 1210; 13B, 8 x 32, 2048 keys 4600 -> 4230; of a 4-layer step over
+// 8000 keys: 7B, 1 x 32 778 -> 720, 13B, 1 x 32 998 -> 894.  Below the line the second launch per layer costs about what it brings
+// or more: 7B, 2 x 8, 512 keys 882 -> 894; 1.1B, 4 x 4, 1024 keys 469 -> 476, and over two tiles of keys (64 keys; 4 layers)
+// 7B, 16 x 1 499 -> 535, 16 x 4 665 -> 664 to 744, 13B, 16 x 1 678 -> 678.
 bool attn_stream_pays(int max_len, int c, int hq, int hkv, int nb) {
   const long long units = (long long)nb * hkv * (((long long)(hq / hkv) * c + 15) / 16);
-  return units >= 64 && units * ((max_len + c + 63) / 64) >= 1000;
+  const int tiles = (max_len + c + 63) / 64;
+  return units >= 64 && tiles >= 3 && units * tiles >= 1000;
 }
 
 int attn_stream_tile_keys() { return kSKeys; }

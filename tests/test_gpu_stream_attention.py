@@ -27,3 +27,11 @@ def test_step_over_streamed_cache(hq, hkv, hd, c, lens):
     # one kernel more per layer than with the fused attention (the vocabulary is no whole number of weight tiles, so that
     # the chained launch takes any number of rows)
     assert dec.fc_last_launch_count() == 3 * cfg.n_layers + 4
+
+
+@pytest.mark.parametrize("heads,c", [(32, 32), (40, 24), (40, 50)])
+def test_one_sequence_with_an_odd_number_of_key_splits(heads, c):
+    """32 and 40 (kv head, query group) pairs: seven and six splits, as many clusters as run at the same time."""
+    cfg = wl.small_config(n_layers=2, n_heads=heads, n_kv_heads=heads, head_dim=128, d_model=256, d_ffn=512, vocab=1000, seed=190 + c)
+    dec, _ = _random_kv_case(cfg, [1471], c, [0])
+    assert dec.fc_last_launch_count() == 3 * cfg.n_layers + 4
