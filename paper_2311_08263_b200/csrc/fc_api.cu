@@ -39,11 +39,13 @@ constexpr int kBulkRows = 1024;           // the same where the dense GEMMs of k
 // 256 rows over 1024 keys 2141, 1800.
 constexpr int kBulkMin = 129;
 
-// Steps of more rows than this add up as the chained launch does (BulkArgs::split): the more rows, the larger the worst of
-// them.  Largest logit difference from the chained launch in units of the logits' rms: 7B, 512 rows, six-block sums 0.0259, split
-// 0.0169, that launch against itself 0.0152 (24 seeds); 13B, 256 rows, six-block sums 0.0150, that launch against itself 0.0212 (5
-// seeds): nothing to gain there.  It costs 3.5 % of the 512-row step (5 % at 256 rows).
-constexpr int kBulkSplit = 256;
+// Steps that store at least this many key and value elements add up as the chained launch does (BulkArgs::split): each of
+// them may fall on the other side of a bf16 rounding boundary and move its row, so the worst row grows with their number.
+// Largest logit difference from the chained launch in units of the logits' rms: 1.34e8 elements (7B, 512 rows, 24 seeds) six-block
+// sums 0.0259, split 0.0169, that launch against itself 0.0152; 1.05e8 (13B, 256 rows, 5 seeds) six-block sums 0.0150, that launch
+// against itself 0.0212: nothing to gain there; 1.1B at 384 rows (4e6) 0.002.  It costs 3.5 % of the 512-row step, 7 % at 294
+// rows of 13B or 1.1B.
+constexpr long long kSplitElems = 120000000;
 
 constexpr int kSyncClaim = kChainMax, kSyncPanel = 2 * kChainMax, kSyncTd = 3 * kChainMax;   // offsets in a group
 
@@ -566,7 +568,7 @@ static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int m
   BulkArgs ba; memset(&ba, 0, sizeof ba);
   ba.slots = ctx->b.bulk_slots; ba.arrived = ctx->b.bulk_arrived;
   ba.pan_rows = d.rows_ws; ba.R = R; ba.eps = s.rms_eps; ba.dn = s.d_model;
-  ba.split = with_head && R > kBulkSplit;
+  ba.split = with_head && 2ll * R * d.kvd * s.n_layers >= kSplitElems;
   const long long stride_h = (long long)s.max_seq * s.head_dim, stride_b = (long long)s.n_kv_heads * stride_h;
   auto norm = [&](const void *gain, float *ss, int cls) {
     ProfScope ps(ctx, cls);

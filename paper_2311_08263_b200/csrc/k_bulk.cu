@@ -17,14 +17,14 @@
 // of 4 layers: chained launch 1.07 / 1.25 / 1.29e-3; whole k range in one accumulator above 1.5e-3; 8 k-blocks 1.09 / 1.32 /
 // 1.28e-3, 1.77 ms; 6: 1.07 / 1.23 / 1.22e-3, 1.82 ms; 4: 1.03 / 1.20 / 1.06e-3, 1.88 ms.
 //
-// Steps of many rows (BulkArgs::split) add up as the chained launch does: a high and a low accumulator over the chained launch's
-// chunks of 16 k-blocks, shares cut between chunks.  Their results differ from that launch's by the order of fp32 additions
-// only.  With other sums the tensor core's rounding differs, which moves more stored K/V values over a bf16 rounding boundary
-// (7.0e-4 of layer 0's instead of 3.4e-5), and one such value moves its row of logits by up to a few per cent.  Largest difference
-// of two steps of 7B from the chained launch, 512 rows, 24 seeds, in units of the logits' rms: six-block sums 0.0259 (median 0.0085),
-// split 0.0169 (0.0041), two runs of the chained launch 0.0152 (0.0022); the distance from 64 bits is the same for all three.  The
-// accumulators cannot alternate then: the high one is added up while the last low products run, and the next chunk waits for
-// the rest (these two steps: six-block sums 30.7 ms, split 31.8, chained launch 35.1).
+// Steps that store very many keys and values (BulkArgs::split) add up as the chained launch does: a high and a low accumulator over
+// that launch's chunks of 16 k-blocks, shares cut between chunks.  Their results differ from that launch's by the order of fp32
+// additions only.  With other sums the tensor core's rounding differs, which moves more stored K/V values over a bf16 rounding
+// boundary (7.0e-4 of layer 0's instead of 3.4e-5), and one such value moves its row of logits by up to a few per cent.  Largest
+// difference of two steps of 7B from the chained launch, 512 rows, 24 seeds, in units of the logits' rms: six-block sums 0.0259
+// (median 0.0087), split 0.0169 (0.0038), two runs of the chained launch 0.0152 (0.0022); the distance from 64 bits is the same for
+// all three.  The accumulators cannot alternate then: the high one is added up while the last low products run, and the next
+// chunk waits for the rest (these two steps: six-block sums 30.7 ms, split 31.8, chained launch 35.1).
 //
 // The tiles of a projection seldom are a whole number of rounds over the pairs: whole rounds run tile by tile, the tiles
 // that are left over are dealt as one run of k-blocks, cut into equal shares for all pairs (a share ends in one tile and may
