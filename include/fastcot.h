@@ -101,7 +101,7 @@ int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weights *weights
             void *kv, size_t kv_bytes, void *ws, size_t ws_bytes, void *cuda_stream);
 
 /* Start `batch` sequences (dropping any previous ones).  prompt_ids: host [batch, p_stride]; prompt_lens:
- * host [batch], each >= 1.  Caches K/V of prompt[0 .. P-2] in blocks of at least 128 rows per forward;
+ * host [batch], each >= 1.  Caches K/V of prompt[0 .. P-2] in blocks of at least 128 rows per forward (or all);
  * prompt[P-1] becomes the pending exact token (window slot 0); slots 1..c-1 are filled by the refill rule.
  * "Overview of FastCoT": the prompt and the window taken from the buffer form the first input. */
 int fc_prefill(fc_ctx *ctx, int32_t batch, const int32_t *prompt_ids, int32_t p_stride,

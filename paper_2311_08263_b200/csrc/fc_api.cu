@@ -42,9 +42,9 @@ constexpr int kBulkMin = 129;
 // Steps that store at least this many key and value elements add up as the chained launch does (BulkArgs::split): each of
 // them may fall on the other side of a bf16 rounding boundary and move its row, so the worst row grows with their number.
 // Largest logit difference from the chained launch in units of the logits' rms: 1.34e8 elements (7B, 512 rows, 24 seeds) six-block
-// sums 0.0259, split 0.0169, that launch against itself 0.0152; 1.05e8 (13B, 256 rows, 5 seeds) six-block sums 0.0150, that launch
-// against itself 0.0212: nothing to gain there; 1.1B at 384 rows (4e6) 0.002.  It costs 3.5 % of the 512-row step, 7 % at 294
-// rows of 13B or 1.1B.
+// sums 0.0259, split 0.0169, two runs of that launch 0.0152; 1.05e8 (13B, 256 rows, 5 seeds) six-block sums 0.0150, two runs of that
+// launch 0.0116, the same behind the other attention kernel 0.0212: nothing to gain there; 1.1B at 384 rows (4e6) 0.002.  It costs
+// 3.5 % of the 512-row step, 7 % at 294 rows of 13B or 1.1B.
 constexpr long long kSplitElems = 120000000;
 
 constexpr int kSyncClaim = kChainMax, kSyncPanel = 2 * kChainMax, kSyncTd = 3 * kChainMax;   // offsets in a group
@@ -801,7 +801,7 @@ static int check_device_error(fc_ctx *ctx) {
 }
 
 // The prompts of a batch one behind the other (n_all rows), cut into as few blocks as the buffers allow, of nearly equal
-// size and, but for the last, whole 128-row tiles.
+// size and, but for the last, whole 128-row tiles.  (A block also ends at kMaxSegs prompts.)
 static int prefill_packed(fc_ctx *ctx, int batch, const int32_t *prompt_lens, long long n_all) {
   const long long n_blk = (n_all + ctx->d.rows_ws - 1) / ctx->d.rows_ws;
   int b = 0, at = 0, blk_no = 0;                                      // next row: id `at` of prompt b
@@ -871,8 +871,9 @@ extern "C" int fc_prefill(fc_ctx *ctx, int32_t batch, const int32_t *prompt_ids,
   FC_CK(cudaMemcpyAsync(ctx->b.n_gen, zeros.data(), sizeof(int32_t) * batch, cudaMemcpyHostToDevice, ctx->st));
   FC_CK(cudaMemcpyAsync(ctx->b.done, zeros.data(), sizeof(int32_t) * batch, cudaMemcpyHostToDevice, ctx->st));
   FC_CK(cudaStreamSynchronize(ctx->st));   // host vectors above go out of scope
-  // K/V of prompt[0 .. P-2]: one sequence at a time, in blocks of as many rows as the activation buffers hold
-  // (at least one 128-row accumulator block, so that a prompt of P ids streams the weights ~P / 128 times)
+  // K/V of prompt[0 .. P-2].  Where the dense GEMMs run and there is enough for them: the prompts one behind the other in as few
+  // blocks as the activation buffers allow.  Else one sequence at a time, in blocks of as many rows as the chained launch (or
+  // the FMA kernels) holds, at least 128: a prompt of P ids then streams the weights ~P / 128 times.
   FC_CK(cudaEventRecord(ctx->ev0, ctx->st));
   long long n_all = 0;
   for (int b = 0; b < batch; ++b) n_all += prompt_lens[b] - 1;

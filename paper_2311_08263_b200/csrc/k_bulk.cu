@@ -500,7 +500,8 @@ cudaError_t launch_norm_pair(const float *x, const void *gain, float *ss, void *
 // k-block takes the slower of its MMAs (4 cycles per row) and its operand loads (about 56 bytes per cycle and
 // SM out of L2); whole rounds take nkb of them, the shares of what is left over `share`, and pieces that have to be stored
 // and added up about 9000 besides.
-// The shares are whole groups of four k-blocks; with split accumulators, whole chunks of them.
+// The shares are whole groups of four k-blocks (an accumulation starts where a share does, so they need not be whole
+// accumulations); with split accumulators, whole chunks.
 static void bulk_plan(int n_wt, int nkb, int R, int n_pairs, bool add, bool may_share, bool split, int &bn, int &rounds, int &share) {
   const int unit = split ? kSplitKb : 4;
   double best = 0;
