@@ -56,6 +56,11 @@ struct Buffers {
   void *qb;
   unsigned int *counters, *err, *chain_bar, *bulk_arrived;
   char *bulk_slots;
+  // up to kClusterRows rows (k_cluster.cu): tensor maps, operand pairs, slots of the sums of squares, grid barriers
+  char *cl_maps;
+  void *cl_pan_x, *cl_pan_a, *cl_pan_h;
+  float *cl_ss_x, *cl_ss_ffn;
+  unsigned int *cl_bar;
   unsigned long long *amax;
   int32_t *window, *kv_len, *n_gen, *done, *acc_count, *acc_tokens, *prompt, *prompt_lens, *out_tokens;
   int32_t *row_tokens;     // tokens of a forward that is not a plain decode step (answer-trigger context; the windows of
@@ -68,6 +73,7 @@ struct Dims {
   int rows_ws;     // rows the activation buffers hold: a decode step or a block of prompts, whichever is larger
   int qd, kvd, ldq, nsplit_max, tk, pan_rows, pan_k, sync_words, q_tiles;
   bool bulk;       // the shape takes the dense GEMMs from kBulkMin rows
+  bool cluster;    // the shape takes the one-writer projections up to kClusterRows rows
   int rows_chain;  // rows the buffers of the chained launch hold
   size_t esz;
 };
@@ -90,12 +96,19 @@ bool bulk_shape(const fc_model_shape *s) {
          s->d_ffn % 256 == 0 && s->n_heads * s->head_dim % 256 == 0 && s->n_kv_heads * s->head_dim % 256 == 0 && s->vocab % 256 == 0;
 }
 
+// bf16 on the tensor cores with head_dim 64 / 128 and whole pairs of k-blocks
+bool cluster_shape(const fc_model_shape *s) {
+  return s->dtype == FC_BF16 && !(s->flags & (FC_FLAG_SIMT_GEMM | FC_FLAG_NO_CHAIN)) && (s->head_dim == 64 || s->head_dim == 128) &&
+         cluster_shape_ok(s->d_model, s->n_heads * s->head_dim, s->n_kv_heads * s->head_dim, s->d_ffn, s->vocab);
+}
+
 Dims dims_of(const fc_model_shape *s) {
   Dims d;
   d.rmax = s->max_batch * s->max_c;
   d.rows_ws = d.rmax > kPrefillRows ? d.rmax : kPrefillRows;
   d.rows_chain = d.rows_ws;
   d.bulk = bulk_shape(s);
+  d.cluster = cluster_shape(s);
   if (d.bulk) {
     d.rows_chain = kPrefillRows;
     const long long all = ((long long)s->max_batch * s->max_seq + 127) / 128 * 128;       // no prompt block is larger
@@ -146,6 +159,14 @@ size_t carve(const fc_model_shape *s, char *base, Buffers *b, std::vector<size_t
   t.pan_ffn = c.take<char>(d.bulk ? (size_t)2 * R * s->d_ffn * 2 : 0); c.guard();
   t.bulk_slots = c.take<char>(d.bulk ? bulk_slot_bytes() : 0); c.guard();
   t.bulk_arrived = c.take<unsigned int>(d.bulk ? kBulkArrived : 0); c.guard();
+  const size_t cl_rows = d.cluster ? 2 * kClusterRows : 0;
+  t.cl_maps = c.take<char>(d.cluster ? cluster_map_bytes(s->n_layers) : 0); c.guard();
+  t.cl_pan_x = c.take<char>(cl_rows * s->d_model * 2); c.guard();
+  t.cl_pan_a = c.take<char>(cl_rows * d.qd * 2); c.guard();
+  t.cl_pan_h = c.take<char>(cl_rows * s->d_ffn * 2); c.guard();
+  t.cl_ss_x = c.take<float>(d.cluster ? kClusterSlots * kClusterRows : 0);
+  t.cl_ss_ffn = c.take<float>(d.cluster ? kClusterSlots * kClusterRows : 0);
+  t.cl_bar = c.take<unsigned int>(d.cluster ? 8 * (size_t)s->n_layers + 2 : 0); c.guard();
   // split-KV partials of the FMA attention kernel
   const size_t Rp = d.bulk ? 0 : R;
   t.part_o = c.take<float>(Rp * s->n_heads * (size_t)d.nsplit_max * s->head_dim); c.guard();
@@ -194,6 +215,7 @@ struct fc_ctx {
   std::vector<UmmaPlan *> plan_gu_half[2], plan_down_half[2];   // the FFN in two halves of d_ffn (chained launch, <= 16 rows)
   bool ffn_split = false;
   UmmaPlan *plan_head = nullptr;
+  ClusterPlan *plan_cl = nullptr;
   float *dbg_logits = nullptr;
   // sequence state mirrored on the host
   int batch = 0, c = 0, refill = 0, pad_id = 0, p_stride = 0;
@@ -266,6 +288,8 @@ static void destroy_plans(fc_ctx *ctx) {
   }
   umma_plan_destroy(ctx->plan_head);
   ctx->plan_head = nullptr;
+  cluster_plan_destroy(ctx->plan_cl);
+  ctx->plan_cl = nullptr;
 }
 
 extern "C" void fc_destroy(fc_ctx *ctx) {
@@ -465,6 +489,14 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
         cudaStreamSynchronize(ctx->st) != cudaSuccess) return fail(FC_ERR_CUDA);
   }
   if (cudaStreamSynchronize(ctx->st) != cudaSuccess) return fail(FC_ERR_CUDA);
+  if (ctx->d.cluster) {          // behind the workspace's clearing: the tensor maps lie in it
+    ClusterModel m; memset(&m, 0, sizeof m);
+    m.n_layers = L; m.d = shape->d_model; m.qd = ctx->d.qd; m.kvd = ctx->d.kvd; m.f = shape->d_ffn; m.vocab = shape->vocab;
+    m.wq = ctx->wq.data(); m.wk = ctx->wk.data(); m.wv = ctx->wv.data(); m.wo = ctx->wo.data();
+    m.w_gate = ctx->w_gate.data(); m.w_up = ctx->w_up.data(); m.w_down = ctx->w_down.data(); m.lm_head = ctx->lm_head;
+    ctx->plan_cl = cluster_plan_create(m, ctx->b.cl_maps, ctx->b.cl_pan_x, ctx->b.cl_pan_a, ctx->b.cl_pan_h, ctx->st);
+    (void)cudaGetLastError();    // without it (a device that does not hold the clusters): the other routes
+  }
   const int B = shape->max_batch;
   ctx->kv_len_h.assign(B, 0); ctx->n_gen_h.assign(B, 0); ctx->pending_h.assign(B, 0); ctx->done_h.assign(B, 0);
   ctx->prompt_h.assign(B, std::vector<int32_t>());
@@ -616,6 +648,82 @@ static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int m
   return FC_OK;
 }
 
+// The two attention routes of the bf16 step for layer l: over rows whose K/V the first kernel stores (streaming), or all in one
+// kernel (fused).  out / out_pan as in FusedAttnArgs; z: buffers to clear on the side.
+static int run_stream_attn(fc_ctx *ctx, int l, const RowSegs &segs, int nb, int rows, int max_len, float *out, void *out_pan, int pan_rows, const ZeroList &z) {
+  const fc_model_shape &s = ctx->s;
+  const Dims &d = ctx->d;
+  const int pdl = ctx->pdl && !ctx->prof;
+  const long long stride_h = (long long)s.max_seq * s.head_dim;
+  QkvFinishArgs qa; memset(&qa, 0, sizeof qa);
+  qa.qkv = ctx->b.qkv; qa.ldq = d.ldq; qa.ss = ctx->b.ss_attn; qa.eps = s.rms_eps; qa.dn = s.d_model; qa.rope = ctx->b.rope;
+  qa.kv_len = ctx->b.kv_len; qa.segs = segs;
+  qa.hq = s.n_heads; qa.hkv = s.n_kv_heads; qa.hd = s.head_dim; qa.q = ctx->b.qb; qa.q_tiles = d.q_tiles;
+  qa.kcache = ctx->kv + (size_t)l * ctx->kv_layer_stride; qa.vcache = (char *)qa.kcache + ctx->kv_half_stride;
+  qa.stride_b = s.n_kv_heads * stride_h; qa.stride_h = stride_h; qa.pdl = pdl; qa.z = z;
+  ++ctx->launches;
+  { ProfScope ps(ctx, FC_CLS_ROPE); FC_CK(launch_qkv_finish(qa, nb * rows, ctx->st)); }
+  StreamAttnArgs sa; memset(&sa, 0, sizeof sa);
+  sa.q = ctx->b.qb; sa.q_tiles = d.q_tiles; sa.kv_len = ctx->b.kv_len; sa.segs = segs; sa.hq = s.n_heads; sa.hkv = s.n_kv_heads;
+  sa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; sa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
+  sa.err = ctx->b.err; sa.out = out; sa.out_pan = out_pan; sa.pan_rows = pan_rows; sa.pdl = pdl;
+  ++ctx->launches;
+  { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_stream(ctx->kv_map_stream, sa, nb, rows, max_len, s.head_dim, ctx->n_sms, ctx->st)); }
+  return FC_OK;
+}
+static int run_fused_attn(fc_ctx *ctx, int l, const RowSegs &segs, int nb, int rows, int max_len, float *out, void *out_pan, int pan_rows, const ZeroList &z) {
+  const fc_model_shape &s = ctx->s;
+  const long long stride_h = (long long)s.max_seq * s.head_dim;
+  FusedAttnArgs fa; memset(&fa, 0, sizeof fa);
+  fa.qkv = ctx->b.qkv; fa.ldq = ctx->d.ldq; fa.ss = ctx->b.ss_attn; fa.eps = s.rms_eps; fa.dn = s.d_model;
+  fa.rope = ctx->b.rope; fa.c_magic = (unsigned int)((0x100000000ull + (unsigned)rows - 1) / (unsigned)rows);
+  fa.kcache = ctx->kv + (size_t)l * ctx->kv_layer_stride; fa.vcache = (char *)fa.kcache + ctx->kv_half_stride;
+  fa.stride_b = s.n_kv_heads * stride_h; fa.stride_h = stride_h;
+  fa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; fa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
+  fa.kv_len = ctx->b.kv_len; fa.b0 = segs.b0; fa.nb = nb; fa.c = rows; fa.hq = s.n_heads; fa.hkv = s.n_kv_heads;
+  fa.seq_map = segs.seq_map;
+  fused_attn_plan(max_len, rows, s.n_heads, s.n_kv_heads, nb, s.head_dim, ctx->n_sms, fa.nsplit, fa.qt);
+  fa.err = ctx->b.err;
+  fa.out = out; fa.pdl = ctx->pdl && !ctx->prof; fa.out_pan = out_pan; fa.pan_rows = pan_rows; fa.z = z;
+  ++ctx->launches;
+  { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_fused(ctx->kv_map, ctx->kv_map, fa, s.head_dim, ctx->st)); }
+  return FC_OK;
+}
+
+// A forward of at most kClusterRows rows: the projections between two attention launches in one launch with one writer per
+// output.  Every buffer is written before it is read: nothing to clear but the counters.
+static int forward_cluster(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, const int32_t *tokens, bool with_head, int max_len) {
+  const fc_model_shape &s = ctx->s;
+  const int L = s.n_layers, R = nb * rows, pdl = ctx->pdl && !ctx->prof;
+  ++ctx->launches;
+  {
+    ProfScope ps(ctx, FC_CLS_EMBED);
+    FC_CK(launch_embed_pair(tokens, ctx->tok_emb, ctx->g_attn[0], ctx->b.x, ctx->b.cl_pan_x, ctx->b.cl_ss_x, ctx->b.cl_bar, 8 * L + 2, R, s.d_model, pdl, ctx->st));
+  }
+  ClusterArgs ca; memset(&ca, 0, sizeof ca);
+  ca.R = R; ca.x = ctx->b.x; ca.qkv = ctx->b.qkv; ca.pan_x = ctx->b.cl_pan_x; ca.pan_h = ctx->b.cl_pan_h;
+  ca.ss_x = ctx->b.cl_ss_x; ca.ss_ffn = ctx->b.cl_ss_ffn; ca.ss_attn = ctx->b.ss_attn; ca.eps = s.rms_eps; ca.bar = ctx->b.cl_bar; ca.err = ctx->b.err;
+  ca.tokens = tokens; ca.perm = s.bias_beta != 0.f ? ctx->bias_perm : nullptr; ca.beta = s.bias_beta; ca.amax = ctx->b.amax; ca.logits = ctx->dbg_logits;
+  auto chain = [&](int first, int last, int cls) {
+    ++ctx->launches;
+    ProfScope ps(ctx, cls);
+    return launch_cluster_chain(ctx->plan_cl, ca, first, last, pdl, ctx->st);
+  };
+  const bool stream = with_head && attn_stream_pays(max_len, rows, s.n_heads, s.n_kv_heads, nb);
+  ZeroList none; memset(&none, 0, sizeof none);
+  FC_CK(chain(0, 1, FC_CLS_QKV));
+  for (int l = 0; l < L; ++l) {
+    int rc = stream ? run_stream_attn(ctx, l, segs, nb, rows, max_len, nullptr, ctx->b.cl_pan_a, kClusterRows, none)
+                    : run_fused_attn(ctx, l, segs, nb, rows, max_len, nullptr, ctx->b.cl_pan_a, kClusterRows, none);
+    if (rc != FC_OK) return rc;
+    if (!with_head && l + 1 == L) break;               // rows that are only cached: nothing reads what follows the last K/V rows
+    ca.g_ffn = ctx->g_ffn[l]; ca.g_next = l + 1 < L ? ctx->g_attn[l + 1] : ctx->g_final;
+    FC_CK(chain(4 * l + 1, l + 1 < L ? 4 * l + 5 : 4 * L, FC_CLS_CHAIN));
+  }
+  if (with_head) FC_CK(chain(4 * L, 4 * L + 1, FC_CLS_HEAD));
+  return FC_OK;
+}
+
 // One decoder forward over nb sequences (b0 .. b0+nb-1) with `rows` rows each.  tokens: device [nb*rows].
 // with_head: LM head + argmax + accept (a decode step); otherwise the rows are committed (prefill chunk).
 // seq_map (device, optional): row block i belongs to sequence seq_map[i] instead of b0 + i (finished sequences skipped).
@@ -635,6 +743,14 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
   }
   if (ctx->d.bulk && R >= kBulkMin) {
     int rc = forward_bulk(ctx, segs, nb, R, rows, max_len_host, tokens, with_head);
+    if (rc != FC_OK) return rc;
+    if (with_head) return run_accept(ctx, b0, nb, rows, seq_map, commit);
+    ++ctx->launches;
+    FC_CK(launch_advance(ctx->b.kv_len, segs, nb, ctx->st));
+    return FC_OK;
+  }
+  if (ctx->plan_cl && R <= kClusterRows) {
+    int rc = forward_cluster(ctx, segs, nb, rows, tokens, with_head, max_len_host);
     if (rc != FC_OK) return rc;
     if (with_head) return run_accept(ctx, b0, nb, rows, seq_map, commit);
     ++ctx->launches;
@@ -663,41 +779,16 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
       FC_CK(run_gemm(ctx, ctx->use_umma ? ctx->plan_qkv[l] : nullptr, args_qkv(ctx, l), R, PRO_GAIN, EPI_ATOMIC_ADD, FC_CLS_QKV, claim_word(ctx, l, GEMM_QKV)));
     void *kc = ctx->kv + (size_t)l * ctx->kv_layer_stride;
     void *vc = ctx->kv + (size_t)l * ctx->kv_layer_stride + ctx->kv_half_stride;
-    if (stream) {
-      QkvFinishArgs qa; memset(&qa, 0, sizeof qa);
-      qa.qkv = ctx->b.qkv; qa.ldq = d.ldq; qa.ss = ctx->b.ss_attn; qa.eps = s.rms_eps; qa.dn = s.d_model; qa.rope = ctx->b.rope;
-      qa.kv_len = ctx->b.kv_len; qa.segs = segs;
-      qa.hq = s.n_heads; qa.hkv = s.n_kv_heads; qa.hd = s.head_dim; qa.q = ctx->b.qb; qa.q_tiles = d.q_tiles;
-      qa.kcache = kc; qa.vcache = vc; qa.stride_b = stride_b; qa.stride_h = stride_h; qa.pdl = ctx->pdl && !ctx->prof;
-      qa.z.p[0] = ctx->b.gu; qa.z.n[0] = Rz * 2 * s.d_ffn;
-      qa.z.p[1] = ctx->b.ss_ffn; qa.z.n[1] = Rz;
-      ++ctx->launches;
-      { ProfScope ps(ctx, FC_CLS_ROPE); FC_CK(launch_qkv_finish(qa, R, ctx->st)); }
-      StreamAttnArgs sa; memset(&sa, 0, sizeof sa);
-      sa.q = ctx->b.qb; sa.q_tiles = d.q_tiles; sa.kv_len = ctx->b.kv_len; sa.segs = qa.segs; sa.hq = s.n_heads; sa.hkv = s.n_kv_heads;
-      sa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; sa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
-      sa.err = ctx->b.err; sa.out = ctx->b.attn; sa.pdl = ctx->pdl && !ctx->prof;
-      if (o_panel) { sa.out_pan = ctx->b.pan; sa.pan_rows = d.pan_rows; }
-      ++ctx->launches;
-      { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_stream(ctx->kv_map_stream, sa, nb, rows, max_len_host, s.head_dim, ctx->n_sms, ctx->st)); }
-    } else if (ctx->fused_attn) {
-      FusedAttnArgs fa; memset(&fa, 0, sizeof fa);
-      fa.qkv = ctx->b.qkv; fa.ldq = d.ldq; fa.ss = ctx->b.ss_attn; fa.eps = s.rms_eps; fa.dn = s.d_model;
-      fa.rope = ctx->b.rope; fa.c_magic = (unsigned int)((0x100000000ull + (unsigned)rows - 1) / (unsigned)rows);
-      fa.kcache = kc; fa.vcache = vc; fa.stride_b = stride_b; fa.stride_h = stride_h;
-      fa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; fa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
-      fa.kv_len = ctx->b.kv_len; fa.b0 = b0; fa.nb = nb; fa.c = rows; fa.hq = s.n_heads; fa.hkv = s.n_kv_heads;
-      fa.seq_map = seq_map;
-      fused_attn_plan(max_len_host, rows, s.n_heads, s.n_kv_heads, nb, s.head_dim, ctx->n_sms, fa.nsplit, fa.qt);
-      fa.err = ctx->b.err;
-      fa.out = ctx->b.attn; fa.pdl = ctx->pdl && !ctx->prof;
-      // more than 16 rows: the chained launch streams its activations from the bf16 panel; the attention kernel writes
-      // its result there directly, which saves the output projection's conversion pass and two grid-wide waits
-      if (o_panel) { fa.out_pan = ctx->b.pan; fa.pan_rows = d.pan_rows; }
-      fa.z.p[0] = ctx->b.gu; fa.z.n[0] = Rz * 2 * s.d_ffn;
-      fa.z.p[1] = ctx->b.ss_ffn; fa.z.n[1] = Rz;
-      ++ctx->launches;
-      { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_fused(ctx->kv_map, ctx->kv_map, fa, s.head_dim, ctx->st)); }
+    ZeroList za; memset(&za, 0, sizeof za);
+    za.p[0] = ctx->b.gu; za.n[0] = Rz * 2 * s.d_ffn;
+    za.p[1] = ctx->b.ss_ffn; za.n[1] = Rz;
+    // more than 16 rows: the chained launch streams its activations from the bf16 panel; the attention kernel writes
+    // its result there directly, which saves the output projection's conversion pass and two grid-wide waits
+    void *o_pan = o_panel ? ctx->b.pan : nullptr;
+    if (ctx->fused_attn) {
+      int rc = stream ? run_stream_attn(ctx, l, segs, nb, rows, max_len_host, ctx->b.attn, o_pan, d.pan_rows, za)
+                      : run_fused_attn(ctx, l, segs, nb, rows, max_len_host, ctx->b.attn, o_pan, d.pan_rows, za);
+      if (rc != FC_OK) return rc;
     } else {
       RopeArgs ra; memset(&ra, 0, sizeof ra);
       ra.qkv = ctx->b.qkv; ra.ldq = d.ldq; ra.ss = ctx->b.ss_attn; ra.eps = s.rms_eps; ra.dn = s.d_model;
@@ -705,8 +796,7 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
       ra.hq = s.n_heads; ra.hkv = s.n_kv_heads; ra.hd = s.head_dim; ra.rope = ctx->b.rope;
       ra.q_out = ctx->b.qb; ra.kcache = kc; ra.vcache = vc;
       ra.stride_b = stride_b; ra.stride_h = stride_h;
-      ra.z.p[0] = ctx->b.gu; ra.z.n[0] = Rz * 2 * s.d_ffn;
-      ra.z.p[1] = ctx->b.ss_ffn; ra.z.n[1] = Rz;
+      ra.z = za;
       ++ctx->launches;
       { ProfScope ps(ctx, FC_CLS_ROPE); FC_CK(launch_rope_kv(ra, s.dtype, ctx->st)); }
       AttnArgs aa; memset(&aa, 0, sizeof aa);

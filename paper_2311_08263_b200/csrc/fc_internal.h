@@ -302,6 +302,37 @@ cudaError_t launch_norm_pair(const float *x, const void *gain, float *ss, void *
 // kv_len[sequence] += rows for every segment
 cudaError_t launch_advance(int32_t *kv_len, const RowSegs &segs, int nseg, cudaStream_t st);
 
+// ---- up to 64 rows: chained projections with one writer per output (k_cluster.cu); d, qd, f multiples of 128, kvd and vocab of 16
+constexpr int kClusterRows = 64;
+constexpr int kClusterSlots = 160;                   // CTAs that the slots of the row sums of squares are laid out for
+struct ClusterModel {
+  int n_layers, d, qd, kvd, f, vocab;
+  const void *const *wq, *const *wk, *const *wv, *const *wo, *const *w_gate, *const *w_up, *const *w_down, *lm_head;   // host arrays of device pointers
+  const void *maps_dev;
+};
+struct ClusterPlan;
+bool cluster_shape_ok(int d, int qd, int kvd, int f, int vocab);
+size_t cluster_map_bytes(int n_layers);
+ClusterPlan *cluster_plan_create(const ClusterModel &m, void *maps_dev, void *pan_x, void *pan_a, void *pan_h, cudaStream_t st);
+void cluster_plan_destroy(ClusterPlan *p);
+struct ClusterArgs {
+  int R;
+  float *x, *qkv;                 // [R, d] residual, [R, qd + 2 kvd] (lacking 1/rms)
+  void *pan_x, *pan_h;            // operand pairs
+  const void *g_ffn, *g_next;     // gains behind the O and the down projection of this launch
+  float *ss_x, *ss_ffn;           // [kClusterSlots][kClusterRows]
+  float *ss_attn;                 // [R], written by the QKV projection
+  float eps;
+  unsigned int *bar;              // [8 * n_layers + 2], zero when a forward starts
+  const int32_t *tokens, *perm; float beta; unsigned long long *amax; float *logits;
+  unsigned int *err;
+};
+// projections [first, last) one after the other: 4 * layer + {0 QKV, 1 O, 2 gate/up, 3 down}, 4 * n_layers: the LM head
+cudaError_t launch_cluster_chain(const ClusterPlan *pl, const ClusterArgs &a, int first, int last, int pdl, cudaStream_t st);
+// x = E[token], pan = x * gain as a pair, ss[r] = sum x^2; words[0 .. n_words) = 0
+cudaError_t launch_embed_pair(const int32_t *tokens, const void *emb, const void *gain, float *x, void *pan, float *ss, unsigned int *words, int n_words,
+                              int R, int d, int pdl, cudaStream_t st);
+
 // Up to four projections in one launch, each consuming the previous one's reduced output; bar: n-1 zeroed words.
 // bar_b: n zeroed words (panel-ready barriers), needed when the rows exceed 16 and the plans have panels.
 // sync (optional, used up to 16 rows): how each projection is tied to the others, instead of a grid barrier

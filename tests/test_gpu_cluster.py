@@ -1,0 +1,43 @@
+"""The projections with one writer per output (up to 64 rows), reached through Jacobi steps, against the oracle: widths 16, 32 and
+64 at their edges, fewer weight units than clusters, column ranges of several tiles, a k range shorter than the cluster's shares,
+cached lengths around the key tiles, grouped queries, both head sizes.  Bars and margin rule as in test_gpu_full_configs.  Nothing
+in this route is added up in the order of arrival: a step repeated gives the same bits (the other tensor-core routes' steps
+differ in their last bits)."""
+import numpy as np
+import pytest
+
+from paper_2311_08263_b200 import workload as wl
+from test_gpu_full_configs import _random_kv_case
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # hq, hkv, hd, d, f, vocab, c, lens
+    (2, 1, 64, 128, 128, 528, 1, [0]),                             # one pair of k-blocks for four shares; one row, no cached key
+    (2, 2, 64, 256, 4480, 9600, 16, [33]),                         # two column ranges of gate and up, three of the LM head
+    (8, 2, 128, 640, 1408, 1040, 1, [700, 31, 0, 1, 32, 95]),      # six rows of a width of 16, grouped queries
+    (4, 4, 128, 512, 9088, 1024, 17, [640]),                       # 17 rows: a width of 32; three ranges, cut in front of the last
+    (10, 5, 64, 640, 896, 4240, 8, [64, 63, 65, 300]),             # 32 rows
+    (2, 2, 128, 256, 4480, 4240, 33, [96]),                        # 33 rows: a width of 64, windows over three 16-key blocks
+    (6, 3, 64, 384, 4480, 9600, 16, [5, 160, 0, 31]),              # 64 rows, passes of two tiles
+    (2, 1, 64, 128, 256, 528, 64, [40]),                           # a window of 64 rows of one sequence
+]
+
+
+@pytest.mark.parametrize("hq,hkv,hd,d,f,vocab,c,lens", CASES)
+def test_step_against_the_oracle_and_again(hq, hkv, hd, d, f, vocab, c, lens):
+    cfg = wl.small_config(n_layers=2, n_heads=hq, n_kv_heads=hkv, head_dim=hd, d_model=d, d_ffn=f, vocab=vocab, seed=2000 + c + hd)
+    dec, _ = _random_kv_case(cfg, lens, c, range(len(lens)))
+    assert dec.fc_last_launch_count() == 2 * cfg.n_layers + 4
+    logits = dec.fc_debug_logits(True)
+    pending = wl.make_random_window(cfg, len(lens), 1, salt=3).numpy()[:, 0]
+    window = wl.make_random_window(cfg, len(lens), c, salt=4).numpy()
+    window[:, 0] = pending
+    seen = []
+    for _ in range(3):
+        dec.fc_debug_set_state(lens, pending, c, pad_id=0)
+        logits.zero_()
+        dec.fc_jacobi_step(window)
+        seen.append(logits[:len(lens) * c].cpu().numpy().copy())
+    assert np.array_equal(seen[0], seen[1]) and np.array_equal(seen[0], seen[2])
+    assert dec.fc_debug_check_guards() == 0
