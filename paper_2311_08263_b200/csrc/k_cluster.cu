@@ -160,8 +160,8 @@ __device__ __forceinline__ void load_4d(uint32_t dst, const CUtensorMap *map, in
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar) : "memory");
 }
-// Arrival on a barrier of another CTA of the cluster, ordering this CTA's shared memory only.  (Release at cluster scope waits for
-// all global stores on their way: 0.7 us per exchange unit.)
+// Arrival on a barrier of another CTA of the cluster that orders nothing in front of it: the caller sees to it that its loads have
+// arrived.  (Release at cluster scope waits for all global stores on their way: 0.7 us per exchange unit.)
 __device__ __forceinline__ void mbar_arrive_far(uint32_t bar_cluster) {
   asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
@@ -208,20 +208,28 @@ __device__ __forceinline__ bool grid_wait(const unsigned int *word, unsigned int
   return true;
 }
 __device__ __forceinline__ void out_meet() { asm volatile("bar.sync 1, 128;" ::: "memory"); }       // the four output warps
+// N columns of the high and of the low products.  One statement: the registers hold nothing before the wait, so nothing that
+// reads them may be moved between the loads and it.
 template <int N>
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t *r) {
+__device__ __forceinline__ void tmem_ld_pair(uint32_t at_hi, uint32_t at_lo, uint32_t (&hi)[N], uint32_t (&lo)[N]) {
   if constexpr (N == 8) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&r"(hi[0]), "=&r"(hi[1]), "=&r"(hi[2]), "=&r"(hi[3]), "=&r"(hi[4]), "=&r"(hi[5]), "=&r"(hi[6]), "=&r"(hi[7]),
+          "=&r"(lo[0]), "=&r"(lo[1]), "=&r"(lo[2]), "=&r"(lo[3]), "=&r"(lo[4]), "=&r"(lo[5]), "=&r"(lo[6]), "=&r"(lo[7])
+        : "r"(at_hi), "r"(at_lo) : "memory");
   } else {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&r"(hi[0]), "=&r"(hi[1]), "=&r"(hi[2]), "=&r"(hi[3]), "=&r"(hi[4]), "=&r"(hi[5]), "=&r"(hi[6]), "=&r"(hi[7]), "=&r"(hi[8]), "=&r"(hi[9]), "=&r"(hi[10]), "=&r"(hi[11]), "=&r"(hi[12]), "=&r"(hi[13]), "=&r"(hi[14]), "=&r"(hi[15]),
+          "=&r"(lo[0]), "=&r"(lo[1]), "=&r"(lo[2]), "=&r"(lo[3]), "=&r"(lo[4]), "=&r"(lo[5]), "=&r"(lo[6]), "=&r"(lo[7]), "=&r"(lo[8]), "=&r"(lo[9]), "=&r"(lo[10]), "=&r"(lo[11]), "=&r"(lo[12]), "=&r"(lo[13]), "=&r"(lo[14]), "=&r"(lo[15])
+        : "r"(at_hi), "r"(at_lo) : "memory");
   }
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ uint32_t pack_pair(float a, float b) {
   __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t *>(&v);
@@ -367,6 +375,10 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
         ok = __shfl_sync(0xffffffffu, ok, 0);
       }
     }
+    // the MMAs' completions of the last round have landed on this CTA's barriers before it leaves
+    if (lane == 0 && ok)
+      for (int i = max(0, issued - S); i < issued; ++i)
+        if (!mbar_wait(smem_u32(&empty_w[i % S]), (uint32_t)(i / S) & 1u, abort_flag)) break;
     if (lane == 0) issued_w_s = issued;
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -457,6 +469,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
             ++issued;
           }
       }
+      for (int i = max(0, issued - NX); i < issued && ok; ++i) ok = mbar_wait(smem_u32(&empty_x[i % NX]), (uint32_t)(i / NX) & 1u, abort_flag);
       issued_x_s = issued;
     }
   } else if (warp < kOutWarp0) {
@@ -492,9 +505,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
 #pragma unroll
               for (int j = 0; j < H; j += N) {
                 uint32_t hi[N], lo[N];
-                tmem_ld<N>(ta + j, hi);
-                tmem_ld<N>(ta + BN + j, lo);
-                tmem_ld_wait();
+                tmem_ld_pair<N>(ta + j, ta + BN + j, hi, lo);
 #pragma unroll
                 for (int i = 0; i < N; ++i) sum[t][j + i] += __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
               }
@@ -522,6 +533,9 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
         e += tn * NCB;
       }
     }
+    // the peers' arrivals of the last units too: one that lands in the next kernel's barrier would let a sender there go too early
+    for (int u = max(0, e - C::NXB); u < e && ok; ++u)
+      if (BN == 16 || (u % NCB) / (NCB / 2 > 0 ? NCB / 2 : 1) == half) ok = mbar_wait_warp(smem_u32(&xc_empty[u % C::NXB]), (uint32_t)(u / C::NXB) & 1u, abort_flag);
   } else {
     // ------------------------------------------------------------ finished values
     const int ot = threadIdx.x - kOutWarp0 * 32, n = ot & 15, mq = ot >> 4;       // row n of a block of 16, weight rows 4 mq .. 4 mq + 3 of this CTA's 32
@@ -597,8 +611,10 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
 #pragma unroll
             for (int k = 1; k < kCl; ++k) v[i] += src[(k * 32 + i) * kXRow];
           }
-          __syncwarp();
-          if (lane < kCl) mbar_arrive_far(far_empty + (uint32_t)b * 8u);
+          // The buffer is free once the loads have arrived, not once they are issued: the vote needs the sums of every lane.  (No sum
+          // has this pattern - the NaN an addition makes has another - but nothing less than a value holds the arrival back.)
+          const bool unread = __any_sync(0xffffffffu, __float_as_uint((v[0] + v[1]) + (v[2] + v[3])) == 0x7fc12345u);
+          if (lane < kCl && !unread) mbar_arrive_far(far_empty + (uint32_t)b * 8u);
           if (kind == PH_O || kind == PH_DOWN) {
             if (mine) {
               v[0] += xr.x; v[1] += xr.y; v[2] += xr.z; v[3] += xr.w;

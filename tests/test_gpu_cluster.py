@@ -41,3 +41,28 @@ def test_step_against_the_oracle_and_again(hq, hkv, hd, d, f, vocab, c, lens):
         seen.append(logits[:len(lens) * c].cpu().numpy().copy())
     assert np.array_equal(seen[0], seen[1]) and np.array_equal(seen[0], seen[2])
     assert dec.fc_debug_check_guards() == 0
+
+
+@pytest.mark.parametrize("b,c,length", [(16, 1, 500), (1, 16, 800), (2, 16, 300), (4, 16, 300), (16, 1, 2048)])
+def test_wide_steps_repeat_bit_for_bit(b, c, length):
+    """Two layers of the 7B shape, fifty times the same step: exchange buffers that are written again before they are read, or
+    read before they are written, show as rows that differ."""
+    import dataclasses
+    import torch
+    from paper_2311_08263_b200 import engine
+    cfg = dataclasses.replace(wl.CONFIGS["7b"], n_layers=2)
+    w = wl.make_weights(cfg, device="cuda")
+    dec = engine.Decoder(cfg, w, b, c, length + c + 8)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    dec.kv_view().normal_(generator=gen)
+    window = wl.make_random_window(cfg, b, c, salt=4).numpy()
+    lens = [length - 31 * i % length for i in range(b)]
+    logits = dec.fc_debug_logits(True)
+    first = None
+    for _ in range(50):
+        dec.fc_debug_set_state(lens, window[:, 0], c, pad_id=0)
+        dec.fc_jacobi_step(window)
+        got = logits[:b * c].clone()
+        first = got if first is None else first
+        assert torch.equal(got, first)
