@@ -690,6 +690,20 @@ static int run_fused_attn(fc_ctx *ctx, int l, const RowSegs &segs, int nb, int r
   return FC_OK;
 }
 
+static int run_short_attn(fc_ctx *ctx, int l, const RowSegs &segs, int nb, int rows, int max_len, void *out_pan, int pan_rows) {
+  const fc_model_shape &s = ctx->s;
+  ShortAttnArgs a; memset(&a, 0, sizeof a);
+  a.qkv = ctx->b.qkv; a.ldq = ctx->d.ldq; a.ss = ctx->b.ss_attn; a.eps = s.rms_eps; a.dn = s.d_model; a.rope = ctx->b.rope;
+  a.kcache = ctx->kv + (size_t)l * ctx->kv_layer_stride; a.vcache = (char *)a.kcache + ctx->kv_half_stride;
+  a.stride_h = (long long)s.max_seq * s.head_dim; a.stride_b = s.n_kv_heads * a.stride_h;
+  a.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; a.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
+  a.kv_len = ctx->b.kv_len; a.seq_map = segs.seq_map; a.b0 = segs.b0; a.c = rows; a.hq = s.n_heads; a.hkv = s.n_kv_heads;
+  a.err = ctx->b.err; a.out_pan = out_pan; a.pan_rows = pan_rows; a.pdl = ctx->pdl && !ctx->prof;
+  ++ctx->launches;
+  { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_short(ctx->kv_map_stream, a, nb, max_len, s.head_dim, ctx->n_sms, ctx->st)); }
+  return FC_OK;
+}
+
 // A forward of at most kClusterRows rows: the projections between two attention launches in one launch with one writer per
 // output.  Every buffer is written before it is read: nothing to clear but the counters.
 static int forward_cluster(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, const int32_t *tokens, bool with_head, int max_len) {
@@ -714,7 +728,7 @@ static int forward_cluster(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, c
   FC_CK(chain(0, 1, FC_CLS_QKV));
   for (int l = 0; l < L; ++l) {
     int rc = stream ? run_stream_attn(ctx, l, segs, nb, rows, max_len, nullptr, ctx->b.cl_pan_a, kClusterRows, none)
-                    : run_fused_attn(ctx, l, segs, nb, rows, max_len, nullptr, ctx->b.cl_pan_a, kClusterRows, none);
+                    : run_short_attn(ctx, l, segs, nb, rows, max_len, ctx->b.cl_pan_a, kClusterRows);
     if (rc != FC_OK) return rc;
     if (!with_head && l + 1 == L) break;               // rows that are only cached: nothing reads what follows the last K/V rows
     ca.g_ffn = ctx->g_ffn[l]; ca.g_next = l + 1 < L ? ctx->g_attn[l + 1] : ctx->g_final;

@@ -161,6 +161,20 @@ struct StreamAttnArgs {   // bf16: window attention over rows whose K/V are in t
   int pdl;
 };
 
+struct ShortAttnArgs {    // bf16: as FusedAttnArgs, for few queries over short caches (k_attn_short.cu); the result is the bf16 pair out_pan
+  const float *qkv; int ldq;
+  const float *ss; float eps; int dn;
+  const float2 *rope;
+  void *kcache, *vcache; long long stride_b, stride_h;
+  int k_plane0, v_plane0;
+  const int32_t *kv_len, *seq_map;
+  int b0, c, hq, hkv;
+  unsigned int *err;
+  void *out_pan; int pan_rows;
+  int stages;             // tiles in flight per warp (set by the launcher)
+  int pdl;
+};
+
 struct AcceptArgs {
   int32_t *window;                 // [batch, c] in/out
   const unsigned long long *amax;  // packed argmax per row, or null
@@ -239,6 +253,7 @@ cudaError_t launch_qkv_finish(const QkvFinishArgs &a, int R, cudaStream_t st);
 // map: boxes of attn_stream_tile_keys() keys; max_rows / max_len: the longest segment and (a bound on) the longest cache
 cudaError_t launch_attn_stream(const KvTensorMap &map, const StreamAttnArgs &a, int nseg, int max_rows, int max_len, int hd,
                                int n_sms, cudaStream_t st);
+cudaError_t launch_attn_short(const KvTensorMap &map, const ShortAttnArgs &a, int nb, int max_len, int hd, int n_sms, cudaStream_t st);
 bool attn_stream_pays(int max_len, int c, int hq, int hkv, int nb);
 int attn_stream_tile_keys();
 size_t attn_stream_q_tiles(int rows, int group, int nseg);      // tiles per kv head for `rows` rows in nseg segments

@@ -1,0 +1,417 @@
+// Window attention of few (sequence, kv head, 16-query) units over short caches, with everything around it in the same
+// kernel: 1/rms and rotation of the queries and of the window's keys out of the fp32 QKV accumulators, K/V rows into the cache.
+//
+// What bounds it: latency from the QKV projection's end to the output projection's operand - the K/V bytes (13 MB per layer of
+// 7B over 800 keys) are on their way before the kernel in front has finished.  So the chain behind that point is
+// kept short: grid (key splits, kv heads x query tiles, sequences), the splits of a unit are one cluster; four warps,
+// each on 32-key tiles of its own (its own ring stages, requested by itself: no producer, no block-wide barrier per tile), queries
+// straight from the accumulators into the registers of MMA A operands, scores and output in registers (the accumulators of Q.K^T are
+// the A operand of P.V as they are), one merge of the warps and one of the splits.  The last split also turns the
+// window's own keys and values into bf16 in shared memory and in the cache; blocks of 16 window keys are causal.
+// q and the probabilities enter the tensor cores as bf16 pairs, so that only the stored K/V are rounded.
+// Row j of a sequence sees keys 0 .. kv_len + j.  Every wait is bounded.
+#include <cstring>
+
+#include "fc_attn.cuh"
+#include "fc_internal.h"
+#include "fc_ptx.cuh"
+
+namespace fc {
+
+namespace {
+constexpr int kShortKeys = 32;                     // keys per tile
+constexpr int kShortWarps = 4, kShortThreads = kShortWarps * 32;
+constexpr int kShortStages = 2;                    // tiles in flight per warp at most
+
+template <int HD>
+struct ShortCfg {
+  static constexpr int SUB = HD / 64;              // 128-byte sub-tiles per row
+  static constexpr uint32_t kSub = kShortKeys * 128;
+  static constexpr uint32_t kHalf = SUB * kSub;    // K (or V) of a tile
+  static constexpr uint32_t kTile = 2 * kHalf;     // 16 KB, 8 KB
+  static constexpr int OLD = HD + 8;               // row pitch of the partial outputs (floats): spreads the banks
+  static_assert(kShortWarps * 16 * OLD * 4 <= kShortWarps * (int)kTile, "partial outputs fit over one stage per warp");
+};
+template <int HD> size_t short_smem(int c, int stages) {
+  return 1024 + (size_t)kShortWarps * stages * ShortCfg<HD>::kTile + (size_t)((c + 15) / 16 * 16) * HD * 4;
+}
+
+// Byte offset of 16-byte piece `ch` of row `r` in sub-tiles of 128-byte rows, `sub` bytes apart, with the TMA's swizzle.
+__device__ __forceinline__ uint32_t piece(int r, int ch, uint32_t sub) {
+  return (uint32_t)(ch >> 3) * sub + (uint32_t)r * 128u + (uint32_t)(((ch & 7) ^ (r & 7)) << 4);
+}
+
+// One block of 8 * NT keys: scores, probabilities, output of a warp's 16 queries.  vis(n, i): key 8 n + 2 (lane & 3) + (i & 1) is
+// visible to the row of accumulator i; all: every key is to every row.
+template <int HD, int NT, typename Vis>
+__device__ __forceinline__ void attend(uint32_t kb, uint32_t vb, uint32_t sub, const uint32_t (&qh)[HD / 16][4], const uint32_t (&ql)[HD / 16][4],
+                                       float (&o)[HD / 8][4], float (&m_run)[2], float (&l_run)[2], float sl2, int lane, bool all, Vis vis) {
+  float s[NT][4];
+#pragma unroll
+  for (int n = 0; n < NT; ++n)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[n][i] = 0.f;
+#pragma unroll
+  for (int k2 = 0; k2 < HD / 32; ++k2) {
+    uint32_t kf[NT][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) ldsm4(kb + piece(n * 8 + (lane & 7), k2 * 4 + (lane >> 3), sub), kf[n]);
+#pragma unroll
+    for (int n = 0; n < NT; ++n) mma16816(s[n], qh[2 * k2], kf[n][0], kf[n][1]);
+#pragma unroll
+    for (int n = 0; n < NT; ++n) mma16816(s[n], ql[2 * k2], kf[n][0], kf[n][1]);
+#pragma unroll
+    for (int n = 0; n < NT; ++n) mma16816(s[n], qh[2 * k2 + 1], kf[n][2], kf[n][3]);
+#pragma unroll
+    for (int n = 0; n < NT; ++n) mma16816(s[n], ql[2 * k2 + 1], kf[n][2], kf[n][3]);
+  }
+  if (!all) {
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (!vis(n, i)) s[n][i] = -INFINITY;
+  }
+  float mx[2] = {m_run[0], m_run[1]};
+#pragma unroll
+  for (int n = 0; n < NT; ++n) {
+    mx[0] = fmaxf(mx[0], fmaxf(s[n][0], s[n][1]));
+    mx[1] = fmaxf(mx[1], fmaxf(s[n][2], s[n][3]));
+  }
+  float mb[2];
+#pragma unroll
+  for (int hh = 0; hh < 2; ++hh) {
+    mx[hh] = fmaxf(mx[hh], __shfl_xor_sync(0xffffffffu, mx[hh], 1));
+    mx[hh] = fmaxf(mx[hh], __shfl_xor_sync(0xffffffffu, mx[hh], 2));
+    const float corr = mx[hh] == -INFINITY ? 1.f : ex2((m_run[hh] - mx[hh]) * sl2);       // first block: 2^-inf = 0
+    l_run[hh] *= corr;
+    m_run[hh] = mx[hh];
+    mb[hh] = mx[hh] == -INFINITY ? 0.f : mx[hh] * sl2;
+#pragma unroll
+    for (int n = 0; n < HD / 8; ++n) { o[n][2 * hh] *= corr; o[n][2 * hh + 1] *= corr; }
+  }
+#pragma unroll
+  for (int n = 0; n < NT; ++n) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[n][i] = ex2(fmaf(s[n][i], sl2, -mb[i >> 1]));
+    l_run[0] += s[n][0] + s[n][1];
+    l_run[1] += s[n][2] + s[n][3];
+  }
+#pragma unroll
+  for (int kk = 0; kk < NT / 2; ++kk) {
+    uint32_t ph[4], pl[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const float p0 = s[2 * kk + (x >> 1)][(x & 1) * 2], p1 = s[2 * kk + (x >> 1)][(x & 1) * 2 + 1];
+      ph[x] = pack2(p0, p1);
+      pl[x] = pack2(p0 - low_half(ph[x]), p1 - high_half(ph[x]));
+    }
+#pragma unroll
+    for (int n4 = 0; n4 < HD / 32; ++n4) {
+      uint32_t vf[2][4];
+      ldsm4t(vb + piece(kk * 16 + (lane & 15), n4 * 4 + (lane >> 4), sub), vf[0]);
+      ldsm4t(vb + piece(kk * 16 + (lane & 15), n4 * 4 + 2 + (lane >> 4), sub), vf[1]);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) mma16816(o[4 * n4 + x], ph, vf[x >> 1][(x & 1) * 2], vf[x >> 1][(x & 1) * 2 + 1]);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) mma16816(o[4 * n4 + x], pl, vf[x >> 1][(x & 1) * 2], vf[x >> 1][(x & 1) * 2 + 1]);
+    }
+  }
+}
+}  // namespace
+
+template <int HD>
+__global__ void __launch_bounds__(kShortThreads, 2)
+attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ ShortAttnArgs a) {
+  using C = ShortCfg<HD>;
+  constexpr int HALF = HD / 2, KS = HD / 16, OLD = C::OLD;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) unsigned long long full_bar[kShortWarps][kShortStages];
+  __shared__ float2 ml[kShortWarps][16];           // (max, sum) per warp and query row
+  __shared__ __align__(8) float2 ml_cta[16];       // after the merge of the CTA's warps
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g4 = lane >> 2, t4 = lane & 3;
+  const int split = blockIdx.x, ns = gridDim.x, NS = a.stages;
+  const int group = a.hq / a.hkv, c = a.c, nq = group * c;
+  const int kvh = blockIdx.y % a.hkv, q0 = (blockIdx.y / a.hkv) * 16;                 // first query of the tile; query q = row * group + head of the group
+  const int bl = blockIdx.z, b = a.seq_map ? a.seq_map[bl] : a.b0 + bl;
+  const int qd = a.hq * HD, kvd = a.hkv * HD;
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  unsigned char *gen = smem_raw + (base - smem_u32(smem_raw));
+  float *obuf = reinterpret_cast<float *>(gen);    // [warps][16][OLD], over the ring
+  const int wrows = (c + 15) & ~15;
+  const uint32_t wsub = (uint32_t)wrows * 128u, win_k = base + (uint32_t)(kShortWarps * NS) * C::kTile, win_v = win_k + C::SUB * wsub;
+
+  const int L = a.kv_len[b];
+  const int n_all = (L + kShortKeys - 1) / kShortKeys;                               // tiles of cached keys
+  const int n_cta = n_all > split ? (n_all - split + ns - 1) / ns : 0;               // this CTA's: split, split + ns, ...
+  const int n_mine = n_cta > warp ? (n_cta - warp + kShortWarps - 1) / kShortWarps : 0;       // this warp's: every fourth of them
+  const int plane_k = a.k_plane0 + b * a.hkv + kvh, plane_v = a.v_plane0 + b * a.hkv + kvh;
+  const uint32_t ring = base + (uint32_t)(warp * NS) * C::kTile;
+  auto key0_of = [&](int i) { return (split + (warp + i * kShortWarps) * ns) * kShortKeys; };
+  auto request = [&](int i) {                      // lane 0
+    const int stage = i % NS;
+    const uint32_t bar = smem_u32(&full_bar[warp][stage]), dst = ring + (uint32_t)stage * C::kTile;
+    const int y = key0_of(i);
+    mbar_expect_tx(bar, C::kTile);
+#pragma unroll
+    for (int s = 0; s < C::SUB; ++s) load_3d(dst + s * C::kSub, &map, s * 64, y, plane_k, bar);
+#pragma unroll
+    for (int s = 0; s < C::SUB; ++s) load_3d(dst + C::kHalf + s * C::kSub, &map, s * 64, y, plane_v, bar);
+  };
+  if (lane == 0) {
+    for (int i = 0; i < kShortStages; ++i) mbar_init(smem_u32(&full_bar[warp][i]), 1);
+    fence_barrier_init();
+    fence_proxy_async();
+    // cached keys were written by earlier steps
+    for (int i = 0; i < NS && i < n_mine; ++i) request(i);
+  }
+  __syncwarp();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  // ---- the window's own keys and values (last split)
+  const bool has_win = split == ns - 1;
+  if (has_win) {
+    const bool store = q0 == 0;                    // one query tile of the kv head writes the cache
+    __nv_bfloat16 *kc = (__nv_bfloat16 *)a.kcache + (long long)b * a.stride_b + (long long)kvh * a.stride_h + (long long)L * HD;
+    __nv_bfloat16 *vc = (__nv_bfloat16 *)a.vcache + (long long)b * a.stride_b + (long long)kvh * a.stride_h + (long long)L * HD;
+    constexpr int PER = HALF / 2;                  // two adjacent pairs per thread and pass
+#pragma unroll 4
+    for (int u = tid; u < wrows * PER; u += kShortThreads) {
+      const int j = u / PER, i = (u % PER) * 2;
+      uint32_t k0 = 0u, k1 = 0u, v0 = 0u, v1 = 0u;                 // rows behind the window: zero (a zero probability meets no NaN pattern)
+      if (j < c) {
+        const int r = bl * c + j;
+        const float *src = a.qkv + (long long)r * a.ldq + qd + kvh * HD + i;
+        const float s = rsqrtf(__ldcg(a.ss + r) / (float)a.dn + a.eps);
+        const float2 x = __ldcg(reinterpret_cast<const float2 *>(src)), y = __ldcg(reinterpret_cast<const float2 *>(src + HALF));
+        const float2 p = __ldcg(reinterpret_cast<const float2 *>(src + kvd)), q = __ldcg(reinterpret_cast<const float2 *>(src + kvd + HALF));
+        const float4 t = __ldg(reinterpret_cast<const float4 *>(a.rope + (long long)(L + j) * HALF + i));
+        const float x0 = x.x * s, x1 = x.y * s, y0 = y.x * s, y1 = y.y * s;
+        k0 = pack2(x0 * t.x - y0 * t.y, x1 * t.z - y1 * t.w);
+        k1 = pack2(x0 * t.y + y0 * t.x, x1 * t.w + y1 * t.z);
+        v0 = pack2(p.x * s, p.y * s); v1 = pack2(q.x * s, q.y * s);
+        if (store) {
+          *reinterpret_cast<uint32_t *>(kc + (long long)j * HD + i) = k0; *reinterpret_cast<uint32_t *>(kc + (long long)j * HD + i + HALF) = k1;
+          *reinterpret_cast<uint32_t *>(vc + (long long)j * HD + i) = v0; *reinterpret_cast<uint32_t *>(vc + (long long)j * HD + i + HALF) = v1;
+        }
+      }
+      const uint32_t o0 = piece(j, i >> 3, wsub) + (uint32_t)(i & 7) * 2u, o1 = piece(j, (i + HALF) >> 3, wsub) + (uint32_t)(i & 7) * 2u;
+      *reinterpret_cast<uint32_t *>(gen + (win_k - base) + o0) = k0; *reinterpret_cast<uint32_t *>(gen + (win_k - base) + o1) = k1;
+      *reinterpret_cast<uint32_t *>(gen + (win_v - base) + o0) = v0; *reinterpret_cast<uint32_t *>(gen + (win_v - base) + o1) = v1;
+    }
+  }
+
+  // ---- queries as MMA A operands: lane holds elements 16 ks + 8 x + 2 t4, + 1 of rows g4 and g4 + 8; the rotation pairs
+  // element e of block ks with the same element of block ks + KS / 2
+  uint32_t qh[KS][4], ql[KS][4];
+#pragma unroll
+  for (int hh = 0; hh < 2; ++hh) {
+    const int q = q0 + g4 + hh * 8;
+    const bool live = q < nq;
+    const int j = live ? q / group : 0, r = bl * c + j;
+    const float *src = a.qkv + (long long)r * a.ldq + (kvh * group + (live ? q - j * group : 0)) * HD;
+    const float2 *rot = a.rope + (long long)(L + j) * HALF;
+    const float s = live ? rsqrtf(__ldcg(a.ss + r) / (float)a.dn + a.eps) : 0.f;
+#pragma unroll
+    for (int ks = 0; ks < KS / 2; ++ks)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int e = ks * 16 + x * 8 + t4 * 2;
+        const float2 u = __ldcg(reinterpret_cast<const float2 *>(src + e)), w = __ldcg(reinterpret_cast<const float2 *>(src + e + HALF));
+        const float4 t = __ldg(reinterpret_cast<const float4 *>(rot + e));
+        const float u0 = u.x * s, u1 = u.y * s, w0 = w.x * s, w1 = w.y * s;
+        const float a0 = u0 * t.x - w0 * t.y, a1 = u1 * t.z - w1 * t.w, b0 = u0 * t.y + w0 * t.x, b1 = u1 * t.w + w1 * t.z;
+        const int g = hh + 2 * x;
+        qh[ks][g] = pack2(a0, a1);
+        ql[ks][g] = pack2(a0 - low_half(qh[ks][g]), a1 - high_half(qh[ks][g]));
+        qh[ks + KS / 2][g] = pack2(b0, b1);
+        ql[ks + KS / 2][g] = pack2(b0 - low_half(qh[ks + KS / 2][g]), b1 - high_half(qh[ks + KS / 2][g]));
+      }
+  }
+  if (has_win) __syncthreads();                    // the window's keys are staged
+
+  const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
+  float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f}, o[HD / 8][4];
+#pragma unroll
+  for (int n = 0; n < HD / 8; ++n)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) o[n][i] = 0.f;
+  bool ok = true;
+  for (int i = 0; i < n_mine; ++i) {
+    const int stage = i % NS, key0 = key0_of(i);
+    if (!__all_sync(0xffffffffu, wait_bounded(smem_u32(&full_bar[warp][stage]), (uint32_t)(i / NS) & 1u))) { ok = false; break; }
+    const uint32_t kb = ring + (uint32_t)stage * C::kTile, vb = kb + C::kHalf;
+    const bool whole = key0 + kShortKeys <= L;
+    if (!whole) {
+      // values beyond the cached keys: whatever the slab holds there may be a NaN pattern
+      unsigned char *vg = gen + (vb - base);
+      for (int e = lane; e < (key0 + kShortKeys - L) * (HD / 8); e += 32)
+        *reinterpret_cast<uint4 *>(vg + piece(L - key0 + e / (HD / 8), e % (HD / 8), C::kSub)) = make_uint4(0, 0, 0, 0);
+      __syncwarp();
+    }
+    attend<HD, kShortKeys / 8>(kb, vb, C::kSub, qh, ql, o, m_run, l_run, sl2, lane, whole,
+                               [&](int n, int x) { return key0 + n * 8 + t4 * 2 + (x & 1) < L; });
+    __syncwarp();
+    if (lane == 0 && i + NS < n_mine) { fence_proxy_async(); request(i + NS); }
+  }
+  if (has_win) {
+    // 16-key blocks of the window, dealt to the warps behind the cached tiles
+    const int j0 = min(q0 + g4, nq - 1) / group, j1 = min(q0 + g4 + 8, nq - 1) / group, j_last = min(q0 + 15, nq - 1) / group;
+    for (int blk = (warp - n_cta % kShortWarps + kShortWarps) % kShortWarps; blk * 16 < wrows; blk += kShortWarps) {
+      if (blk * 16 > j_last) break;
+      attend<HD, 2>(win_k + (uint32_t)blk * 2048u, win_v + (uint32_t)blk * 2048u, wsub, qh, ql, o, m_run, l_run, sl2, lane, false,
+                    [&](int n, int x) { return blk * 16 + n * 8 + t4 * 2 + (x & 1) <= (x >> 1 ? j1 : j0); });
+    }
+  }
+#pragma unroll
+  for (int hh = 0; hh < 2; ++hh) {
+    l_run[hh] += __shfl_xor_sync(0xffffffffu, l_run[hh], 1);
+    l_run[hh] += __shfl_xor_sync(0xffffffffu, l_run[hh], 2);
+  }
+  if (!__syncthreads_and(ok ? 1 : 0)) {
+    // a tile did not arrive: no result; copies on their way stay inside this CTA's ring, which outlives them as far as the bound
+    if (lane == 0) {
+      atomicExch(a.err, 1u);
+      const unsigned long long t0 = clock64();
+      for (int i = 0; i < NS && i < n_mine; ++i)
+        while (!mbar_try(smem_u32(&full_bar[warp][i]), (uint32_t)((n_mine - 1 - i) / NS) & 1u))
+          if ((unsigned long long)(clock64() - t0) > kSpinBudget / 4) break;
+    }
+    __syncthreads();
+  }
+
+  // ---- partial results of the warps
+  {
+    float *ob = obuf + warp * 16 * OLD;
+#pragma unroll
+    for (int n = 0; n < HD / 8; ++n) {
+      *reinterpret_cast<float2 *>(ob + g4 * OLD + n * 8 + t4 * 2) = make_float2(o[n][0], o[n][1]);
+      *reinterpret_cast<float2 *>(ob + (g4 + 8) * OLD + n * 8 + t4 * 2) = make_float2(o[n][2], o[n][3]);
+    }
+    if (t4 == 0) { ml[warp][g4] = make_float2(m_run[0], l_run[0]); ml[warp][g4 + 8] = make_float2(m_run[1], l_run[1]); }
+  }
+  __syncthreads();
+  auto store = [&](int row, int c4, float4 v) {
+    const int q = q0 + row, j = q / group, h = kvh * group + q - j * group;
+    const long long at = (long long)(bl * c + j) * qd + h * HD + c4 * 4;
+    const uint2 hi = make_uint2(pack2(v.x, v.y), pack2(v.z, v.w));
+    __nv_bfloat16 *p = (__nv_bfloat16 *)a.out_pan + at;
+    *reinterpret_cast<uint2 *>(p) = hi;
+    *reinterpret_cast<uint2 *>(p + (long long)a.pan_rows * qd) =
+        make_uint2(pack2(v.x - low_half(hi.x), v.y - high_half(hi.x)), pack2(v.z - low_half(hi.y), v.w - high_half(hi.y)));
+  };
+  for (int u = tid; u < 16 * (HD / 4); u += kShortThreads) {
+    const int row = u / (HD / 4), c4 = u - row * (HD / 4);
+    float M = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kShortWarps; ++k) M = fmaxf(M, ml[k][row].x);
+    float den = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < kShortWarps; ++k) {
+      const float2 v = ml[k][row];
+      const float w = v.x == -INFINITY ? 0.f : ex2((v.x - M) * sl2);
+      const float4 x = *reinterpret_cast<const float4 *>(obuf + (k * 16 + row) * OLD + c4 * 4);
+      den = fmaf(v.y, w, den);
+      acc.x = fmaf(w, x.x, acc.x); acc.y = fmaf(w, x.y, acc.y); acc.z = fmaf(w, x.z, acc.z); acc.w = fmaf(w, x.w, acc.w);
+    }
+    if (ns == 1) {
+      if (q0 + row < nq) {
+        const float inv = 1.0f / den;
+        store(row, c4, make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
+      }
+    } else {
+      *reinterpret_cast<float4 *>(obuf + row * OLD + c4 * 4) = acc;                     // only this thread reads these
+      if (c4 == 0) ml_cta[row] = make_float2(M, den);
+    }
+  }
+  if (ns > 1) {
+    // ---- merge of the key splits through the cluster's shared memory
+    __syncwarp();
+    cluster_sync_all();
+    const uint32_t ml_addr = smem_u32(ml_cta);
+    for (int u = split * kShortThreads + tid; u < 16 * (HD / 4); u += ns * kShortThreads) {
+      const int row = u / (HD / 4), c4 = u - row * (HD / 4);
+      if (q0 + row >= nq) continue;
+      float2 mv[8];
+      float4 ov[8];
+#pragma unroll
+      for (int sp = 0; sp < 8; ++sp) {
+        mv[sp] = make_float2(-INFINITY, 0.f);
+        ov[sp] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (sp < ns) {
+          mv[sp] = ld_cluster_f2(map_to_cta(ml_addr + (uint32_t)row * 8u, (uint32_t)sp));
+          ov[sp] = ld_cluster_f4(map_to_cta(base + (uint32_t)(row * OLD + c4 * 4) * 4u, (uint32_t)sp));
+        }
+      }
+      float M = -INFINITY;
+#pragma unroll
+      for (int sp = 0; sp < 8; ++sp) M = fmaxf(M, mv[sp].x);
+      float den = 0.f;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int sp = 0; sp < 8; ++sp) {
+        const float w = mv[sp].x == -INFINITY ? 0.f : ex2((mv[sp].x - M) * sl2);
+        den = fmaf(mv[sp].y, w, den);
+        acc.x = fmaf(w, ov[sp].x, acc.x); acc.y = fmaf(w, ov[sp].y, acc.y);
+        acc.z = fmaf(w, ov[sp].z, acc.z); acc.w = fmaf(w, ov[sp].w, acc.w);
+      }
+      const float inv = 1.0f / den;
+      store(row, c4, make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
+    }
+    __syncwarp();
+    cluster_sync_all();                            // the other splits may still be reading this CTA's memory
+  }
+}
+
+// ------------------------------------------------------------------------------------ host side
+template <int HD>
+static cudaError_t launch_short_t(const KvTensorMap &map, const ShortAttnArgs &a, int ns, int nqt, int nb, cudaStream_t st) {
+  const size_t smem = short_smem<HD>(a.c, a.stages);
+  static size_t attr_smem[kMaxDevices] = {0};
+  const int dev = current_device_slot();
+  if (smem > attr_smem[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(attn_short_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr_smem[dev] = smem;
+  }
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3(ns, a.hkv * nqt, nb); cfg.blockDim = dim3(kShortThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int na = 0;
+  if (a.pdl) {
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  if (ns > 1) {
+    attr[na].id = cudaLaunchAttributeClusterDimension;
+    attr[na].val.clusterDim.x = (unsigned)ns; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  cfg.attrs = attr; cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, attn_short_kernel<HD>, *reinterpret_cast<const CUtensorMap *>(&map), a);
+}
+
+// map: boxes of attn_stream_tile_keys() keys.
+cudaError_t launch_attn_short(const KvTensorMap &map, const ShortAttnArgs &a, int nb, int max_len, int hd, int n_sms, cudaStream_t st) {
+  if (nb < 1 || nb > 65535 || a.c < 1 || a.c > 64 || !a.err || !a.out_pan || (hd != 64 && hd != 128)) return cudaErrorInvalidValue;
+  const int nqt = ((a.hq / a.hkv) * a.c + 15) / 16;
+  if ((long long)a.hkv * nqt > 65535) return cudaErrorInvalidValue;
+  const long long units = (long long)nb * a.hkv * nqt;
+  const int tiles = (max_len + kShortKeys - 1) / kShortKeys;
+  // one CTA per SM, or two where that leaves a warp more than two tiles
+  long long ns = n_sms / units;
+  if (ns < 1) ns = 1;
+  if (tiles > 2 * kShortWarps * ns) ns = 2ll * n_sms / units;
+  if (ns > 8) ns = 8;
+  if (ns > (tiles + kShortWarps - 1) / kShortWarps) ns = (tiles + kShortWarps - 1) / kShortWarps;
+  if (ns < 1) ns = 1;
+  ShortAttnArgs args = a;
+  args.stages = units * ns > n_sms ? 1 : kShortStages;           // more than one CTA per SM: two have to fit
+  return hd == 128 ? launch_short_t<128>(map, args, (int)ns, nqt, nb, st) : launch_short_t<64>(map, args, (int)ns, nqt, nb, st);
+}
+
+}  // namespace fc
