@@ -4,9 +4,8 @@
 // What bounds it: latency from the QKV projection's end to the output projection's operand - the K/V bytes (13 MB per layer of
 // 7B over 800 keys) are on their way before the kernel in front has finished.  So the chain behind that point is
 // kept short: grid (key splits, kv heads x query tiles, sequences), the splits of a unit are one cluster; four warps,
-// each on 32-key tiles of its own (its own ring stages, requested by itself: no producer, no block-wide barrier per tile), queries
-// straight from the accumulators into the registers of MMA A operands, scores and output in registers (the accumulators of Q.K^T are
-// the A operand of P.V as they are), one merge of the warps and one of the splits.  The last split also turns the
+// each on 32-key tiles of its own (its own ring stages, requested by itself: no producer, no block-wide barrier per tile), queries in
+// the registers of MMA A operands, scores and output in registers (the accumulators of Q.K^T are the A operand of P.V as they are), one merge of the warps and one of the splits.  The last split also turns the
 // window's own keys and values into bf16 in shared memory and in the cache; blocks of 16 window keys are causal.
 // q and the probabilities enter the tensor cores as bf16 pairs, so that only the stored K/V are rounded.
 // Row j of a sequence sees keys 0 .. kv_len + j.  Every wait is bounded.
@@ -29,11 +28,12 @@ struct ShortCfg {
   static constexpr uint32_t kSub = kShortKeys * 128;
   static constexpr uint32_t kHalf = SUB * kSub;    // K (or V) of a tile
   static constexpr uint32_t kTile = 2 * kHalf;     // 16 KB, 8 KB
+  static constexpr uint32_t kQ = 16 * HD * 4;      // 16 queries, high and low
   static constexpr int OLD = HD + 8;               // row pitch of the partial outputs (floats): spreads the banks
   static_assert(kShortWarps * 16 * OLD * 4 <= kShortWarps * (int)kTile, "partial outputs fit over one stage per warp");
 };
 template <int HD> size_t short_smem(int c, int stages) {
-  return 1024 + (size_t)kShortWarps * stages * ShortCfg<HD>::kTile + (size_t)((c + 15) / 16 * 16) * HD * 4;
+  return 1024 + (size_t)kShortWarps * stages * ShortCfg<HD>::kTile + (size_t)((c + 15) / 16 * 16) * HD * 4 + ShortCfg<HD>::kQ;
 }
 
 // Byte offset of 16-byte piece `ch` of row `r` in sub-tiles of 128-byte rows, `sub` bytes apart, with the TMA's swizzle.
@@ -140,6 +140,7 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
   float *obuf = reinterpret_cast<float *>(gen);    // [warps][16][OLD], over the ring
   const int wrows = (c + 15) & ~15;
   const uint32_t wsub = (uint32_t)wrows * 128u, win_k = base + (uint32_t)(kShortWarps * NS) * C::kTile, win_v = win_k + C::SUB * wsub;
+  unsigned char *q_area = gen + (win_v - base) + C::SUB * wsub;
 
   const int L = a.kv_len[b];
   const int n_all = (L + kShortKeys - 1) / kShortKeys;                               // tiles of cached keys
@@ -169,67 +170,77 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
+  // Queries and window keys by loops of few instructions over the block: code that runs once per launch costs its fetch (each warp
+  // straight from the accumulators into its registers, 128 loads unrolled: 4 us).
+  // ---- queries, in the order in which a warp holds them as MMA A operands: [high, low][16-wide k block][lane][4 registers]
+  {
+    constexpr int PT = HALF / 8;                   // pairs (i, i + HALF) per thread: 8 or 4 adjacent ones
+    const int rr = tid >> 3, q = q0 + rr;
+    const bool live = q < nq;
+    const int j = live ? q / group : 0, r = bl * c + j, i0 = (tid & 7) * PT;
+    const float *src = a.qkv + (long long)r * a.ldq + (kvh * group + (live ? q - j * group : 0)) * HD + i0;
+    const float4 *rot = reinterpret_cast<const float4 *>(a.rope + (long long)(L + j) * HALF + i0);
+    float4 u[PT / 4], w[PT / 4], t[PT / 2];
+    const float ss = __ldcg(a.ss + r);
+#pragma unroll
+    for (int k = 0; k < PT / 4; ++k) { u[k] = __ldcg(reinterpret_cast<const float4 *>(src) + k); w[k] = __ldcg(reinterpret_cast<const float4 *>(src + HALF) + k); }
+#pragma unroll
+    for (int k = 0; k < PT / 2; ++k) t[k] = __ldg(rot + k);
+    const float s = live ? rsqrtf(ss / (float)a.dn + a.eps) : 0.f;
+    uint32_t *qs = reinterpret_cast<uint32_t *>(q_area);
+#pragma unroll
+    for (int k = 0; k < PT / 2; ++k) {             // two adjacent pairs: one register of the low, one of the high half of the head
+      const float u0 = ((k & 1) ? u[k >> 1].z : u[k >> 1].x) * s, u1 = ((k & 1) ? u[k >> 1].w : u[k >> 1].y) * s;
+      const float w0 = ((k & 1) ? w[k >> 1].z : w[k >> 1].x) * s, w1 = ((k & 1) ? w[k >> 1].w : w[k >> 1].y) * s;
+      const float a0 = u0 * t[k].x - w0 * t[k].y, a1 = u1 * t[k].z - w1 * t[k].w, b0 = u0 * t[k].y + w0 * t[k].x, b1 = u1 * t[k].w + w1 * t[k].z;
+      const int e = i0 + 2 * k, at = ((e >> 4) * 32 + (rr & 7) * 4 + ((e & 7) >> 1)) * 4 + (rr >> 3) + 2 * ((e & 15) >> 3);
+      const uint32_t h0 = pack2(a0, a1), h1 = pack2(b0, b1);
+      qs[at] = h0; qs[at + (KS / 2) * 128] = h1;
+      qs[at + KS * 128] = pack2(a0 - low_half(h0), a1 - high_half(h0));
+      qs[at + (KS + KS / 2) * 128] = pack2(b0 - low_half(h1), b1 - high_half(h1));
+    }
+  }
   // ---- the window's own keys and values (last split)
   const bool has_win = split == ns - 1;
   if (has_win) {
     const bool store = q0 == 0;                    // one query tile of the kv head writes the cache
     __nv_bfloat16 *kc = (__nv_bfloat16 *)a.kcache + (long long)b * a.stride_b + (long long)kvh * a.stride_h + (long long)L * HD;
     __nv_bfloat16 *vc = (__nv_bfloat16 *)a.vcache + (long long)b * a.stride_b + (long long)kvh * a.stride_h + (long long)L * HD;
-    constexpr int PER = HALF / 2;                  // two adjacent pairs per thread and pass
-#pragma unroll 4
+    constexpr int PER = HALF / 4;                  // four adjacent pairs per thread and pass
+#pragma unroll 2
     for (int u = tid; u < wrows * PER; u += kShortThreads) {
-      const int j = u / PER, i = (u % PER) * 2;
-      uint32_t k0 = 0u, k1 = 0u, v0 = 0u, v1 = 0u;                 // rows behind the window: zero (a zero probability meets no NaN pattern)
+      const int j = u / PER, i = (u % PER) * 4;
+      uint2 k0 = make_uint2(0u, 0u), k1 = k0, v0 = k0, v1 = k0;    // rows behind the window: zero (a zero probability meets no NaN pattern)
       if (j < c) {
         const int r = bl * c + j;
         const float *src = a.qkv + (long long)r * a.ldq + qd + kvh * HD + i;
+        const float4 x = __ldcg(reinterpret_cast<const float4 *>(src)), y = __ldcg(reinterpret_cast<const float4 *>(src + HALF));
+        const float4 p = __ldcg(reinterpret_cast<const float4 *>(src + kvd)), q = __ldcg(reinterpret_cast<const float4 *>(src + kvd + HALF));
+        const float4 *rp = reinterpret_cast<const float4 *>(a.rope + (long long)(L + j) * HALF + i);
+        const float4 t0 = __ldg(rp), t1 = __ldg(rp + 1);
         const float s = rsqrtf(__ldcg(a.ss + r) / (float)a.dn + a.eps);
-        const float2 x = __ldcg(reinterpret_cast<const float2 *>(src)), y = __ldcg(reinterpret_cast<const float2 *>(src + HALF));
-        const float2 p = __ldcg(reinterpret_cast<const float2 *>(src + kvd)), q = __ldcg(reinterpret_cast<const float2 *>(src + kvd + HALF));
-        const float4 t = __ldg(reinterpret_cast<const float4 *>(a.rope + (long long)(L + j) * HALF + i));
-        const float x0 = x.x * s, x1 = x.y * s, y0 = y.x * s, y1 = y.y * s;
-        k0 = pack2(x0 * t.x - y0 * t.y, x1 * t.z - y1 * t.w);
-        k1 = pack2(x0 * t.y + y0 * t.x, x1 * t.w + y1 * t.z);
-        v0 = pack2(p.x * s, p.y * s); v1 = pack2(q.x * s, q.y * s);
+        const float x0 = x.x * s, x1 = x.y * s, x2 = x.z * s, x3 = x.w * s, y0 = y.x * s, y1 = y.y * s, y2 = y.z * s, y3 = y.w * s;
+        k0 = make_uint2(pack2(x0 * t0.x - y0 * t0.y, x1 * t0.z - y1 * t0.w), pack2(x2 * t1.x - y2 * t1.y, x3 * t1.z - y3 * t1.w));
+        k1 = make_uint2(pack2(x0 * t0.y + y0 * t0.x, x1 * t0.w + y1 * t0.z), pack2(x2 * t1.y + y2 * t1.x, x3 * t1.w + y3 * t1.z));
+        v0 = make_uint2(pack2(p.x * s, p.y * s), pack2(p.z * s, p.w * s)); v1 = make_uint2(pack2(q.x * s, q.y * s), pack2(q.z * s, q.w * s));
         if (store) {
-          *reinterpret_cast<uint32_t *>(kc + (long long)j * HD + i) = k0; *reinterpret_cast<uint32_t *>(kc + (long long)j * HD + i + HALF) = k1;
-          *reinterpret_cast<uint32_t *>(vc + (long long)j * HD + i) = v0; *reinterpret_cast<uint32_t *>(vc + (long long)j * HD + i + HALF) = v1;
+          *reinterpret_cast<uint2 *>(kc + (long long)j * HD + i) = k0; *reinterpret_cast<uint2 *>(kc + (long long)j * HD + i + HALF) = k1;
+          *reinterpret_cast<uint2 *>(vc + (long long)j * HD + i) = v0; *reinterpret_cast<uint2 *>(vc + (long long)j * HD + i + HALF) = v1;
         }
       }
       const uint32_t o0 = piece(j, i >> 3, wsub) + (uint32_t)(i & 7) * 2u, o1 = piece(j, (i + HALF) >> 3, wsub) + (uint32_t)(i & 7) * 2u;
-      *reinterpret_cast<uint32_t *>(gen + (win_k - base) + o0) = k0; *reinterpret_cast<uint32_t *>(gen + (win_k - base) + o1) = k1;
-      *reinterpret_cast<uint32_t *>(gen + (win_v - base) + o0) = v0; *reinterpret_cast<uint32_t *>(gen + (win_v - base) + o1) = v1;
+      *reinterpret_cast<uint2 *>(gen + (win_k - base) + o0) = k0; *reinterpret_cast<uint2 *>(gen + (win_k - base) + o1) = k1;
+      *reinterpret_cast<uint2 *>(gen + (win_v - base) + o0) = v0; *reinterpret_cast<uint2 *>(gen + (win_v - base) + o1) = v1;
     }
   }
-
-  // ---- queries as MMA A operands: lane holds elements 16 ks + 8 x + 2 t4, + 1 of rows g4 and g4 + 8; the rotation pairs
-  // element e of block ks with the same element of block ks + KS / 2
+  __syncthreads();
   uint32_t qh[KS][4], ql[KS][4];
 #pragma unroll
-  for (int hh = 0; hh < 2; ++hh) {
-    const int q = q0 + g4 + hh * 8;
-    const bool live = q < nq;
-    const int j = live ? q / group : 0, r = bl * c + j;
-    const float *src = a.qkv + (long long)r * a.ldq + (kvh * group + (live ? q - j * group : 0)) * HD;
-    const float2 *rot = a.rope + (long long)(L + j) * HALF;
-    const float s = live ? rsqrtf(__ldcg(a.ss + r) / (float)a.dn + a.eps) : 0.f;
-#pragma unroll
-    for (int ks = 0; ks < KS / 2; ++ks)
-#pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        const int e = ks * 16 + x * 8 + t4 * 2;
-        const float2 u = __ldcg(reinterpret_cast<const float2 *>(src + e)), w = __ldcg(reinterpret_cast<const float2 *>(src + e + HALF));
-        const float4 t = __ldg(reinterpret_cast<const float4 *>(rot + e));
-        const float u0 = u.x * s, u1 = u.y * s, w0 = w.x * s, w1 = w.y * s;
-        const float a0 = u0 * t.x - w0 * t.y, a1 = u1 * t.z - w1 * t.w, b0 = u0 * t.y + w0 * t.x, b1 = u1 * t.w + w1 * t.z;
-        const int g = hh + 2 * x;
-        qh[ks][g] = pack2(a0, a1);
-        ql[ks][g] = pack2(a0 - low_half(qh[ks][g]), a1 - high_half(qh[ks][g]));
-        qh[ks + KS / 2][g] = pack2(b0, b1);
-        ql[ks + KS / 2][g] = pack2(b0 - low_half(qh[ks + KS / 2][g]), b1 - high_half(qh[ks + KS / 2][g]));
-      }
+  for (int ks = 0; ks < KS; ++ks) {
+    const uint4 h = reinterpret_cast<const uint4 *>(q_area)[ks * 32 + lane], w = reinterpret_cast<const uint4 *>(q_area)[(KS + ks) * 32 + lane];
+    qh[ks][0] = h.x; qh[ks][1] = h.y; qh[ks][2] = h.z; qh[ks][3] = h.w;
+    ql[ks][0] = w.x; ql[ks][1] = w.y; ql[ks][2] = w.z; ql[ks][3] = w.w;
   }
-  if (has_win) __syncthreads();                    // the window's keys are staged
 
   const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
   float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f}, o[HD / 8][4];

@@ -347,7 +347,11 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   tc_fence_before();
   __syncthreads();
   __syncwarp();                                    // the cluster's barrier counts warps
-  cluster_sync_all();                              // the peers' barriers exist before anything arrives on them
+  // The peers' barriers have to exist before anything arrives on them: only the warps that send across the cluster wait for that
+  // now (1.5 us that the first activations need not wait), the others before the meeting at the end.
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  const bool sends = warp >= kDrainWarp0;
+  if (sends) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -446,13 +450,11 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     if (lane == 0) {
       int issued = 0;
       bool ok = true;
-      asm volatile("griddepcontrol.wait;" ::: "memory");
       for (int id = p.first; id < p.last && ok; ++id) {
         const Phase ph = phase_of(p, id, cl, rank);
         const CUtensorMap *map = &maps.x[ph.kind == PH_O ? 1 : ph.kind == PH_DOWN ? 2 : 0];
         const unsigned int *word = p.bar + 2 * (id - 1);          // results of the projection in front: [all, first column ranges]
-        int seen = id == p.first ? 2 : 0;                         // of its two words
-        if (id == p.first) asm volatile("fence.proxy.async.global;" ::: "memory");      // rows stored by the kernel in front, read by the TMA
+        int seen = 0;                                             // of its two words
         for (int t0 = 0; t0 < ph.n_tiles && ok; t0 = ph.pass_end<T>(t0))
           for (int i = 0; i < ph.np * 2 / C::XK; ++i) {
             const int pr = i * C::XK / 2, sl = issued % NX;
@@ -461,7 +463,8 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
             mbar_expect_tx(bar, C::kXSlot);
             const int need = ph.kind == PH_DOWN && pr < ph.np0 ? 1 : 2;
             if (seen < need) {
-              if (!grid_wait(word + (need == 1 ? 1 : 0), gridDim.x, abort_flag)) { ok = false; break; }
+              if (id == p.first) asm volatile("griddepcontrol.wait;" ::: "memory");     // they are the kernel's in front
+              else if (!grid_wait(word + (need == 1 ? 1 : 0), gridDim.x, abort_flag)) { ok = false; break; }
               asm volatile("fence.proxy.async.global;" ::: "memory");      // rows stored by other CTAs, read by the TMA
               seen = need;
             }
@@ -689,6 +692,8 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   }
 
   // ---------------------------------------------------------------- teardown
+  __syncwarp();
+  if (!sends) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   __syncthreads();
   if (abort_s) {
     if (threadIdx.x == 0) {
