@@ -160,6 +160,7 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
     for (int s = 0; s < C::SUB; ++s) load_3d(dst + C::kHalf + s * C::kSub, &map, s * 64, y, plane_v, bar);
   };
   if (lane == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map) : "memory");
     for (int i = 0; i < kShortStages; ++i) mbar_init(smem_u32(&full_bar[warp][i]), 1);
     fence_barrier_init();
     fence_proxy_async();
@@ -372,7 +373,10 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
       store(row, c4, make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
     }
     __syncwarp();
-    cluster_sync_all();                            // the other splits may still be reading this CTA's memory
+    // The other splits may still be reading this CTA's memory.  (Relaxed: what was read has arrived, it is in the stores; a release
+    // would wait for these too.)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
 }
 

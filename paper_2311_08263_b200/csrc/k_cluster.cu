@@ -50,7 +50,9 @@ constexpr int kMapsPerLayer = 7 * kTileUnits;      // wq, wk, wv, wo, gate, up, 
 
 template <int BN>
 struct ClCfg {
-  static constexpr int T = BN == 64 ? 2 : 4;                      // tiles whose sums a warp holds at a time
+  // Tiles whose sums a warp holds at a time: gate and up of a column range.  (Four, activations loaded half as often: 7B, 16 rows
+  // 2814 us a step against 2796, 2 x 16 rows 3105 against 3059 - the drain loop is unrolled over them.)
+  static constexpr int T = 2;
   static constexpr int H = BN / 2;                                // rows (accumulator columns) per drain warp
   static constexpr int kAcc = 2 * BN;
   static constexpr int NACC = BN == 64 ? 4 : 8;
@@ -58,6 +60,8 @@ struct ClCfg {
   static constexpr int XK = BN == 64 ? 1 : 2;                     // k-blocks per activation slot
   static constexpr int kXBlock = 2 * BN * 128;                    // a k-block, high and low
   static constexpr int kXSlot = XK * kXBlock;
+  // Activation slots.  (16 rows: three 2842 us a step, four 2814, five the same; 64 rows: four 4879, five 4794; 32 rows, nine of one
+  // k-block instead of four of two: 3142 against 3105.)
   static constexpr int NX = BN == 64 ? 5 : 4;
   static constexpr int NCB = BN / 16;                             // exchange units per tile
   static constexpr int NXB = NCB > 2 ? NCB : 2;                   // exchange buffers: unit u of a launch takes buffer u modulo NXB, so a
@@ -341,6 +345,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     // an exchange buffer is free again when the four output warps of all four CTAs have read theirs
     if (lane < C::NXB) { mbar_init(smem_u32(&xc_full[lane]), 1); mbar_init(smem_u32(&xc_empty[lane]), 4 * kCl); }
     fence_barrier_init();
+    if (lane < 3) asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.x[lane]) : "memory");
     __syncwarp();
   }
   if (warp == 1) tmem_alloc(smem_u32(&tmem_base_s), C::kCols);
@@ -349,7 +354,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   __syncwarp();                                    // the cluster's barrier counts warps
   // The peers' barriers have to exist before anything arrives on them: only the warps that send across the cluster wait for that
   // now (1.5 us that the first activations need not wait), the others before the meeting at the end.
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");      // the barriers themselves were released by their fence
   const bool sends = warp >= kDrainWarp0;
   if (sends) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   tc_fence_after();
@@ -718,7 +723,10 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   tc_fence_before();
   __syncthreads();
   __syncwarp();
-  cluster_sync_all();                              // no CTA leaves while a peer may still write to it
+  // No CTA leaves while a peer may still write to it.  (Relaxed: what goes across the cluster has been waited for above; a release would
+  // also wait for the last global stores, which the end of the grid does.)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, C::kCols);
