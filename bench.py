@@ -30,7 +30,7 @@ from paper_2311_08263_b200 import workload as wl  # noqa: E402
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu capture
 # summarised under profiles/ (None until a capture of the current kernel exists)
-TRAFFIC_BYTES_PER_LAUNCH = {"7b": 415.7e6}     # profiles/gemm_umma_chain_7b_4layers.txt (same shapes per launch)
+TRAFFIC_BYTES_PER_LAUNCH = {}
 
 METRIC = "accepted_tokens_per_s"
 UNIT = "tokens/s"
@@ -279,7 +279,7 @@ def run_ours(args, cfg, rank, world, local):
     chain_ms, chain_n = prof.get("chain", (0.0, 0))
     if chain_n > 0:
         chain_bytes = s * (L * (d * qd + 3 * d * f) + (L - 1) * (qd + 2 * kvd) * d)
-        kname = "gemm_umma_kernel<EPI_ATOMIC_ADD> (chained O + gate/up + down + next-QKV projections)"
+        kname = ("cluster_chain_kernel" if B * c <= 64 else "gemm_umma_kernel<EPI_ATOMIC_ADD>") + " (chained O + gate/up + down + next-QKV projections)"
         k_ms, k_n, k_bytes = chain_ms, chain_n, chain_bytes / chain_n
     else:
         k_ms, k_n = prof["gateup"]
