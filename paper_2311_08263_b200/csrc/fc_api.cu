@@ -723,7 +723,7 @@ static int forward_cluster(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, c
     ProfScope ps(ctx, cls);
     return launch_cluster_chain(ctx->plan_cl, ca, first, last, pdl, ctx->st);
   };
-  const bool stream = with_head && attn_stream_pays(max_len, rows, s.n_heads, s.n_kv_heads, nb);
+  const bool stream = with_head && !attn_short_pays(max_len, rows, s.n_heads, s.n_kv_heads, nb, s.head_dim);
   ZeroList none; memset(&none, 0, sizeof none);
   FC_CK(chain(0, 1, FC_CLS_QKV));
   for (int l = 0; l < L; ++l) {

@@ -20,7 +20,7 @@ namespace fc {
 namespace {
 constexpr int kShortKeys = 32;                     // keys per tile
 constexpr int kShortWarps = 4, kShortThreads = kShortWarps * 32;
-constexpr int kShortStages = 2;                    // tiles in flight per warp at most
+constexpr int kShortStages = 4;                    // tiles in flight per warp at most
 
 template <int HD>
 struct ShortCfg {
@@ -417,16 +417,30 @@ cudaError_t launch_attn_short(const KvTensorMap &map, const ShortAttnArgs &a, in
   if ((long long)a.hkv * nqt > 65535) return cudaErrorInvalidValue;
   const long long units = (long long)nb * a.hkv * nqt;
   const int tiles = (max_len + kShortKeys - 1) / kShortKeys;
-  // one CTA per SM, or two where that leaves a warp more than two tiles
-  long long ns = n_sms / units;
+  // One CTA per SM with 128 KB of tiles in flight, or two with half of that each where one leaves a warp more than two tiles and the
+  // clusters of the finer cut fit (32 clusters of eight run in two rounds beside the last CTAs of the kernel in front).  Measured, a step, one ->
+  // two: 7B, 2 x 16 rows over 803 keys (64 units, clusters of 2 -> 4) 3042 -> 3022 us, 1 x 32 over 8000 4150 -> 3995; 1 x 16 over 8000 (32
+  // units, 4 -> 8) 3280 -> 3873; 13B, 1 x 16 over 8000 (40 units, 3 -> 7) 6434 -> 7084; 7B, 4 x 16 over 2048 (128 units, 1 -> 2) 4665 -> 4723;
+  // 1.1B, 1 x 16 over 8000 (head_dim 64, 4 -> 8) 1195 -> 1158.
+  long long ns = n_sms / units, two = 2ll * n_sms / units;
   if (ns < 1) ns = 1;
-  if (tiles > 2 * kShortWarps * ns) ns = 2ll * n_sms / units;
+  if (tiles > 2 * kShortWarps * ns && (hd == 64 || (ns > 1 && two <= 4))) ns = two;
   if (ns > 8) ns = 8;
   if (ns > (tiles + kShortWarps - 1) / kShortWarps) ns = (tiles + kShortWarps - 1) / kShortWarps;
   if (ns < 1) ns = 1;
   ShortAttnArgs args = a;
-  args.stages = units * ns > n_sms ? 1 : kShortStages;           // more than one CTA per SM: two have to fit
+  args.stages = (units * ns > n_sms ? 1 : 2) * (hd == 64 ? 2 : 1);
   return hd == 128 ? launch_short_t<128>(map, args, (int)ns, nqt, nb, st) : launch_short_t<64>(map, args, (int)ns, nqt, nb, st);
+}
+
+// The streaming pair reads faster where there is much to read (two CTAs of 96 KB of tiles per SM) but takes a second launch per layer, about
+// 4 us.  Measured, a step, short -> pair, by 16-query units x 64-key tiles.  head_dim 128: 7B, 2 x 16 rows over 1500 keys (1536) 3125 us ->
+// 3233; 4 x 16 over 2048 (4224) 4665 -> 4802; 1 x 16 over 8000 (4032) 3280 -> 3391; 4 x 8 over 4000 (8064) 4186 -> 4233; 16 x 1 over 1024 (8704) 3933
+// -> 3931, over 2048 (16896) 5061 -> 4979.  head_dim 64: 1.1B, 16 x 4 over 1024 (2176) 1659 -> 1703; 1 x 16 over 8000 (4032) 1158 -> 1579;
+// 4 x 16 over 4000 (8064) 2000 -> 1967; 16 x 4 over 8000 (16128) 2482 -> 2243.
+bool attn_short_pays(int max_len, int c, int hq, int hkv, int nb, int hd) {
+  const long long units = (long long)nb * hkv * (((long long)(hq / hkv) * c + 15) / 16);
+  return units * ((max_len + c + 63) / 64) < (hd == 128 ? 8600 : 4600);
 }
 
 }  // namespace fc

@@ -21,6 +21,11 @@ CASES = [
     (2, 2, 128, 256, 4480, 4240, 33, [96]),                        # 33 rows: a width of 64, windows over three 16-key blocks
     (6, 3, 64, 384, 4480, 9600, 16, [5, 160, 0, 31]),              # 64 rows, passes of two tiles
     (2, 1, 64, 128, 256, 528, 64, [40]),                           # a window of 64 rows of one sequence
+    (32, 32, 128, 256, 512, 1040, 16, [1471]),                     # 32 units, four key splits, rings that wrap
+    (32, 32, 128, 256, 512, 1040, 8, [700, 33]),                   # 64 units, four key splits of half the ring
+    (32, 4, 64, 256, 512, 1040, 16, [2500]),                       # head_dim 64, eight key splits
+    (16, 16, 128, 256, 512, 1040, 1, [2300] + [31 + 61 * i for i in range(15)]),       # 256 units x 36 tiles: the streaming pair
+    (32, 32, 128, 256, 512, 1040, 4, [1100, 0, 1, 31, 32, 33, 63, 64, 65, 95, 96, 97, 191, 192, 193, 1023]),     # 64 rows, 512 x 18: the same
 ]
 
 
@@ -28,7 +33,8 @@ CASES = [
 def test_step_against_the_oracle_and_again(hq, hkv, hd, d, f, vocab, c, lens):
     cfg = wl.small_config(n_layers=2, n_heads=hq, n_kv_heads=hkv, head_dim=hd, d_model=d, d_ffn=f, vocab=vocab, seed=2000 + c + hd)
     dec, _ = _random_kv_case(cfg, lens, c, range(len(lens)))
-    assert dec.fc_last_launch_count() == 2 * cfg.n_layers + 4
+    units, tiles = len(lens) * hkv * ((hq // hkv * c + 15) // 16), (max(lens) + c + 63) // 64
+    assert dec.fc_last_launch_count() == (3 if units * tiles >= 8600 else 2) * cfg.n_layers + 4
     logits = dec.fc_debug_logits(True)
     pending = wl.make_random_window(cfg, len(lens), 1, salt=3).numpy()[:, 0]
     window = wl.make_random_window(cfg, len(lens), c, salt=4).numpy()
