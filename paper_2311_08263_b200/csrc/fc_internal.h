@@ -254,7 +254,7 @@ cudaError_t launch_qkv_finish(const QkvFinishArgs &a, int R, cudaStream_t st);
 cudaError_t launch_attn_stream(const KvTensorMap &map, const StreamAttnArgs &a, int nseg, int max_rows, int max_len, int hd,
                                int n_sms, cudaStream_t st);
 cudaError_t launch_attn_short(const KvTensorMap &map, const ShortAttnArgs &a, int nb, int max_len, int hd, int n_sms, cudaStream_t st);
-bool attn_short_pays(int max_len, int c, int hq, int hkv, int nb, int hd);      // against the streaming pair, behind the one-writer projections
+bool attn_short_pays(int max_len, int c, int hq, int hkv, int nb, int hd, int n_sms);      // against the streaming pair, behind the one-writer projections
 bool attn_stream_pays(int max_len, int c, int hq, int hkv, int nb);
 int attn_stream_tile_keys();
 size_t attn_stream_q_tiles(int rows, int group, int nseg);      // tiles per kv head for `rows` rows in nseg segments

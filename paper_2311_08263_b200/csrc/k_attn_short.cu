@@ -436,11 +436,12 @@ cudaError_t launch_attn_short(const KvTensorMap &map, const ShortAttnArgs &a, in
 // The streaming pair reads faster where there is much to read (two CTAs of 96 KB of tiles per SM) but takes a second launch per layer, about
 // 4 us.  Measured, a step, short -> pair, by 16-query units x 64-key tiles.  head_dim 128: 7B, 2 x 16 rows over 1500 keys (1536) 3125 us ->
 // 3233; 4 x 16 over 2048 (4224) 4665 -> 4802; 1 x 16 over 8000 (4032) 3280 -> 3391; 4 x 8 over 4000 (8064) 4186 -> 4233; 16 x 1 over 1024 (8704) 3933
-// -> 3931, over 2048 (16896) 5061 -> 4979.  head_dim 64: 1.1B, 16 x 4 over 1024 (2176) 1659 -> 1703; 1 x 16 over 8000 (4032) 1158 -> 1579;
+// -> 3931, over 2048 (16896) 5061 -> 4979.  More units than SMs leave the short kernel a second round: 5 x 8 over 3000 (160 units, 7680) 5488 -> 5306,
+// over 2000 (5120) 4962 -> 4949 behind the chained launch.  head_dim 64: 1.1B, 16 x 4 over 1024 (2176) 1659 -> 1703; 1 x 16 over 8000 (4032) 1158 -> 1579;
 // 4 x 16 over 4000 (8064) 2000 -> 1967; 16 x 4 over 8000 (16128) 2482 -> 2243.
-bool attn_short_pays(int max_len, int c, int hq, int hkv, int nb, int hd) {
+bool attn_short_pays(int max_len, int c, int hq, int hkv, int nb, int hd, int n_sms) {
   const long long units = (long long)nb * hkv * (((long long)(hq / hkv) * c + 15) / 16);
-  return units * ((max_len + c + 63) / 64) < (hd == 128 ? 8600 : 4600);
+  return units * ((max_len + c + 63) / 64) < (hd == 128 ? (units > n_sms ? 6000 : 8600) : 4600);
 }
 
 }  // namespace fc

@@ -72,3 +72,27 @@ def test_wide_steps_repeat_bit_for_bit(b, c, length):
         got = logits[:b * c].clone()
         first = got if first is None else first
         assert torch.equal(got, first)
+
+
+def test_rows_where_the_route_changes():
+    """Two layers as wide as 13B: 9 and 32 rows take these projections, 8 and 33 the chained launch.  A row's logits depend on the rows in front of it
+    only, so the shorter window's rows are the longer one's first."""
+    import dataclasses
+    import torch
+    from paper_2311_08263_b200 import engine
+    cfg = dataclasses.replace(wl.CONFIGS["13b"], n_layers=2, vocab=2048)
+    w = wl.make_weights(cfg, device="cuda")
+    window = wl.make_random_window(cfg, 1, 33, salt=4).numpy()
+    got = {}
+    for c in (8, 9, 32, 33):
+        dec = engine.Decoder(cfg, w, 1, c, 300)
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(5)
+        dec.kv_view().normal_(generator=gen)
+        dec.fc_debug_set_state([200], window[:, 0], c, pad_id=0)
+        logits = dec.fc_debug_logits(True)
+        dec.fc_jacobi_step(window[:, :c].copy())
+        got[c] = logits[:c].float().cpu().clone()
+        assert dec.fc_debug_check_guards() == 0
+    for c in (8, 9, 32):
+        assert float((got[c] - got[33][:c]).abs().max()) < 3e-2 * float(got[33].pow(2).mean().sqrt())
