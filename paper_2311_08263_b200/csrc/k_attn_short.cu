@@ -417,14 +417,15 @@ cudaError_t launch_attn_short(const KvTensorMap &map, const ShortAttnArgs &a, in
   if ((long long)a.hkv * nqt > 65535) return cudaErrorInvalidValue;
   const long long units = (long long)nb * a.hkv * nqt;
   const int tiles = (max_len + kShortKeys - 1) / kShortKeys;
-  // One CTA per SM with 128 KB of tiles in flight, or two with half of that each where one leaves a warp more than two tiles and the
-  // clusters of the finer cut fit (32 clusters of eight run in two rounds beside the last CTAs of the kernel in front).  Measured, a step, one ->
-  // two: 7B, 2 x 16 rows over 803 keys (64 units, clusters of 2 -> 4) 3042 -> 3022 us, 1 x 32 over 8000 4150 -> 3995; 1 x 16 over 8000 (32
-  // units, 4 -> 8) 3280 -> 3873; 13B, 1 x 16 over 8000 (40 units, 3 -> 7) 6434 -> 7084; 7B, 4 x 16 over 2048 (128 units, 1 -> 2) 4665 -> 4723;
-  // 1.1B, 1 x 16 over 8000 (head_dim 64, 4 -> 8) 1195 -> 1158.
+  // One CTA per SM with 128 KB of tiles in flight, or two with half of that each where one leaves a warp more than two tiles, the finer cut
+  // gives clusters of three or four and a tenth of the slots stays free (what does not fit beside the last CTAs of the kernel in front is a second
+  // round).  Measured, a step, one -> two: 7B, 2 x 16 rows over 803 keys (64 units, clusters of 2 -> 4) 3042 -> 3022 us, 1 x 32 over 8000 4150
+  // -> 3995; 13B, 2 x 16 over 4000 (80 units, 1 -> 3) 7439 -> 6962; but 7B, 3 x 16 over 2000 (96 units, 1 -> 3, 288 of 296 slots) 4507 -> 4870;
+  // 1 x 16 over 8000 (32 units, 4 -> 8) 3280 -> 3873; 13B, 1 x 16 over 8000 (40 units, 3 -> 7) 6434 -> 7084; 7B, 4 x 16 over 2048 (128 units,
+  // 1 -> 2) 4665 -> 4723.  head_dim 64 has half the bytes per tile: 1.1B, 1 x 16 over 8000 (4 -> 8) 1195 -> 1158.
   long long ns = n_sms / units, two = 2ll * n_sms / units;
   if (ns < 1) ns = 1;
-  if (tiles > 2 * kShortWarps * ns && (hd == 64 || (ns > 1 && two <= 4))) ns = two;
+  if (tiles > 2 * kShortWarps * ns && (hd == 64 || ((two == 3 || two == 4) && 10 * units * two <= 18ll * n_sms))) ns = two;
   if (ns > 8) ns = 8;
   if (ns > (tiles + kShortWarps - 1) / kShortWarps) ns = (tiles + kShortWarps - 1) / kShortWarps;
   if (ns < 1) ns = 1;

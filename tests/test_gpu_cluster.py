@@ -23,6 +23,8 @@ CASES = [
     (2, 1, 64, 128, 256, 528, 64, [40]),                           # a window of 64 rows of one sequence
     (32, 32, 128, 256, 512, 1040, 16, [1471]),                     # 32 units, four key splits, rings that wrap
     (32, 32, 128, 256, 512, 1040, 8, [700, 33]),                   # 64 units, four key splits of half the ring
+    (40, 40, 128, 256, 512, 1040, 16, [1300, 64]),                 # 80 units, three key splits of half the ring
+    (24, 24, 128, 256, 512, 1040, 12, [1300, 64, 5, 900]),         # 96 units, no split
     (32, 4, 64, 256, 512, 1040, 16, [2500]),                       # head_dim 64, eight key splits
     (16, 16, 128, 256, 512, 1040, 1, [2300] + [31 + 61 * i for i in range(15)]),       # 256 units x 36 tiles: the streaming pair
     (32, 32, 128, 256, 512, 1040, 4, [1100, 0, 1, 31, 32, 33, 63, 64, 65, 95, 96, 97, 191, 192, 193, 1023]),     # 64 rows, 512 x 18: the same
