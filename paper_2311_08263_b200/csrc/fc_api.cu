@@ -56,8 +56,7 @@ struct Buffers {
   void *qb;
   unsigned int *counters, *err, *chain_bar, *bulk_arrived;
   char *bulk_slots;
-  // up to kClusterRows rows (k_cluster.cu): tensor maps, operand pairs, slots of the sums of squares, grid barriers
-  char *cl_maps;
+  // up to kClusterRows rows (k_cluster.cu): operand pairs, slots of the sums of squares, grid barriers
   void *cl_pan_x, *cl_pan_a, *cl_pan_h;
   float *cl_ss_x, *cl_ss_ffn;
   unsigned int *cl_bar;
@@ -160,7 +159,6 @@ size_t carve(const fc_model_shape *s, char *base, Buffers *b, std::vector<size_t
   t.bulk_slots = c.take<char>(d.bulk ? bulk_slot_bytes() : 0); c.guard();
   t.bulk_arrived = c.take<unsigned int>(d.bulk ? kBulkArrived : 0); c.guard();
   const size_t cl_rows = d.cluster ? 2 * kClusterRows : 0;
-  t.cl_maps = c.take<char>(d.cluster ? cluster_map_bytes(s->n_layers) : 0); c.guard();
   t.cl_pan_x = c.take<char>(cl_rows * s->d_model * 2); c.guard();
   t.cl_pan_a = c.take<char>(cl_rows * d.qd * 2); c.guard();
   t.cl_pan_h = c.take<char>(cl_rows * s->d_ffn * 2); c.guard();
@@ -489,12 +487,12 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
         cudaStreamSynchronize(ctx->st) != cudaSuccess) return fail(FC_ERR_CUDA);
   }
   if (cudaStreamSynchronize(ctx->st) != cudaSuccess) return fail(FC_ERR_CUDA);
-  if (ctx->d.cluster) {          // behind the workspace's clearing: the tensor maps lie in it
+  if (ctx->d.cluster) {
     ClusterModel m; memset(&m, 0, sizeof m);
     m.n_layers = L; m.d = shape->d_model; m.qd = ctx->d.qd; m.kvd = ctx->d.kvd; m.f = shape->d_ffn; m.vocab = shape->vocab;
     m.wq = ctx->wq.data(); m.wk = ctx->wk.data(); m.wv = ctx->wv.data(); m.wo = ctx->wo.data();
     m.w_gate = ctx->w_gate.data(); m.w_up = ctx->w_up.data(); m.w_down = ctx->w_down.data(); m.lm_head = ctx->lm_head;
-    ctx->plan_cl = cluster_plan_create(m, ctx->b.cl_maps, ctx->b.cl_pan_x, ctx->b.cl_pan_a, ctx->b.cl_pan_h, ctx->st);
+    ctx->plan_cl = cluster_plan_create(m, ctx->b.cl_pan_x, ctx->b.cl_pan_a, ctx->b.cl_pan_h);
     (void)cudaGetLastError();    // without it (a device that does not hold the clusters): the other routes
   }
   const int B = shape->max_batch;

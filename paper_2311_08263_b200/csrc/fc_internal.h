@@ -326,12 +326,10 @@ constexpr int kClusterSlots = 160;                   // CTAs that the slots of t
 struct ClusterModel {
   int n_layers, d, qd, kvd, f, vocab;
   const void *const *wq, *const *wk, *const *wv, *const *wo, *const *w_gate, *const *w_up, *const *w_down, *lm_head;   // host arrays of device pointers
-  const void *maps_dev;
 };
 struct ClusterPlan;
 bool cluster_shape_ok(int d, int qd, int kvd, int f, int vocab);
-size_t cluster_map_bytes(int n_layers);
-ClusterPlan *cluster_plan_create(const ClusterModel &m, void *maps_dev, void *pan_x, void *pan_a, void *pan_h, cudaStream_t st);
+ClusterPlan *cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a, void *pan_h);
 void cluster_plan_destroy(ClusterPlan *p);
 struct ClusterArgs {
   int R;
@@ -345,7 +343,7 @@ struct ClusterArgs {
   const int32_t *tokens, *perm; float beta; unsigned long long *amax; float *logits;
   unsigned int *err;
 };
-// projections [first, last) one after the other: 4 * layer + {0 QKV, 1 O, 2 gate/up, 3 down}, 4 * n_layers: the LM head
+// projections [first, last), four at most, one after the other: 4 * layer + {0 QKV, 1 O, 2 gate/up, 3 down}, 4 * n_layers: the LM head
 cudaError_t launch_cluster_chain(const ClusterPlan *pl, const ClusterArgs &a, int first, int last, int pdl, cudaStream_t st);
 // x = E[token], pan = x * gain as a pair, ss[r] = sum x^2; words[0 .. n_words) = 0
 cudaError_t launch_embed_pair(const int32_t *tokens, const void *emb, const void *gain, float *x, void *pan, float *ss, unsigned int *words, int n_words,

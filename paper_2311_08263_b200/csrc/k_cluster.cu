@@ -25,6 +25,7 @@
 // Warps: 0 weights, 1 MMA and tensor memory, 2 activations, 3-10 accumulators -> registers -> cluster, 11-14 cluster -> results.
 // Every wait is bounded.  The grid barrier between projections needs every cluster resident: the grid is what
 // cudaOccupancyMaxActiveClusters reports.
+#include <array>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -46,7 +47,7 @@ constexpr int kXRow = 16;                          // floats per weight row in a
 constexpr int kXBuf = kCl * 32 * kXRow * 4;        // one exchange unit: 32 weight rows x 16 rows from four CTAs
 constexpr size_t kMaxSmem = 227 * 1024 - 3 * 1024; // dynamic: the static part takes less than 3 KB
 enum { PH_QKV = 0, PH_O = 1, PH_GU = 2, PH_DOWN = 3, PH_HEAD = 4 };
-constexpr int kMapsPerLayer = 7 * kTileUnits;      // wq, wk, wv, wo, gate, up, down: one map per tile height
+constexpr int kMats = 7;                           // wq (or the LM head), wk, wv, wo, gate, up, down: the matrices of a launch
 
 template <int BN>
 struct ClCfg {
@@ -71,7 +72,12 @@ struct ClCfg {
   static_assert(kSmem <= kMaxSmem, "shared memory");
 };
 
-struct ClMaps { CUtensorMap x[3]; };               // operand pairs: residual x gain (K = d), attention (qd), feed-forward (f)
+// By value in the launch's parameters, as in all kernels here: a map that lies in global memory would need a proxy fence in every
+// block before its first use.
+struct ClMaps {
+  CUtensorMap x[3];                                // operand pairs: residual x gain (K = d), attention (qd), feed-forward (f)
+  CUtensorMap w[kMats][2];                         // weights, boxes of the matrix's two tile heights
+};
 
 // One kind of projection, as far as it is the same for all clusters (made on the host: integer divisions and their code cost
 // every role of every launch).
@@ -80,7 +86,7 @@ struct Kind {
   unsigned int inv_parts;                          // reciprocal() of parts
   int early;                                       // gate/up: tiles in front of the last column range (their results are published first)
   int pairs, first;                                // pairs of k-blocks; down: those in front of the last column range of gate/up
-  int map;                                         // tensor maps of the layer in front of this projection's
+  int mat0, h0;                                    // ClMaps::w: first matrix; the lower of the tile heights (the other is one more)
 };
 
 struct ClParams {
@@ -89,7 +95,6 @@ struct ClParams {
   unsigned int inv_ncl;                            // reciprocal() of the clusters
   int first, last;                                 // projections [first, last): 4 * layer + PH_*, 4 * n_layers: the LM head
   int n_layers, d, qd, kvd, f, vocab, R;
-  const CUtensorMap *w;                            // [layer][matrix][height - 1], then the LM head
   float *x, *qkv;
   __nv_bfloat16 *pan_x, *pan_h;                    // [2][kClusterRows][d], [2][kClusterRows][f]
   const __nv_bfloat16 *g_ffn, *g_next;             // gains applied behind O and behind down
@@ -117,7 +122,6 @@ __host__ __device__ inline void tile_units(const Kind &k, int t, int cl, unsigne
 struct Phase {
   int kind, n_tiles, early, cl;
   int p0, np0, q0, np;                             // this CTA's np pairs of k-blocks: np0 from pair p0, the rest from pair q0
-  const CUtensorMap *maps;
   // tile t: matrix, first unit, height (0 to 8 units; 0: nothing, for a range of fewer units than clusters)
   __device__ __forceinline__ void tile(const ClParams &p, int t, int &mat, int &u, int &h) const {
     const Kind &k = p.kind[kind];
@@ -150,7 +154,6 @@ __device__ __forceinline__ Phase phase_of(const ClParams &p, int id, int cl, int
   ph.np0 = (rank + 1) * k.first / kCl - ph.p0;
   ph.q0 = k.first + rank * rest / kCl;
   ph.np = ph.np0 + k.first + (rank + 1) * rest / kCl - ph.q0;
-  ph.maps = p.w + (size_t)l * kMapsPerLayer + k.map;
   return ph;
 }
 
@@ -308,11 +311,13 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   const int rank = (int)cluster_rank(), cl = blockIdx.x / kCl;
   volatile int *abort_flag = &abort_s;
 
-  // Tiles of a pass for the thread that requests weights: (first weight row, height in units | map << 8).
+  // Tiles of a pass for the thread that requests weights: (first weight row, height in units | index into ClMaps::w << 8).
   auto list_tiles = [&](const Phase &ph, int t0, int t1) {
     int mat, u, h;
     ph.tile(p, min(t0 + lane, t1 - 1), mat, u, h);
-    if (lane < T) tiles_s[lane] = make_int2(u * kUnit, h | (mat * kTileUnits + h - 1) << 8);
+    const Kind &k = p.kind[ph.kind];
+    const int h0 = ph.kind == PH_QKV && mat > 0 ? p.kv.h0 : k.h0;
+    if (lane < T) tiles_s[lane] = make_int2(u * kUnit, h | (2 * (k.mat0 + mat) + h - h0) << 8);
     __syncwarp();
   };
   auto request = [&](const Phase &ph, int st, int t, int pr) {
@@ -320,7 +325,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     const int h = ti.y & 0xff;
     const uint32_t bar = smem_u32(&full_w[st]);
     mbar_expect_tx(bar, (uint32_t)h * (2 * kUnit * 128));
-    if (h > 0) load_3d(base + st * kStageW, ph.maps + (ti.y >> 8), 0, ti.x, 2 * ph.pair(pr), bar);
+    if (h > 0) load_3d(base + st * kStageW, &maps.w[0][0] + (ti.y >> 8), 0, ti.x, 2 * ph.pair(pr), bar);
   };
   // The ring's first round of weights is requested before everything else: the rest of the set-up takes about 3 us (tensor memory,
   // barriers, the cluster's meeting).
@@ -752,7 +757,8 @@ struct ClusterPlan {
   ClusterModel m;
   int ncl;
   Kind kind[5], kv;
-  ClMaps x[3];                                     // boxes of 16, 32, 64 rows
+  ClMaps maps[3];                                  // operand boxes of 16, 32, 64 rows; the weights' are filled in per launch
+  std::vector<std::array<CUtensorMap, 2>> w;       // [layer][kMats], then the LM head
 };
 
 template <int BN>
@@ -786,10 +792,9 @@ static int cluster_fit() {
 bool cluster_shape_ok(int d, int qd, int kvd, int f, int vocab) {
   return d % 128 == 0 && qd % 128 == 0 && f % 128 == 0 && kvd % kUnit == 0 && vocab % kUnit == 0;
 }
-size_t cluster_map_bytes(int n_layers) { return ((size_t)n_layers * kMapsPerLayer + kTileUnits) * sizeof(CUtensorMap); }
 
-// maps_dev: cluster_map_bytes() of device memory, 64-byte aligned; pairs: [2][kClusterRows][d | qd | f].  Null: the device does not hold it.
-ClusterPlan *cluster_plan_create(const ClusterModel &m, void *maps_dev, void *pan_x, void *pan_a, void *pan_h, cudaStream_t st) {
+// Pairs: [2][kClusterRows][d | qd | f].  Null: the device does not hold it.
+ClusterPlan *cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a, void *pan_h) {
   EncodeTiledFn enc = encode_fn();
   int ncl = cluster_fit<16>();
   for (int n : {cluster_fit<32>(), cluster_fit<64>(), kClusterSlots / kCl}) ncl = n < ncl ? n : ncl;
@@ -797,13 +802,14 @@ ClusterPlan *cluster_plan_create(const ClusterModel &m, void *maps_dev, void *pa
   ClusterPlan *pl = new (std::nothrow) ClusterPlan();
   if (!pl) return nullptr;
   pl->m = m; pl->ncl = ncl;
-  std::vector<CUtensorMap> host((size_t)m.n_layers * kMapsPerLayer + kTileUnits);
-  memset((void *)host.data(), 0, host.size() * sizeof(CUtensorMap));
+  pl->w.resize((size_t)m.n_layers * kMats + 1);
+  memset((void *)pl->w.data(), 0, pl->w.size() * sizeof pl->w[0]);
   bool ok = true;
-  auto kind_of = [&](int N, int K, int map) {
+  auto kind_of = [&](int N, int K, int mat0) {
     Kind k; memset(&k, 0, sizeof k);
     k.units = N / kUnit; k.parts = k.n_tiles = n_parts(k.units, ncl); k.inv_parts = reciprocal(k.parts);
-    k.pairs = k.first = K >> 7; k.map = map * kTileUnits;
+    k.pairs = k.first = K >> 7; k.mat0 = mat0;
+    k.h0 = k.units / k.parts / ncl;                // ranges differ by one unit, and so do the tiles of a range
     return k;
   };
   pl->kv = kind_of(m.kvd, m.d, 0);
@@ -814,34 +820,26 @@ ClusterPlan *cluster_plan_create(const ClusterModel &m, void *maps_dev, void *pa
   pl->kind[PH_DOWN] = kind_of(m.d, m.f, 6);
   pl->kind[PH_DOWN].first = (gu.parts - 1) * gu.units / gu.parts * kUnit >> 7;
   pl->kind[PH_HEAD] = kind_of(m.vocab, m.d, 0);
-  auto weight_maps = [&](CUtensorMap *out, const void *w, int N, int K) {
-    bool used[kTileUnits + 1] = {false};
-    const Kind k = kind_of(N, K, 0);
-    for (int t = 0; t < k.parts; ++t)
-      for (int c = 0; c < ncl; ++c) {
-        int u, h;
-        tile_units(k, t, c, reciprocal(ncl), u, h);
-        used[h] = true;
-      }
-    for (int h = 1; h <= kTileUnits && ok; ++h) {
-      if (!used[h]) continue;
+  auto weight_maps = [&](std::array<CUtensorMap, 2> &out, const void *w, int N, int K) {
+    const int h0 = kind_of(N, K, 0).h0;
+    for (int h = h0 > 1 ? h0 : 1; h <= h0 + 1 && h <= kTileUnits && ok; ++h) {
       cuuint64_t gdim[3] = {64, (cuuint64_t)N, (cuuint64_t)K / 64}, gstr[2] = {(cuuint64_t)K * 2, 128};
       cuuint32_t box[3] = {64, (cuuint32_t)(h * kUnit), 2}, estr[3] = {1, 1, 1};
-      ok = enc(&out[h - 1], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(w), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+      ok = enc(&out[h - h0], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(w), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
   };
   for (int l = 0; l < m.n_layers && ok; ++l) {
-    CUtensorMap *o = host.data() + (size_t)l * kMapsPerLayer;
-    weight_maps(o, m.wq[l], m.qd, m.d);
-    weight_maps(o + kTileUnits, m.wk[l], m.kvd, m.d);
-    weight_maps(o + 2 * kTileUnits, m.wv[l], m.kvd, m.d);
-    weight_maps(o + 3 * kTileUnits, m.wo[l], m.d, m.qd);
-    weight_maps(o + 4 * kTileUnits, m.w_gate[l], m.f, m.d);
-    weight_maps(o + 5 * kTileUnits, m.w_up[l], m.f, m.d);
-    weight_maps(o + 6 * kTileUnits, m.w_down[l], m.d, m.f);
+    std::array<CUtensorMap, 2> *o = pl->w.data() + (size_t)l * kMats;
+    weight_maps(o[0], m.wq[l], m.qd, m.d);
+    weight_maps(o[1], m.wk[l], m.kvd, m.d);
+    weight_maps(o[2], m.wv[l], m.kvd, m.d);
+    weight_maps(o[3], m.wo[l], m.d, m.qd);
+    weight_maps(o[4], m.w_gate[l], m.f, m.d);
+    weight_maps(o[5], m.w_up[l], m.f, m.d);
+    weight_maps(o[6], m.w_down[l], m.d, m.f);
   }
-  weight_maps(host.data() + (size_t)m.n_layers * kMapsPerLayer, m.lm_head, m.vocab, m.d);
+  weight_maps(pl->w.back(), m.lm_head, m.vocab, m.d);
   void *pans[3] = {pan_x, pan_a, pan_h};
   const int ks[3] = {m.d, m.qd, m.f};
   for (int b = 0; b < 3; ++b)
@@ -849,13 +847,10 @@ ClusterPlan *cluster_plan_create(const ClusterModel &m, void *maps_dev, void *pa
       const cuuint64_t K = (cuuint64_t)ks[i];
       cuuint64_t gdim[4] = {64, (cuuint64_t)kClusterRows, 2, K / 64}, gstr[3] = {K * 2, K * 2 * kClusterRows, 128};
       cuuint32_t box[4] = {64, (cuuint32_t)(16 << b), 2, (cuuint32_t)(b == 2 ? ClCfg<64>::XK : ClCfg<16>::XK)}, estr[4] = {1, 1, 1, 1};
-      ok = enc(&pl->x[b].x[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, pans[i], gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+      ok = enc(&pl->maps[b].x[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, pans[i], gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
-  if (ok) ok = cudaMemcpyAsync(maps_dev, host.data(), host.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st) == cudaSuccess &&
-               cudaStreamSynchronize(st) == cudaSuccess;
   if (!ok) { delete pl; return nullptr; }
-  pl->m.maps_dev = maps_dev;
   return pl;
 }
 void cluster_plan_destroy(ClusterPlan *p) { delete p; }
@@ -883,21 +878,27 @@ static cudaError_t launch_cluster_t(const ClMaps &maps, const ClParams &p, int n
 
 cudaError_t launch_cluster_chain(const ClusterPlan *pl, const ClusterArgs &a, int first, int last, int pdl, cudaStream_t st) {
   const ClusterModel &m = pl->m;
-  if (a.R < 1 || a.R > kClusterRows || first < 0 || first >= last || last > 4 * m.n_layers + 1) return cudaErrorInvalidValue;
+  if (a.R < 1 || a.R > kClusterRows || first < 0 || first >= last || last > 4 * m.n_layers + 1 || last - first > 4) return cudaErrorInvalidValue;
   ClParams p;
   memset(&p, 0, sizeof p);
   memcpy(p.kind, pl->kind, sizeof p.kind);
   p.kv = pl->kv; p.inv_ncl = reciprocal(pl->ncl);
   p.first = first; p.last = last; p.n_layers = m.n_layers; p.d = m.d; p.qd = m.qd; p.kvd = m.kvd; p.f = m.f; p.vocab = m.vocab; p.R = a.R;
-  p.w = (const CUtensorMap *)m.maps_dev;
   p.x = a.x; p.qkv = a.qkv; p.pan_x = (__nv_bfloat16 *)a.pan_x; p.pan_h = (__nv_bfloat16 *)a.pan_h;
   p.g_ffn = (const __nv_bfloat16 *)a.g_ffn; p.g_next = (const __nv_bfloat16 *)a.g_next;
   p.ss_x = a.ss_x; p.ss_ffn = a.ss_ffn; p.ss_attn = a.ss_attn; p.first_slots = 1;
   p.eps = a.eps; p.dn = m.d; p.bar = a.bar; p.err = a.err;
   p.tokens = a.tokens; p.perm = a.perm; p.beta = a.beta; p.amax = a.amax; p.logits = a.logits;
-  if (a.R <= 16) return launch_cluster_t<16>(pl->x[0], p, pl->ncl, pdl, st);
-  if (a.R <= 32) return launch_cluster_t<32>(pl->x[1], p, pl->ncl, pdl, st);
-  return launch_cluster_t<64>(pl->x[2], p, pl->ncl, pdl, st);
+  const int width = a.R <= 16 ? 0 : a.R <= 32 ? 1 : 2;
+  ClMaps maps = pl->maps[width];
+  for (int id = first; id < last; ++id) {          // every matrix at most once in four projections
+    const int l = id >> 2, kind = l == m.n_layers ? (int)PH_HEAD : id & 3, mat0 = pl->kind[kind].mat0;
+    const int n = kind == PH_QKV ? 3 : kind == PH_GU ? 2 : 1;
+    for (int i = 0; i < n; ++i) memcpy(maps.w[mat0 + i], &pl->w[(size_t)l * kMats + mat0 + i], sizeof maps.w[0]);
+  }
+  if (width == 0) return launch_cluster_t<16>(maps, p, pl->ncl, pdl, st);
+  if (width == 1) return launch_cluster_t<32>(maps, p, pl->ncl, pdl, st);
+  return launch_cluster_t<64>(maps, p, pl->ncl, pdl, st);
 }
 
 }  // namespace fc

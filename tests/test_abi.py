@@ -101,3 +101,12 @@ def test_workspace_of_the_dense_route_holds_whole_row_tiles(cdll, rows):
     assert got[0] <= got[1] <= got[0] + (full - batch * c) * per_seq + slack
     row = 4 * (512 + 3 * 512)
     assert (full - batch * c) * row > slack
+
+
+def test_workspace_holds_no_tensor_maps(cdll):
+    """A kernel that takes a tensor map from memory that was copied to needs a proxy fence in front; maps go by value in the
+    launch's parameters.  What a layer adds to the workspace are its synchronisation words, a few hundred bytes."""
+    cdll.fc_workspace_bytes.restype = C.c_size_t
+    shape = dict(dtype=lib.FC_BF16, d_model=512, n_heads=8, n_kv_heads=8, head_dim=64, d_ffn=1536, vocab=1024, max_c=16, max_seq=80)
+    few, many = (cdll.fc_workspace_bytes(C.byref(_shape(**shape, n_layers=n))) for n in (8, 40))
+    assert many - few < 32 * 512 + 1024

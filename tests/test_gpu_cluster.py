@@ -98,3 +98,36 @@ def test_rows_where_the_route_changes():
         assert dec.fc_debug_check_guards() == 0
     for c in (8, 9, 32):
         assert float((got[c] - got[33][:c]).abs().max()) < 3e-2 * float(got[33].pow(2).mean().sqrt())
+
+
+def test_second_model_in_the_buffers_of_the_first():
+    """fc_init on the K/V slab and workspace that another context's projections ran from, with weights elsewhere: the step is
+    that of the second model bit for bit, as in buffers of its own."""
+    import ctypes as C
+    import dataclasses
+    import torch
+    from paper_2311_08263_b200 import engine, lib as _l
+    cfg = wl.small_config(n_layers=3, n_heads=8, n_kv_heads=8, head_dim=64, d_model=512, d_ffn=1536, vocab=1024, seed=61)
+    first, second = (wl.make_weights(c, device="cuda") for c in (cfg, dataclasses.replace(cfg, seed=62)))
+    B, c, lens = 2, 16, [70, 33]
+    window = wl.make_random_window(cfg, B, c, salt=4).numpy()
+
+    def step(dec):
+        dec.kv_view().normal_(generator=torch.Generator(device="cuda").manual_seed(5))
+        dec.fc_debug_set_state(lens, window[:, 0], c)
+        logits = dec.fc_debug_logits(True)
+        dec.fc_jacobi_step(window)
+        return logits.cpu().numpy().copy()
+
+    want = step(engine.Decoder(cfg, second, B, c, 100))
+    dec = engine.Decoder(cfg, first, B, c, 100)
+    other = step(dec)
+    donor = engine.Decoder(cfg, second, B, c, 100)
+    dec.close()
+    h = C.c_void_p()
+    assert dec.lib.fc_init(C.byref(h), C.byref(dec.shape), C.byref(donor.weights), dec.kv.data_ptr(), dec._kv_bytes,
+                           dec.ws.data_ptr(), dec._ws_bytes, dec.stream.cuda_stream) == _l.FC_OK
+    dec.h = h
+    got = step(dec)
+    assert np.array_equal(got, want) and not np.array_equal(got, other)
+    assert dec.fc_debug_check_guards() == 0
