@@ -13,6 +13,7 @@
 
 #include "fc_attn.cuh"
 #include "fc_internal.h"
+#include "fc_plan.h"
 #include "fc_ptx.cuh"
 
 namespace fc {
@@ -250,6 +251,7 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
 #pragma unroll
     for (int i = 0; i < 4; ++i) o[n][i] = 0.f;
   bool ok = true;
+  int issued = min(NS, n_mine);
   for (int i = 0; i < n_mine; ++i) {
     const int stage = i % NS, key0 = key0_of(i);
     if (!__all_sync(0xffffffffu, wait_bounded(smem_u32(&full_bar[warp][stage]), (uint32_t)(i / NS) & 1u))) { ok = false; break; }
@@ -265,7 +267,10 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
     attend<HD, kShortKeys / 8>(kb, vb, C::kSub, qh, ql, o, m_run, l_run, sl2, lane, whole,
                                [&](int n, int x) { return key0 + n * 8 + t4 * 2 + (x & 1) < L; });
     __syncwarp();
-    if (lane == 0 && i + NS < n_mine) { fence_proxy_async(); request(i + NS); }
+    if (i + NS < n_mine) {
+      if (lane == 0) { fence_proxy_async(); request(i + NS); }
+      ++issued;
+    }
   }
   if (has_win) {
     // 16-key blocks of the window, dealt to the warps behind the cached tiles
@@ -282,12 +287,12 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
     l_run[hh] += __shfl_xor_sync(0xffffffffu, l_run[hh], 2);
   }
   if (!__syncthreads_and(ok ? 1 : 0)) {
-    // a tile did not arrive: no result; copies on their way stay inside this CTA's ring, which outlives them as far as the bound
+    // a tile did not arrive: no result; this warp's copies on their way are waited for (bounded)
     if (lane == 0) {
       atomicExch(a.err, 1u);
       const unsigned long long t0 = clock64();
-      for (int i = 0; i < NS && i < n_mine; ++i)
-        while (!mbar_try(smem_u32(&full_bar[warp][i]), (uint32_t)((n_mine - 1 - i) / NS) & 1u))
+      for (int i = 0; i < NS && i < issued; ++i)
+        while (!mbar_try(smem_u32(&full_bar[warp][i]), last_copy_parity(issued, NS, i)))
           if ((unsigned long long)(clock64() - t0) > kSpinBudget / 4) break;
     }
     __syncthreads();

@@ -20,6 +20,7 @@
 
 #include "fc_attn.cuh"
 #include "fc_internal.h"
+#include "fc_plan.h"
 #include "fc_ptx.cuh"
 
 namespace fc {
@@ -148,6 +149,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
 
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long full_bar[S], empty_bar[S];
+  __shared__ int issued_s;                         // tiles that the producer requested
   __shared__ float2 ml[kSWarps][16];              // (max, sum) per warp and query row
   __shared__ __align__(8) float2 ml_cta[ROWS];    // after the merge of the CTA's key groups
 
@@ -196,7 +198,8 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
     if (lane == 0) {
       const int plane_k = a.k_plane0 + b * a.hkv + kvh, plane_v = a.v_plane0 + b * a.hkv + kvh;
       bool waited = false;
-      for (int t = 0; t < nt; ++t) {
+      int t = 0;
+      for (; t < nt; ++t) {
         const int stage = t % S;
         if (t >= S && !wait_bounded(smem_u32(&empty_bar[stage]), (uint32_t)(t / S - 1) & 1u)) { ok = false; break; }
         const int y = (t_begin + t) * kSKeys;
@@ -212,6 +215,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
 #pragma unroll
         for (int s = 0; s < SUB; ++s) load_3d(dst + C::kHalf + s * C::kSub, &map, s * 64, y, plane_v, bar);
       }
+      issued_s = t;
     }
   } else {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -342,16 +346,13 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
     }
   }
   if (!__syncthreads_and(ok ? 1 : 0)) {
-    // a tile did not arrive: no result.  Copies that are still on their way stay inside this CTA's ring, which outlives
-    // them as far as the bound below.
+    // a tile did not arrive: no result.  Copies on their way are waited for (bounded).
     if (tid == 0) {
       atomicExch(a.err, 1u);
       const unsigned long long t0 = clock64();
-      for (int i = 0; i < S && i < nt; ++i) {
-        const int last = (nt - 1 - i) / S;
-        while (!mbar_try(smem_u32(&full_bar[i]), (uint32_t)last & 1u))
+      for (int i = 0; i < S && i < issued_s; ++i)
+        while (!mbar_try(smem_u32(&full_bar[i]), last_copy_parity(issued_s, S, i)))
           if ((unsigned long long)(clock64() - t0) > kSpinBudget / 4) break;
-      }
     }
     __syncthreads();
   }
