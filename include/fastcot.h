@@ -159,6 +159,10 @@ int fc_get_state(fc_ctx *ctx, int32_t *kv_lens, int32_t *n_gen);
  * separated by canary bands written at fc_init; *n_damaged (host) receives how many of them no longer hold the
  * pattern (0 = no kernel wrote outside its slice). */
 int fc_debug_inject_timeout(fc_ctx *ctx);
+/* The next forward of up to 64 rows through the one-writer projections waits, at the grid barriers of one launch, for an
+ * arrival that no CTA makes: its bounded waits run out (0.2 s) and the step returns FC_ERR_DEVICE_TIMEOUT.  FC_ERR_STATE if
+ * this context has no such projections. */
+int fc_debug_withhold_arrival(fc_ctx *ctx);
 int fc_debug_check_guards(fc_ctx *ctx, int32_t *n_damaged);
 
 /* Enqueue `n_steps` iterations back to back with no host round trip in between and return the

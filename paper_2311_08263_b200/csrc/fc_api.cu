@@ -223,6 +223,7 @@ struct fc_ctx {
   int gen_max_tokens = 0, gen_eos = -1;
   float ms_prefill = 0.f;        // device time of the most recent fc_prefill
   bool inject_timeout = false;   // test aid: the next step's accept kernel raises the device error word
+  bool withhold = false;         // test aid: the next one-writer launch of several projections waits for an arrival that nobody makes
   char *ws_base = nullptr;
   std::vector<size_t> guards;    // offsets of the canary bands inside the workspace
   // pinned staging: [count | tokens | window | err]
@@ -741,6 +742,8 @@ static int forward_cluster(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, c
     if (rc != FC_OK) return rc;
     if (!with_head && l + 1 == L) break;               // rows that are only cached: nothing reads what follows the last K/V rows
     ca.g_ffn = ctx->g_ffn[l]; ca.g_next = l + 1 < L ? ctx->g_attn[l + 1] : ctx->g_final;
+    ca.withheld = ctx->withhold ? 1 : 0;
+    ctx->withhold = false;
     FC_CK(chain(4 * l + 1, l + 1 < L ? 4 * l + 5 : 4 * L, FC_CLS_CHAIN));
   }
   if (with_head) FC_CK(chain(4 * L, 4 * L + 1, FC_CLS_HEAD));
@@ -1247,6 +1250,13 @@ extern "C" int fc_finish_with_trigger(fc_ctx *ctx, const int32_t *trigger_ids, i
   }
   ctx->launches = launches;
   return check_device_error(ctx);
+}
+
+extern "C" int fc_debug_withhold_arrival(fc_ctx *ctx) {
+  if (!ctx) return FC_ERR_ARG;
+  if (!ctx->plan_cl) return FC_ERR_STATE;
+  ctx->withhold = true;
+  return FC_OK;
 }
 
 extern "C" int fc_debug_inject_timeout(fc_ctx *ctx) {

@@ -340,6 +340,7 @@ struct ClusterArgs {
   float *ss_attn;                 // [R], written by the QKV projection
   float eps;
   unsigned int *bar;              // [8 * n_layers + 2], zero when a forward starts
+  int withheld;                   // test aid: arrivals that the launch's grid barriers wait for and nobody makes
   const int32_t *tokens, *perm; float beta; unsigned long long *amax; float *logits;
   unsigned int *err;
 };

@@ -102,6 +102,7 @@ struct ClParams {
   int first_slots;                                 // slots of ss_x in front of layer 0
   float eps; int dn;
   unsigned int *bar;                               // two counters per projection (all results, the first column ranges), zero when a forward starts
+  unsigned int arrivals;                           // that complete a counter: the CTAs (a test may ask for one more)
   const int32_t *tokens, *perm; float beta;
   unsigned long long *amax; float *logits;
   unsigned int *err;
@@ -194,6 +195,17 @@ __device__ __forceinline__ bool elect_one() {
   uint32_t one;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(one));
   return one != 0;
+}
+__device__ __forceinline__ void mbar_complete_tx(uint32_t bar, uint32_t bytes) {      // as if that many bytes had arrived
+  asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
 }
 __device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, float a, float b, float c, float d) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
@@ -305,6 +317,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   __shared__ int2 tiles_s[T];                      // warp 0
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s, issued_w_s, issued_x_s;
+  __shared__ int sent_s[8], taken_s, expected_s, peer_abort_s;      // exchange units; used only after a wait has run out
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   const uint32_t xs_base = base + S * kStageW, xc_base = xs_base + NX * C::kXSlot;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -344,7 +357,8 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     __syncwarp();
   } else if (warp == 2) {
     // the other barriers, one per lane
-    if (lane == 0) { abort_s = 0; issued_w_s = 0; issued_x_s = 0; mbar_init(smem_u32(&drain_bar), 1); }
+    if (lane == 0) { abort_s = 0; peer_abort_s = 0; taken_s = 0; expected_s = 0; issued_w_s = 0; issued_x_s = 0; mbar_init(smem_u32(&drain_bar), 1); }
+    if (lane < 8) sent_s[lane] = 0;
     if (lane < NX) { mbar_init(smem_u32(&full_x[lane]), 1); mbar_init(smem_u32(&empty_x[lane]), 1); }
     if (lane < NACC) { mbar_init(smem_u32(&acc_full[lane]), 1); mbar_init(smem_u32(&acc_empty[lane]), 8); }
     // an exchange buffer is free again when the four output warps of all four CTAs have read theirs
@@ -474,7 +488,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
             const int need = ph.kind == PH_DOWN && pr < ph.np0 ? 1 : 2;
             if (seen < need) {
               if (id == p.first) asm volatile("griddepcontrol.wait;" ::: "memory");     // they are the kernel's in front
-              else if (!grid_wait(word + (need == 1 ? 1 : 0), gridDim.x, abort_flag)) { ok = false; break; }
+              else if (!grid_wait(word + (need == 1 ? 1 : 0), p.arrivals, abort_flag)) { ok = false; break; }
               asm volatile("fence.proxy.async.global;" ::: "memory");      // rows stored by other CTAs, read by the TMA
               seen = need;
             }
@@ -539,6 +553,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
                 const float *v = &sum[t][BN > 16 ? (cb % (NCB / 2 > 0 ? NCB / 2 : 1)) * 16 : 0];
 #pragma unroll
                 for (int i = 0; i < N; i += 4) st_async_v4(to + (uint32_t)((BN > 16 ? 0 : half * H) + i) * 4u, bar, v[i], v[i + 1], v[i + 2], v[i + 3]);
+                if (lane == 0) sent_s[warp - kDrainWarp0] = u + 1;
               }
             }
           }
@@ -561,7 +576,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     for (int id = p.first; id < p.last; ++id) {
       const Phase ph = phase_of(p, id, cl, rank);
       const int kind = ph.kind;
-      if (id != p.first && ot == 0) (void)grid_wait(p.bar + 2 * (id - 1), gridDim.x, abort_flag);
+      if (id != p.first && ot == 0) (void)grid_wait(p.bar + 2 * (id - 1), p.arrivals, abort_flag);
       out_meet();
       if (kind == PH_GU || kind == PH_HEAD || (kind == PH_QKV && blockIdx.x == 0)) {
         // row sums of squares over the slots of all CTAs, in a fixed order
@@ -613,9 +628,10 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
           const bool mine = live && r < p.R;
           float4 xr = make_float4(0.f, 0.f, 0.f, 0.f);
           if (mine && (kind == PH_O || kind == PH_DOWN)) xr = __ldcg(reinterpret_cast<const float4 *>(p.x + (long long)r * p.d + col));
-          if (ok && ot == 0) mbar_expect_tx(smem_u32(&xc_full[b]), kCl * 32 * 16 * 4);
+          if (ok && ot == 0) { mbar_expect_tx(smem_u32(&xc_full[b]), kXBuf); expected_s = e + 1; }
           if (ok) ok = mbar_wait_warp(smem_u32(&xc_full[b]), (uint32_t)(e / C::NXB) & 1u, abort_flag);
           if (!ok) continue;
+          if (ot == 0) taken_s = e + 1;
           const float *src = reinterpret_cast<const float *>(xc_gen + b * kXBuf) + (mq * 4) * kXRow + n;
           float v[4];
 #pragma unroll
@@ -708,6 +724,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   if (abort_s) {
     if (threadIdx.x == 0) {
       atomicExch(p.err, 1u);
+      for (int r = 0; r < kCl; ++r) st_cluster_u32(map_to_cta(smem_u32(&peer_abort_s), (uint32_t)r), 1u);
       const unsigned long long t0 = clock64();                    // copies still in flight (bounded)
       for (int i = max(0, issued_w_s - S); i < issued_w_s; ++i)
         while (!mbar_try(smem_u32(&full_w[i % S]), (uint32_t)(i / S) & 1u))
@@ -730,8 +747,36 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   __syncwarp();
   // No CTA leaves while a peer may still write to it.  (Relaxed: what goes across the cluster has been waited for above; a release would
   // also wait for the last global stores, which the end of the grid does.)
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  if (abort_s) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  else asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (*(volatile int *)&peer_abort_s) {
+    // A wait ran out in this cluster, so not everything that was sent has been waited for.  Every CTA learns from its peers how far
+    // they sent, lets each buffer expect that and no more, and waits (bounded) for it to land.
+    cluster_sync_all();
+    if (threadIdx.x == 0) {
+      const unsigned long long t0 = clock64();
+      for (int b = 0; b < C::NXB; ++b) {
+        int u = taken_s;                                          // the first unit of this buffer that was not taken
+        while (u % C::NXB != b) ++u;
+        uint32_t bytes = 0;
+        for (int r = 0; r < kCl; ++r)
+          for (int w = 0; w < 8; ++w)                             // the senders whose weight rows are this CTA's
+            if (((w + kDrainWarp0) & 3) == rank && u < (int)ld_cluster_u32(map_to_cta(smem_u32(&sent_s[w]), (uint32_t)r)) &&
+                (BN == 16 || (u % NCB) / (NCB / 2 > 0 ? NCB / 2 : 1) == w >> 2))
+              bytes += 32 * (BN == 16 ? H : 16) * 4;
+        const uint32_t bar = smem_u32(&xc_full[b]);
+        if (u < expected_s) { if (bytes < (uint32_t)kXBuf) mbar_complete_tx(bar, (uint32_t)kXBuf - bytes); }
+        else if (bytes > 0) mbar_expect_tx(bar, bytes);
+        else continue;
+        while (!mbar_try(bar, (uint32_t)(u / C::NXB) & 1u))
+          if ((unsigned long long)(clock64() - t0) > kSpinBudget / 4) break;
+      }
+    }
+    __syncthreads();
+    __syncwarp();
+    cluster_sync_all();
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, C::kCols);
@@ -887,7 +932,7 @@ cudaError_t launch_cluster_chain(const ClusterPlan *pl, const ClusterArgs &a, in
   p.x = a.x; p.qkv = a.qkv; p.pan_x = (__nv_bfloat16 *)a.pan_x; p.pan_h = (__nv_bfloat16 *)a.pan_h;
   p.g_ffn = (const __nv_bfloat16 *)a.g_ffn; p.g_next = (const __nv_bfloat16 *)a.g_next;
   p.ss_x = a.ss_x; p.ss_ffn = a.ss_ffn; p.ss_attn = a.ss_attn; p.first_slots = 1;
-  p.eps = a.eps; p.dn = m.d; p.bar = a.bar; p.err = a.err;
+  p.eps = a.eps; p.dn = m.d; p.bar = a.bar; p.arrivals = (unsigned int)(pl->ncl * kCl + a.withheld); p.err = a.err;
   p.tokens = a.tokens; p.perm = a.perm; p.beta = a.beta; p.amax = a.amax; p.logits = a.logits;
   const int width = a.R <= 16 ? 0 : a.R <= 32 ? 1 : 2;
   ClMaps maps = pl->maps[width];

@@ -142,6 +142,9 @@ class Decoder:
     def fc_debug_inject_timeout(self):
         self._check(self.lib.fc_debug_inject_timeout(self.h), "fc_debug_inject_timeout")
 
+    def fc_debug_withhold_arrival(self):
+        self._check(self.lib.fc_debug_withhold_arrival(self.h), "fc_debug_withhold_arrival")
+
     def fc_debug_check_guards(self) -> int:
         """Number of damaged canary bands: those between the workspace slices (kept by the library) plus the ones
         this binding keeps around the K/V slab and the workspace."""

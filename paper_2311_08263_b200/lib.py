@@ -21,7 +21,7 @@ FC_ERR_ARG, FC_ERR_SHAPE, FC_ERR_CAPACITY, FC_ERR_TOKEN_RANGE = -1, -2, -3, -4
 FC_ERR_STATE, FC_ERR_BAD_WINDOW, FC_ERR_DEVICE_TIMEOUT, FC_ERR_CUDA = -5, -6, -7, -8
 
 EXPORTS = ["fc_kv_bytes", "fc_workspace_bytes", "fc_init", "fc_prefill", "fc_jacobi_step", "fc_generate",
-           "fc_set_window", "fc_finish_with_trigger", "fc_debug_inject_timeout", "fc_debug_check_guards",
+           "fc_set_window", "fc_finish_with_trigger", "fc_debug_inject_timeout", "fc_debug_withhold_arrival", "fc_debug_check_guards",
            "fc_debug_set_state", "fc_debug_logits", "fc_get_state", "fc_bench_steps", "fc_profile_step",
            "fc_last_launch_count", "fc_destroy", "fc_strerror", "fc_last_cuda_error",
            "fc_op_linear", "fc_op_accept", "fc_op_window_attention",
@@ -76,6 +76,7 @@ def load() -> C.CDLL:
     lib.fc_set_window.argtypes = [vp, i32]
     lib.fc_finish_with_trigger.argtypes = [vp, i32p, i32, i32, i32, i32p, i32p]
     lib.fc_debug_inject_timeout.argtypes = [vp]
+    lib.fc_debug_withhold_arrival.argtypes = [vp]
     lib.fc_debug_check_guards.argtypes = [vp, C.POINTER(C.c_int32)]
     lib.fc_debug_set_state.argtypes = [vp, i32, i32p, i32p, i32, i32]
     lib.fc_debug_logits.argtypes = [vp, vp]

@@ -131,3 +131,26 @@ def test_second_model_in_the_buffers_of_the_first():
     got = step(dec)
     assert np.array_equal(got, want) and not np.array_equal(got, other)
     assert dec.fc_debug_check_guards() == 0
+
+
+@pytest.mark.parametrize("c", [16, 24, 50])
+def test_wait_that_runs_out_is_reported_and_the_next_prompt_is_as_before(c):
+    """A grid barrier that one arrival is missing from (widths 16, 32, 64): the waits of every CTA run out, the exchange and the copies
+    on their way are waited for, the step reports it.  The buffers and the context are as good as new."""
+    from paper_2311_08263_b200 import engine, lib as _l
+    cfg = wl.small_config(n_layers=2, n_heads=8, n_kv_heads=8, head_dim=64, d_model=512, d_ffn=4608, vocab=1024, prompt_len=60, seed=71)
+    ids = wl.make_prompts(cfg)[0][0].numpy()
+    dec = engine.Decoder(cfg, wl.make_weights(cfg, device="cuda"), 1, c, 60 + 4 * c)
+    logits = dec.fc_debug_logits(True)
+    dec.fc_prefill(ids, [60], c)
+    want = dec.fc_jacobi_step()
+    first = logits.clone()
+    dec.fc_debug_withhold_arrival()
+    with pytest.raises(engine.FcError) as e:
+        dec.fc_jacobi_step()
+    assert e.value.code == _l.FC_ERR_DEVICE_TIMEOUT
+    assert dec.fc_debug_check_guards() == 0
+    dec.fc_prefill(ids, [60], c)
+    got = dec.fc_jacobi_step()
+    assert all(np.array_equal(a, b) for a, b in zip(got, want)) and bool((logits == first).all())
+    assert dec.fc_debug_check_guards() == 0
