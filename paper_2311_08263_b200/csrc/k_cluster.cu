@@ -317,7 +317,8 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   __shared__ int2 tiles_s[T];                      // warp 0
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s, issued_w_s, issued_x_s;
-  __shared__ int sent_s[8], taken_s, expected_s, peer_abort_s;      // exchange units; used only after a wait has run out
+  // Exchange units sent, taken and expected, for the end of a launch in which a wait ran out: written where a role fails or ends.
+  __shared__ int sent_s[8], taken_s, expected_s, peer_abort_s;
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   const uint32_t xs_base = base + S * kStageW, xc_base = xs_base + NX * C::kXSlot;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -357,8 +358,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     __syncwarp();
   } else if (warp == 2) {
     // the other barriers, one per lane
-    if (lane == 0) { abort_s = 0; peer_abort_s = 0; taken_s = 0; expected_s = 0; issued_w_s = 0; issued_x_s = 0; mbar_init(smem_u32(&drain_bar), 1); }
-    if (lane < 8) sent_s[lane] = 0;
+    if (lane == 0) { abort_s = 0; peer_abort_s = 0; issued_w_s = 0; issued_x_s = 0; mbar_init(smem_u32(&drain_bar), 1); }
     if (lane < NX) { mbar_init(smem_u32(&full_x[lane]), 1); mbar_init(smem_u32(&empty_x[lane]), 1); }
     if (lane < NACC) { mbar_init(smem_u32(&acc_full[lane]), 1); mbar_init(smem_u32(&acc_empty[lane]), 8); }
     // an exchange buffer is free again when the four output warps of all four CTAs have read theirs
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
             if (ph.np > 0) {
               const int ab = use % NACC;
               ok = mbar_wait_warp(smem_u32(&acc_full[ab]), (uint32_t)(use / NACC) & 1u, abort_flag);
-              if (!ok) continue;
+              if (!ok) { if (lane == 0) sent_s[warp - kDrainWarp0] = e + (sg + 1 == nseg ? t * NCB : 0); continue; }
               tc_fence_after();
               const uint32_t ta = t_lane + (uint32_t)(ab * C::kAcc);
               constexpr int N = H < 16 ? 8 : 16;
@@ -546,14 +546,16 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
               for (int cb = 0; cb < NCB; ++cb) {
                 if (BN > 16 && cb / (NCB / 2 > 0 ? NCB / 2 : 1) != half) continue;       // the other half's rows
                 const int u = e + t * NCB + cb, b = u % C::NXB;
-                if (u >= C::NXB && ok) ok = mbar_wait_warp(smem_u32(&xc_empty[b]), (uint32_t)(u / C::NXB - 1) & 1u, abort_flag);
+                if (u >= C::NXB && ok) {
+                  ok = mbar_wait_warp(smem_u32(&xc_empty[b]), (uint32_t)(u / C::NXB - 1) & 1u, abort_flag);
+                  if (!ok && lane == 0) sent_s[warp - kDrainWarp0] = u;
+                }
                 if (!ok) continue;
                 const uint32_t to = dst + (uint32_t)(b * kXBuf), bar = dbar + (uint32_t)b * 8u;
                 constexpr int N = H < 16 ? H : 16;
                 const float *v = &sum[t][BN > 16 ? (cb % (NCB / 2 > 0 ? NCB / 2 : 1)) * 16 : 0];
 #pragma unroll
                 for (int i = 0; i < N; i += 4) st_async_v4(to + (uint32_t)((BN > 16 ? 0 : half * H) + i) * 4u, bar, v[i], v[i + 1], v[i + 2], v[i + 3]);
-                if (lane == 0) sent_s[warp - kDrainWarp0] = u + 1;
               }
             }
           }
@@ -561,6 +563,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
         e += tn * NCB;
       }
     }
+    if (ok && lane == 0) sent_s[warp - kDrainWarp0] = e;
     // the peers' arrivals of the last units too: one that lands in the next kernel's barrier would let a sender there go too early
     for (int u = max(0, e - C::NXB); u < e && ok; ++u)
       if (BN == 16 || (u % NCB) / (NCB / 2 > 0 ? NCB / 2 : 1) == half) ok = mbar_wait_warp(smem_u32(&xc_empty[u % C::NXB]), (uint32_t)(u / C::NXB) & 1u, abort_flag);
@@ -628,10 +631,12 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
           const bool mine = live && r < p.R;
           float4 xr = make_float4(0.f, 0.f, 0.f, 0.f);
           if (mine && (kind == PH_O || kind == PH_DOWN)) xr = __ldcg(reinterpret_cast<const float4 *>(p.x + (long long)r * p.d + col));
-          if (ok && ot == 0) { mbar_expect_tx(smem_u32(&xc_full[b]), kXBuf); expected_s = e + 1; }
-          if (ok) ok = mbar_wait_warp(smem_u32(&xc_full[b]), (uint32_t)(e / C::NXB) & 1u, abort_flag);
+          if (ok && ot == 0) mbar_expect_tx(smem_u32(&xc_full[b]), kXBuf);
+          if (ok) {
+            ok = mbar_wait_warp(smem_u32(&xc_full[b]), (uint32_t)(e / C::NXB) & 1u, abort_flag);
+            if (!ok && ot == 0) { taken_s = e; expected_s = e + 1; }
+          }
           if (!ok) continue;
-          if (ot == 0) taken_s = e + 1;
           const float *src = reinterpret_cast<const float *>(xc_gen + b * kXBuf) + (mq * 4) * kXRow + n;
           float v[4];
 #pragma unroll
@@ -714,6 +719,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
       }
       if (id + 1 < p.last) publish(p.bar + 2 * id);
     }
+    if (ok && ot == 0) { taken_s = e; expected_s = e; }
     asm volatile("fence.proxy.async.global;" ::: "memory");       // for the TMA reads of the next kernel
   }
 
@@ -756,11 +762,14 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     cluster_sync_all();
     if (threadIdx.x == 0) {
       const unsigned long long t0 = clock64();
+#pragma unroll 1
       for (int b = 0; b < C::NXB; ++b) {
         int u = taken_s;                                          // the first unit of this buffer that was not taken
         while (u % C::NXB != b) ++u;
         uint32_t bytes = 0;
+#pragma unroll 1
         for (int r = 0; r < kCl; ++r)
+#pragma unroll 1
           for (int w = 0; w < 8; ++w)                             // the senders whose weight rows are this CTA's
             if (((w + kDrainWarp0) & 3) == rank && u < (int)ld_cluster_u32(map_to_cta(smem_u32(&sent_s[w]), (uint32_t)r)) &&
                 (BN == 16 || (u % NCB) / (NCB / 2 > 0 ? NCB / 2 : 1) == w >> 2))
