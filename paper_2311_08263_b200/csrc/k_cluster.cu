@@ -168,10 +168,36 @@ __device__ __forceinline__ void load_4d(uint32_t dst, const CUtensorMap *map, in
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar) : "memory");
 }
-// Arrival on a barrier of another CTA of the cluster that orders nothing in front of it: the caller sees to it that its loads have
-// arrived.  (Release at cluster scope waits for all global stores on their way: 0.7 us per exchange unit.)
+// Arrival on a barrier of another CTA of the cluster, behind this warp's accesses to its own CTA's shared memory.  (The release is
+// restricted to those: an unrestricted one waits for all global stores on their way too, 0.7 us per exchange unit; 8 layers of 1.1B, 16 rows
+// 387 us against 350, 64 rows 774 against 594.)
 __device__ __forceinline__ void mbar_arrive_far(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+  asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+}
+// Bounded wait of a converged warp for what other CTAs of the cluster signal: acquires at cluster scope.
+__device__ __forceinline__ bool mbar_try_far(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool wait_far(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+  bool ok = true;
+  if (!mbar_try_far(bar, parity)) {
+    const unsigned long long t0 = clock64();
+    unsigned int spins = 0;
+    while (!mbar_try_far(bar, parity)) {
+      if ((++spins & 0xFFu) == 0u) {
+        if (*abort_flag) { ok = false; break; }
+        if ((unsigned long long)(clock64() - t0) > kSpinBudget) { *abort_flag = 1; ok = false; break; }
+      }
+    }
+  }
+  return __all_sync(0xffffffffu, ok);
 }
 // Every lane that looks waits for its own barrier; one verdict for the warp.
 __device__ __forceinline__ bool lanes_wait(uint32_t bar, uint32_t parity, bool looks, volatile int *abort_flag) {
@@ -547,7 +573,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
                 if (BN > 16 && cb / (NCB / 2 > 0 ? NCB / 2 : 1) != half) continue;       // the other half's rows
                 const int u = e + t * NCB + cb, b = u % C::NXB;
                 if (u >= C::NXB && ok) {
-                  ok = mbar_wait_warp(smem_u32(&xc_empty[b]), (uint32_t)(u / C::NXB - 1) & 1u, abort_flag);
+                  ok = wait_far(smem_u32(&xc_empty[b]), (uint32_t)(u / C::NXB - 1) & 1u, abort_flag);
                   if (!ok && lane == 0) sent_s[warp - kDrainWarp0] = u;
                 }
                 if (!ok) continue;
@@ -566,7 +592,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     if (ok && lane == 0) sent_s[warp - kDrainWarp0] = e;
     // the peers' arrivals of the last units too: one that lands in the next kernel's barrier would let a sender there go too early
     for (int u = max(0, e - C::NXB); u < e && ok; ++u)
-      if (BN == 16 || (u % NCB) / (NCB / 2 > 0 ? NCB / 2 : 1) == half) ok = mbar_wait_warp(smem_u32(&xc_empty[u % C::NXB]), (uint32_t)(u / C::NXB) & 1u, abort_flag);
+      if (BN == 16 || (u % NCB) / (NCB / 2 > 0 ? NCB / 2 : 1) == half) ok = wait_far(smem_u32(&xc_empty[u % C::NXB]), (uint32_t)(u / C::NXB) & 1u, abort_flag);
   } else {
     // ------------------------------------------------------------ finished values
     const int ot = threadIdx.x - kOutWarp0 * 32, n = ot & 15, mq = ot >> 4;       // row n of a block of 16, weight rows 4 mq .. 4 mq + 3 of this CTA's 32
@@ -633,7 +659,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
           if (mine && (kind == PH_O || kind == PH_DOWN)) xr = __ldcg(reinterpret_cast<const float4 *>(p.x + (long long)r * p.d + col));
           if (ok && ot == 0) mbar_expect_tx(smem_u32(&xc_full[b]), kXBuf);
           if (ok) {
-            ok = mbar_wait_warp(smem_u32(&xc_full[b]), (uint32_t)(e / C::NXB) & 1u, abort_flag);
+            ok = wait_far(smem_u32(&xc_full[b]), (uint32_t)(e / C::NXB) & 1u, abort_flag);
             if (!ok && ot == 0) { taken_s = e; expected_s = e + 1; }
           }
           if (!ok) continue;
@@ -645,10 +671,9 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
 #pragma unroll
             for (int k = 1; k < kCl; ++k) v[i] += src[(k * 32 + i) * kXRow];
           }
-          // The buffer is free once the loads have arrived, not once they are issued: the vote needs the sums of every lane.  (No sum
-          // has this pattern - the NaN an addition makes has another - but nothing less than a value holds the arrival back.)
-          const bool unread = __any_sync(0xffffffffu, __float_as_uint((v[0] + v[1]) + (v[2] + v[3])) == 0x7fc12345u);
-          if (lane < kCl && !unread) mbar_arrive_far(far_empty + (uint32_t)b * 8u);
+          // the buffer is free: every lane's loads are in front of the arrival (a barrier of the warp, then the release)
+          __syncwarp();
+          if (lane < kCl) mbar_arrive_far(far_empty + (uint32_t)b * 8u);
           if (kind == PH_O || kind == PH_DOWN) {
             if (mine) {
               v[0] += xr.x; v[1] += xr.y; v[2] += xr.z; v[3] += xr.w;

@@ -51,7 +51,7 @@ def test_step_against_the_oracle_and_again(hq, hkv, hd, d, f, vocab, c, lens):
     assert dec.fc_debug_check_guards() == 0
 
 
-@pytest.mark.parametrize("b,c,length", [(16, 1, 500), (1, 16, 800), (2, 16, 300), (4, 16, 300), (16, 1, 2048)])
+@pytest.mark.parametrize("b,c,length", [(16, 1, 500), (1, 16, 800), (2, 16, 300), (1, 24, 300), (1, 33, 500), (4, 16, 300), (16, 1, 2048)])
 def test_wide_steps_repeat_bit_for_bit(b, c, length):
     """Two layers of the 7B shape, fifty times the same step: exchange buffers that are written again before they are read, or
     read before they are written, show as rows that differ."""
