@@ -1,5 +1,7 @@
 // Integer arithmetic of the launch plans and of the waits, without CUDA types (the tests compile it with the host compiler).
 #pragma once
+#include <cstddef>
+#include <mutex>
 
 #ifdef __CUDACC__
 #define FC_HD __host__ __device__ inline
@@ -12,5 +14,20 @@ namespace fc {
 // A ring of `stages` stages into which `issued` copies have been requested, copy j into stage j % stages: the parity of the phase that
 // the last copy into `stage` completes (stage < issued).
 FC_HD unsigned int last_copy_parity(int issued, int stages, int stage) { return (unsigned int)((issued - 1 - stage) / stages) & 1u; }
+
+// A limit per device that only rises (a kernel's dynamic shared memory), set and remembered by one thread at a time: a thread that sets
+// a lower one after another has remembered its higher one would have that one's next launch refused.
+struct RisingLimit {
+  std::mutex m;
+  size_t done[64] = {0};
+  template <typename Set>
+  auto raise(int dev, size_t bytes, Set set) -> decltype(set(bytes)) {      // set: 0 is success
+    std::lock_guard<std::mutex> lock(m);
+    if (bytes <= done[dev]) return (decltype(set(bytes)))0;
+    auto e = set(bytes);
+    if (e == (decltype(e))0) done[dev] = bytes;
+    return e;
+  }
+};
 
 }  // namespace fc

@@ -27,6 +27,7 @@
 #include <cstring>
 
 #include "fc_internal.h"
+#include "fc_plan.h"
 
 namespace fc {
 
@@ -694,13 +695,11 @@ static cudaError_t launch_fused_t(const KvTensorMap &kmap, const KvTensorMap &vm
   }
   const size_t smem = attn_smem_bytes<HD>(a.c, QT, args.stages);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  static size_t attr_smem[kMaxDevices] = {0};
-  const int dev = current_device_slot();
-  if (smem > attr_smem[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(attn_tma_kernel<HD, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_smem[dev] = smem;
-  }
+  static RisingLimit limit;
+  const cudaError_t set = limit.raise(current_device_slot(), smem, [](size_t n) {
+    return cudaFuncSetAttribute(attn_tma_kernel<HD, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+  });
+  if (set != cudaSuccess) return set;
   const int nqt = ((a.hq / a.hkv) * a.c + 15) / 16;
   const int nqg = (nqt + QT - 1) / QT;
   cudaLaunchConfig_t cfg;

@@ -389,13 +389,11 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
 template <int HD>
 static cudaError_t launch_short_t(const KvTensorMap &map, const ShortAttnArgs &a, int ns, int nqt, int nb, cudaStream_t st) {
   const size_t smem = short_smem<HD>(a.c, a.stages);
-  static size_t attr_smem[kMaxDevices] = {0};
-  const int dev = current_device_slot();
-  if (smem > attr_smem[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(attn_short_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_smem[dev] = smem;
-  }
+  static RisingLimit limit;
+  const cudaError_t set = limit.raise(current_device_slot(), smem, [](size_t n) {
+    return cudaFuncSetAttribute(attn_short_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+  });
+  if (set != cudaSuccess) return set;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3(ns, a.hkv * nqt, nb); cfg.blockDim = dim3(kShortThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;

@@ -21,6 +21,7 @@
 #include <cstring>
 
 #include "fc_internal.h"
+#include "fc_plan.h"
 #include "fc_ptx.cuh"
 
 namespace fc {
@@ -920,13 +921,11 @@ cudaError_t make_pair_tensor_map(CUtensorMap *out, const void *pan, int pan_rows
 template <int EPI, int BN, bool PANEL>
 static cudaError_t launch_one(const MapPack &maps, const UmmaParams &p, int grid, cudaStream_t st) {
   const size_t smem = (size_t)p.stages * (kWBytes + x_parts(BN) * BN * 128) + 1024;
-  static size_t attr_smem[kMaxDevices] = {0};
-  const int dev = current_device_slot();
-  if (smem > attr_smem[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_umma_kernel<EPI, BN, PANEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_smem[dev] = smem;
-  }
+  static RisingLimit limit;
+  const cudaError_t set = limit.raise(current_device_slot(), smem, [](size_t n) {
+    return cudaFuncSetAttribute(gemm_umma_kernel<EPI, BN, PANEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+  });
+  if (set != cudaSuccess) return set;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;

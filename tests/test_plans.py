@@ -9,8 +9,23 @@ from paper_2311_08263_b200 import build
 
 WRAP = """
 #include "fc_plan.h"
+#include <chrono>
+#include <thread>
 extern "C" {
 unsigned int last_copy_parity(int issued, int stages, int stage) { return fc::last_copy_parity(issued, stages, stage); }
+// Two threads raise a limit to `a` and, begun a little later but finished at once, to `b`; the limit that stands.
+long long raised_by_two(long long a, long long b) {
+  fc::RisingLimit limit;
+  long long stands = 0;
+  auto raise = [&](long long n, int ms) {
+    limit.raise(3, (size_t)n, [&](size_t v) { std::this_thread::sleep_for(std::chrono::milliseconds(ms)); stands = (long long)v; return 0; });
+  };
+  std::thread t(raise, a, 60);
+  std::this_thread::sleep_for(std::chrono::milliseconds(20));
+  raise(b, 0);
+  t.join();
+  return stands;
+}
 }
 """
 
@@ -21,7 +36,7 @@ def plan(tmp_path_factory):
     src, so = os.path.join(d, "wrap.cpp"), os.path.join(d, "plan.so")
     with open(src, "w") as f:
         f.write(WRAP)
-    subprocess.check_call(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", build.CSRC, src, "-o", so])
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-pthread", "-shared", "-fPIC", "-I", build.CSRC, src, "-o", so])
     return C.CDLL(so)
 
 
@@ -34,3 +49,10 @@ def test_parity_that_a_wait_for_the_copies_in_flight_asks_for(plan, stages):
             phases = len(range(stage, issued, stages))
             p = plan.last_copy_parity(issued, stages, stage)
             assert (phases - 1 - 1) % 2 != p and (phases - 1) % 2 == p
+
+
+@pytest.mark.parametrize("a,b", [(100, 200), (200, 100)])
+def test_limit_raised_by_two_threads_is_the_higher_one(plan, a, b):
+    """Shared-memory limits of a kernel: contexts on different threads, windows of different length."""
+    plan.raised_by_two.restype = C.c_longlong
+    assert plan.raised_by_two(C.c_longlong(a), C.c_longlong(b)) == 200
