@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "fc_internal.h"
+#include "fc_plan.h"
 #include "fc_ptx.cuh"
 
 namespace fc {
@@ -40,6 +41,7 @@ namespace {
 constexpr int kCl = 4;                             // CTAs per cluster = shares of the k range
 constexpr int kUnit = 16;                          // weight rows per unit
 constexpr int kTileUnits = 8;                      // units per tile at most (M = 128)
+constexpr int kFewestClusters = 16;                // a B200 holds 33
 constexpr int kThreadsCl = 480;
 constexpr int kDrainWarp0 = 3, kOutWarp0 = 11;
 constexpr int kStageW = 2 * kTileM * kTileK * 2;   // 32 KB: two k-blocks
@@ -110,10 +112,6 @@ struct ClParams {
 
 // The units of a matrix are cut into column ranges of nearly equal size, and every range into one tile per cluster: so
 // all clusters have the same number of tiles, and with the tiles of one index a whole range of columns is finished.
-int n_parts(int units, int ncl) { return ((units + ncl - 1) / ncl + kTileUnits - 1) / kTileUnits; }
-// x / n == x * reciprocal(n) >> 32 for x < 2^32 / n (the products here are below 2^24)
-unsigned int reciprocal(int n) { return n == 1 ? 0u : (unsigned int)((0x100000000ull + (unsigned)n - 1) / (unsigned)n); }
-__host__ __device__ inline int quotient(int x, unsigned int inv) { return inv ? (int)((unsigned long long)(unsigned)x * inv >> 32) : x; }
 __host__ __device__ inline void tile_units(const Kind &k, int t, int cl, unsigned int inv_ncl, int &u, int &h) {
   const int b = quotient(t * k.units, k.inv_parts), n = quotient((t + 1) * k.units, k.inv_parts) - b;
   u = b + quotient(cl * n, inv_ncl);
@@ -869,6 +867,8 @@ static int cluster_fit() {
 }
 
 bool cluster_shape_ok(int d, int qd, int kvd, int f, int vocab) {
+  for (int n : {d, qd, kvd, f, vocab})
+    if (!ranges_exact(n / kUnit, kFewestClusters, kTileUnits)) return false;
   return d % 128 == 0 && qd % 128 == 0 && f % 128 == 0 && kvd % kUnit == 0 && vocab % kUnit == 0;
 }
 
@@ -877,7 +877,7 @@ ClusterPlan *cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a
   EncodeTiledFn enc = encode_fn();
   int ncl = cluster_fit<16>();
   for (int n : {cluster_fit<32>(), cluster_fit<64>(), kClusterSlots / kCl}) ncl = n < ncl ? n : ncl;
-  if (!enc || ncl < 1 || !cluster_shape_ok(m.d, m.qd, m.kvd, m.f, m.vocab)) return nullptr;
+  if (!enc || ncl < kFewestClusters || !cluster_shape_ok(m.d, m.qd, m.kvd, m.f, m.vocab)) return nullptr;
   ClusterPlan *pl = new (std::nothrow) ClusterPlan();
   if (!pl) return nullptr;
   pl->m = m; pl->ncl = ncl;
@@ -886,7 +886,7 @@ ClusterPlan *cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a
   bool ok = true;
   auto kind_of = [&](int N, int K, int mat0) {
     Kind k; memset(&k, 0, sizeof k);
-    k.units = N / kUnit; k.parts = k.n_tiles = n_parts(k.units, ncl); k.inv_parts = reciprocal(k.parts);
+    k.units = N / kUnit; k.parts = k.n_tiles = column_ranges(k.units, ncl, kTileUnits); k.inv_parts = reciprocal(k.parts);
     k.pairs = k.first = K >> 7; k.mat0 = mat0;
     k.h0 = k.units / k.parts / ncl;                // ranges differ by one unit, and so do the tiles of a range
     return k;

@@ -110,3 +110,12 @@ def test_workspace_holds_no_tensor_maps(cdll):
     shape = dict(dtype=lib.FC_BF16, d_model=512, n_heads=8, n_kv_heads=8, head_dim=64, d_ffn=1536, vocab=1024, max_c=16, max_seq=80)
     few, many = (cdll.fc_workspace_bytes(C.byref(_shape(**shape, n_layers=n))) for n in (8, 40))
     assert many - few < 32 * 512 + 1024
+
+
+def test_workspace_without_the_operands_of_a_route_that_the_vocabulary_is_too_large_for(cdll):
+    """Two million ids are beyond what the one-writer projections' tile arithmetic is exact for: as with a vocabulary that is no multiple
+    of 16, no operands for them."""
+    cdll.fc_workspace_bytes.restype = C.c_size_t
+    shape = dict(dtype=lib.FC_BF16, d_model=512, n_heads=8, n_kv_heads=8, head_dim=64, d_ffn=1536, max_c=16, max_seq=80)
+    large, ragged, small = (cdll.fc_workspace_bytes(C.byref(_shape(**shape, vocab=n))) for n in (2000000, 2000001, 32016))
+    assert large == ragged < small
