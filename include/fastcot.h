@@ -184,6 +184,15 @@ int fc_profile_step(fc_ctx *ctx, float *ms_by_class, int32_t *launches_by_class)
 /* Number of kernels the most recent step / prefill / bench call launched. */
 int64_t fc_last_launch_count(const fc_ctx *ctx);
 
+/* Which kernels the most recent forward ran: one FC_ROUTE_* (the projections) | one FC_ATTN_* (not with FC_ROUTE_SMALL); 0 before the
+ * first forward.  For tests and for naming what was timed; which forward takes which is the library's choice. */
+enum { FC_ROUTE_SMALL = 1 /* fp32, everything in one kernel */, FC_ROUTE_SEPARATE = 2 /* a launch per projection */,
+       FC_ROUTE_CHAIN = 3 /* a layer's projections in one launch, sums added up in L2 */,
+       FC_ROUTE_ONE_WRITER = 4 /* the same in clusters with one writer per output */, FC_ROUTE_DENSE = 5 /* dense GEMMs */,
+       FC_ROUTE_MASK = 15, FC_ATTN_SPLIT = 16 /* FMA kernel over key splits */, FC_ATTN_FUSED = 32, FC_ATTN_STREAM = 48, FC_ATTN_SHORT = 64,
+       FC_ATTN_MASK = 240 };
+int fc_last_route(const fc_ctx *ctx);
+
 void fc_destroy(fc_ctx *ctx);
 const char *fc_strerror(int status);
 const char *fc_last_cuda_error(const fc_ctx *ctx);   /* text of the last CUDA failure, or "" */

@@ -233,6 +233,7 @@ struct fc_ctx {
   bool small = false;            // fp32 model whose forward is one kernel (up to a number of keys: small_forward_pays)
   int32_t *pin_map = nullptr;    // pinned [max_batch]: the live sequences of a compacted step
   int64_t launches = 0;
+  int route = 0;                 // FC_ROUTE_* | FC_ATTN_* of the most recent forward
   char cuda_err[256] = {0};
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // per-launch profiling (fc_profile_step)
@@ -278,6 +279,7 @@ extern "C" const char *fc_strerror(int st) {
 
 extern "C" const char *fc_last_cuda_error(const fc_ctx *ctx) { return ctx ? ctx->cuda_err : ""; }
 extern "C" int64_t fc_last_launch_count(const fc_ctx *ctx) { return ctx ? ctx->launches : 0; }
+extern "C" int fc_last_route(const fc_ctx *ctx) { return ctx ? ctx->route : 0; }
 
 static void destroy_plans(fc_ctx *ctx) {
   for (auto *v : {&ctx->plan_qkv, &ctx->plan_o, &ctx->plan_gu, &ctx->plan_down, &ctx->plan_gu_half[0], &ctx->plan_gu_half[1],
@@ -493,8 +495,13 @@ extern "C" int fc_init(fc_ctx **out, const fc_model_shape *shape, const fc_weigh
     m.n_layers = L; m.d = shape->d_model; m.qd = ctx->d.qd; m.kvd = ctx->d.kvd; m.f = shape->d_ffn; m.vocab = shape->vocab;
     m.wq = ctx->wq.data(); m.wk = ctx->wk.data(); m.wv = ctx->wv.data(); m.wo = ctx->wo.data();
     m.w_gate = ctx->w_gate.data(); m.w_up = ctx->w_up.data(); m.w_down = ctx->w_down.data(); m.lm_head = ctx->lm_head;
-    ctx->plan_cl = cluster_plan_create(m, ctx->b.cl_pan_x, ctx->b.cl_pan_a, ctx->b.cl_pan_h);
-    (void)cudaGetLastError();    // without it (a device that does not hold the clusters): the other routes
+    // without a plan (a device that holds too few of the clusters): the other routes
+    const cudaError_t e = cluster_plan_create(m, ctx->b.cl_pan_x, ctx->b.cl_pan_a, ctx->b.cl_pan_h, &ctx->plan_cl);
+    if (e != cudaSuccess) {
+      fprintf(stderr, "fc_init: plan of the one-writer projections: %s\n", cudaGetErrorString(e));
+      (void)cudaGetLastError();
+      return fail(FC_ERR_CUDA);
+    }
   }
   const int B = shape->max_batch;
   ctx->kv_len_h.assign(B, 0); ctx->n_gen_h.assign(B, 0); ctx->pending_h.assign(B, 0); ctx->done_h.assign(B, 0);
@@ -577,6 +584,7 @@ static int forward_small(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, con
   a.x = ctx->b.x; a.q = (float *)ctx->b.qb; a.attn = ctx->b.attn; a.h = ctx->b.gu;
   a.with_head = with_head; a.perm = s.bias_beta != 0.f ? ctx->bias_perm : nullptr; a.beta = s.bias_beta; a.logits = ctx->dbg_logits;
   if (with_head) a.accept = accept_args(ctx, segs.b0, nb, rows, segs.seq_map, commit);
+  ctx->route = FC_ROUTE_SMALL;
   ++ctx->launches;
   ProfScope ps(ctx, FC_CLS_CHAIN);
   FC_CK(launch_small_forward(a, ctx->st));
@@ -590,6 +598,7 @@ static int forward_bulk(fc_ctx *ctx, const RowSegs &segs, int nseg, int R, int m
   const fc_model_shape &s = ctx->s;
   const Dims &d = ctx->d;
   if (R < 1 || R > d.rows_ws) return FC_ERR_CAPACITY;
+  ctx->route = FC_ROUTE_DENSE | FC_ATTN_STREAM;
   const int pdl = ctx->pdl && !ctx->prof;
   EmbedArgs ea; memset(&ea, 0, sizeof ea);
   ea.tokens = tokens; ea.emb = ctx->tok_emb; ea.x = ctx->b.x; ea.R = R; ea.d = s.d_model;
@@ -734,6 +743,7 @@ static int forward_cluster(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, c
     return launch_cluster_chain(ctx->plan_cl, ca, first, last, pdl, ctx->st);
   };
   const bool stream = with_head && !attn_short_pays(max_len, rows, s.n_heads, s.n_kv_heads, nb, s.head_dim, ctx->n_sms);
+  ctx->route = FC_ROUTE_ONE_WRITER | (stream ? FC_ATTN_STREAM : FC_ATTN_SHORT);
   ZeroList none; memset(&none, 0, sizeof none);
   FC_CK(chain(0, 1, FC_CLS_QKV));
   for (int l = 0; l < L; ++l) {
@@ -800,6 +810,7 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
   const bool chained = ctx->chain;
   const bool o_panel = chained && ctx->fused_attn && R > 16 && ctx->d.pan_rows >= R;
   const bool stream = with_head && ctx->fused_attn && attn_stream_pays(max_len_host, rows, s.n_heads, s.n_kv_heads, nb);
+  ctx->route = (chained ? FC_ROUTE_CHAIN : FC_ROUTE_SEPARATE) | (stream ? FC_ATTN_STREAM : ctx->fused_attn ? FC_ATTN_FUSED : FC_ATTN_SPLIT);
   for (int l = 0; l < s.n_layers; ++l) {
     if (!chained || l == 0)
       FC_CK(run_gemm(ctx, ctx->use_umma ? ctx->plan_qkv[l] : nullptr, args_qkv(ctx, l), R, PRO_GAIN, EPI_ATOMIC_ADD, FC_CLS_QKV, claim_word(ctx, l, GEMM_QKV)));

@@ -329,7 +329,7 @@ struct ClusterModel {
 };
 struct ClusterPlan;
 bool cluster_shape_ok(int d, int qd, int kvd, int f, int vocab);
-ClusterPlan *cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a, void *pan_h);
+cudaError_t cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a, void *pan_h, ClusterPlan **out);
 void cluster_plan_destroy(ClusterPlan *p);
 struct ClusterArgs {
   int R;

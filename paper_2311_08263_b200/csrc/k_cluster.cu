@@ -856,14 +856,16 @@ static cudaError_t cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (
   cfg.attrs = attr; cfg.numAttrs = pdl ? 2 : 1;
   return cudaSuccess;
 }
+// most = min(most, clusters that run at the same time)
 template <int BN>
-static int cluster_fit() {
+static cudaError_t cluster_fit(int &most) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   int n = 0;
-  if (cluster_config<BN>(cfg, attr, 1, 0, nullptr) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, cluster_chain_kernel<BN>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
-  return n;
+  cudaError_t e = cluster_config<BN>(cfg, attr, 1, 0, nullptr);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, cluster_chain_kernel<BN>, &cfg);
+  if (e == cudaSuccess && n < most) most = n;
+  return e;
 }
 
 bool cluster_shape_ok(int d, int qd, int kvd, int f, int vocab) {
@@ -872,14 +874,18 @@ bool cluster_shape_ok(int d, int qd, int kvd, int f, int vocab) {
   return d % 128 == 0 && qd % 128 == 0 && f % 128 == 0 && kvd % kUnit == 0 && vocab % kUnit == 0;
 }
 
-// Pairs: [2][kClusterRows][d | qd | f].  Null: the device does not hold it.
-ClusterPlan *cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a, void *pan_h) {
+// Pairs: [2][kClusterRows][d | qd | f].  *out is null where the device holds too few of the clusters; anything else that fails is an error.
+cudaError_t cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a, void *pan_h, ClusterPlan **out) {
+  *out = nullptr;
   EncodeTiledFn enc = encode_fn();
-  int ncl = cluster_fit<16>();
-  for (int n : {cluster_fit<32>(), cluster_fit<64>(), kClusterSlots / kCl}) ncl = n < ncl ? n : ncl;
-  if (!enc || ncl < kFewestClusters || !cluster_shape_ok(m.d, m.qd, m.kvd, m.f, m.vocab)) return nullptr;
+  if (!enc || !cluster_shape_ok(m.d, m.qd, m.kvd, m.f, m.vocab)) return cudaErrorNotSupported;
+  int ncl = kClusterSlots / kCl;
+  cudaError_t e = cluster_fit<16>(ncl);
+  if (e == cudaSuccess) e = cluster_fit<32>(ncl);
+  if (e == cudaSuccess) e = cluster_fit<64>(ncl);
+  if (e != cudaSuccess || ncl < kFewestClusters) return e;
   ClusterPlan *pl = new (std::nothrow) ClusterPlan();
-  if (!pl) return nullptr;
+  if (!pl) return cudaErrorMemoryAllocation;
   pl->m = m; pl->ncl = ncl;
   pl->w.resize((size_t)m.n_layers * kMats + 1);
   memset((void *)pl->w.data(), 0, pl->w.size() * sizeof pl->w[0]);
@@ -929,8 +935,9 @@ ClusterPlan *cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a
       ok = enc(&pl->maps[b].x[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, pans[i], gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
-  if (!ok) { delete pl; return nullptr; }
-  return pl;
+  if (!ok) { delete pl; return cudaErrorInvalidValue; }
+  *out = pl;
+  return cudaSuccess;
 }
 void cluster_plan_destroy(ClusterPlan *p) { delete p; }
 

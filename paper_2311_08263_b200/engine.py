@@ -195,6 +195,9 @@ class Decoder:
     def fc_last_launch_count(self) -> int:
         return int(self.lib.fc_last_launch_count(self.h))
 
+    def fc_last_route(self) -> int:
+        return int(self.lib.fc_last_route(self.h))
+
     # ---- K/V slab view for the window-step sweep (the caller writes random K/V into it) --------
     def kv_view(self) -> torch.Tensor:
         s = self.shape

@@ -14,6 +14,8 @@ LIB_PATH = os.path.join(_HERE, "libfastcot.so")
 FC_F32, FC_BF16 = 0, 1
 FC_REFILL_PROMPT_CYCLE, FC_REFILL_PAD = 0, 1
 FC_FLAG_SIMT_GEMM, FC_FLAG_NO_PDL, FC_FLAG_NO_CHAIN, FC_FLAG_NO_FFN_SPLIT, FC_FLAG_NO_CTA_PAIRS = 1, 4, 8, 16, 32
+FC_ROUTE_SMALL, FC_ROUTE_SEPARATE, FC_ROUTE_CHAIN, FC_ROUTE_ONE_WRITER, FC_ROUTE_DENSE, FC_ROUTE_MASK = 1, 2, 3, 4, 5, 15
+FC_ATTN_SPLIT, FC_ATTN_FUSED, FC_ATTN_STREAM, FC_ATTN_SHORT, FC_ATTN_MASK = 16, 32, 48, 64, 240
 FC_OK = 0
 FC_NOALLOC_SCRATCH_BYTES = 8 << 20
 FC_CLASSES = ["embed", "qkv", "rope", "attn", "oproj", "gateup", "down", "head", "accept", "chain"]
@@ -23,7 +25,7 @@ FC_ERR_STATE, FC_ERR_BAD_WINDOW, FC_ERR_DEVICE_TIMEOUT, FC_ERR_CUDA = -5, -6, -7
 EXPORTS = ["fc_kv_bytes", "fc_workspace_bytes", "fc_init", "fc_prefill", "fc_jacobi_step", "fc_generate",
            "fc_set_window", "fc_finish_with_trigger", "fc_debug_inject_timeout", "fc_debug_withhold_arrival", "fc_debug_check_guards",
            "fc_debug_set_state", "fc_debug_logits", "fc_get_state", "fc_bench_steps", "fc_profile_step",
-           "fc_last_launch_count", "fc_destroy", "fc_strerror", "fc_last_cuda_error",
+           "fc_last_launch_count", "fc_last_route", "fc_destroy", "fc_strerror", "fc_last_cuda_error",
            "fc_op_linear", "fc_op_accept", "fc_op_window_attention",
            "fc_op_window_attention_scratch_bytes", "fc_op_window_attention_noalloc",
            "fc_op_fused_window_attention", "fc_op_fused_window_attention_scratch_bytes"]
@@ -85,6 +87,7 @@ def load() -> C.CDLL:
     lib.fc_profile_step.argtypes = [vp, C.POINTER(C.c_float), C.POINTER(C.c_int32)]
     lib.fc_last_launch_count.restype = C.c_int64
     lib.fc_last_launch_count.argtypes = [vp]
+    lib.fc_last_route.argtypes = [vp]
     lib.fc_destroy.restype = None
     lib.fc_destroy.argtypes = [vp]
     lib.fc_strerror.restype = C.c_char_p

@@ -6,7 +6,7 @@ differ in their last bits)."""
 import numpy as np
 import pytest
 
-from paper_2311_08263_b200 import workload as wl
+from paper_2311_08263_b200 import lib as _l, workload as wl
 from test_gpu_full_configs import _random_kv_case
 
 pytestmark = pytest.mark.gpu
@@ -35,6 +35,7 @@ CASES = [
 def test_step_against_the_oracle_and_again(hq, hkv, hd, d, f, vocab, c, lens):
     cfg = wl.small_config(n_layers=2, n_heads=hq, n_kv_heads=hkv, head_dim=hd, d_model=d, d_ffn=f, vocab=vocab, seed=2000 + c + hd)
     dec, _ = _random_kv_case(cfg, lens, c, range(len(lens)))
+    assert dec.fc_last_route() & _l.FC_ROUTE_MASK == _l.FC_ROUTE_ONE_WRITER
     units, tiles = len(lens) * hkv * ((hq // hkv * c + 15) // 16), (max(lens) + c + 63) // 64
     assert dec.fc_last_launch_count() == (3 if units * tiles >= 8600 else 2) * cfg.n_layers + 4
     logits = dec.fc_debug_logits(True)
@@ -95,6 +96,7 @@ def test_rows_where_the_route_changes():
         logits = dec.fc_debug_logits(True)
         dec.fc_jacobi_step(window[:, :c].copy())
         got[c] = logits[:c].float().cpu().clone()
+        assert dec.fc_last_route() & _l.FC_ROUTE_MASK == (_l.FC_ROUTE_ONE_WRITER if 9 <= c <= 32 else _l.FC_ROUTE_CHAIN)
         assert dec.fc_debug_check_guards() == 0
     for c in (8, 9, 32):
         assert float((got[c] - got[33][:c]).abs().max()) < 3e-2 * float(got[33].pow(2).mean().sqrt())
@@ -106,7 +108,7 @@ def test_second_model_in_the_buffers_of_the_first():
     import ctypes as C
     import dataclasses
     import torch
-    from paper_2311_08263_b200 import engine, lib as _l
+    from paper_2311_08263_b200 import engine
     cfg = wl.small_config(n_layers=3, n_heads=8, n_kv_heads=8, head_dim=64, d_model=512, d_ffn=1536, vocab=1024, seed=61)
     first, second = (wl.make_weights(c, device="cuda") for c in (cfg, dataclasses.replace(cfg, seed=62)))
     B, c, lens = 2, 16, [70, 33]
@@ -137,7 +139,7 @@ def test_second_model_in_the_buffers_of_the_first():
 def test_wait_that_runs_out_is_reported_and_the_next_prompt_is_as_before(c):
     """A grid barrier that one arrival is missing from (widths 16, 32, 64): the waits of every CTA run out, the exchange and the copies
     on their way are waited for, the step reports it.  The buffers and the context are as good as new."""
-    from paper_2311_08263_b200 import engine, lib as _l
+    from paper_2311_08263_b200 import engine
     cfg = wl.small_config(n_layers=2, n_heads=8, n_kv_heads=8, head_dim=64, d_model=512, d_ffn=4608, vocab=1024, prompt_len=60, seed=71)
     ids = wl.make_prompts(cfg)[0][0].numpy()
     dec = engine.Decoder(cfg, wl.make_weights(cfg, device="cuda"), 1, c, 60 + 4 * c)
