@@ -27,6 +27,28 @@ inline bool ranges_exact(int units, int clusters, int tile) {
   return parts * units * (parts - 1) < (1ll << 32);
 }
 
+// Key splits of the short attention (the CTAs of a unit, one cluster): `units` units of (sequence, kv head, 16 queries), `tiles` key tiles
+// for the `warps` warps of a CTA.  fit(splits, deep): clusters that run at the same time, with one CTA per SM and the whole ring of tiles
+// (deep) or with two per SM and half of it.  Either cut is taken back until all clusters run at once: clusters do not cross groups of SMs, and
+// what does not fit is a second round.
+template <typename Fit>
+void short_plan(int tiles, long long units, int head_dim, int warps, int n_sms, Fit fit, int &splits, bool &deep) {
+  const int most = tiles < 8 * warps ? (tiles + warps - 1) / warps : 8;
+  auto cut = [&](long long slots, bool d) {
+    int s = (int)(slots / units < most ? slots / units : most);
+    while (s > 1 && units > fit(s, d)) --s;
+    return s > 1 ? s : 1;
+  };
+  splits = cut(n_sms, true);
+  deep = units * splits <= n_sms;
+  // Two CTAs per SM where one leaves a warp more than two tiles: always at head_dim 64 (half the bytes per tile), at 128 where it makes three or
+  // more of one or two.
+  if (tiles > 2 * warps * splits) {
+    const int half = cut(2ll * n_sms, false);
+    if (half > splits && units * half > n_sms && (head_dim == 64 || (splits <= 2 && half >= 3))) { splits = half; deep = false; }
+  }
+}
+
 // A limit per device that only rises (a kernel's dynamic shared memory), set and remembered by one thread at a time: a thread that sets
 // a lower one after another has remembered its higher one would have that one's next launch refused.
 struct RisingLimit {

@@ -30,6 +30,7 @@ struct ShortCfg {
   static constexpr uint32_t kHalf = SUB * kSub;    // K (or V) of a tile
   static constexpr uint32_t kTile = 2 * kHalf;     // 16 KB, 8 KB
   static constexpr uint32_t kQ = 16 * HD * 4;      // 16 queries, high and low
+  static constexpr int stages(bool deep) { return (deep ? 2 : 1) * (HD == 64 ? 2 : 1); }      // tiles in flight per warp
   static constexpr int OLD = HD + 8;               // row pitch of the partial outputs (floats): spreads the banks
   static_assert(kShortWarps * 16 * OLD * 4 <= kShortWarps * (int)kTile, "partial outputs fit over one stage per warp");
 };
@@ -387,19 +388,16 @@ attn_short_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant
 
 // ------------------------------------------------------------------------------------ host side
 template <int HD>
-static cudaError_t launch_short_t(const KvTensorMap &map, const ShortAttnArgs &a, int ns, int nqt, int nb, cudaStream_t st) {
-  const size_t smem = short_smem<HD>(a.c, a.stages);
+static cudaError_t short_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int ns, int ny, int nz, size_t smem, bool pdl, cudaStream_t st) {
   static RisingLimit limit;
   const cudaError_t set = limit.raise(current_device_slot(), smem, [](size_t n) {
     return cudaFuncSetAttribute(attn_short_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
   });
   if (set != cudaSuccess) return set;
-  cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3(ns, a.hkv * nqt, nb); cfg.blockDim = dim3(kShortThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute attr[2];
+  cfg.gridDim = dim3(ns, ny, nz); cfg.blockDim = dim3(kShortThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
   int na = 0;
-  if (a.pdl) {
+  if (pdl) {
     attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[na].val.programmaticStreamSerializationAllowed = 1;
     ++na;
@@ -410,7 +408,40 @@ static cudaError_t launch_short_t(const KvTensorMap &map, const ShortAttnArgs &a
     ++na;
   }
   cfg.attrs = attr; cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, attn_short_kernel<HD>, *reinterpret_cast<const CUtensorMap *>(&map), a);
+  return cudaSuccess;
+}
+
+// Clusters of ns CTAs that run at the same time (B200, one CTA per SM: 74 of two, 45 of three, 33 of four, 26 22 15 15; two: 148 93 71 56 45 37 33).
+// With two per SM a sixteenth is left out, because CTAs of the kernel in front still hold slots when they are placed (36 of 37 clusters of seven ran
+// in two rounds).
+template <int HD>
+static int short_clusters(int ns, bool deep, int c) {
+  static int known[kMaxDevices][9][2][4] = {};
+  int &n = known[current_device_slot()][ns][deep][(c - 1) / 16];
+  if (n == 0) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    int fit = 0;
+    if (short_config<HD>(cfg, attr, ns, 1, 1, short_smem<HD>(c, ShortCfg<HD>::stages(deep)), false, nullptr) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&fit, attn_short_kernel<HD>, &cfg) != cudaSuccess || fit < 1) {
+      (void)cudaGetLastError();
+      fit = 1;
+    }
+    n = !deep && fit > 15 ? fit * 15 / 16 : fit;
+  }
+  return n;
+}
+
+template <int HD>
+static cudaError_t launch_short_t(const KvTensorMap &map, ShortAttnArgs a, int tiles, int nqt, int nb, int n_sms, cudaStream_t st) {
+  int ns;
+  bool deep;
+  short_plan(tiles, (long long)nb * a.hkv * nqt, HD, kShortWarps, n_sms, [&](int s, bool d) { return (long long)short_clusters<HD>(s, d, a.c); }, ns, deep);
+  a.stages = ShortCfg<HD>::stages(deep);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  cudaError_t e = short_config<HD>(cfg, attr, ns, a.hkv * nqt, nb, short_smem<HD>(a.c, a.stages), a.pdl != 0, st);
+  return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, attn_short_kernel<HD>, *reinterpret_cast<const CUtensorMap *>(&map), a) : e;
 }
 
 // map: boxes of attn_stream_tile_keys() keys.
@@ -418,23 +449,15 @@ cudaError_t launch_attn_short(const KvTensorMap &map, const ShortAttnArgs &a, in
   if (nb < 1 || nb > 65535 || a.c < 1 || a.c > 64 || !a.err || !a.out_pan || (hd != 64 && hd != 128)) return cudaErrorInvalidValue;
   const int nqt = ((a.hq / a.hkv) * a.c + 15) / 16;
   if ((long long)a.hkv * nqt > 65535) return cudaErrorInvalidValue;
-  const long long units = (long long)nb * a.hkv * nqt;
   const int tiles = (max_len + kShortKeys - 1) / kShortKeys;
-  // One CTA per SM with 128 KB of tiles in flight, or two with half of that each where one leaves a warp more than two tiles, the finer cut
-  // gives clusters of three or four and a tenth of the slots stays free (what does not fit beside the last CTAs of the kernel in front is a second
-  // round).  Measured, a step, one -> two: 7B, 2 x 16 rows over 803 keys (64 units, clusters of 2 -> 4) 3042 -> 3022 us, 1 x 32 over 8000 4150
-  // -> 3995; 13B, 2 x 16 over 4000 (80 units, 1 -> 3) 7439 -> 6962; but 7B, 3 x 16 over 2000 (96 units, 1 -> 3, 288 of 296 slots) 4507 -> 4870;
-  // 1 x 16 over 8000 (32 units, 4 -> 8) 3280 -> 3873; 13B, 1 x 16 over 8000 (40 units, 3 -> 7) 6434 -> 7084; 7B, 4 x 16 over 2048 (128 units,
-  // 1 -> 2) 4665 -> 4723.  head_dim 64 has half the bytes per tile: 1.1B, 1 x 16 over 8000 (4 -> 8) 1195 -> 1158.
-  long long ns = n_sms / units, two = 2ll * n_sms / units;
-  if (ns < 1) ns = 1;
-  if (tiles > 2 * kShortWarps * ns && (hd == 64 || ((two == 3 || two == 4) && 10 * units * two <= 18ll * n_sms))) ns = two;
-  if (ns > 8) ns = 8;
-  if (ns > (tiles + kShortWarps - 1) / kShortWarps) ns = (tiles + kShortWarps - 1) / kShortWarps;
-  if (ns < 1) ns = 1;
-  ShortAttnArgs args = a;
-  args.stages = (units * ns > n_sms ? 1 : 2) * (hd == 64 ? 2 : 1);
-  return hd == 128 ? launch_short_t<128>(map, args, (int)ns, nqt, nb, st) : launch_short_t<64>(map, args, (int)ns, nqt, nb, st);
+  // One CTA per SM with 128 KB of tiles in flight, or two with half of that each (short_plan).  Measured, a step, one -> two: 7B, 2 x 16 rows over
+  // 803 keys (64 units, clusters of 2 -> 4) 3042 -> 3022 us, 1 x 32 over 8000 4150 -> 3995; 13B, 2 x 16 over 4000 (80 units, 1 -> 3) 7439 ->
+  // 6962; but 1 x 16 over 8000 (32 units, 4 -> 8) 3280 -> 3873; 13B, 1 x 16 over 8000 (40 units, 3 -> 7) 6434 -> 7084; 7B, 4 x 16 over 2048
+  // (128 units, 1 -> 2) 4665 -> 4723.  head_dim 64: 1.1B, 1 x 16 over 8000 (4 -> 8) 1195 -> 1158.
+  // Splits that do not all fit against the next fewer that do, 8 layers of 1.1B, one sequence: 10 rows over 1000 keys (20 units, 7 -> 6) 394 -> 359 us,
+  // 12 rows (24, 6 -> 5) 394 -> 361, 18 rows (36, 4 -> 3) 454 -> 417, over 3000 (8 -> 6) 478 -> 436; 6 layers of 24 query and 8 kv heads of 128 (201 MB),
+  // 32 rows over 3000 keys (48, 3 -> 5 with two CTAs per SM) 560 -> 466.
+  return hd == 128 ? launch_short_t<128>(map, a, tiles, nqt, nb, n_sms, st) : launch_short_t<64>(map, a, tiles, nqt, nb, n_sms, st);
 }
 
 // The streaming pair reads faster where there is much to read (two CTAs of 96 KB of tiles per SM) but takes a second launch per layer, about

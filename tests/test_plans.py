@@ -27,6 +27,13 @@ int wrong_bounds(int units, int clusters, int *most) {
   }
   return wrong;
 }
+// fit: [2][9], clusters of 0 .. 8 CTAs with two CTAs per SM, then with one; returns splits, negative with half the ring
+int short_plan(int tiles, int units, int head_dim, const int *fit) {
+  int splits;
+  bool deep;
+  fc::short_plan(tiles, units, head_dim, 4, 148, [&](int s, bool d) { return (long long)fit[(d ? 9 : 0) + s]; }, splits, deep);
+  return deep ? splits : -splits;
+}
 // Two threads raise a limit to `a` and, begun a little later but finished at once, to `b`; the limit that stands.
 long long raised_by_two(long long a, long long b) {
   fc::RisingLimit limit;
@@ -83,3 +90,33 @@ def test_column_ranges_by_reciprocals_are_exact_where_they_are_used(plan, cluste
             assert most.value <= 8 * clusters
     assert plan.wrong_bounds(125000, 33, C.byref(most)) > 0 and not plan.ranges_exact(125000, 33)
     assert plan.ranges_exact(16032, clusters) and plan.ranges_exact(1792, clusters)
+
+
+# what cudaOccupancyMaxActiveClusters says on a B200 (with two CTAs per SM less a sixteenth)
+FIT = (C.c_int * 18)(0, 296, 138, 87, 66, 52, 42, 34, 30, 0, 148, 74, 45, 33, 26, 22, 15, 15)
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+def test_key_splits_all_run_at_once(plan, head_dim):
+    """Whatever the units and tiles: no more clusters than run at the same time, no CTA without a tile for its warps, never more than
+    eight splits; and units of at most an SM each keep the whole ring unless a warp has more than two tiles."""
+    for units in range(1, 400):
+        for tiles in list(range(0, 70)) + [94, 250, 1000]:
+            got = plan.short_plan(tiles, units, head_dim, FIT)
+            s = abs(got)
+            assert 1 <= s <= 8 and (s == 1 or s <= (tiles + 3) // 4)
+            if s > 1:
+                assert units <= FIT[(9 if got > 0 else 0) + s]
+            if got > 0:
+                assert units * s <= 148
+            elif units <= 148:
+                assert tiles > 8
+
+
+@pytest.mark.parametrize("head_dim,units,tiles,want", [
+    (128, 32, 25, 4), (128, 32, 250, 4), (128, 40, 250, 3), (128, 64, 25, -4), (128, 80, 125, -3), (128, 96, 63, 1), (128, 128, 64, 1), (128, 160, 90, -1),
+    (64, 32, 20, 4), (64, 32, 94, -7), (64, 64, 32, -4), (64, 128, 64, -2),
+    (64, 20, 32, 6), (64, 24, 32, 5), (64, 28, 32, 4), (64, 36, 22, 3), (64, 36, 57, -6), (128, 16, 47, 6), (128, 24, 25, 5), (128, 48, 47, -5), (128, 48, 10, 2),
+])
+def test_key_splits_of_the_measured_shapes(plan, head_dim, units, tiles, want):
+    assert plan.short_plan(tiles, units, head_dim, FIT) == want
