@@ -712,17 +712,6 @@ static int run_short_attn(fc_ctx *ctx, int l, const RowSegs &segs, int nb, int r
   return FC_OK;
 }
 
-// Where the one-writer projections are faster than the chained launch, by the rows and a layer's weights.  Their weight stream is slower the larger
-// the layer, that of the chained launch the more rows share it.  Measured, a step, chained launch -> one writer.  1.1B (88 MB a layer) and
-// 7B (405 MB): every row count, 7B 1 row 2869 -> 2638 us, 3 rows 2866 -> 2583, 40 rows 4564 -> 4383, 64 rows 4521 -> 4133.  13B (634 MB):
-// 1 row 4890 -> 5295, 4 rows 4956 -> 5190, 8 rows 5222 -> 5293 (8 x 1 5753 -> 5728), 16 rows 5796 -> 5454, 18 rows 6276 -> 6058, 32 rows 6654 -> 6445,
-// 40 rows 7572 -> 8997, 64 rows 7827 -> 8968.  The line between 405 and 634 MB lies where straight lines through both cross for more than 32 rows.
-static bool cluster_pays(const fc_model_shape &s, int R) {
-  const long long qd = (long long)s.n_heads * s.head_dim, kvd = (long long)s.n_kv_heads * s.head_dim;
-  const long long layer_bytes = 2 * s.d_model * (2 * qd + 2 * kvd + 3ll * s.d_ffn);
-  return layer_bytes < 450000000 || (R > 8 && R <= 32);
-}
-
 // A forward of at most kClusterRows rows: the projections between two attention launches in one launch with one writer per
 // output.  Every buffer is written before it is read: nothing to clear but the counters.
 static int forward_cluster(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, const int32_t *tokens, bool with_head, int max_len) {
@@ -785,7 +774,7 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
     FC_CK(launch_advance(ctx->b.kv_len, segs, nb, ctx->st));
     return FC_OK;
   }
-  if (ctx->plan_cl && R <= kClusterRows && cluster_pays(s, R)) {
+  if (cluster_pays(ctx->plan_cl, R)) {
     int rc = forward_cluster(ctx, segs, nb, rows, tokens, with_head, max_len_host);
     if (rc != FC_OK) return rc;
     if (with_head) return run_accept(ctx, b0, nb, rows, seq_map, commit);

@@ -27,6 +27,33 @@ inline bool ranges_exact(int units, int clusters, int tile) {
   return parts * units * (parts - 1) < (1ll << 32);
 }
 
+// Share of the one-writer projections' ring stages that is weights: a stage takes two k-blocks of a tile however few of its 8 x 16 weight
+// rows the tile has.  shape: pairs (weight rows, k) of a layer's n matrices.
+inline double stage_fill(const int (*shape)[2], int n, int clusters) {
+  double bytes = 0, room = 0;
+  for (int i = 0; i < n; ++i) {
+    bytes += (double)shape[i][0] * shape[i][1];
+    room += (double)column_ranges(shape[i][0] / 16, clusters, 8) * 128 * clusters * shape[i][1];
+  }
+  return bytes / room;
+}
+
+// Where the one-writer projections are faster than the chained launch, by how full their stages are, a layer's weight bytes and the rows.
+// Measured, a step, chained launch -> one writer, us (layer MB, fill; 1.1B, 7B whole, others 2 to 8 layers).  Full stages, up to 32 rows
+// always: 7B (405, .92) 1 row 2869 -> 2638, 40 rows 4564 -> 4383, 64 rows 4521 -> 4133; 1070 MB, .81: 1 row 649 -> 644, 16 728 -> 655; 1711, .92:
+// 678 -> 648, 770 -> 664.  From 33 rows the activations' loads grow with the stages: 625, .84: 40 rows 790 -> 791, 64 850 -> 812; 906, .82: 775 ->
+// 857, 812 -> 890; 1070, .81: 911 -> 997.  Stages half to two thirds full: 294, .58: 1 row 345 -> 395, 16 396 -> 426, 32 499 -> 451, 40 527 -> 618;
+// 402, .59: 406 -> 508, 456 -> 517, 571 -> 551, 629 -> 767; 510, .68: 468 -> 548, 531 -> 556, 648 -> 591, 696 -> 810; 567, .65: 515 -> 571, 580 ->
+// 576, 696 -> 640, 738 -> 919; 13B (634, .69): 553 -> 582, 8 rows 593 -> 587, 16 624 -> 593, 32 738 -> 658, 40 797 -> 942; 721, .72: 482 -> 499, 539 ->
+// 508, 629 -> 556, 662 -> 781.  Small layers, where the chained launch's latency counts: 1.1B (88, .47) 1 row 47 -> 43 a layer, 40 rows 83 -> 73;
+// 170, .62: 379 -> 398, 436 -> 406, 571 -> 427, 622 -> 589; 201, .73: 71 -> 60 a layer, 105 -> 98.
+inline bool one_writer_pays(double fill, long long layer_bytes, int rows) {
+  if (layer_bytes < 210000000 || (rows > 16 && rows <= 32)) return true;
+  const bool full = fill >= 0.74;
+  if (rows <= 16) return full || (rows > 8 && layer_bytes >= 550000000);
+  return full && layer_bytes < 750000000;
+}
+
 // Key splits of the short attention (the CTAs of a unit, one cluster): `units` units of (sequence, kv head, 16 queries), `tiles` key tiles
 // for the `warps` warps of a CTA.  fit(splits, deep): clusters that run at the same time, with one CTA per SM and the whole ring of tiles
 // (deep) or with two per SM and half of it.  Either cut is taken back until all clusters run at once: clusters do not cross groups of SMs, and

@@ -833,6 +833,8 @@ static EncodeTiledFn encode_fn() {
 struct ClusterPlan {
   ClusterModel m;
   int ncl;
+  double fill;                                     // stage_fill() of a layer
+  long long layer_bytes;
   Kind kind[5], kv;
   ClMaps maps[3];                                  // operand boxes of 16, 32, 64 rows; the weights' are filled in per launch
   std::vector<std::array<CUtensorMap, 2>> w;       // [layer][kMats], then the LM head
@@ -887,6 +889,9 @@ cudaError_t cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a,
   ClusterPlan *pl = new (std::nothrow) ClusterPlan();
   if (!pl) return cudaErrorMemoryAllocation;
   pl->m = m; pl->ncl = ncl;
+  const int shape[7][2] = {{m.qd, m.d}, {m.kvd, m.d}, {m.kvd, m.d}, {m.d, m.qd}, {m.f, m.d}, {m.f, m.d}, {m.d, m.f}};
+  pl->fill = stage_fill(shape, 7, ncl);
+  pl->layer_bytes = 2ll * m.d * (2ll * m.qd + 2ll * m.kvd + 3ll * m.f);
   pl->w.resize((size_t)m.n_layers * kMats + 1);
   memset((void *)pl->w.data(), 0, pl->w.size() * sizeof pl->w[0]);
   bool ok = true;
@@ -940,6 +945,7 @@ cudaError_t cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a,
   return cudaSuccess;
 }
 void cluster_plan_destroy(ClusterPlan *p) { delete p; }
+bool cluster_pays(const ClusterPlan *pl, int R) { return pl && R <= kClusterRows && one_writer_pays(pl->fill, pl->layer_bytes, R); }
 
 cudaError_t launch_embed_pair(const int32_t *tokens, const void *emb, const void *gain, float *x, void *pan, float *ss, unsigned int *words, int n_words,
                               int R, int d, int pdl, cudaStream_t st) {

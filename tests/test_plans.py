@@ -34,6 +34,10 @@ int short_plan(int tiles, int units, int head_dim, const int *fit) {
   fc::short_plan(tiles, units, head_dim, 4, 148, [&](int s, bool d) { return (long long)fit[(d ? 9 : 0) + s]; }, splits, deep);
   return deep ? splits : -splits;
 }
+int one_writer_pays(int d, int qd, int kvd, int f, int rows) {
+  const int shape[7][2] = {{qd, d}, {kvd, d}, {kvd, d}, {d, qd}, {f, d}, {f, d}, {d, f}};
+  return fc::one_writer_pays(fc::stage_fill(shape, 7, 33), 2ll * d * (2ll * qd + 2ll * kvd + 3ll * f), rows);
+}
 // Two threads raise a limit to `a` and, begun a little later but finished at once, to `b`; the limit that stands.
 long long raised_by_two(long long a, long long b) {
   fc::RisingLimit limit;
@@ -120,3 +124,25 @@ def test_key_splits_all_run_at_once(plan, head_dim):
 ])
 def test_key_splits_of_the_measured_shapes(plan, head_dim, units, tiles, want):
     assert plan.short_plan(tiles, units, head_dim, FIT) == want
+
+
+@pytest.mark.parametrize("shape,few,mid,many", [
+    # d, heads x head_dim, kv heads x head_dim, d_ffn: rows up to 8, 9 to 16, 33 to 64 through one writer (17 to 32 always)
+    ((2048, 2048, 256, 5632), 1, 1, 1),
+    ((4096, 4096, 4096, 11008), 1, 1, 1),
+    ((5120, 5120, 5120, 13824), 0, 1, 0),
+    ((4352, 4352, 256, 8192), 0, 0, 0),            # a little over 33 x 8 units of 16 rows: two column ranges, stages half full
+    ((4608, 4608, 512, 9216), 0, 0, 0),
+    ((4352, 4352, 4352, 9600), 0, 0, 0),
+    ((4608, 4608, 4608, 12288), 0, 0, 0),
+    ((4864, 4864, 4864, 12928), 0, 1, 0),
+    ((4224, 4224, 4224, 11264), 1, 1, 1),
+    ((4096, 4096, 1024, 22016), 1, 1, 1),
+    ((6656, 6656, 6656, 17920), 1, 1, 0),
+    ((8192, 8192, 1024, 28672), 1, 1, 0),
+    ((1024, 1024, 256, 2816), 1, 1, 1),
+    ((3072, 3072, 1024, 8192), 1, 1, 1),
+])
+def test_route_of_the_measured_shapes(plan, shape, few, mid, many):
+    for rows, want in ((1, few), (8, few), (9, mid), (16, mid), (17, 1), (32, 1), (33, many), (64, many)):
+        assert plan.one_writer_pays(*shape, rows) == want, rows
