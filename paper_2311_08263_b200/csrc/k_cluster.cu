@@ -341,7 +341,8 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
   __shared__ int2 tiles_s[T];                      // warp 0
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s, issued_w_s, issued_x_s;
-  // Exchange units sent, taken and expected, for the end of a launch in which a wait ran out: written where a role fails or ends.
+  // Exchange units sent, taken and expected, for the end of a launch in which a wait ran out.  (Branches for it in the exchange's loops, and its
+  // code in front of the way out, cost 1 to 4 % of a step: 8 layers of 1.1B, 64 rows 620 us, now 606.)
   __shared__ int sent_s[8], taken_s, expected_s, peer_abort_s;
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   const uint32_t xs_base = base + S * kStageW, xc_base = xs_base + NX * C::kXSlot;
@@ -530,7 +531,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     // weight rows 32 q .. of a tile go to CTA q of the cluster
     const uint32_t dst = map_to_cta(xc_base, (uint32_t)q) + (uint32_t)((rank * 32 + lane) * kXRow * 4);
     const uint32_t dbar = map_to_cta(smem_u32(&xc_full[0]), (uint32_t)q);
-    int use = 0, e = 0;
+    int use = 0, e = 0, sent = 0;                                 // sent: units of this half
     bool ok = true;
     for (int id = p.first; id < p.last && ok; ++id) {
       const Phase ph = phase_of(p, id, cl, rank);
@@ -549,7 +550,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
             if (ph.np > 0) {
               const int ab = use % NACC;
               ok = mbar_wait_warp(smem_u32(&acc_full[ab]), (uint32_t)(use / NACC) & 1u, abort_flag);
-              if (!ok) { if (lane == 0) sent_s[warp - kDrainWarp0] = e + (sg + 1 == nseg ? t * NCB : 0); continue; }
+              if (!ok) continue;
               tc_fence_after();
               const uint32_t ta = t_lane + (uint32_t)(ab * C::kAcc);
               constexpr int N = H < 16 ? 8 : 16;
@@ -572,12 +573,13 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
                 const int u = e + t * NCB + cb, b = u % C::NXB;
                 if (u >= C::NXB && ok) {
                   ok = wait_far(smem_u32(&xc_empty[b]), (uint32_t)(u / C::NXB - 1) & 1u, abort_flag);
-                  if (!ok && lane == 0) sent_s[warp - kDrainWarp0] = u;
                 }
                 if (!ok) continue;
                 const uint32_t to = dst + (uint32_t)(b * kXBuf), bar = dbar + (uint32_t)b * 8u;
                 constexpr int N = H < 16 ? H : 16;
                 const float *v = &sum[t][BN > 16 ? (cb % (NCB / 2 > 0 ? NCB / 2 : 1)) * 16 : 0];
+#pragma unroll
+                sent += 1;
 #pragma unroll
                 for (int i = 0; i < N; i += 4) st_async_v4(to + (uint32_t)((BN > 16 ? 0 : half * H) + i) * 4u, bar, v[i], v[i + 1], v[i + 2], v[i + 3]);
               }
@@ -587,7 +589,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
         e += tn * NCB;
       }
     }
-    if (ok && lane == 0) sent_s[warp - kDrainWarp0] = e;
+    if (lane == 0) sent_s[warp - kDrainWarp0] = sent;
     // the peers' arrivals of the last units too: one that lands in the next kernel's barrier would let a sender there go too early
     for (int u = max(0, e - C::NXB); u < e && ok; ++u)
       if (BN == 16 || (u % NCB) / (NCB / 2 > 0 ? NCB / 2 : 1) == half) ok = wait_far(smem_u32(&xc_empty[u % C::NXB]), (uint32_t)(u / C::NXB) & 1u, abort_flag);
@@ -650,7 +652,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
         uint2 gq = make_uint2(0u, 0u);
         if (live && (kind == PH_O || kind == PH_DOWN)) gq = __ldg(reinterpret_cast<const uint2 *>(gain + col));
 #pragma unroll
-        for (int cb = 0; cb < NCB; ++cb, ++e) {
+        for (int cb = 0; cb < NCB; ++cb, e += ok) {      // a wait that ran out: e stays at its unit
           const int r = cb * 16 + n, b = e % C::NXB;
           const bool mine = live && r < p.R;
           float4 xr = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -658,7 +660,6 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
           if (ok && ot == 0) mbar_expect_tx(smem_u32(&xc_full[b]), kXBuf);
           if (ok) {
             ok = wait_far(smem_u32(&xc_full[b]), (uint32_t)(e / C::NXB) & 1u, abort_flag);
-            if (!ok && ot == 0) { taken_s = e; expected_s = e + 1; }
           }
           if (!ok) continue;
           const float *src = reinterpret_cast<const float *>(xc_gen + b * kXBuf) + (mq * 4) * kXRow + n;
@@ -742,7 +743,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
       }
       if (id + 1 < p.last) publish(p.bar + 2 * id);
     }
-    if (ok && ot == 0) { taken_s = e; expected_s = e; }
+    if (ot == 0) { taken_s = e; expected_s = e + !ok; }
     asm volatile("fence.proxy.async.global;" ::: "memory");       // for the TMA reads of the next kernel
   }
 
@@ -770,16 +771,20 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
         if ((unsigned long long)(clock64() - t0) > kSpinBudget / 4) break;
     }
     __syncthreads();
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");      // the peers' flags, in front of the closing barrier
   }
   tc_fence_before();
   __syncthreads();
   __syncwarp();
   // No CTA leaves while a peer may still write to it.  (Relaxed: what goes across the cluster has been waited for above; a release would
   // also wait for the last global stores, which the end of the grid does.)
-  if (abort_s) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  else asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  if (*(volatile int *)&peer_abort_s) {
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, C::kCols);
+  }
+  if (__builtin_expect(*(volatile int *)&peer_abort_s, 0)) {
     // A wait ran out in this cluster, so not everything that was sent has been waited for.  Every CTA learns from its peers how far
     // they sent, lets each buffer expect that and no more, and waits (bounded) for it to land.
     cluster_sync_all();
@@ -789,12 +794,13 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
       for (int b = 0; b < C::NXB; ++b) {
         int u = taken_s;                                          // the first unit of this buffer that was not taken
         while (u % C::NXB != b) ++u;
+        const int u_half = BN == 16 ? u : u / NCB * (NCB / 2) + u % (NCB / 2 > 0 ? NCB / 2 : 1);      // its number among a half's units
         uint32_t bytes = 0;
 #pragma unroll 1
         for (int r = 0; r < kCl; ++r)
 #pragma unroll 1
           for (int w = 0; w < 8; ++w)                             // the senders whose weight rows are this CTA's
-            if (((w + kDrainWarp0) & 3) == rank && u < (int)ld_cluster_u32(map_to_cta(smem_u32(&sent_s[w]), (uint32_t)r)) &&
+            if (((w + kDrainWarp0) & 3) == rank && u_half < (int)ld_cluster_u32(map_to_cta(smem_u32(&sent_s[w]), (uint32_t)r)) &&
                 (BN == 16 || (u % NCB) / (NCB / 2 > 0 ? NCB / 2 : 1) == w >> 2))
               bytes += 32 * (BN == 16 ? H : 16) * 4;
         const uint32_t bar = smem_u32(&xc_full[b]);
@@ -808,10 +814,6 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
     __syncthreads();
     __syncwarp();
     cluster_sync_all();
-  }
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tmem_base, C::kCols);
   }
 }
 
