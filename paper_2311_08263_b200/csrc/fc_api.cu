@@ -674,7 +674,7 @@ static int run_stream_attn(fc_ctx *ctx, int l, const RowSegs &segs, int nb, int 
   StreamAttnArgs sa; memset(&sa, 0, sizeof sa);
   sa.q = ctx->b.qb; sa.q_tiles = d.q_tiles; sa.kv_len = ctx->b.kv_len; sa.segs = segs; sa.hq = s.n_heads; sa.hkv = s.n_kv_heads;
   sa.k_plane0 = (l * 2) * s.max_batch * s.n_kv_heads; sa.v_plane0 = (l * 2 + 1) * s.max_batch * s.n_kv_heads;
-  sa.err = ctx->b.err; sa.out = out; sa.out_pan = out_pan; sa.pan_rows = pan_rows; sa.pdl = pdl;
+  sa.err = ctx->b.err; sa.out = out; sa.out_pan = out_pan; sa.pan_rows = pan_rows; sa.spare = 1; sa.pdl = pdl;
   ++ctx->launches;
   { ProfScope ps(ctx, FC_CLS_ATTN); FC_CK(launch_attn_stream(ctx->kv_map_stream, sa, nb, rows, max_len, s.head_dim, ctx->n_sms, ctx->st)); }
   return FC_OK;
@@ -731,6 +731,8 @@ static int forward_cluster(fc_ctx *ctx, const RowSegs &segs, int nb, int rows, c
     ProfScope ps(ctx, cls);
     return launch_cluster_chain(ctx->plan_cl, ca, first, last, pdl, ctx->st);
   };
+  // (Rows that are only cached: the short kernel whatever the length.  A trigger's context, short against pair: 1.1B, 28 rows over 8000 keys 546 us
+  // against 666, 52 rows 846 against 827; 7B, 28 rows 488 against 489, 52 rows 783 against 774, for 8 and 4 layers.)
   const bool stream = with_head && !attn_short_pays(max_len, rows, s.n_heads, s.n_kv_heads, nb, s.head_dim, ctx->n_sms);
   ctx->route = FC_ROUTE_ONE_WRITER | (stream ? FC_ATTN_STREAM : FC_ATTN_SHORT);
   ZeroList none; memset(&none, 0, sizeof none);

@@ -158,6 +158,7 @@ struct StreamAttnArgs {   // bf16: window attention over rows whose K/V are in t
   float *out;             // [R, hq * hd] fp32, or
   void *out_pan;          // the bf16 pair [2][pan_rows][hq * hd]
   int pan_rows;
+  int spare;              // behind a persistent launch: key splits leave room beside that kernel's last CTAs
   int pdl;
 };
 

@@ -76,6 +76,22 @@ void short_plan(int tiles, long long units, int head_dim, int warps, int n_sms, 
   }
 }
 
+// Key splits of the streaming attention: the fewest rounds of clusters times a CTA's length in tile times, where start, query loads and merge
+// cost about as much as six tiles.  fit(splits): clusters that run at the same time.  spare: where all run at once, a thirty-second more
+// has to fit.
+template <typename Fit>
+int stream_splits(int tiles, long long units, bool spare, Fit fit) {
+  long long best = 0;
+  int ns = 1;
+  for (int s = 1; s <= 8 && s <= tiles; ++s) {
+    const long long n = fit(s);
+    const long long rounds = spare && s > 1 && units <= n && units + units / 32 > n ? 2 : (units + n - 1) / n;
+    const long long cost = rounds * ((tiles + s - 1) / s + 6 + (s > 1 ? 2 : 0));
+    if (s == 1 || cost < best) { best = cost; ns = s; }
+  }
+  return ns;
+}
+
 // A limit per device that only rises (a kernel's dynamic shared memory), set and remembered by one thread at a time: a thread that sets
 // a lower one after another has remembered its higher one would have that one's next launch refused.
 struct RisingLimit {

@@ -516,7 +516,7 @@ static int stream_clusters(int hd, int wq, int ns, int n_sms) {
 }
 
 // Query tiles per CTA and key splits for `nb` segments of at most `rows` rows behind at most max_len keys.
-static void stream_plan(int max_len, int rows, int group, int hkv, int nb, int hd, int n_sms, int &wq, int &ns) {
+static void stream_plan(int max_len, int rows, int group, int hkv, int nb, int hd, int n_sms, bool spare, int &wq, int &ns) {
   const int nqt = (group * rows + 15) / 16;
   wq = nqt >= 3 ? 4 : nqt;
   const long long units = (long long)nb * hkv * ((nqt + wq - 1) / wq);
@@ -524,16 +524,12 @@ static void stream_plan(int max_len, int rows, int group, int hkv, int nb, int h
   // Rounds of clusters times a CTA's length in tile times; start, query loads and merge cost about as much as six tiles.  Measured
   // by splits, 4 layers over 8000 keys: 7B, 1 x 32 rows (32 units) 4 splits 825 us, 6 742, 7 720, 8 822; 13B, 1 x 32 (40 units) 5
   // 931, 6 894, 7 1028; 13B, 2 x 16 (80 units) 2 957, 3 914, 4 1002; 7B, 4 x 16 (128 units) 1 1084, 2 940, 3 1003.
-  long long best = 0;
-  ns = 1;
-  for (int s = 1; s <= 8 && s <= tiles; ++s) {
-    const int fit = stream_clusters(hd, wq, s, n_sms);
-    // (A thirty-second more where all should run at once: behind the one-writer projections 52 clusters of five that only just fitted ran in two
-    // rounds; 1.1B, 13 x 4 rows over 5000 keys 2176 -> 1988 us a step.  With two rounds or more the edge does not show: 13 x 16 over 4000 3626 -> 3793.)
-    const long long rounds = s > 1 && units <= fit && units + units / 32 > fit ? 2 : (units + fit - 1) / fit;
-    const long long cost = rounds * ((tiles + s - 1) / s + 6 + (s > 1 ? 2 : 0));
-    if (s == 1 || cost < best) { best = cost; ns = s; }
-  }
+  // Behind a persistent launch of projections, where clusters that only just fit run in two rounds (spare): one-writer, 1.1B, 13 x 4 rows over 5000 keys
+  // (52 clusters of five) 2176 -> 1988 us a step, 26 heads of 128 (268 MB, 6 layers), 2 x 32 over 8000
+  // 1235 -> 1128; chained, 2 x 40 over 2000 1039 -> 1010, over 8000 1610 -> 1551; 34 clusters of seven, 1 x 64 over 8000 992 -> 965.  Behind the dense
+  // GEMMs, whose clusters leave one by one, it only takes splits away: 22 heads, 3 x 48 over 4000 891 -> 973, 34 heads, 4 x 40 1496 -> 1668 (4 layers).
+  // (With two rounds or more the edge does not show: 1.1B, 13 x 16 over 4000 3626 -> 3793.)
+  ns = stream_splits(tiles, units, spare, [&](int s) { return stream_clusters(hd, wq, s, n_sms); });
 }
 
 template <int HD, int WQ>
@@ -549,7 +545,7 @@ cudaError_t launch_attn_stream(const KvTensorMap &map, const StreamAttnArgs &a, 
   if (nseg < 1 || nseg > 65535 || max_rows < 1 || !a.err || a.segs.n > kMaxSegs || (hd != 64 && hd != 128)) return cudaErrorInvalidValue;
   const int group = a.hq / a.hkv;
   int wq, ns;
-  stream_plan(max_len, max_rows, group, a.hkv, nseg, hd, n_sms, wq, ns);
+  stream_plan(max_len, max_rows, group, a.hkv, nseg, hd, n_sms, a.spare != 0, wq, ns);
   const int nqg = (group * max_rows + wq * 16 - 1) / (wq * 16);
   if ((long long)a.hkv * nqg > 65535) return cudaErrorInvalidValue;
   if (hd == 128) {

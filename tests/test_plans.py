@@ -38,6 +38,9 @@ int one_writer_pays(int d, int qd, int kvd, int f, int rows) {
   const int shape[7][2] = {{qd, d}, {kvd, d}, {kvd, d}, {d, qd}, {f, d}, {f, d}, {d, f}};
   return fc::one_writer_pays(fc::stage_fill(shape, 7, 33), 2ll * d * (2ll * qd + 2ll * kvd + 3ll * f), rows);
 }
+int stream_splits(int tiles, int units, int spare, const int *fit) {
+  return fc::stream_splits(tiles, units, spare != 0, [&](int s) { return fit[s]; });
+}
 // Two threads raise a limit to `a` and, begun a little later but finished at once, to `b`; the limit that stands.
 long long raised_by_two(long long a, long long b) {
   fc::RisingLimit limit;
@@ -146,3 +149,15 @@ def test_key_splits_of_the_measured_shapes(plan, head_dim, units, tiles, want):
 def test_route_of_the_measured_shapes(plan, shape, few, mid, many):
     for rows, want in ((1, few), (8, few), (9, mid), (16, mid), (17, 1), (32, 1), (33, many), (64, many)):
         assert plan.one_writer_pays(*shape, rows) == want, rows
+
+
+def test_streaming_splits_leave_a_spare_only_where_it_is_asked_for(plan):
+    """Two CTAs per SM, a sixteenth left out.  Behind the dense GEMMs 66 units take four splits and 136 two, which just fit; behind a
+    persistent launch they take fewer or more, whatever leaves a thirty-second free.  Elsewhere the spare changes nothing."""
+    for units, tiles, splits in ((66, 127, 4), (136, 126, 2), (42, 63, 6), (52, 63, 5), (34, 126, 7)):
+        assert plan.stream_splits(tiles, units, 0, FIT) == splits
+        with_spare = plan.stream_splits(tiles, units, 1, FIT)
+        assert with_spare != splits and (units + units // 32 <= FIT[with_spare] or units > FIT[with_spare] or with_spare == 1)
+    for units in (32, 40, 64, 80, 96, 128, 160, 320):
+        for tiles in (1, 2, 8, 26, 63, 126, 250):
+            assert plan.stream_splits(tiles, units, 0, FIT) == plan.stream_splits(tiles, units, 1, FIT)
