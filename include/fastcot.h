@@ -228,7 +228,7 @@ int fc_op_window_attention(const void *q, const void *kcache, const void *vcache
                            int32_t head_dim, int32_t max_seq, int32_t max_len, int32_t dtype,
                            void *scratch, size_t scratch_bytes, void *cuda_stream);
 
-/* The attention kernel of the bf16 step as it runs inside fc_jacobi_step (head_dim 64 or 128): applies the deferred
+/* The attention kernel in front of the chained projections as it runs inside fc_jacobi_step (head_dim 64 or 128): applies the deferred
  * RMSNorm factor 1/sqrt(sumsq[r] / d_norm + rms_eps) to the q, k and v accumulators of every window row, rotates q and k
  * at position kv_len[b] + j (pairs i <-> i + head_dim/2, angle pos * rope_theta^(-2i/head_dim)), stores the window's k and v
  * rows as bf16 at cache slots kv_len[b] .. kv_len[b]+c-1, and computes the window attention of Eq. 4's forward as
@@ -247,6 +247,15 @@ int fc_op_fused_window_attention(float *qkv_acc, float *sumsq, float rms_eps, in
                                  int32_t c, int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, int32_t max_seq,
                                  int32_t max_len, int32_t n_splits, int32_t q_tiles, void *scratch,
                                  size_t scratch_bytes, void *cuda_stream);
+
+/* The attention kernel behind the one-writer projections (up to 64 rows over short caches), as fc_op_fused_window_attention but for the
+ * result, which is what the output projection reads: out_pair, bf16 [2][batch*c][n_heads*head_dim], high and low part (their sum is the
+ * value).  The accumulators and sums of squares are left as they are.  c <= 64; vcache lies whole (sequence, kv head) planes behind
+ * kcache; scratch of fc_op_fused_window_attention_scratch_bytes(...). */
+int fc_op_short_window_attention(const float *qkv_acc, const float *sumsq, float rms_eps, int32_t d_norm, float rope_theta,
+                                 void *kcache, void *vcache, const int32_t *kv_len, void *out_pair, int32_t batch,
+                                 int32_t c, int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, int32_t max_seq,
+                                 int32_t max_len, void *scratch, size_t scratch_bytes, void *cuda_stream);
 
 /* The same window attention for callers that may not allocate device memory (the paper has no
  * counterpart; this exists for hosts whose device memory is owned by someone else, e.g. a serving

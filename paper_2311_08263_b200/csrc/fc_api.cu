@@ -1495,6 +1495,25 @@ static void fused_layout(int hd, int max_seq, size_t off[3]) {
   off[1] = off[0] + align_up((size_t)max_seq * (hd / 2) * sizeof(float2));      // error word
   off[2] = off[1] + align_up(sizeof(unsigned int));                             // end
 }
+// Scratch of the attention kernels as operations: rotary table exactly as fc_init builds it, a cleared error word; the device's SMs.
+static int fused_scratch(char *base, const size_t off[3], float rope_theta, int head_dim, int max_seq, int &sms, cudaStream_t st) {
+  const int half = head_dim / 2;
+  std::vector<float2> table((size_t)max_seq * half);
+  for (int i = 0; i < half; ++i) {
+    const float inv_freq = powf(rope_theta, -2.0f * (float)i / (float)head_dim);
+    for (int pos = 0; pos < max_seq; ++pos) {
+      const float ang = (float)pos * inv_freq;
+      table[(size_t)pos * half + i] = make_float2(cosf(ang), sinf(ang));
+    }
+  }
+  if (cudaMemcpyAsync(base + off[0], table.data(), table.size() * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaMemsetAsync(base + off[1], 0, off[2] - off[1], st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+    return FC_ERR_CUDA;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return FC_ERR_CUDA;
+  return FC_OK;
+}
 }  // namespace fc
 
 extern "C" size_t fc_op_fused_window_attention_scratch_bytes(int32_t batch, int32_t c, int32_t n_heads, int32_t n_kv_heads,
@@ -1520,22 +1539,8 @@ extern "C" int fc_op_fused_window_attention(float *qkv_acc, float *sumsq, float 
   if (scratch_bytes < off[2]) return FC_ERR_CAPACITY;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char *base = (char *)scratch;
-  // rotary table exactly as fc_init builds it
-  const int half = head_dim / 2;
-  std::vector<float2> table((size_t)max_seq * half);
-  for (int i = 0; i < half; ++i) {
-    const float inv_freq = powf(rope_theta, -2.0f * (float)i / (float)head_dim);
-    for (int pos = 0; pos < max_seq; ++pos) {
-      const float ang = (float)pos * inv_freq;
-      table[(size_t)pos * half + i] = make_float2(cosf(ang), sinf(ang));
-    }
-  }
-  if (cudaMemcpyAsync(base + off[0], table.data(), table.size() * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemsetAsync(base + off[1], 0, off[2] - off[1], st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
-    return FC_ERR_CUDA;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return FC_ERR_CUDA;
+  int sms = 0;
+  if (int rc = fused_scratch(base, off, rope_theta, head_dim, max_seq, sms, st)) return rc;
   KvTensorMap kmap, vmap;
   const long long planes = (long long)batch * n_kv_heads;
   if (make_kv_tensor_map(&kmap, kcache, head_dim, max_seq, planes, attn_fused_tile_keys()) != cudaSuccess ||
@@ -1560,6 +1565,38 @@ extern "C" int fc_op_fused_window_attention(float *qkv_acc, float *sumsq, float 
       cudaMemsetAsync(sumsq, 0, (size_t)batch * c * sizeof(float), st) != cudaSuccess ||
       cudaMemcpyAsync(&herr, fa.err, sizeof herr, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess) return FC_ERR_CUDA;
+  return herr ? FC_ERR_DEVICE_TIMEOUT : FC_OK;
+}
+
+extern "C" int fc_op_short_window_attention(const float *qkv_acc, const float *sumsq, float rms_eps, int32_t d_norm, float rope_theta,
+                                            void *kcache, void *vcache, const int32_t *kv_len, void *out_pair, int32_t batch,
+                                            int32_t c, int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, int32_t max_seq,
+                                            int32_t max_len, void *scratch, size_t scratch_bytes, void *cuda_stream) {
+  if (!qkv_acc || !sumsq || !kcache || !vcache || !kv_len || !out_pair || !scratch || d_norm < 1) return FC_ERR_ARG;
+  if (!fused_shape_ok(batch, c, n_heads, n_kv_heads, head_dim, max_seq, max_len) || c > 64) return FC_ERR_ARG;
+  if (max_len + c > max_seq) return FC_ERR_CAPACITY;
+  if ((uintptr_t)scratch % kAlign || ((uintptr_t)kcache | (uintptr_t)vcache | (uintptr_t)qkv_acc | (uintptr_t)out_pair) % 16) return FC_ERR_ARG;
+  // one tensor map covers K and V: the values lie whole planes behind the keys
+  const long long planes = (long long)batch * n_kv_heads, plane_bytes = (long long)max_seq * head_dim * 2;
+  const long long behind = (long long)((intptr_t)vcache - (intptr_t)kcache);
+  if (behind < planes * plane_bytes || behind % plane_bytes || behind / plane_bytes > 0x3fffffff) return FC_ERR_ARG;
+  size_t off[3];
+  fused_layout(head_dim, max_seq, off);
+  if (scratch_bytes < off[2]) return FC_ERR_CAPACITY;
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  char *base = (char *)scratch;
+  int sms = 0;
+  if (int rc = fused_scratch(base, off, rope_theta, head_dim, max_seq, sms, st)) return rc;
+  KvTensorMap map;
+  if (make_kv_tensor_map(&map, kcache, head_dim, max_seq, behind / plane_bytes + planes, attn_stream_tile_keys()) != cudaSuccess) return FC_ERR_CUDA;
+  ShortAttnArgs a; memset(&a, 0, sizeof a);
+  a.qkv = qkv_acc; a.ldq = (n_heads + 2 * n_kv_heads) * head_dim; a.ss = sumsq; a.eps = rms_eps; a.dn = d_norm; a.rope = (const float2 *)(base + off[0]);
+  a.kcache = kcache; a.vcache = vcache; a.stride_h = (long long)max_seq * head_dim; a.stride_b = n_kv_heads * a.stride_h;
+  a.k_plane0 = 0; a.v_plane0 = (int)(behind / plane_bytes); a.kv_len = kv_len; a.c = c; a.hq = n_heads; a.hkv = n_kv_heads;
+  a.err = (unsigned int *)(base + off[1]); a.out_pan = out_pair; a.pan_rows = batch * c;
+  unsigned int herr = 0;
+  if (launch_attn_short(map, a, batch, max_len, head_dim, sms, st) != cudaSuccess ||
+      cudaMemcpyAsync(&herr, a.err, sizeof herr, cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return FC_ERR_CUDA;
   return herr ? FC_ERR_DEVICE_TIMEOUT : FC_OK;
 }
 

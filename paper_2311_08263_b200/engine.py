@@ -272,3 +272,22 @@ def fc_op_fused_window_attention(qkv_acc: torch.Tensor, sumsq: torch.Tensor, rms
     if rc != _l.FC_OK:
         raise FcError(rc, "fc_op_fused_window_attention")
     return out
+
+
+def fc_op_short_window_attention(qkv_acc: torch.Tensor, sumsq: torch.Tensor, rms_eps: float, d_norm: int, rope_theta: float,
+                                 kv: torch.Tensor, kv_len: torch.Tensor, c: int, n_heads: int, max_len: int) -> torch.Tensor:
+    """The attention kernel behind the one-writer projections as one operation.  kv: bf16 [2, B, hkv, max_seq, hd], keys and values;
+    receives the window's rows.  Returns fp32 [B*c, hq*hd], the sum of the bf16 pair that the kernel writes."""
+    lib = _l.load()
+    _, B, hkv, max_seq, hd = kv.shape
+    nbytes = lib.fc_op_fused_window_attention_scratch_bytes(B, c, n_heads, hkv, hd, max_seq, max_len)
+    if nbytes == 0:
+        raise FcError(_l.FC_ERR_ARG, "fc_op_fused_window_attention_scratch_bytes")
+    scratch = torch.empty(nbytes, dtype=torch.uint8, device=kv.device)
+    pair = torch.empty(2, B * c, n_heads * hd, dtype=torch.bfloat16, device=kv.device)
+    rc = lib.fc_op_short_window_attention(qkv_acc.data_ptr(), sumsq.data_ptr(), rms_eps, d_norm, rope_theta, kv[0].data_ptr(),
+                                          kv[1].data_ptr(), kv_len.data_ptr(), pair.data_ptr(), B, c, n_heads, hkv, hd, max_seq,
+                                          max_len, scratch.data_ptr(), nbytes, torch.cuda.current_stream().cuda_stream)
+    if rc != _l.FC_OK:
+        raise FcError(rc, "fc_op_short_window_attention")
+    return pair.float().sum(0)

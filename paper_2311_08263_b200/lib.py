@@ -28,7 +28,7 @@ EXPORTS = ["fc_kv_bytes", "fc_workspace_bytes", "fc_init", "fc_prefill", "fc_jac
            "fc_last_launch_count", "fc_last_route", "fc_destroy", "fc_strerror", "fc_last_cuda_error",
            "fc_op_linear", "fc_op_accept", "fc_op_window_attention",
            "fc_op_window_attention_scratch_bytes", "fc_op_window_attention_noalloc",
-           "fc_op_fused_window_attention", "fc_op_fused_window_attention_scratch_bytes"]
+           "fc_op_fused_window_attention", "fc_op_short_window_attention", "fc_op_fused_window_attention_scratch_bytes"]
 
 
 class fc_model_shape(C.Structure):
@@ -103,6 +103,8 @@ def load() -> C.CDLL:
     lib.fc_op_fused_window_attention_scratch_bytes.restype = C.c_size_t
     lib.fc_op_fused_window_attention_scratch_bytes.argtypes = [i32] * 7
     lib.fc_op_fused_window_attention.argtypes = [vp, vp, C.c_float, i32, C.c_float, vp, vp, vp, vp] + [i32] * 9 + \
+                                                [vp, C.c_size_t, vp]
+    lib.fc_op_short_window_attention.argtypes = [vp, vp, C.c_float, i32, C.c_float, vp, vp, vp, vp] + [i32] * 7 + \
                                                 [vp, C.c_size_t, vp]
     _lib = lib
     return lib

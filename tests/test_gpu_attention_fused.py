@@ -1,5 +1,6 @@
-"""Element-wise parity of the attention kernel that the bf16 step launches (fused 1/rms + rotary embedding + K/V
-write + split-KV window attention), through fc_op_fused_window_attention, against the CPU oracle's layer-0 trace.
+"""Element-wise parity of the attention kernels of the bf16 step that do everything in one launch (1/rms + rotary embedding + K/V write +
+split-KV window attention), against the CPU oracle's layer-0 trace: the one in front of the chained projections through
+fc_op_fused_window_attention, the one in front of the one-writer projections (up to 64 rows) through fc_op_short_window_attention.
 
 The oracle runs a one-layer model: prefill of L tokens, then a forward over a window with tracing, which gives the
 rotated queries, the attention output and the K/V cache (committed rows + the window's rows, rounded to bf16 where
@@ -81,22 +82,11 @@ CASES = [
 ]
 
 
-@pytest.mark.parametrize("hq,hkv,hd,c,lens,splits,q_tiles", CASES)
-def test_fused_window_attention_vs_oracle_trace(hq, hkv, hd, c, lens, splits, q_tiles):
-    cfg, acc, ss, kc, vc, max_seq, want_attn, want_k, want_v = _case(hq, hkv, hd, c, lens, seed=40 + c)
-    B = len(lens)
-    kcd = kc.to(torch.bfloat16).cuda().contiguous()
-    vcd = vc.to(torch.bfloat16).cuda().contiguous()
-    assert torch.equal(kcd.float().cpu(), kc)                   # the oracle's cached rows are bf16 values
-    accd, ssd = acc.cuda().contiguous(), ss.cuda().contiguous()
-    out = engine.fc_op_fused_window_attention(accd, ssd, cfg.rms_eps, cfg.d_model, cfg.rope_theta, kcd, vcd,
-                                              torch.tensor(lens, dtype=torch.int32).cuda(), c, hq, max(lens), splits, q_tiles)
-    out = out.cpu().numpy().reshape(B, c, hq * hd)
-    assert float(accd.abs().max()) == 0.0 and float(ssd.abs().max()) == 0.0      # consumed
+def _check(out, kcd, vcd, lens, c, kvd, vc, want_attn, want_k, want_v):
     for b, L in enumerate(lens):
         # the window's K/V rows as stored: within one bf16 step of the oracle's, nearly all identical
         for got_t, want in ((kcd, want_k[b]), (vcd, want_v[b])):
-            got = got_t[b, :, L:L + c].float().cpu().transpose(0, 1).reshape(c, hkv * hd).numpy()
+            got = got_t[b, :, L:L + c].float().cpu().transpose(0, 1).reshape(c, kvd).numpy()
             # one step of an 8-bit significand at most; elements that are small through cancellation carry the fp32
             # summation-order difference of their 256 terms instead (absolute, ~1e-6)
             step = np.maximum(np.abs(want) * 2.0 ** -7, 1e-5)
@@ -109,6 +99,21 @@ def test_fused_window_attention_vs_oracle_trace(hq, hkv, hd, c, lens, splits, q_
     # rows beyond the window stay untouched (zero) in the cache
     for b, L in enumerate(lens):
         assert float(kcd[b, :, L + c:].float().abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("hq,hkv,hd,c,lens,splits,q_tiles", CASES)
+def test_fused_window_attention_vs_oracle_trace(hq, hkv, hd, c, lens, splits, q_tiles):
+    cfg, acc, ss, kc, vc, max_seq, want_attn, want_k, want_v = _case(hq, hkv, hd, c, lens, seed=40 + c)
+    B = len(lens)
+    kcd = kc.to(torch.bfloat16).cuda().contiguous()
+    vcd = vc.to(torch.bfloat16).cuda().contiguous()
+    assert torch.equal(kcd.float().cpu(), kc)                   # the oracle's cached rows are bf16 values
+    accd, ssd = acc.cuda().contiguous(), ss.cuda().contiguous()
+    out = engine.fc_op_fused_window_attention(accd, ssd, cfg.rms_eps, cfg.d_model, cfg.rope_theta, kcd, vcd,
+                                              torch.tensor(lens, dtype=torch.int32).cuda(), c, hq, max(lens), splits, q_tiles)
+    out = out.cpu().numpy().reshape(B, c, hq * hd)
+    assert float(accd.abs().max()) == 0.0 and float(ssd.abs().max()) == 0.0      # consumed
+    _check(out, kcd, vcd, lens, c, hkv * hd, vc, want_attn, want_k, want_v)
 
 
 def test_fused_window_attention_rejects_bad_arguments():
@@ -127,3 +132,30 @@ def test_fused_window_attention_rejects_bad_arguments():
     assert l.fc_op_fused_window_attention(t.data_ptr(), t.data_ptr(), 1e-5, 8, 1e4, t.data_ptr(), t.data_ptr(),
                                           t.data_ptr(), t.data_ptr(), 1, 8, 4, 4, 64, 64, 60, 0, 0, t.data_ptr(), n,
                                           st) == lib.FC_ERR_CAPACITY
+
+
+SHORT_CASES = [
+    # hq, hkv, hd, c, lens                            units (sequence, kv head, 16 queries), key splits
+    (4, 4, 128, 16, [127, 128, 129, 0, 1, 31, 33]),   # 28; lengths around the 32-key tiles, empty cache, one key
+    (8, 2, 64, 5, [260, 1, 2047]),                    # 12: eight asked for, fewer run at once; odd window, splits without a tile
+    (4, 4, 128, 1, [77, 130, 2047]),                  # 12, c = 1
+    (8, 2, 64, 33, [300, 4000]),                      # 36, with two CTAs per SM; windows over three 16-key blocks
+    (4, 2, 128, 64, [513, 40]),                       # 32, a window of 64 rows
+    (32, 32, 128, 16, [1000]),                        # the benchmark's attention shape: 32 units, four splits
+    (12, 12, 128, 16, [1200, 64, 7, 600]),            # 48: five with two CTAs per SM
+    (16, 16, 64, 16, [70, 1, 130, 257, 64] * 2),      # 160: more units than SMs, no split
+]
+
+
+@pytest.mark.parametrize("hq,hkv,hd,c,lens", SHORT_CASES)
+def test_short_window_attention_vs_oracle_trace(hq, hkv, hd, c, lens):
+    cfg, acc, ss, kc, vc, max_seq, want_attn, want_k, want_v = _case(hq, hkv, hd, c, lens, seed=60 + c)
+    kv = torch.stack([kc, vc]).to(torch.bfloat16).cuda()
+    accd, ssd = acc.cuda().contiguous(), ss.cuda().contiguous()
+    out = engine.fc_op_short_window_attention(accd, ssd, cfg.rms_eps, cfg.d_model, cfg.rope_theta, kv,
+                                              torch.tensor(lens, dtype=torch.int32).cuda(), c, hq, max(lens))
+    out = out.cpu().numpy().reshape(len(lens), c, hq * hd)
+    # the pair carries 16 bits of the value: 2^-17 of it, far below the bounds
+    _check(out, kv[0], kv[1], lens, c, hkv * hd, vc, want_attn, want_k, want_v)
+    for b, L in enumerate(lens):
+        assert float(kv[1, b, :, L + c:].float().abs().max()) == 0.0
