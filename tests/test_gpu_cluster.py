@@ -27,6 +27,13 @@ CASES = [
     (24, 24, 128, 256, 512, 1040, 12, [1300, 64, 5, 900]),         # 96 units, no split
     (32, 4, 64, 256, 512, 1040, 16, [2500]),                       # head_dim 64, eight key splits
     (16, 16, 128, 256, 512, 1040, 1, [2300] + [31 + 61 * i for i in range(15)]),       # 256 units x 36 tiles: the streaming pair
+    (32, 4, 64, 256, 512, 1040, 16, [2200, 5, 64, 300]),           # head_dim 64: 128 units x 35 tiles, short
+    (32, 4, 64, 256, 512, 1040, 16, [2290, 5, 64, 300]),           # 128 x 37: the streaming pair
+    (40, 40, 128, 256, 512, 1040, 16, [2300, 5, 64, 300]),         # more units than SMs: 160 x 37, short
+    (40, 40, 128, 256, 512, 1040, 16, [2420, 5, 64, 300]),         # 160 x 39: the streaming pair
+    (20, 20, 128, 256, 512, 1040, 16, [900]),                      # 20 units: six key splits
+    (8, 4, 64, 256, 512, 1040, 64, [1300]),                        # 64 rows of one sequence, 32 units, ring halves
+    (12, 12, 128, 256, 512, 1040, 13, [1300, 64, 5, 900]),         # 48 units: five key splits of half the ring
     (32, 32, 128, 256, 512, 1040, 4, [1100, 0, 1, 31, 32, 33, 63, 64, 65, 95, 96, 97, 191, 192, 193, 1023]),     # 64 rows, 512 x 18: the same
 ]
 
@@ -37,7 +44,9 @@ def test_step_against_the_oracle_and_again(hq, hkv, hd, d, f, vocab, c, lens):
     dec, _ = _random_kv_case(cfg, lens, c, range(len(lens)))
     assert dec.fc_last_route() & _l.FC_ROUTE_MASK == _l.FC_ROUTE_ONE_WRITER
     units, tiles = len(lens) * hkv * ((hq // hkv * c + 15) // 16), (max(lens) + c + 63) // 64
-    assert dec.fc_last_launch_count() == (3 if units * tiles >= 8600 else 2) * cfg.n_layers + 4
+    stream = units * tiles >= (4600 if hd == 64 else 6000 if units > 148 else 8600)
+    assert dec.fc_last_route() & _l.FC_ATTN_MASK == (_l.FC_ATTN_STREAM if stream else _l.FC_ATTN_SHORT)
+    assert dec.fc_last_launch_count() == (3 if stream else 2) * cfg.n_layers + 4
     logits = dec.fc_debug_logits(True)
     pending = wl.make_random_window(cfg, len(lens), 1, salt=3).numpy()[:, 0]
     window = wl.make_random_window(cfg, len(lens), c, salt=4).numpy()

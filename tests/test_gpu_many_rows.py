@@ -132,6 +132,8 @@ COMPACTED = [
     ("dense", 8, 4, 64, 1024, 16, [60, 33, 70, 1, 64, 60, 20, 95, 31, 60, 47, 80]),              # 192 rows, then 144
     ("dense", 4, 4, 128, 1024, 40, [30, 33, 70, 2, 64, 30, 20, 95, 31, 30, 47, 80]),             # 480, then 360
     ("stream", 8, 8, 64, 1000, 2, [40, 33, 960, 1, 64, 40, 20, 95, 31, 40, 47, 500]),            # 72 units x 16 tiles of 64 keys
+    ("short", 4, 4, 128, 1008, 5, [40, 33, 300, 1, 64, 40, 20, 95, 31, 40, 47, 80]),             # 60 rows, then 45
+    ("one-writer-stream", 16, 16, 64, 1008, 5, [40, 29, 2140, 1, 64, 40, 20, 95, 31, 40, 47, 80]),     # 144 units x 34 tiles
 ]
 
 
@@ -159,7 +161,10 @@ def test_finished_sequences_leave_the_rows_of_the_many_row_routes(route, hq, hkv
     for b in range(B):
         assert out[b, :out_lens[b]].tolist() == first[b]
     cnt, tok, win = dec.fc_jacobi_step()
-    assert dec.fc_last_launch_count() == (8 if route == "dense" else 3) * cfg.n_layers + 4 + 1      # and the gather of the windows
+    assert dec.fc_last_launch_count() == {"dense": 8, "short": 2}.get(route, 3) * cfg.n_layers + 4 + 1      # and the gather of the windows
+    assert dec.fc_last_route() == {"dense": _l.FC_ROUTE_DENSE | _l.FC_ATTN_STREAM, "stream": _l.FC_ROUTE_CHAIN | _l.FC_ATTN_STREAM,
+                                   "short": _l.FC_ROUTE_ONE_WRITER | _l.FC_ATTN_SHORT,
+                                   "one-writer-stream": _l.FC_ROUTE_ONE_WRITER | _l.FC_ATTN_STREAM}[route]
     lg = logits[:(B - len(gone)) * c].cpu().numpy().reshape(B - len(gone), c, vocab)
     live = [b for b in range(B) if b not in gone]
     for i, b in enumerate(live):
@@ -195,8 +200,8 @@ def test_more_prompts_than_segments_of_a_block():
 
 
 def test_dense_and_chained_steps_after_a_reported_timeout():
-    """Dense step that reports a timeout, prompts again, then a chained step (64 rows) and a dense one (132 rows) over the same
-    buffers."""
+    """Dense step that reports a timeout, prompts again, then a one-writer step (64 rows), a chained one (96) and a dense one (132) over
+    the same buffers."""
     cfg = _cfg(8, 4, 64, seed=1400, prompt_len=60)
     B, c, lens = 4, 33, [60, 41, 3, 50]
     w = wl.make_weights(cfg)
@@ -213,10 +218,11 @@ def test_dense_and_chained_steps_after_a_reported_timeout():
     for b, P in enumerate(lens):
         orc.append(oracle.Oracle(cfg, w, 60 + 4 * c))
         orc[b].prefill(ids[b, :P], c)
-    for width, per_layer in ((16, 2), (c, 8)):
+    for width, per_layer, route in ((16, 2, _l.FC_ROUTE_ONE_WRITER), (24, 2, _l.FC_ROUTE_CHAIN), (c, 8, _l.FC_ROUTE_DENSE)):
         dec.fc_set_window(width)
         cnt, tok, win = dec.fc_jacobi_step()
         assert dec.fc_last_launch_count() == per_layer * cfg.n_layers + 4
+        assert dec.fc_last_route() & _l.FC_ROUTE_MASK == route
         lg = logits[:B * width].cpu().numpy().reshape(B, width, cfg.vocab)
         for b in range(B):
             orc[b].set_window(width)

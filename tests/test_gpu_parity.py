@@ -114,12 +114,13 @@ def _compare_stream_with_resync(cfg, w, dec, prompt, c, n_tokens, max_seq):
 @pytest.mark.parametrize("flags", [lib.FC_FLAG_SIMT_GEMM, 0, lib.FC_FLAG_NO_PDL | lib.FC_FLAG_NO_CHAIN,
                                    lib.FC_FLAG_NO_FFN_SPLIT],
                          ids=["fma", "tensor", "tensor-unchained", "tensor-ffn-unsplit"])
-@pytest.mark.parametrize("shape", ["gqa64", "mha128", "gqa32"])
+@pytest.mark.parametrize("shape", ["gqa64", "mha128", "gqa32", "gqa64-v1008", "mha128-v1008"])
 def test_small_bf16_logits_and_stream(flags, shape):
+    """Vocabulary 1000: up to 64 rows through the chained launch.  1008 (whole units of 16 rows): through the one-writer projections."""
     kw = {"gqa64": dict(n_heads=4, n_kv_heads=2, head_dim=64, d_model=256, d_ffn=512),
           "mha128": dict(n_heads=2, n_kv_heads=2, head_dim=128, d_model=256, d_ffn=640),
-          "gqa32": dict(n_heads=8, n_kv_heads=2, head_dim=32, d_model=320, d_ffn=328)}[shape]
-    cfg = wl.small_config(vocab=1000, n_layers=3, prompt_len=150, c=8, gen_tokens=24, **kw)
+          "gqa32": dict(n_heads=8, n_kv_heads=2, head_dim=32, d_model=320, d_ffn=328)}[shape.split("-")[0]]
+    cfg = wl.small_config(vocab=1008 if shape.endswith("v1008") else 1000, n_layers=3, prompt_len=150, c=8, gen_tokens=24, **kw)
     w, dec, max_seq = _setup(cfg, flags=flags)
     prompt = wl.make_prompts(cfg)[0][0].numpy()
     o = oracle.Oracle(cfg, w, max_seq)
@@ -130,6 +131,8 @@ def test_small_bf16_logits_and_stream(flags, shape):
         k, acc, wnew, lg = o.jacobi_step(want_logits=True)
         cnt, tok, wg = dec.fc_jacobi_step()
         got = logits[:cfg.c].cpu().numpy()
+        one_writer = shape.endswith("v1008") and not flags & (lib.FC_FLAG_SIMT_GEMM | lib.FC_FLAG_NO_CHAIN)
+        assert (dec.fc_last_route() & lib.FC_ROUTE_MASK == lib.FC_ROUTE_ONE_WRITER) == one_writer
         assert np.abs(got - lg).max() < LOGIT_TOL
         srt = np.sort(lg, axis=1)
         if (srt[:, -1] - srt[:, -2]).min() > MARGIN_TOL:
@@ -165,8 +168,9 @@ def test_bf16_window_sizes_one_and_sixteen(c):
     _compare_stream_with_resync(cfg, w, dec, prompt, c, cfg.gen_tokens, max_seq)
 
 
-def test_batch_ragged_prompts_independent_accepts():
-    cfg = wl.small_config(vocab=600, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256, d_ffn=512,
+@pytest.mark.parametrize("vocab,route", [(600, lib.FC_ROUTE_CHAIN), (608, lib.FC_ROUTE_ONE_WRITER)])
+def test_batch_ragged_prompts_independent_accepts(vocab, route):
+    cfg = wl.small_config(vocab=vocab, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256, d_ffn=512,
                           prompt_len=70, c=6, gen_tokens=20)
     B = 4
     lens = [70, 33, 1, 50]
@@ -176,6 +180,7 @@ def test_batch_ragged_prompts_independent_accepts():
     ids, lens_t = wl.make_prompts(cfg, batch=B, lens=lens)
     dec.fc_prefill(ids.numpy(), lens, cfg.c)
     toks, out_lens, st = dec.fc_generate(cfg.gen_tokens)
+    assert dec.fc_last_route() & lib.FC_ROUTE_MASK == route
     for b in range(B):
         o = oracle.Oracle(cfg, w, max_seq)
         ar, margins = o.ar_generate(ids[b, :lens[b]].numpy(), cfg.gen_tokens)
@@ -320,14 +325,14 @@ def test_injected_device_timeout_is_reported_and_prefill_recovers():
     assert dec.fc_debug_check_guards() == 0
 
 
-@pytest.mark.parametrize("which", ["tiny", "bf16-batch"])
+@pytest.mark.parametrize("which", ["tiny", "bf16-batch", "bf16-batch-one-writer"])
 def test_canary_bands_intact_after_prefill_steps_and_generate(which):
     """Canary bands around the K/V slab, around the workspace and between its slices must hold their pattern after
     every kind of call (the stand-in for an out-of-bounds checker); damaging one on purpose from the host is seen."""
     if which == "tiny":
         cfg, B, c = wl.CONFIGS["tiny"], 1, 8
     else:
-        cfg, B, c = wl.small_config(vocab=600, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256,
+        cfg, B, c = wl.small_config(vocab=608 if which.endswith("one-writer") else 600, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256,
                                     d_ffn=512, prompt_len=150, c=12, gen_tokens=20), 3, 12
     w = wl.make_weights(cfg)
     max_seq = 150 + 40 + c + 8
@@ -414,10 +419,11 @@ def test_finish_with_trigger_fp32_exact(n_trig, c):
     assert dec.fc_debug_check_guards() == 0
 
 
-def test_finish_with_trigger_bf16_batch_ragged_with_eos():
+@pytest.mark.parametrize("vocab,route", [(600, lib.FC_ROUTE_CHAIN), (608, lib.FC_ROUTE_ONE_WRITER)])
+def test_finish_with_trigger_bf16_batch_ragged_with_eos(vocab, route):
     """Three sequences of different lengths on the tensor-core path: each answer equals the oracle's, or leaves it
     only at a position whose margin in the oracle's greedy run over the same context is below the tolerance."""
-    cfg = wl.small_config(vocab=600, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256, d_ffn=512,
+    cfg = wl.small_config(vocab=vocab, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256, d_ffn=512,
                           prompt_len=70, c=6, gen_tokens=20)
     B, lens = 3, [70, 33, 5]
     w = wl.make_weights(cfg)
@@ -430,6 +436,7 @@ def test_finish_with_trigger_bf16_batch_ragged_with_eos():
     wins = dec.fc_jacobi_step()[2]            # the windows whose approximate tokens get handed over
     kl, ng = dec.fc_get_state()
     got, glens = dec.fc_finish_with_trigger(trigger, 12)
+    assert dec.fc_last_route() & lib.FC_ROUTE_MASK == route
     for b in range(B):
         o = oracle.Oracle(cfg, w, 200)
         ar, _ = o.ar_generate(ids[b, :lens[b]].numpy(), int(ng[b]))
@@ -509,10 +516,10 @@ def test_fp32_stream_exact_at_positions_in_the_thousands():
 @pytest.mark.parametrize("flags", [0, lib.FC_FLAG_NO_FFN_SPLIT], ids=["ffn-split", "ffn-unsplit"])
 def test_bf16_step_run_to_run_spread_is_bounded(flags):
     """Partial sums are added in L2 in whatever order they arrive, so two runs of the same step differ in the last
-    bits.  The spread of the logits over repeated runs must stay two orders of magnitude under the parity tolerance
+    bits (vocabulary 2008: no whole units of 16 rows, so the chained launch).  The spread of the logits over repeated runs must stay two orders of magnitude under the parity tolerance
     (a lost update or a read of a half-added residual would be far larger), with the feed-forward block run as two
     halves and as one."""
-    cfg = wl.small_config(vocab=2000, n_layers=8, n_heads=16, n_kv_heads=4, head_dim=64, d_model=1024, d_ffn=2816,
+    cfg = wl.small_config(vocab=2008, n_layers=8, n_heads=16, n_kv_heads=4, head_dim=64, d_model=1024, d_ffn=2816,
                           prompt_len=300, c=16, gen_tokens=8)
     w = wl.make_weights(cfg, device="cuda")
     prompt = wl.make_prompts(cfg)[0][0].numpy()
@@ -528,7 +535,38 @@ def test_bf16_step_run_to_run_spread_is_bounded(flags):
         if ref is None:
             ref = lg
         spread = max(spread, float((lg - ref).abs().max()))
+    assert dec.fc_last_route() & lib.FC_ROUTE_MASK == lib.FC_ROUTE_CHAIN
     assert spread < 3e-4, spread
+
+
+@pytest.mark.parametrize("flags", [0, lib.FC_FLAG_NO_FFN_SPLIT], ids=["ffn-split", "ffn-unsplit"])
+@pytest.mark.parametrize("c", [1, 8])
+def test_chained_steps_as_wide_as_13b_repeat_and_agree_with_the_oracle(c, flags):
+    """Two layers of the 13B shape, up to 8 rows: long enough phases for the feed-forward block in two halves, whose sums meet in the residual.
+    Twenty repeats within a small spread, the first against the oracle."""
+    import dataclasses
+    cfg = dataclasses.replace(wl.CONFIGS["13b"], n_layers=2, vocab=2048)
+    w = wl.make_weights(cfg, device="cuda")
+    ids = wl.make_prompts(cfg, batch=1, lens=[40])[0].numpy()[:, :40]
+    dec = engine.Decoder(cfg, w, 1, c, 64, flags=flags)
+    logits = dec.fc_debug_logits(True)
+    dec.fc_prefill(ids, [40], c)
+    wc = {k: [t.cpu() for t in v] if isinstance(v, list) else v.cpu() for k, v in w.items()}
+    o = oracle.Oracle(cfg, wc, 64)
+    o.prefill(ids[0], c)
+    _, _, _, lg = o.jacobi_step(want_logits=True)
+    o.close()
+    first, spread = None, 0.0
+    for _ in range(20):
+        dec.fc_bench_steps(1, commit=False)
+        torch.cuda.synchronize()
+        assert dec.fc_last_route() == lib.FC_ROUTE_CHAIN | lib.FC_ATTN_FUSED
+        got = logits[:c].clone()
+        first = got if first is None else first
+        spread = max(spread, float((got - first).abs().max()))
+    assert np.abs(first.cpu().numpy() - lg).max() < LOGIT_TOL
+    # sums in another order move logits by some 1e-5; a lost partial sum, or a read of a half-added residual, by 1e-2 and more
+    assert spread < 1e-3, spread
 
 
 @pytest.mark.parametrize("flags", [0, lib.FC_FLAG_NO_CTA_PAIRS], ids=["cta-pairs", "single-cta-tiles"])
@@ -565,7 +603,7 @@ def test_bf16_many_row_step_spread_and_agreement_of_the_two_tilings(flags):
         o.close()
 
 
-@pytest.mark.parametrize("kind", ["fp32", "bf16"])
+@pytest.mark.parametrize("kind", ["fp32", "bf16", "bf16-one-writer"])
 def test_finished_sequences_are_skipped_and_the_others_unaffected(kind):
     """A batch in which sequences finish at different times (one on an EOS early in its stream, the others at
     max_tokens): finished sequences no longer take rows of the forward - the step runs over the live ones only,
@@ -575,7 +613,7 @@ def test_finished_sequences_are_skipped_and_the_others_unaffected(kind):
         cfg = wl.CONFIGS["tiny"]
         c, n_gen = 4, 24
     else:
-        cfg = wl.small_config(vocab=600, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256, d_ffn=512,
+        cfg = wl.small_config(vocab=600 if kind == "bf16" else 608, n_layers=2, n_heads=4, n_kv_heads=2, head_dim=64, d_model=256, d_ffn=512,
                               prompt_len=70, c=6, gen_tokens=20)
         c, n_gen = cfg.c, cfg.gen_tokens
     B = 4
@@ -609,8 +647,9 @@ def test_finished_sequences_are_skipped_and_the_others_unaffected(kind):
                 assert len(got) == len(want[b])
     # steps after sequence 1 ended carry a gather launch and fewer attention CTAs; the count of launches per step is
     # the plain step's + 1 for those steps
-    per_step = (2 * cfg.n_layers + 4) if kind == "bf16" else None
+    per_step = (2 * cfg.n_layers + 4) if kind != "fp32" else None
     if per_step:
+        assert dec.fc_last_route() & lib.FC_ROUTE_MASK == (lib.FC_ROUTE_CHAIN if kind == "bf16" else lib.FC_ROUTE_ONE_WRITER)
         assert st.steps * per_step < dec.fc_last_launch_count() <= st.steps * (per_step + 1)
     cnt, _, _ = dec.fc_jacobi_step()
     assert cnt.tolist() == [0] * B
