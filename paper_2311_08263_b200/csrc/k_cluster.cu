@@ -578,7 +578,6 @@ __global__ void __launch_bounds__(kThreadsCl, 1) cluster_chain_kernel(const __gr
                 const uint32_t to = dst + (uint32_t)(b * kXBuf), bar = dbar + (uint32_t)b * 8u;
                 constexpr int N = H < 16 ? H : 16;
                 const float *v = &sum[t][BN > 16 ? (cb % (NCB / 2 > 0 ? NCB / 2 : 1)) * 16 : 0];
-#pragma unroll
                 sent += 1;
 #pragma unroll
                 for (int i = 0; i < N; i += 4) st_async_v4(to + (uint32_t)((BN > 16 ? 0 : half * H) + i) * 4u, bar, v[i], v[i + 1], v[i + 2], v[i + 3]);
