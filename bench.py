@@ -26,11 +26,11 @@ sys.path.insert(0, ROOT)
 import numpy as np  # noqa: E402
 import torch  # noqa: E402
 
-from paper_2311_08263_b200 import workload as wl  # noqa: E402
+from paper_2311_08263_b200 import lib, workload as wl  # noqa: E402
 
-# dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu capture
-# summarised under profiles/ (None until a capture of the current kernel exists)
-TRAFFIC_BYTES_PER_LAUNCH = {}
+# dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, by (workload, route of the projections), from the
+# ncu capture summarised in profiles/cluster_chain_7b_4layers.txt: steps of up to 16 rows
+TRAFFIC_BYTES_PER_LAUNCH = {("7b", lib.FC_ROUTE_ONE_WRITER): 411.3e6}
 
 METRIC = "accepted_tokens_per_s"
 UNIT = "tokens/s"
@@ -267,6 +267,7 @@ def run_ours(args, cfg, rank, world, local):
     # ---- per-kernel-class device times (events around every launch of one step)
     prof = dec.fc_profile_step()
     prof = dec.fc_profile_step()
+    route = dec.fc_last_route() & lib.FC_ROUTE_MASK
     kv_mid = [int((a + b) // 2) for a, b in zip(kv0, kv1)]
     sbytes = step_bytes(cfg, B, c, kv_mid)
     peak, peak_kind = measured_peaks()
@@ -279,7 +280,7 @@ def run_ours(args, cfg, rank, world, local):
     chain_ms, chain_n = prof.get("chain", (0.0, 0))
     if chain_n > 0:
         chain_bytes = s * (L * (d * qd + 3 * d * f) + (L - 1) * (qd + 2 * kvd) * d)
-        kname = ("cluster_chain_kernel" if B * c <= 64 else "gemm_umma_kernel<EPI_ATOMIC_ADD>") + " (chained O + gate/up + down + next-QKV projections)"
+        kname = ("cluster_chain_kernel" if route == lib.FC_ROUTE_ONE_WRITER else "gemm_umma_kernel<EPI_ATOMIC_ADD>") + " (chained O + gate/up + down + next-QKV projections)"
         k_ms, k_n, k_bytes = chain_ms, chain_n, chain_bytes / chain_n
     else:
         k_ms, k_n = prof["gateup"]
@@ -288,7 +289,7 @@ def run_ours(args, cfg, rank, world, local):
     achieved = k_bytes * k_n / (k_ms * 1e-3) / 1e9 if k_ms > 0 else 0.0
     roofline = {"bound": "hbm", "kernel": kname,
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "peak_kind": f"of {peak_kind}", "traffic": TRAFFIC_BYTES_PER_LAUNCH.get(cfg.name),
+                "peak_kind": f"of {peak_kind}", "traffic": TRAFFIC_BYTES_PER_LAUNCH.get((cfg.name, route)) if B * c <= 16 else None,
                 "bytes_per_launch": k_bytes, "ms_per_launch": k_ms / max(k_n, 1), "launches": k_n}
     step_ms = ms_max / steps
     step_gbs = sbytes / (step_ms * 1e-3) / 1e9
