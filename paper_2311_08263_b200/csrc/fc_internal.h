@@ -321,7 +321,7 @@ cudaError_t launch_advance(int32_t *kv_len, const RowSegs &segs, int nseg, cudaS
 
 // ---- up to 64 rows: chained projections with one writer per output (k_cluster.cu); d, qd, f multiples of 128, kvd and vocab of 16
 // The width the kernel is built for at most (64 activation rows high and low are one MMA operand of 128).  One step of 7B against the
-// chained launch it replaces: 1 row over 512 keys 2603 us, 2812; 16 over 803 2707, 3237; 2 x 16 3022, 4096; 4 x 16 over 2048 4763, 4893.
+// chained launch it replaces: 1 row over 512 keys 2612 us, 2803; 16 over 803 2718, 3235; 2 x 16 3024, 4079; 4 x 16 over 2048 4615, 4882.
 constexpr int kClusterRows = 64;
 constexpr int kClusterSlots = 160;                   // CTAs that the slots of the row sums of squares are laid out for
 struct ClusterModel {
