@@ -30,7 +30,7 @@ from paper_2311_08263_b200 import lib, workload as wl  # noqa: E402
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, by (workload, route of the projections), from the
 # ncu capture summarised in profiles/cluster_chain_7b_4layers.txt: steps of up to 16 rows
-TRAFFIC_BYTES_PER_LAUNCH = {("7b", lib.FC_ROUTE_ONE_WRITER): 411.3e6}
+TRAFFIC_BYTES_PER_LAUNCH = {("7b", lib.FC_ROUTE_ONE_WRITER): 407.5e6}
 
 METRIC = "accepted_tokens_per_s"
 UNIT = "tokens/s"
