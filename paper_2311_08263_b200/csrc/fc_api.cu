@@ -776,7 +776,9 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
     FC_CK(launch_advance(ctx->b.kv_len, segs, nb, ctx->st));
     return FC_OK;
   }
-  if (cluster_pays(ctx->plan_cl, R)) {
+  // in front of the chained launch: streaming or fused attention
+  const bool stream = with_head && ctx->fused_attn && attn_stream_pays(max_len_host, rows, s.n_heads, s.n_kv_heads, nb);
+  if (cluster_pays(ctx->plan_cl, R, max_len_host, !stream)) {
     int rc = forward_cluster(ctx, segs, nb, rows, tokens, with_head, max_len_host);
     if (rc != FC_OK) return rc;
     if (with_head) return run_accept(ctx, b0, nb, rows, seq_map, commit);
@@ -800,7 +802,6 @@ static int forward(fc_ctx *ctx, int b0, int nb, int rows, const int32_t *tokens,
   const long long stride_b = (long long)s.n_kv_heads * stride_h;
   const bool chained = ctx->chain;
   const bool o_panel = chained && ctx->fused_attn && R > 16 && ctx->d.pan_rows >= R;
-  const bool stream = with_head && ctx->fused_attn && attn_stream_pays(max_len_host, rows, s.n_heads, s.n_kv_heads, nb);
   ctx->route = (chained ? FC_ROUTE_CHAIN : FC_ROUTE_SEPARATE) | (stream ? FC_ATTN_STREAM : ctx->fused_attn ? FC_ATTN_FUSED : FC_ATTN_SPLIT);
   for (int l = 0; l < s.n_layers; ++l) {
     if (!chained || l == 0)

@@ -332,7 +332,8 @@ struct ClusterPlan;
 bool cluster_shape_ok(int d, int qd, int kvd, int f, int vocab);
 cudaError_t cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a, void *pan_h, ClusterPlan **out);
 void cluster_plan_destroy(ClusterPlan *p);
-bool cluster_pays(const ClusterPlan *pl, int R);     // against the chained launch; false without a plan
+// Against the chained launch; false without a plan.  fused: that launch would have the fused attention in front of it.
+bool cluster_pays(const ClusterPlan *pl, int R, int max_len, bool fused);
 struct ClusterArgs {
   int R;
   float *x, *qkv;                 // [R, d] residual, [R, qd + 2 kvd] (lacking 1/rms)

@@ -38,7 +38,8 @@ inline double stage_fill(const int (*shape)[2], int n, int clusters) {
   return bytes / room;
 }
 
-// Where the one-writer projections are faster than the chained launch, by how full their stages are, a layer's weight bytes and the rows.
+// Where the one-writer projections are faster than the chained launch, by how full their stages are, a layer's weight bytes, the rows and
+// (up to 16 rows) the cached keys.
 // Measured, a step, chained launch -> one writer, us (layer MB, fill; 1.1B, 7B whole, others 2 to 8 layers).  Full stages, up to 32 rows
 // always: 7B (405, .92) 1 row 2869 -> 2638, 40 rows 4564 -> 4383, 64 rows 4521 -> 4133; 1070 MB, .81: 1 row 649 -> 644, 16 728 -> 655; 1711, .92:
 // 678 -> 648, 770 -> 664.  From 33 rows the activations' loads grow with the stages: 625, .84: 40 rows 790 -> 791, 64 850 -> 812; 906, .82: 775 ->
@@ -47,11 +48,17 @@ inline double stage_fill(const int (*shape)[2], int n, int clusters) {
 // 576, 696 -> 640, 738 -> 919; 13B (634, .69): 553 -> 582, 8 rows 593 -> 587, 16 624 -> 593, 32 738 -> 658, 40 797 -> 942; 721, .72: 482 -> 499, 539 ->
 // 508, 629 -> 556, 662 -> 781.  Small layers, where the chained launch's latency counts: 1.1B (88, .47) 1 row 47 -> 43 a layer, 40 rows 83 -> 73;
 // 170, .62: 379 -> 398, 436 -> 406, 571 -> 427, 622 -> 589; 201, .73: 71 -> 60 a layer, 105 -> 98.
-inline bool one_writer_pays(double fill, long long layer_bytes, int rows) {
+// Where the chained launch would have the fused attention kernel in front of it (`fused`: few units), the short kernel's lead grows with the
+// cached keys.  Up to 16 rows, 1000 / 3000 / 5000 / 8000 keys, chained -> one writer, 4 layers: 402 MB, 1 row 426 -> 498, 508 -> 523, 559 -> 552, 623 -> 588,
+// 8 rows 452 -> 500, 532 -> 525, 584 -> 552, 649 -> 589, 16 rows 475 -> 505, 562 -> 530; 510 MB, 1 row 486 -> 537, 569 -> 556, 8 rows 521 -> 537, 608 -> 560;
+// 13B, 1 row 565 -> 591, 642 -> 616, 708 -> 645, 800 -> 681, 8 rows 607 -> 595, 688 -> 620.  The line is a plane through these crossings.
+inline bool one_writer_pays(double fill, long long layer_bytes, int rows, int cached, bool fused) {
   if (layer_bytes < 210000000 || (rows > 16 && rows <= 32)) return true;
   const bool full = fill >= 0.74;
-  if (rows <= 16) return full || (rows > 8 && layer_bytes >= 550000000);
-  return full && layer_bytes < 750000000;
+  if (rows > 16) return full && layer_bytes < 750000000;
+  if (full || (rows > 8 && layer_bytes >= 550000000)) return true;
+  const long long over = layer_bytes > 400000000 ? (layer_bytes - 400000000) / 100000 : 0;
+  return fused && cached >= 4000 - 150 * rows - over;
 }
 
 // Key splits of the short attention (the CTAs of a unit, one cluster): `units` units of (sequence, kv head, 16 queries), `tiles` key tiles

@@ -946,7 +946,9 @@ cudaError_t cluster_plan_create(const ClusterModel &m, void *pan_x, void *pan_a,
   return cudaSuccess;
 }
 void cluster_plan_destroy(ClusterPlan *p) { delete p; }
-bool cluster_pays(const ClusterPlan *pl, int R) { return pl && R <= kClusterRows && one_writer_pays(pl->fill, pl->layer_bytes, R); }
+bool cluster_pays(const ClusterPlan *pl, int R, int max_len, bool fused) {
+  return pl && R <= kClusterRows && one_writer_pays(pl->fill, pl->layer_bytes, R, max_len, fused);
+}
 
 cudaError_t launch_embed_pair(const int32_t *tokens, const void *emb, const void *gain, float *x, void *pan, float *ss, unsigned int *words, int n_words,
                               int R, int d, int pdl, cudaStream_t st) {

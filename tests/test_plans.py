@@ -34,9 +34,9 @@ int short_plan(int tiles, int units, int head_dim, const int *fit) {
   fc::short_plan(tiles, units, head_dim, 4, 148, [&](int s, bool d) { return (long long)fit[(d ? 9 : 0) + s]; }, splits, deep);
   return deep ? splits : -splits;
 }
-int one_writer_pays(int d, int qd, int kvd, int f, int rows) {
+int one_writer_pays(int d, int qd, int kvd, int f, int rows, int cached, int fused) {
   const int shape[7][2] = {{qd, d}, {kvd, d}, {kvd, d}, {d, qd}, {f, d}, {f, d}, {d, f}};
-  return fc::one_writer_pays(fc::stage_fill(shape, 7, 33), 2ll * d * (2ll * qd + 2ll * kvd + 3ll * f), rows);
+  return fc::one_writer_pays(fc::stage_fill(shape, 7, 33), 2ll * d * (2ll * qd + 2ll * kvd + 3ll * f), rows, cached, fused != 0);
 }
 int stream_splits(int tiles, int units, int spare, const int *fit) {
   return fc::stream_splits(tiles, units, spare != 0, [&](int s) { return fit[s]; });
@@ -148,7 +148,8 @@ def test_key_splits_of_the_measured_shapes(plan, head_dim, units, tiles, want):
 ])
 def test_route_of_the_measured_shapes(plan, shape, few, mid, many):
     for rows, want in ((1, few), (8, few), (9, mid), (16, mid), (17, 1), (32, 1), (33, many), (64, many)):
-        assert plan.one_writer_pays(*shape, rows) == want, rows
+        assert plan.one_writer_pays(*shape, rows, 100, 1) == want, rows
+        assert plan.one_writer_pays(*shape, rows, 8000, 0) == want, rows
 
 
 def test_streaming_splits_leave_a_spare_only_where_it_is_asked_for(plan):
@@ -161,3 +162,15 @@ def test_streaming_splits_leave_a_spare_only_where_it_is_asked_for(plan):
     for units in (32, 40, 64, 80, 96, 128, 160, 320):
         for tiles in (1, 2, 8, 26, 63, 126, 250):
             assert plan.stream_splits(tiles, units, 0, FIT) == plan.stream_splits(tiles, units, 1, FIT)
+
+
+@pytest.mark.parametrize("shape,rows,crossing", [
+    # cached keys where the two routes cost the same (measured between 1000, 3000, 5000 and 8000)
+    ((4352, 4352, 4352, 9600), 1, 4300), ((4352, 4352, 4352, 9600), 8, 2800), ((4352, 4352, 4352, 9600), 16, 2000),
+    ((4352, 4352, 4352, 11520), 1, 4000), ((4352, 4352, 4352, 11520), 8, 2400), ((4608, 4608, 4608, 12288), 1, 2600),
+    ((5120, 5120, 5120, 13824), 1, 2000), ((5120, 5120, 5120, 13824), 8, 600),
+])
+def test_long_caches_in_front_of_the_fused_attention_change_the_route(plan, shape, rows, crossing):
+    assert plan.one_writer_pays(*shape, rows, crossing + 800, 1) == 1
+    assert plan.one_writer_pays(*shape, rows, max(crossing - 800, 0), 1) == 0
+    assert plan.one_writer_pays(*shape, rows, 8000, 0) == 0
