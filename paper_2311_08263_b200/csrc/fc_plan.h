@@ -57,7 +57,8 @@ inline bool one_writer_pays(double fill, long long layer_bytes, int rows, int ca
   const bool full = fill >= 0.74;
   if (rows > 16) return full && layer_bytes < 750000000;
   if (full || (rows > 8 && layer_bytes >= 550000000)) return true;
-  const long long over = layer_bytes > 400000000 ? (layer_bytes - 400000000) / 100000 : 0;
+  long long over = layer_bytes > 400000000 ? (layer_bytes - 400000000) / 100000 : 0;
+  if (over > 2000) over = 2000;                    // 721 MB, .72: 1 row 1000 keys 492 -> 506, 3000 521 -> 524, 5000 552 -> 547
   return fused && cached >= 4000 - 150 * rows - over;
 }
 
